@@ -35,6 +35,11 @@ sys.path.insert(0, ROOT)
 
 FLOPS_PER_CAND_SAMPLE = 14          # conj product 6 + derotation 6 + accumulation 2
 CDFT_COMBINE_FLOPS = 30             # per candidate x super-chunk: 6-bin interpolation 22 + phase MAC 8
+# per candidate and snapshot of a surface looked up in delay-Doppler maps:
+# geometry (Eq. 3-10, two ranges and two range rates) about 60, six-bin
+# interpolation with its weights and |.|^2 about 40; the maps' own FFT work is
+# not counted
+MAP_LOOKUP_FLOPS = 100
 FP32_PROBE_ITERS = 50000           # ~50 ms per probe launch on a GB300
 METRIC = "candidate·sample correlations/s"
 UNIT = "cand·samples/s"
@@ -456,7 +461,25 @@ def run_dg(a, rank, world, local_rank):
     kernels = {}
     alu_peak = fp["tflops"]
     issued_per_step = None
-    if a.algo == "cdft":
+    # a surface from delay-Doppler maps (dg_map.cu) plans nothing on the device
+    maps = a.algo == "cdft" and kt["plan"][1] == 0
+    if maps:
+        flops_per_step = MAP_LOOKUP_FLOPS * G_rank * scene.k_steps
+        corr_ms = kt["contract"][0] + kt["combine"][0]
+        corr_launches = kt["contract"][1] + kt["combine"][1]
+        roof_kernel = "k_map_spec + k_map_corr + k_map_expand + k_map_lookup (FP32 CUDA cores)"
+        roof_basis = (f"{MAP_LOOKUP_FLOPS} flop per candidate x snapshot (geometry, six-bin interpolation); the "
+                      "maps' FFT work is not counted")
+        roof_bound, roof_peak, roof_unit = "alu", alu_peak, "TFLOP/s"
+        for name in ("contract", "combine"):
+            kernels[name] = {"ms_per_step": kt[name][0] / a.steps,
+                             "kernels": {"contract": "k_map_spec, k_map_corr, k_map_expand (the maps)",
+                                         "combine": "k_map_lookup (geometry and interpolation per candidate)"}[name]}
+        ach = flops_per_step * a.steps / (kt["combine"][0] / 1e3) / 1e12
+        kernels["combine"].update(bound="alu", achieved=ach, peak=alu_peak, unit="TFLOP/s", frac=ach / alu_peak,
+                                  basis=roof_basis)
+        dom = "combine"
+    elif a.algo == "cdft":
         # every kernel of the chunked-DFT path against its own roofline; the
         # dominant one is the headline
         # with the automatic choice every batch of this workload took the
@@ -537,7 +560,7 @@ def run_dg(a, rank, world, local_rank):
             "ms_per_step_synchronous_calls": sync_ms_per_step,
             "steps": a.steps, "warmup": a.warmup, "ms_per_step": 1e3 * dev_s / a.steps,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": CONTRACT_DTYPE[a.contract] if a.algo == "cdft" else "f32",
+            "dtype": CONTRACT_DTYPE[a.contract] if a.algo == "cdft" and not maps else "f32",
             "data": "synthetic",
             "config": {"workload": desc, "G": G_rank * world, "K": scene.k_steps, "N": scene.n_samples,
                        "fmt": scene.fmt, "delay": "integer", "algo": a.algo, "acc": "power",
@@ -573,7 +596,8 @@ def run_dg(a, rank, world, local_rank):
                          "achieved_basis": roof_basis + " / CUDA-event time of the launches",
                          **launch_fields(a, dom if a.algo == "cdft" else "corr", corr_launches, corr_s)},
             "kernel_ms_per_step": {n: v[0] / a.steps for n, v in kt.items() if v[1]},
-            "cdft_work": ({"lag_chunk_rows": bucket_chunks, "candidate_superchunks": cand_chunks}
+            "cdft_work": ({"lag_block_pairs": bucket_chunks, "candidate_lookups": cand_chunks} if maps else
+                          {"lag_chunk_rows": bucket_chunks, "candidate_superchunks": cand_chunks}
                           if a.algo == "cdft" else None),
             "kernels": kernels,
             "device": {"name": torch.cuda.get_device_name(dev), "sm_count": fp["sm_count"],
@@ -740,7 +764,9 @@ def run_batch(a, rank, world, local_rank):
     step_s = statistics.median(dev_ms) / 1e3
     # issued tensor flops: 512 x chunk per (lag, chunk) row of every context
     # algorithmic contraction flops: 512 x chunk per (lag, chunk) row of every context
-    flops = sum(512 * g.cdft_work()[0] * g.cdft_chunks()[1] for g in gs) if a.contract != "fp32" else 0
+    # (none where the surfaces come from delay-Doppler maps: no shared rounds)
+    flops = (sum(512 * g.cdft_work()[0] * g.cdft_chunks()[1] for g in gs)
+             if a.contract != "fp32" and batch.rounds() else 0)
     clocks = clk.summary()
     if rank == 0:
         line = {

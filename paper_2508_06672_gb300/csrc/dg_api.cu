@@ -62,11 +62,36 @@ struct CdftRun {  // one chunked-DFT surface, phase by phase (run_surface_cdft)
     std::vector<int> Ms;  // chunk of each batch of snapshots
 };
 
+struct GridRange {  // what a grid's nodes can take in one snapshot
+    double d_lo, d_hi;    // D (samples)
+    double nu_lo, nu_hi;  // FDOA (cycles per sample)
+};
+
+struct MapPlan {  // shapes of the delay-Doppler maps of the main grid (dg_map.cu)
+    uint64_t gen = 0;   // steps_gen it was made for (0: none)
+    bool ok = false;    // the grid and captures suit the maps
+    int logn = 0, Mb = 0, Cmax = 0, P = 0, Q = 0, LT = 0, ntile = 0, NLpad = 0, S = 0;
+    bool c64 = false;
+    int chunk_min = 0, chunk_max = 0;  // what dg_cdft_chunks reports
+    int64_t rows = 0;                  // (lag, block) pairs of one surface
+    double xnode[kMapMaxNodes] = {};
+};
+
+struct MapBufs {  // their device tables and scratch, grown on demand
+    MapSnap *snap = nullptr;
+    float2 *tw = nullptr, *F2 = nullptr, *U = nullptr, *X = nullptr, *phase = nullptr;
+    float *T = nullptr;
+    int *bad = nullptr;
+    size_t snap_cap = 0, tw_cap = 0, F2_cap = 0, U_cap = 0, X_cap = 0, phase_cap = 0, T_cap = 0, bad_cap = 0;
+    int tw_logn = 0, T_P = 0, T_Q = 0;  // what tw and T hold
+};
+
 struct CdftBufs {  // chunked-DFT scratch, grown on demand
     int *lr = nullptr;
     CdftLayout main_layout, loc_layout;
     std::vector<double> main_span;  // FDOA span estimates per snapshot (main grid)
     std::vector<double> main_lags;  // and lag-count estimates
+    std::vector<GridRange> main_range;  // and lag / FDOA bounds
     CdftRun main_run;               // the main surface's last run (its batches' arguments)
     int *layout = nullptr, *Mcs = nullptr;
     unsigned long long *work = nullptr;
@@ -153,6 +178,9 @@ struct dg_ctx {
     unsigned *err_h = nullptr;          // pinned mirror
     LocalGrid loc;
     CdftBufs cd;
+    MapPlan mp;
+    MapBufs mb;
+    bool last_map = false;  // the last CDFT surface came from the maps
     CoarseBufs co;
     int cd_chunk_min = 0, cd_chunk_max = 0;              // chunks it used
     // whole-step CUDA graph (dg_graph_*)
@@ -296,12 +324,31 @@ static std::atomic<unsigned> g_tc_wait_polls{0};
 
 dg_status run_surface_cdft(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *surf, void *out,
                            bool refine);
+static dg_status map_plan(dg_ctx *c);
+static dg_status run_surface_map(dg_ctx *c, void *out);
+
+// Surfaces whose candidates look their correlations up in delay-Doppler maps
+// (dg_map.cu) instead of the per-lag DFT rows of the contraction: the main
+// grid of a context that leaves the launch shape to the library (chunk 0,
+// DG_TILES_AUTO) with an arithmetic that is FP32 or claims its accuracy (the
+// split forms). The single 16-bit forms keep the tensor-core products the
+// caller asked for.
+static bool map_eligible(const dg_ctx *c)
+{
+    return c->opt.algo == DG_ALGO_CDFT && c->opt.chunk == 0 && c->opt.tiles == DG_TILES_AUTO &&
+           c->opt.contract != DG_CONTRACT_BF16 && c->opt.contract != DG_CONTRACT_FP16 && c->G >= kMapMinNodes;
+}
 
 dg_status run_surface(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *surf, void *out,
                       bool refine)
 {
+    dg_status st;
+    if (!refine && map_eligible(c)) {
+        if ((st = map_plan(c)) != DG_OK) return st;
+        if (c->mp.ok) return run_surface_map(c, out);
+    }
     if (c->opt.algo == DG_ALGO_CDFT) return run_surface_cdft(c, gd, xyz, G, surf, out, refine);
-    dg_status st = push_steps(c);
+    st = push_steps(c);
     if (st != DG_OK) return st;
     bool same_fmt = true;
     for (int k = 1; k < c->K; ++k) same_fmt &= c->steps[k].fmt == c->steps[0].fmt;
@@ -381,7 +428,7 @@ static int lag_slots(const dg_ephem &e, double fs, double diam)
     return (int)std::ceil(span) + 6;
 }
 
-// FP64 WGS-84 node position and Eq. 3-10 FDOA on the host (planning only).
+// FP64 WGS-84 node position on the host (planning only).
 static void host_node_ecef(const GridDev &g, double i, double j, double p[3])
 {
     const double e2 = kF * (2.0 - kF);
@@ -393,17 +440,6 @@ static void host_node_ecef(const GridDev &g, double i, double j, double p[3])
     p[0] = n * std::cos(lat) * std::cos(lon);
     p[1] = n * std::cos(lat) * std::sin(lon);
     p[2] = n * (1.0 - e2) * sl;
-}
-
-static double host_nu(const double p[3], const dg_ephem &e, double fs, double lambda)
-{
-    double f[2];
-    for (int r = 0; r < 2; ++r) {
-        const double *pp = r ? e.p2 : e.p1, *vv = r ? e.v2 : e.v1;
-        const double x = pp[0] - p[0], y = pp[1] - p[1], z = pp[2] - p[2];
-        f[r] = -(x * vv[0] + y * vv[1] + z * vv[2]) / (std::sqrt(x * x + y * y + z * z) * lambda);
-    }
-    return (f[1] - f[0]) / fs;
 }
 
 // Diameter bound of the shard: the largest distance between its corners and
@@ -428,9 +464,18 @@ static double grid_diameter(const GridDev &g)
 // corners, edges and interior; the FDOA field is smooth at these scales): up
 // to 65 x 65 nodes, fewer on small shards (at least 9 x 9, about one lattice
 // node per 8 grid nodes), the node positions computed once for all
-// snapshots.
+// snapshots. lags: the lattice's lag counts. range: bounds of D and the FDOA
+// that hold at every node of the shard: the lattice's extremes widened by the
+// fields' Lipschitz bounds times the largest distance h of a node from the
+// lattice (half a cell's diagonal). With unit vectors u_i to the receivers at
+// distances >= rho, |grad D| = |u_2 - u_1| fs / c <= (|p2 - p1| / rho) fs / c;
+// the gradient of u . v is (v - u (u . v)) / rho, whose change over the
+// receivers' separation is at most 3 |v| |p2 - p1| / rho^2, so |grad nu| <=
+// (|v2 - v1| / rho + 3 |v| |p2 - p1| / rho^2) / (lambda fs). An infinite range
+// marks a snapshot whose receivers come within a cell or each other's
+// distance of the nodes.
 static void fdoa_spans(const dg_ctx *c, const GridDev &g, std::vector<double> &span,
-                       std::vector<double> *lags = nullptr)
+                       std::vector<double> *lags = nullptr, std::vector<GridRange> *range = nullptr)
 {
     const int side = std::max(g.nrows, g.nlon);
     const int lattice = std::min(65, std::max(9, side / 8 + 1));
@@ -442,30 +487,63 @@ static void fdoa_spans(const dg_ctx *c, const GridDev &g, std::vector<double> &s
             const double j = nj > 1 ? (double)b * (g.nlon - 1) / (nj - 1) : 0.0;
             host_node_ecef(g, std::round(i), std::round(j), &p[3 * ((size_t)a * nj + b)]);
         }
+    double h = 0.0;  // half the longest cell diagonal, with 5 % for the curvature within a cell
+    if (range) {
+        auto dist2 = [&](size_t q, size_t r) {
+            const double *x = &p[3 * q], *y = &p[3 * r];
+            return (x[0] - y[0]) * (x[0] - y[0]) + (x[1] - y[1]) * (x[1] - y[1]) + (x[2] - y[2]) * (x[2] - y[2]);
+        };
+        double hi = 0.0, hj = 0.0;
+        for (int a = 0; a < ni; ++a)
+            for (int b = 0; b < nj; ++b) {
+                const size_t q = (size_t)a * nj + b;
+                if (a + 1 < ni) hi = std::max(hi, dist2(q, q + nj));
+                if (b + 1 < nj) hj = std::max(hj, dist2(q, q + 1));
+            }
+        h = 0.5 * 1.05 * std::sqrt(hi + hj);
+        range->assign(c->K, GridRange{});
+    }
     span.assign(c->K, 0.0);
     if (lags) lags->assign(c->K, 1.0);
     for (int k = 0; k < c->K; ++k) {
-        double lo = 1e300, hi = -1e300, dlo = 1e300, dhi = -1e300;
+        double lo = 1e300, hi = -1e300, dlo = 1e300, dhi = -1e300, rmin = 1e300;
         const dg_ephem &e = c->eph_host[k];
         for (size_t q = 0; q < (size_t)ni * nj; ++q) {
             const double *x = &p[3 * q];
-            const double nu = host_nu(x, e, c->fs, c->lambda);
+            double f[2], r[2];  // Eq. 6-8 and 4, 7
+            for (int t = 0; t < 2; ++t) {
+                const double *pp = t ? e.p2 : e.p1, *vv = t ? e.v2 : e.v1;
+                const double dx = pp[0] - x[0], dy = pp[1] - x[1], dz = pp[2] - x[2];
+                r[t] = std::sqrt(dx * dx + dy * dy + dz * dz);
+                f[t] = -(dx * vv[0] + dy * vv[1] + dz * vv[2]) / (r[t] * c->lambda);
+            }
+            const double nu = (f[1] - f[0]) / c->fs;
             lo = std::min(lo, nu);
             hi = std::max(hi, nu);
             if (lags) {  // Eq. 7 and 9: the lattice's lag range
-                double r[2];
-                for (int t = 0; t < 2; ++t) {
-                    const double *pp = t ? e.p2 : e.p1;
-                    r[t] = std::sqrt((pp[0] - x[0]) * (pp[0] - x[0]) + (pp[1] - x[1]) * (pp[1] - x[1]) +
-                                     (pp[2] - x[2]) * (pp[2] - x[2]));
-                }
                 const double D = (r[1] - r[0]) * c->fs / kC;
                 dlo = std::min(dlo, D);
                 dhi = std::max(dhi, D);
+                rmin = std::min(rmin, std::min(r[0], r[1]));
             }
         }
         span[k] = hi - lo;
         if (lags) (*lags)[k] = std::floor(dhi + 0.5) - std::floor(dlo + 0.5) + 1.0;
+        if (lags && range) {
+            auto norm = [](double x, double y, double z) { return std::sqrt(x * x + y * y + z * z); };
+            const double sep = norm(e.p2[0] - e.p1[0], e.p2[1] - e.p1[1], e.p2[2] - e.p1[2]);
+            const double dv = norm(e.v2[0] - e.v1[0], e.v2[1] - e.v1[1], e.v2[2] - e.v1[2]);
+            const double v = std::max(norm(e.v1[0], e.v1[1], e.v1[2]), norm(e.v2[0], e.v2[1], e.v2[2]));
+            const double rho = rmin - h - 0.5 * sep;  // also along the receivers' segment
+            GridRange &R = (*range)[k];
+            if (rho > 0.0) {
+                const double md = sep / rho * c->fs / kC * h;
+                const double mn = (dv / rho + 3.0 * v * sep / (rho * rho)) / (c->lambda * c->fs) * h;
+                R = GridRange{dlo - md, dhi + md, lo - mn, hi + mn};
+            } else {
+                R = GridRange{-1e300, 1e300, -1e300, 1e300};
+            }
+        }
     }
 }
 
@@ -499,21 +577,14 @@ static int auto_chunk(const dg_ctx *c, const std::vector<double> &span, const st
     return M;
 }
 
-// The batches of a surface and their bucket / combine-group bases: static for
-// a grid size G (the main grid and the refinement grid each keep one).
-static dg_status cdft_layout(dg_ctx *c, const GridDev &gd, int64_t G, CdftLayout &L)
+// The batches of snapshots of a surface of G nodes (same IQ format, scratch
+// within the context's target) and their bucket / combine-group bases.
+// Snapshots per batch: per-candidate arrays (16 B per candidate) and the
+// per-lag DFTs (lag slots x chunks x 512 B, chunks at the longest automatic
+// chunk unless one is fixed) within the scratch target.
+static dg_status cdft_batches(dg_ctx *c, int64_t G, double diam, CdftLayout &L, std::vector<int> &bb,
+                              std::vector<int> &gb)
 {
-    const double diam = grid_diameter(gd);
-    if (L.G == G && L.diam >= diam && !L.batches.empty()) return DG_OK;
-    int *old_bb = L.bbase, *old_gb = L.gbase;
-    L = CdftLayout{};
-    L.G = G;
-    L.diam = diam;
-    L.bbase = old_bb;
-    L.gbase = old_gb;
-    // snapshots per batch: per-candidate arrays (16 B per candidate) and the
-    // per-lag DFTs (lag slots x chunks x 512 B, chunks at the longest
-    // automatic chunk unless one is fixed) within the scratch target
     const double budget = (double)(c->opt.scratch_mib ? c->opt.scratch_mib : 12288) * 1048576.0;
     int64_t nmax = 1;
     int slots_max = 1;
@@ -525,7 +596,6 @@ static dg_status cdft_layout(dg_ctx *c, const GridDev &gd, int64_t G, CdftLayout
     const double per_snap = 16.0 * (double)G + (double)slots_max * (double)((nmax + m_est - 1) / m_est) * 512.0;
     int s_max = (int)std::max<int64_t>(1, std::min<int64_t>(c->K, (int64_t)(budget / per_snap)));
     if (c->opt.contract != DG_CONTRACT_FP32) s_max = std::min(s_max, kTcMaxSnapshots);
-    std::vector<int> bb, gb;
     for (int k0 = 0; k0 < c->K;) {
         int S = 1;  // same format, at most s_max snapshots
         while (k0 + S < c->K && S < s_max && c->steps[k0 + S].fmt == c->steps[k0].fmt) ++S;
@@ -549,6 +619,24 @@ static dg_status cdft_layout(dg_ctx *c, const GridDev &gd, int64_t G, CdftLayout
         L.groups_max = std::max<int64_t>(L.groups_max, ng);
         k0 += S;
     }
+    return DG_OK;
+}
+
+// The batches of a surface and their bucket / combine-group bases: static for
+// a grid size G (the main grid and the refinement grid each keep one).
+static dg_status cdft_layout(dg_ctx *c, const GridDev &gd, int64_t G, CdftLayout &L)
+{
+    const double diam = grid_diameter(gd);
+    if (L.G == G && L.diam >= diam && !L.batches.empty()) return DG_OK;
+    int *old_bb = L.bbase, *old_gb = L.gbase;
+    L = CdftLayout{};
+    L.G = G;
+    L.diam = diam;
+    L.bbase = old_bb;
+    L.gbase = old_gb;
+    std::vector<int> bb, gb;
+    dg_status bst = cdft_batches(c, G, diam, L, bb, gb);
+    if (bst != DG_OK) return bst;
     dg_status st;
     if ((st = grow(c, &L.bbase, bb.size())) != DG_OK) return st;
     if ((st = grow(c, &L.gbase, gb.size())) != DG_OK) return st;
@@ -619,7 +707,7 @@ static dg_status cdft_setup(dg_ctx *c, CdftRun &r)
     const bool mma = c->opt.contract != DG_CONTRACT_FP32;
     r.mma = mma;
     if (c->opt.chunk == 0 && (span.size() != (size_t)c->K || b.main_lags.size() != (size_t)c->K))
-        fdoa_spans(c, c->gd, span, &b.main_lags);
+        fdoa_spans(c, c->gd, span, &b.main_lags, &b.main_range);
     std::vector<int> &Ms = r.Ms;
     Ms.assign(L.batches.size(), 0);
     int M_max = 64, B_max = 1;
@@ -890,11 +978,253 @@ static dg_status cdft_finish(dg_ctx *c, const CdftRun &r)
     return DG_OK;
 }
 
+// ---------------------------------------------------------------------------
+// Delay-Doppler maps (dg_map.cu): the plan of a context's main grid, made on
+// the host from the grid, the ephemerides and the capture lengths only, and
+// the surface.
+// ---------------------------------------------------------------------------
+
+// Doppler nodes of a block of Mb samples over a band of half width w: the
+// Chebyshev interpolant of e^{j 2 pi nu m}, |nu| <= w, |m| <= Mb / 2, is off by
+// at most 4 (theta / 2)^P / P!, theta = pi w Mb (the tail of its Bessel
+// coefficients). 0 if more than kMapMaxNodes would be needed.
+static int map_nodes(double halfw, int Mb)
+{
+    const double x = 0.5 * kPi * halfw * Mb;
+    double term = 4.0;
+    for (int P = 1; P <= kMapMaxNodes; ++P) {
+        term *= x / P;
+        if (P >= 2 && P > x && term <= 2e-7) return P;
+    }
+    return 0;
+}
+
+// Shapes: the FFT length n = 2^logn, the lag tile LT and the block
+// Mb = n - LT + 1 that take the fewest SM cycles by a model of the kernels
+// (FFT butterflies at 0.35 of the FP32 rate, expansion at 0.5, a floor for the
+// chain of one CTA).
+static dg_status map_plan(dg_ctx *c)
+{
+    MapPlan &m = c->mp;
+    if (m.gen == c->steps_gen) return DG_OK;
+    m = MapPlan{};
+    CdftBufs &b = c->cd;
+    if (b.main_span.size() != (size_t)c->K || b.main_lags.size() != (size_t)c->K ||
+        b.main_range.size() != (size_t)c->K)
+        fdoa_spans(c, c->gd, b.main_span, &b.main_lags, &b.main_range);
+    const bool frac = c->opt.delay != DG_DELAY_INTEGER;
+    std::vector<MapSnap> snap((size_t)c->K);
+    int nmax = 1, nlmax = 1;
+    double Qd = 8.0;
+    m.gen = c->steps_gen;  // whatever the outcome, it holds until the shapes change
+    for (int k = 0; k < c->K; ++k) {
+        const GridRange &R = b.main_range[k];
+        if (c->steps[k].n > (1 << 24)) return DG_OK;
+        // 0.01 samples absorb the rounding of D; Lagrange4 reaches L - 1 .. L + 2
+        if (!(std::fabs(R.d_lo) < 4e6 && std::fabs(R.d_hi) < 4e6)) return DG_OK;
+        const int lo = (int)std::floor(R.d_lo - 0.51) - (frac ? 1 : 0), hi = (int)std::ceil(R.d_hi + 0.51) + (frac ? 2 : 0);
+        snap[k].L0 = lo;
+        snap[k].NL = hi - lo + 1;
+        nlmax = std::max(nlmax, snap[k].NL);
+        nmax = std::max(nmax, (int)c->steps[k].n);
+        const double w = (R.nu_hi - R.nu_lo) * (1.0 + 1e-5) + 1e-13;
+        if (!(w < 0.046)) return DG_OK;  // wider than the 64 bins of the contraction's shortest chunk take: refused there
+        Qd = std::max(Qd, 6.0 + std::ceil(w * (double)c->steps[k].n / kMapNDelta));
+        m.c64 |= c->steps[k].fmt == DG_IQ_C64;
+    }
+    if (Qd > 8192.0 || nlmax > 65536) return DG_OK;
+    m.Q = (int)Qd;
+    double halfw = 0.0;
+    for (int k = 0; k < c->K; ++k) {
+        MapSnap &s = snap[k];
+        const GridRange &R = b.main_range[k];
+        s.delta = ((R.nu_hi - R.nu_lo) * (1.0 + 1e-5) + 1e-13) / (m.Q - 6);
+        s.nu0 = 0.5 * (R.nu_lo + R.nu_hi) - 0.5 * (m.Q - 1) * s.delta;
+        s.nuc = 0.5 * (R.nu_lo + R.nu_hi);
+        s.halfw = 0.5 * (m.Q - 1) * s.delta;
+        s.nu0_hi = (float)s.nu0;
+        s.nu0_lo = (float)(s.nu0 - (double)s.nu0_hi);
+        s.inv_delta = (float)(1.0 / s.delta);
+        halfw = std::max(halfw, s.halfw);
+    }
+    double best = 1e300;
+    for (int logn = 10; logn <= 14; ++logn) {
+        const int n = 1 << logn;
+        for (int nt = 1; nt <= 64; ++nt) {
+            int LT = (nlmax + nt - 1) / nt;
+            LT = (LT + 31) / 32 * 32;
+            const int Mb = (n - LT) & ~1;
+            if (Mb < n / 8) continue;
+            const int P = map_nodes(halfw, Mb);
+            if (P == 0) continue;
+            double ffts = 0.0, exps = 0.0, cmax = 0.0;
+            for (int k = 0; k < c->K; ++k) {
+                const double C = std::ceil((double)c->steps[k].n / Mb);
+                ffts += C * std::ceil((double)snap[k].NL / LT) * (1 + 2 * P);
+                exps += (double)snap[k].NL * m.Q * C * (2 * P + 4);
+                cmax = std::max(cmax, C);
+            }
+            const double t_fft = ffts * n * logn * 5.0 / (128 * 0.35) / c->sm_count;
+            const double cost = std::max(t_fft, 3.0 * (4000.0 + 1.6 * n)) + exps / (128 * 0.5) / c->sm_count +
+                                cmax * P * 40.0;
+            if (cost < best) {
+                best = cost;
+                m.logn = logn;
+                m.Mb = Mb;
+                m.LT = LT;
+                m.P = P;
+            }
+            if (nt * 32 >= nlmax) break;
+        }
+    }
+    if (best == 1e300) return DG_OK;
+    m.ntile = (nlmax + m.LT - 1) / m.LT;
+    m.NLpad = (nlmax + 31) / 32 * 32;
+    m.Cmax = (nmax + m.Mb - 1) / m.Mb;
+    for (int k = 0; k < c->K; ++k) m.rows += (int64_t)snap[k].NL * ((c->steps[k].n + m.Mb - 1) / m.Mb);
+    // the chunk the contraction would take (dg_cdft_chunks), and its limit on the per-lag DFT buffer
+    {
+        CdftLayout L;
+        std::vector<int> bb, gb;
+        if (cdft_batches(c, c->G, grid_diameter(c->gd), L, bb, gb) != DG_OK) return DG_OK;
+        const bool tc = c->opt.contract != DG_CONTRACT_FP32;
+        m.chunk_min = INT_MAX;
+        int64_t B = 1;
+        for (const auto &t : L.batches) {
+            const int M = auto_chunk(c, b.main_span, b.main_lags, t.k0, t.S, tc);
+            m.chunk_min = std::min(m.chunk_min, M);
+            m.chunk_max = std::max(m.chunk_max, M);
+            for (int s = 0; s < t.S; ++s) B = std::max<int64_t>(B, (c->steps[t.k0 + s].n + M - 1) / M);
+        }
+        if ((double)L.nbt_max * (double)B * 512.0 > (double)((size_t)64 << 30)) return DG_OK;
+    }
+    const size_t n = (size_t)1 << m.logn;
+    const double per = 8.0 * ((double)m.ntile * m.Cmax * n + (double)m.Cmax * m.P * m.NLpad + (double)m.Q * m.NLpad +
+                              (double)m.Cmax * m.Q);
+    const double budget = (double)(c->opt.scratch_mib ? c->opt.scratch_mib : 12288) * 1048576.0;
+    m.S = (int)std::max(1.0, std::min((double)c->K, std::floor(budget / per)));
+    // device tables and scratch (never inside a captured graph: a graph is
+    // captured after one uncaptured call of the same shape)
+    MapBufs &d = c->mb;
+    dg_status st;
+    const size_t S = (size_t)m.S;
+    if ((st = ensure(c, (void **)&d.snap, &d.snap_cap, sizeof(MapSnap) * (size_t)c->K)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&d.tw, &d.tw_cap, sizeof(float2) * n)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&d.T, &d.T_cap, sizeof(float) * (size_t)m.P * m.Q)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&d.F2, &d.F2_cap, sizeof(float2) * S * m.ntile * m.Cmax * n)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&d.U, &d.U_cap, sizeof(float2) * S * m.Cmax * m.P * m.NLpad)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&d.X, &d.X_cap, sizeof(float2) * S * m.Q * m.NLpad)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&d.phase, &d.phase_cap, sizeof(float2) * S * m.Cmax * m.Q)) != DG_OK) return st;
+    if (m.c64 && (st = ensure(c, (void **)&d.bad, &d.bad_cap, sizeof(int) * 4 * S)) != DG_OK) return st;
+    if ((st = ensure_ephf(c)) != DG_OK) return st;
+    // pageable sources: staged before the calls return
+    CK(c, cudaMemcpyAsync(d.snap, snap.data(), sizeof(MapSnap) * snap.size(), cudaMemcpyHostToDevice, c->stream));
+    if (d.tw_logn != m.logn) {
+        CK(c, launch_map_twiddles(d.tw, m.logn, c->stream));
+        ++c->launches;
+        d.tw_logn = m.logn;
+    }
+    for (int p = 0; p < m.P; ++p) m.xnode[p] = std::cos(kPi * (p + 0.5) / m.P);
+    if (d.T_P != m.P || d.T_Q != m.Q) {
+        std::vector<float> T((size_t)m.P * m.Q);
+        for (int p = 0; p < m.P; ++p)
+            for (int q = 0; q < m.Q; ++q) {
+                const double x = -1.0 + 2.0 * q / (m.Q - 1);
+                double t = 1.0;
+                for (int r = 0; r < m.P; ++r)
+                    if (r != p) t *= (x - m.xnode[r]) / (m.xnode[p] - m.xnode[r]);
+                T[(size_t)p * m.Q + q] = (float)t;
+            }
+        CK(c, cudaMemcpyAsync(d.T, T.data(), sizeof(float) * T.size(), cudaMemcpyHostToDevice, c->stream));
+        d.T_P = m.P;
+        d.T_Q = m.Q;
+    }
+    m.ok = true;
+    return DG_OK;
+}
+
+static dg_status run_surface_map(dg_ctx *c, void *out)
+{
+    const MapPlan &m = c->mp;
+    MapBufs &d = c->mb;
+    dg_status st = push_steps(c);
+    if (st != DG_OK) return st;
+    c->cd_chunk_min = m.chunk_min;
+    c->cd_chunk_max = m.chunk_max;
+    c->last_map = true;
+    auto split = [](double v, float &h, float &l) {
+        h = (float)v;
+        l = (float)(v - (double)h);
+    };
+    for (int k0 = 0; k0 < c->K; k0 += m.S) {
+        MapArgs a{};
+        a.S = std::min(m.S, c->K - k0);
+        a.sd = c->steps_d + k0;
+        a.snap = d.snap + k0;
+        a.xyz = c->xyz;
+        a.eph = c->eph + 12 * (size_t)k0;
+        a.ephf = c->cd.ephf + 24 * (size_t)k0;
+        split(c->fs / kC, a.fsc_hi, a.fsc_lo);
+        split(1.0 / (c->lambda * c->fs), a.ilf_hi, a.ilf_lo);
+        a.fs = c->fs;
+        a.lambda = c->lambda;
+        a.G = c->G;
+        a.nrows = c->gd.nrows;
+        a.nlon = c->gd.nlon;
+        a.logn = m.logn;
+        a.Mb = m.Mb;
+        a.Cmax = m.Cmax;
+        a.P = m.P;
+        a.Q = m.Q;
+        a.LT = m.LT;
+        a.ntile = m.ntile;
+        a.NLpad = m.NLpad;
+        a.delay = c->opt.delay;
+        a.acc = c->opt.acc;
+        a.first = k0 == 0;
+        a.tw = d.tw;
+        a.T = d.T;
+        std::memcpy(a.xnode, m.xnode, sizeof a.xnode);
+        a.F2 = d.F2;
+        a.U = d.U;
+        a.X = d.X;
+        a.phase = d.phase;
+        a.bad = m.c64 ? d.bad : nullptr;
+        a.out = (float *)out;
+        a.err = c->err_d;
+        {
+            Timed t(c, DG_K_CDFT_CONTRACT);
+            int n = 1;
+            CK(c, launch_map_tables(a, c->stream, &n));
+            CK(c, launch_map_expand(a, c->stream));
+            t.done(n);
+        }
+        {
+            Timed t(c, DG_K_CDFT_COMBINE);
+            CK(c, launch_map_lookup(a, c->stream));
+            t.done(1);
+        }
+    }
+    CK(c, cudaMemcpyAsync(c->err_h, c->err_d, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+    return DG_OK;
+}
+
+// The per-snapshot surfaces [K][G] of a main surface (the maps need none).
+static dg_status ensure_surf(dg_ctx *c)
+{
+    if (map_eligible(c)) {
+        const dg_status st = map_plan(c);
+        if (st != DG_OK || c->mp.ok) return st;
+    }
+    const size_t esz = c->opt.prec == DG_PREC_FP64 ? 8 : 4;
+    return ensure(c, &c->surf, &c->surf_bytes, esz * (size_t)c->G * c->K);
+}
 
 dg_status run_surface_cdft(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *surf, void *out,
                            bool refine)
 {
     CdftRun r;
+    if (!refine) c->last_map = false;
     r.gd = gd;
     r.xyz = xyz;
     r.G = G;
@@ -1096,6 +1426,7 @@ dg_status dg_set_grid(dg_ctx *c, const dg_grid *grid)
     c->G = G;
     c->cd.main_span.clear();  // FDOA spans and lag counts of the old grid
     c->cd.main_lags.clear();
+    c->cd.main_range.clear();
     ++c->steps_gen;           // graphs and batches recorded on the old grid are stale
     {
         Timed t(c, DG_K_GRID);
@@ -1149,8 +1480,7 @@ dg_status dg_cost_surface(dg_ctx *c, void *out)
     if (!out) return fail(c, DG_EINVAL, "out is NULL");
     for (int k = 0; k < c->K; ++k)
         if (!c->steps[k].loaded) return fail(c, DG_ESTATE, "snapshot %d has not been loaded", k);
-    const size_t esz = c->opt.prec == DG_PREC_FP64 ? 8 : 4;
-    dg_status st = ensure(c, &c->surf, &c->surf_bytes, esz * (size_t)c->G * c->K);
+    dg_status st = ensure_surf(c);
     if (st != DG_OK) return st;
     return run_surface(c, c->gd, c->xyz, c->G, c->surf, out, false);
 }
@@ -1334,8 +1664,7 @@ static dg_status prepare_step(dg_ctx *c, int half)
 {
     for (int k = 0; k < c->K; ++k)
         if (!c->steps[k].loaded) return fail(c, DG_ESTATE, "snapshot %d has not been loaded", k);
-    const size_t esz = c->opt.prec == DG_PREC_FP64 ? 8 : 4;
-    dg_status st = ensure(c, &c->surf, &c->surf_bytes, esz * (size_t)c->G * c->K);
+    dg_status st = ensure_surf(c);
     if (st != DG_OK) return st;
     const int n = 2 * half + 1;
     const int64_t Gl = half > 0 ? (int64_t)n * n : 0;
@@ -1435,7 +1764,7 @@ static dg_status tc_rounds(dg_ctx *const *ctxs, int n, TcRounds &R, bool &ok)
     for (int i = 0; i < n; ++i) {
         dg_ctx *c = ctxs[i];
         if (c->opt.algo != DG_ALGO_CDFT || c->opt.contract == DG_CONTRACT_FP32 || c->opt.tiles == DG_TILES_HANKEL ||
-            c->opt.contract != contract || !c->cd.main_run.L)
+            c->opt.contract != contract || !c->cd.main_run.L || c->last_map)
             return DG_OK;
         for (int k = 0; k < c->K; ++k)
             if (c->steps[k].fmt != fmt) return DG_OK;
@@ -1984,7 +2313,10 @@ dg_status dg_cdft_work(const dg_ctx *c, int64_t *bucket_chunks, int64_t *candida
 {
     if (!c) return fail(nullptr, DG_EINVAL, "ctx is NULL");
     unsigned long long w[2] = {0, 0};
-    if (c->cd.work) {  // counted on the device by the plan: wait for the stream
+    if (c->last_map) {  // (lag, block) pairs correlated, candidates looked up
+        w[0] = (unsigned long long)c->mp.rows;
+        w[1] = (unsigned long long)c->G * c->K;
+    } else if (c->cd.work) {  // counted on the device by the plan: wait for the stream
         if (cudaMemcpyAsync(w, c->cd.work, sizeof w, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
             cudaStreamSynchronize(c->stream) != cudaSuccess)
             return fail(nullptr, DG_ECUDA, "reading the CDFT work counters failed");
@@ -2023,6 +2355,14 @@ dg_status dg_destroy(dg_ctx *c)
     fr(c->loc.cost);
     fr(c->cd.lr);
     fr(c->reg_res);
+    fr(c->mb.snap);
+    fr(c->mb.tw);
+    fr(c->mb.T);
+    fr(c->mb.F2);
+    fr(c->mb.U);
+    fr(c->mb.X);
+    fr(c->mb.phase);
+    fr(c->mb.bad);
     fr(c->co.lag);
     fr(c->co.nu);
     fr(c->co.lmm);
@@ -2243,7 +2583,7 @@ dg_status dg_search_regions(dg_ctx *c, const dg_grid *regions, int32_t n, void *
     dg_status st;
     for (int r = 0; r < n; ++r) {
         if ((st = dg_set_grid(c, &regions[r])) != DG_OK) return st;
-        if ((st = ensure(c, &c->surf, &c->surf_bytes, esz * (size_t)G * c->K)) != DG_OK) return st;
+        if ((st = ensure_surf(c)) != DG_OK) return st;
         if ((st = ensure(c, &c->amax_tmp, &c->amax_tmp_bytes, argmax_tmp_bytes(G))) != DG_OK) return st;
         void *cr = (char *)costs + esz * (size_t)G * r;
         if ((st = run_surface(c, c->gd, c->xyz, G, c->surf, cr, false)) != DG_OK) return st;

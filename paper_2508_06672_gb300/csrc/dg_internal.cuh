@@ -154,8 +154,8 @@ __device__ __forceinline__ dfl df_div_fast(dfl a, dfl b)
 // of a cancelling sum, an error of 1e-9 cycles per sample already shows at
 // 1e-4 in |C|^2. So the range rates r_i . v_i / rho_i and their difference
 // are double-float too, and nu is rounded to FP32 once, at the end.
-__device__ __forceinline__ void geometry_df(dfl x, dfl y, dfl z, const dfl *e, dfl fs_over_c, dfl inv_lam_fs,
-                                            dfl &D, float &nu)
+__device__ __forceinline__ void geometry_dfl(dfl x, dfl y, dfl z, const dfl *e, dfl fs_over_c, dfl inv_lam_fs,
+                                             dfl &D, dfl &nu)
 {
     const dfl r1x = df_sub_fast(e[0], x), r1y = df_sub_fast(e[1], y), r1z = df_sub_fast(e[2], z);
     const dfl r2x = df_sub_fast(e[6], x), r2y = df_sub_fast(e[7], y), r2z = df_sub_fast(e[8], z);
@@ -164,7 +164,13 @@ __device__ __forceinline__ void geometry_df(dfl x, dfl y, dfl z, const dfl *e, d
     D = df_mul(df_sub_fast(rho2, rho1), fs_over_c);
     const dfl q1 = df_div_fast(df_add_fast(df_add_fast(df_mul(r1x, e[3]), df_mul(r1y, e[4])), df_mul(r1z, e[5])), rho1);
     const dfl q2 = df_div_fast(df_add_fast(df_add_fast(df_mul(r2x, e[9]), df_mul(r2y, e[10])), df_mul(r2z, e[11])), rho2);
-    const dfl n = df_mul(df_sub_fast(q1, q2), inv_lam_fs);  // (f2 - f1) lambda / (lambda fs)
+    nu = df_mul(df_sub_fast(q1, q2), inv_lam_fs);  // (f2 - f1) lambda / (lambda fs)
+}
+__device__ __forceinline__ void geometry_df(dfl x, dfl y, dfl z, const dfl *e, dfl fs_over_c, dfl inv_lam_fs,
+                                            dfl &D, float &nu)
+{
+    dfl n;
+    geometry_dfl(x, y, z, e, fs_over_c, inv_lam_fs, D, n);
     nu = n.hi + n.lo;
 }
 
@@ -468,6 +474,53 @@ constexpr int kCdftRefineMaxChunk = 256;
 constexpr double kCdftMDelta = 5.0e-2;
 constexpr int kCdftBinPad = 2;                  // bins outside the FDOA range on each side
 constexpr int kCdftBinSpan = 63 - 2 * kCdftBinPad;  // bin steps across the FDOA range
+
+// ---------------------------------------------------------------------------
+// Delay-Doppler maps of the grid's own lags and FDOAs, looked up per
+// candidate (dg_map.cu): the chunked-DFT path of grids with many nodes.
+// ---------------------------------------------------------------------------
+constexpr int kMapMaxNodes = 24;  // Chebyshev Doppler nodes per block
+// Smallest grid that takes the maps. They are the faster side below it too
+// (surface of K = 4, N = 20000: 45^2 nodes 52 us against 167, 64^2 50 against
+// 132, 90^2 49 against 134); small grids keep the contraction because batches
+// of many small contexts share its launches (dg_batch_capture's rounds) and
+// the bounded waits behind DG_ETIMEOUT are its own.
+constexpr int64_t kMapMinNodes = 8192;
+// Bin spacing x samples of a table (cycles): its 6-point interpolation error
+// is at most 4.9e-3 (pi x this)^6 = 8.4e-7 of the coherent sum (the capture's
+// centre is the phase origin, so the derivative bound has N / 2).
+constexpr double kMapNDelta = 7.5e-2;
+struct MapSnap {                  // one snapshot's table
+    double nu0, delta;            // bins nu0 + q delta, q < Q (cycles per sample)
+    double nuc, halfw;            // the bins' centre and half width: nodes nuc + halfw xnode[p]
+    float nu0_hi, nu0_lo, inv_delta;
+    int L0, NL;                   // lags L0 .. L0 + NL - 1
+};
+struct MapArgs {
+    const StepDesc *sd;           // [S] captures
+    const MapSnap *snap;          // [S]
+    const double *xyz, *eph;      // [3][G] node ECEF, [S][12]
+    const float *ephf;            // [S][24]
+    float fsc_hi, fsc_lo, ilf_hi, ilf_lo;  // as in CdftBatch
+    double fs, lambda;
+    int64_t G;
+    int nrows, nlon;
+    int S, logn, Mb, Cmax;        // FFT points 2^logn; block of samples; most blocks of a snapshot
+    int P, Q;                     // Doppler nodes per block, bins
+    int LT, ntile, NLpad;         // lags per tile, tiles, lag stride (a multiple of 32)
+    int delay, acc, first;        // first: the sum starts here (else it continues out)
+    const float2 *tw;             // [2^logn] e^{-j 2 pi i / n}
+    const float *T;               // [P][Q] node polynomials at the bins
+    double xnode[kMapMaxNodes];   // Chebyshev nodes on [-1, 1]
+    float2 *F2, *U, *X, *phase;   // [S][ntile][Cmax][n], [S][Cmax][P][NLpad], [S][Q][NLpad], [S][Cmax][Q]
+    int *bad;                     // [S][4] first / last sample of y1, y2 that is not finite (NULL: no c64 capture)
+    float *out;                   // [G]
+    unsigned *err;
+};
+cudaError_t launch_map_twiddles(float2 *tw, int logn, cudaStream_t s);
+cudaError_t launch_map_tables(const MapArgs &a, cudaStream_t s, int *launches);
+cudaError_t launch_map_expand(const MapArgs &a, cudaStream_t s);
+cudaError_t launch_map_lookup(const MapArgs &a, cudaStream_t s);
 
 // Threshold detection (dg_detect.cu). cap: power of two <= kDetectCap candidates
 // (the sort keeps value + index of each in static shared memory, 32 KiB).

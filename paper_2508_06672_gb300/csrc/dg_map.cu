@@ -1,0 +1,594 @@
+// dg_map.cu -- Eq. 11 from delay-Doppler maps: the chunked-DFT evaluation
+// (DG_ALGO_CDFT) of a grid of many nodes with FP32 arithmetic.
+//
+// Every candidate c of snapshot k needs the cross-ambiguity function
+//     X(l, nu) = sum_n y1[n] conj(y2[n + l]) e^{j 2 pi nu (n - N/2)}
+// at its own integer lag l (Eq. 9) and FDOA nu (Eq. 10), up to the unit phase
+// e^{j pi nu N} that |.| removes. The grid's lags and FDOAs cover a narrow
+// rectangle, so X is tabulated once per snapshot on every lag of it and on Q
+// Doppler bins, and each candidate interpolates the table in Doppler.
+//
+//   spec    FFT (n points) of each y2 window of a block of Mb samples, and
+//           the block's phases e^{j 2 pi nu_q t_c} at the bins;
+//   corr    per (block c, Doppler node p): the block of y1 turned at nu_p,
+//           its FFT times the window's conjugate spectrum, and a second FFT:
+//           U[c][p][l] = sum_m y1[cMb + m] e^{j 2 pi nu_p (m - Mb/2)}
+//           conj(y2[cMb + m + l]) for all lags of a tile at once. Over one
+//           block X is smooth in nu (its phase turns by less than one
+//           or two cycles across the band), so P Chebyshev nodes nu_p fix it;
+//   expand  X[q][l] = sum_c e^{j 2 pi nu_q t_c} sum_p T_p(nu_q) U[c][p][l],
+//           T_p the nodes' Lagrange polynomials at the bins, t_c the block's
+//           centre relative to the capture's;
+//   lookup  per candidate, snapshots in order: geometry, six bins around its
+//           FDOA (Lagrange), |.|^2 or |.|, summed in a register.
+//
+// A correlation of n lags through two FFTs costs about 10 n log2 n flop where
+// the contraction of dg_cdft_mma.cu costs 512 flop per (lag, sample): the
+// 4001^2-node, 50-snapshot workload needs 0.1 TFLOP for its tables instead of
+// 18. The lookup gathers from tables stored lag-fastest: neighbouring nodes of
+// a grid row have neighbouring lags and nearly the same FDOA, so a warp's
+// loads fall into a few cache lines and nothing has to be sorted.
+//
+// FFT: the Stockham autosort form (Govindaraju et al., "High performance
+// discrete Fourier transforms on graphics processors", 2008): 16 points per
+// thread, radix-16 passes in registers with one shared-memory exchange
+// between passes (one pad element per 16 keeps the stride-16 stores of the
+// first exchange free of bank conflicts), the remaining radix last, so input
+// and output have the same distribution (element t + T e in thread t).
+#include "dg_internal.cuh"
+
+namespace dg {
+namespace {
+
+__device__ __forceinline__ float2 cmul(float2 a, float2 b)
+{
+    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+
+// e^{j 2 pi f x} for a frequency f = hi + lo (cycles per sample) and an
+// integer-valued x, |x| < 2^24.
+__device__ __forceinline__ float2 cis_df(float hi, float lo, float x)
+{
+    float s, c;
+    sincospif(2.0f * (frac_mul(hi, x) + lo * x), &s, &c);
+    return make_float2(c, s);
+}
+
+// Forward DFTs of 2, 4, 8 and 16 points in registers; output k of fft16 is
+// v[4 (k % 4) + k / 4], of fft8 v[2 (k % 4) + k / 4].
+__device__ __forceinline__ void fft2(float2 &a, float2 &b)
+{
+    const float2 t = a;
+    a = cadd(t, b);
+    b = csub(t, b);
+}
+__device__ __forceinline__ void fft4(float2 &a, float2 &b, float2 &c, float2 &d)
+{
+    const float2 s = cadd(a, c), t = csub(a, c), u = cadd(b, d), w = csub(b, d);
+    a = cadd(s, u);
+    b = make_float2(t.x + w.y, t.y - w.x);  // t - j w
+    c = csub(s, u);
+    d = make_float2(t.x - w.y, t.y + w.x);
+}
+constexpr float kC8 = 0.70710678118654752f, kC16 = 0.92387953251128674f, kS16 = 0.38268343236508977f;
+__device__ __forceinline__ float2 rot8(float2 a)  // times e^{-j pi / 4}
+{
+    return make_float2(kC8 * (a.x + a.y), kC8 * (a.y - a.x));
+}
+__device__ __forceinline__ float2 rotj(float2 a) { return make_float2(a.y, -a.x); }  // times -j
+
+__device__ __forceinline__ void fft16(float2 (&v)[16])
+{
+#pragma unroll
+    for (int a = 0; a < 4; ++a) fft4(v[a], v[a + 4], v[a + 8], v[a + 12]);
+    // v[a + 4 k] times e^{-j 2 pi a k / 16}
+    const float2 w1 = make_float2(kC16, -kS16), w3 = make_float2(kS16, -kC16);
+    v[5] = cmul(v[5], w1);
+    v[6] = rot8(v[6]);
+    v[7] = cmul(v[7], w3);
+    v[9] = rot8(v[9]);
+    v[10] = rotj(v[10]);
+    v[11] = rotj(rot8(v[11]));
+    v[13] = cmul(v[13], w3);
+    v[14] = rotj(rot8(v[14]));
+    v[15] = cmul(v[15], make_float2(-kC16, kS16));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) fft4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+}
+__device__ __forceinline__ constexpr int pos16(int k) { return 4 * (k & 3) + (k >> 2); }
+
+// The last pass of radix R < 16: 16 / R butterflies of elements i + r (16 / R).
+template <int R> __device__ __forceinline__ void fft_small(float2 (&v)[16])
+{
+    constexpr int S = 16 / R;
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+        if constexpr (R == 2) {
+            fft2(v[i], v[i + S]);
+        } else if constexpr (R == 4) {
+            fft4(v[i], v[i + S], v[i + 2 * S], v[i + 3 * S]);
+        } else {
+            float2 e0 = v[i], e1 = v[i + 2 * S], e2 = v[i + 4 * S], e3 = v[i + 6 * S];
+            float2 o0 = v[i + S], o1 = v[i + 3 * S], o2 = v[i + 5 * S], o3 = v[i + 7 * S];
+            fft4(e0, e1, e2, e3);
+            fft4(o0, o1, o2, o3);
+            o1 = rot8(o1);
+            o2 = rotj(o2);
+            o3 = rotj(rot8(o3));
+            v[i] = cadd(e0, o0);
+            v[i + S] = cadd(e1, o1);
+            v[i + 2 * S] = cadd(e2, o2);
+            v[i + 3 * S] = cadd(e3, o3);
+            v[i + 4 * S] = csub(e0, o0);
+            v[i + 5 * S] = csub(e1, o1);
+            v[i + 6 * S] = csub(e2, o2);
+            v[i + 7 * S] = csub(e3, o3);
+        }
+    }
+}
+
+__device__ __forceinline__ int pad16(int i) { return i + (i >> 4); }
+
+// v[e] times w^{e idx} of a radix-R butterfly, w = e^{-j 2 pi / n}: the
+// powers 1, 2, 4, 8 from the table, the others as one product each.
+template <int R, int STRIDE>
+__device__ __forceinline__ void twiddle(float2 *v, const float2 *__restrict__ tw, int idx)
+{
+    const float2 w1 = __ldg(tw + idx);
+    v[STRIDE] = cmul(v[STRIDE], w1);
+    if constexpr (R >= 4) {
+        const float2 w2 = __ldg(tw + 2 * idx), w3 = cmul(w1, w2);
+        v[2 * STRIDE] = cmul(v[2 * STRIDE], w2);
+        v[3 * STRIDE] = cmul(v[3 * STRIDE], w3);
+        if constexpr (R >= 8) {
+            const float2 w4 = __ldg(tw + 4 * idx);
+            v[4 * STRIDE] = cmul(v[4 * STRIDE], w4);
+            v[5 * STRIDE] = cmul(v[5 * STRIDE], cmul(w4, w1));
+            v[6 * STRIDE] = cmul(v[6 * STRIDE], cmul(w4, w2));
+            v[7 * STRIDE] = cmul(v[7 * STRIDE], cmul(w4, w3));
+            if constexpr (R >= 16) {
+                const float2 w8 = __ldg(tw + 8 * idx), w12 = cmul(w8, w4);
+                v[8] = cmul(v[8], w8);
+                v[9] = cmul(v[9], cmul(w8, w1));
+                v[10] = cmul(v[10], cmul(w8, w2));
+                v[11] = cmul(v[11], cmul(w8, w3));
+                v[12] = cmul(v[12], w12);
+                v[13] = cmul(v[13], cmul(w12, w1));
+                v[14] = cmul(v[14], cmul(w12, w2));
+                v[15] = cmul(v[15], cmul(w12, w3));
+            }
+        }
+    }
+}
+
+// n = 2^LOGN point forward DFT of the CTA's n / 16 threads, in place; s holds
+// pad16(n) elements. Enters and leaves with s free (a barrier before each use).
+template <int LOGN> __device__ __forceinline__ void fft_cta(float2 (&v)[16], float2 *s, const float2 *__restrict__ tw)
+{
+    constexpr int n = 1 << LOGN, T = n / 16, full = LOGN / 4, rest = LOGN % 4;
+    const int t = threadIdx.x;
+#pragma unroll
+    for (int p = 0; p < full; ++p) {
+        const int Ns = 1 << (4 * p);
+        if (p > 0) twiddle<16, 1>(v, tw, (t & (Ns - 1)) << (LOGN - 4 * p - 4));
+        fft16(v);
+        if (p + 1 < full || rest) {
+            const int d = ((t >> (4 * p)) << (4 * p + 4)) + (t & (Ns - 1));
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < 16; ++r) s[pad16(d + r * Ns)] = v[pos16(r)];
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] = s[pad16(t + e * T)];
+        } else {
+            float2 u[16];
+#pragma unroll
+            for (int r = 0; r < 16; ++r) u[r] = v[pos16(r)];
+#pragma unroll
+            for (int r = 0; r < 16; ++r) v[r] = u[r];
+        }
+    }
+    if constexpr (rest > 0) {
+        constexpr int R = 1 << rest, S = 16 / R;
+#pragma unroll
+        for (int i = 0; i < S; ++i) twiddle<R, S>(v + i, tw, t + i * T);  // Ns = n / R: index j
+        fft_small<R>(v);
+    }
+}
+
+// Sample i of a capture as FP32; a value that is not finite counts as zero
+// (only c64 captures can hold one; its lags are flagged apart).
+__device__ __forceinline__ float2 load_sample(const void *b, int fmt, int i)
+{
+    if (fmt == DG_IQ_CI16) return IQ<DG_IQ_CI16>::load(b, i);
+    if (fmt == DG_IQ_CI8) return IQ<DG_IQ_CI8>::load(b, i);
+    const float2 v = IQ<DG_IQ_C64>::load(b, i);
+    return isfinite(v.x) && isfinite(v.y) ? v : make_float2(0.f, 0.f);
+}
+
+}  // namespace
+
+__global__ void k_map_twiddles(float2 *tw, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float s, c;
+    sincospif(-2.0f * (float)i / (float)n, &s, &c);  // i / n is exact
+    tw[i] = make_float2(c, s);
+}
+
+// First and last sample of each capture that is not finite (c64 captures).
+__global__ void k_map_bad_init(int *bad, int S)
+{
+    for (int i = threadIdx.x; i < S; i += blockDim.x) {
+        bad[4 * i] = bad[4 * i + 2] = 0x7fffffff;
+        bad[4 * i + 1] = bad[4 * i + 3] = -1;
+    }
+}
+__global__ void __launch_bounds__(256) k_map_bad(MapArgs a)
+{
+    const int s = blockIdx.y, r = blockIdx.z;
+    const StepDesc sd = a.sd[s];
+    if (sd.fmt != DG_IQ_C64) return;
+    const float2 *y = reinterpret_cast<const float2 *>(r ? sd.y2 : sd.y1);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < sd.n; i += gridDim.x * blockDim.x) {
+        const float2 v = __ldg(y + i);
+        if (!(isfinite(v.x) && isfinite(v.y))) {
+            atomicMin(a.bad + 4 * s + 2 * r, i);
+            atomicMax(a.bad + 4 * s + 2 * r + 1, i);
+        }
+    }
+}
+
+template <int LOGN> __global__ void __launch_bounds__((1 << LOGN) / 16) k_map_spec(MapArgs a)
+{
+    constexpr int n = 1 << LOGN, T = n / 16;
+    extern __shared__ __align__(16) float2 sm[];
+    const int t = threadIdx.x, c = blockIdx.x, tile = blockIdx.y, s = blockIdx.z;
+    const StepDesc sd = a.sd[s];
+    const MapSnap ms = a.snap[s];
+    if ((int64_t)c * a.Mb >= sd.n || tile * a.LT >= ms.NL) return;
+    if (tile == 0) {  // the block's phases at the bins
+        const double tc = (double)((int64_t)c * a.Mb + a.Mb / 2 - sd.n / 2);
+        for (int q = t; q < a.Q; q += T) {
+            const double ph = (ms.nu0 + q * ms.delta) * tc;
+            float sn, cs;
+            sincospif((float)(2.0 * (ph - floor(ph))), &sn, &cs);
+            a.phase[((size_t)s * a.Cmax + c) * a.Q + q] = make_float2(cs, sn);
+        }
+    }
+    const int64_t i0 = (int64_t)c * a.Mb + ms.L0 + (int64_t)tile * a.LT;
+    float2 v[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        const int64_t i = i0 + t + T * e;
+        v[e] = i >= 0 && i < sd.n ? load_sample(sd.y2, sd.fmt, (int)i) : make_float2(0.f, 0.f);
+    }
+    fft_cta<LOGN>(v, sm, a.tw);
+    float2 *F = a.F2 + (((size_t)s * a.ntile + tile) * a.Cmax + c) * n + t;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) F[T * e] = v[e];
+}
+
+template <int LOGN>
+__global__ void __launch_bounds__((1 << LOGN) / 16, LOGN == 14 ? 1 : LOGN == 13 ? 2 : 768 * 16 / (1 << LOGN)) k_map_corr(MapArgs a)
+{
+    constexpr int n = 1 << LOGN, T = n / 16;
+    extern __shared__ __align__(16) float2 sm[];
+    __shared__ float2 s_step[16];
+    __shared__ float s_nu[2];
+    const int t = threadIdx.x, p = blockIdx.x % a.P, c = blockIdx.x / a.P, tile = blockIdx.y, s = blockIdx.z;
+    const StepDesc sd = a.sd[s];
+    const MapSnap ms = a.snap[s];
+    const int64_t n0 = (int64_t)c * a.Mb;
+    if (n0 >= sd.n || tile * a.LT >= ms.NL) return;
+    // the node's frequency and the phasors of the thread's samples,
+    // e^{j 2 pi nu_p (t - Mb/2)} e^{j 2 pi nu_p T e}
+    if (t == 0) {
+        const double nup = ms.nuc + ms.halfw * a.xnode[p];
+        s_nu[0] = (float)nup;
+        s_nu[1] = (float)(nup - (double)s_nu[0]);
+    }
+    __syncthreads();
+    const float nh = s_nu[0], nl = s_nu[1];
+    if (t < 16) s_step[t] = cis_df(nh, nl, (float)(T * t));
+    const float2 base = cis_df(nh, nl, (float)(t - a.Mb / 2));
+    __syncthreads();
+    const int len = (int)min((int64_t)a.Mb, sd.n - n0);
+    float2 v[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        const int m = t + T * e;
+        v[e] = m < len ? load_sample(sd.y1, sd.fmt, (int)(n0 + m)) : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = cmul(v[e], cmul(base, s_step[e]));
+    const float2 *F = a.F2 + (((size_t)s * a.ntile + tile) * a.Cmax + c) * n + t;
+    constexpr float inv = 1.0f / (float)n;
+    // both transforms through one copy of the code: inlined twice, the
+    // compiler keeps the first one's twiddles in registers for the second
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        fft_cta<LOGN>(v, sm, a.tw);
+        if (pass == 0) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                const float2 f = __ldg(F + T * e);
+                v[e] = make_float2(fmaf(v[e].x, f.x, v[e].y * f.y) * inv, fmaf(v[e].y, f.x, -v[e].x * f.y) * inv);
+            }
+        }
+    }
+    float2 *U = a.U + (((size_t)s * a.Cmax + c) * a.P + p) * a.NLpad;
+    const int l0 = tile * a.LT, nl_t = min(a.LT, ms.NL - l0);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        const int l = t + T * e;
+        if (l < nl_t) U[l0 + l] = v[e];
+    }
+}
+
+// X[q][l]: a warp takes 32 lags and kExpQ bins; 8 warps share the lags (their
+// U loads hit L1) and take 8 kExpQ consecutive bins.
+constexpr int kExpQ = 8;
+constexpr int kExpWarps = 8;
+constexpr int kExpBins = kExpQ * kExpWarps;
+
+__global__ void __launch_bounds__(32 * kExpWarps) k_map_expand(MapArgs a)
+{
+    __shared__ __align__(16) float sT[kMapMaxNodes][kExpBins];
+    const int s = blockIdx.z, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const StepDesc sd = a.sd[s];
+    const MapSnap ms = a.snap[s];
+    const int qb = blockIdx.y * kExpBins, P = a.P;
+    if (blockIdx.x * 32 >= ms.NL) return;
+    for (int i = threadIdx.x; i < P * kExpBins; i += 32 * kExpWarps) {
+        const int q = qb + i % kExpBins;
+        sT[i / kExpBins][i % kExpBins] = q < a.Q ? __ldg(a.T + (i / kExpBins) * a.Q + q) : 0.f;
+    }
+    __syncthreads();
+    const int q0 = qb + kExpQ * warp;
+    if (q0 >= a.Q) return;
+    const int l = blockIdx.x * 32 + lane;
+    const int C = (sd.n + a.Mb - 1) / a.Mb;
+    const float2 *U = a.U + (size_t)s * a.Cmax * P * a.NLpad + l;
+    const float2 *E = a.phase + (size_t)s * a.Cmax * a.Q;
+    float2 x[kExpQ];
+#pragma unroll
+    for (int i = 0; i < kExpQ; ++i) x[i] = make_float2(0.f, 0.f);
+    for (int c = 0; c < C; ++c) {
+        float2 y[kExpQ];
+#pragma unroll
+        for (int i = 0; i < kExpQ; ++i) y[i] = make_float2(0.f, 0.f);
+#pragma unroll 4
+        for (int p = 0; p < P; ++p) {
+            const float2 u = U[((size_t)c * P + p) * a.NLpad];
+            const float4 ta = *reinterpret_cast<const float4 *>(&sT[p][kExpQ * warp]);
+            const float4 tb = *reinterpret_cast<const float4 *>(&sT[p][kExpQ * warp + 4]);
+            const float w[kExpQ] = {ta.x, ta.y, ta.z, ta.w, tb.x, tb.y, tb.z, tb.w};
+#pragma unroll
+            for (int i = 0; i < kExpQ; ++i) {
+                y[i].x = fmaf(w[i], u.x, y[i].x);
+                y[i].y = fmaf(w[i], u.y, y[i].y);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kExpQ; ++i) {
+            const float2 e = __ldg(E + (size_t)c * a.Q + min(q0 + i, a.Q - 1));
+            x[i].x = fmaf(e.x, y[i].x, fmaf(-e.y, y[i].y, x[i].x));
+            x[i].y = fmaf(e.x, y[i].y, fmaf(e.y, y[i].x, x[i].y));
+        }
+    }
+    if (l >= ms.NL) return;
+    const int L = ms.L0 + l;
+    const bool none = L >= sd.n || L <= -sd.n;  // no overlap: exactly zero
+#pragma unroll
+    for (int i = 0; i < kExpQ; ++i)
+        if (q0 + i < a.Q)
+            a.X[((size_t)s * a.Q + q0 + i) * a.NLpad + l] = none ? make_float2(0.f, 0.f) : x[i];
+}
+
+// Whether lag L's overlap touches a sample that is not finite: n runs over
+// [max(0, -L), min(N, N - L)), y2's index over [max(0, L), min(N, N + L)).
+__device__ __forceinline__ bool lag_bad(int4 b, int L, int N)
+{
+    if (L >= N || L <= -N) return false;
+    return L >= 0 ? (b.x < N - L || b.w >= L) : (b.y >= -L || b.z < N + L);
+}
+
+// One candidate and snapshot: |C|^2 or |C|.
+template <bool FRAC>
+__device__ __forceinline__ float map_value(const MapArgs &a, const MapSnap &ms, int s, int L, float mu, float u)
+{
+    // 6-point Lagrange interpolation on bins q0 - 2 .. q0 + 3 (see the
+    // combine of dg_cdft.cu); the host pads the bins so that q0 is inside
+    const int q0 = max(2, min(a.Q - 4, __float2int_rd(u)));
+    const float t = u - (float)q0;
+    const float a2 = t + 2.f, a1 = t + 1.f, b1 = t - 1.f, b2 = t - 2.f, b3 = t - 3.f;
+    const float t01 = t * b1, t23 = b2 * b3, s21 = a2 * a1;
+    const float w[6] = {-(a1 * t01 * t23) * (1.f / 120.f), (a2 * t01 * t23) * (1.f / 24.f),
+                        -(s21 * b1 * t23) * (1.f / 12.f),  (s21 * t * t23) * (1.f / 12.f),
+                        -(s21 * t01 * b3) * (1.f / 24.f),  (s21 * t01 * b2) * (1.f / 120.f)};
+    const int l = max(FRAC ? 1 : 0, min(ms.NL - (FRAC ? 3 : 1), L - ms.L0));
+    const float2 *X = a.X + ((size_t)s * a.Q + q0 - 2) * a.NLpad + l;
+    float cx = 0.f, cy = 0.f;
+    if (!FRAC) {
+#pragma unroll
+        for (int e = 0; e < 6; ++e) {
+            const float2 v = __ldg(X + (size_t)e * a.NLpad);
+            cx = fmaf(w[e], v.x, cx);
+            cy = fmaf(w[e], v.y, cy);
+        }
+    } else {
+        const float lw[4] = {-mu * (mu - 1.f) * (mu - 2.f) * (1.f / 6.f), (mu + 1.f) * (mu - 1.f) * (mu - 2.f) * 0.5f,
+                             -(mu + 1.f) * mu * (mu - 2.f) * 0.5f, (mu + 1.f) * mu * (mu - 1.f) * (1.f / 6.f)};
+#pragma unroll
+        for (int e = 0; e < 6; ++e) {
+            const float2 *R = X + (size_t)e * a.NLpad;
+            float zx = 0.f, zy = 0.f;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const float2 v = __ldg(R + m - 1);
+                zx = fmaf(lw[m], v.x, zx);
+                zy = fmaf(lw[m], v.y, zy);
+            }
+            cx = fmaf(w[e], zx, cx);
+            cy = fmaf(w[e], zy, cy);
+        }
+    }
+    if (a.bad) {
+        const int4 b = __ldg(reinterpret_cast<const int4 *>(a.bad) + s);
+        const int N = a.sd[s].n;
+        bool bad = lag_bad(b, L, N);
+        if (FRAC) bad |= lag_bad(b, L - 1, N) || lag_bad(b, L + 1, N) || lag_bad(b, L + 2, N);
+        if (bad) return __int_as_float(0x7fc00000);
+    }
+    const float pw = fmaf(cx, cx, cy * cy);
+    return a.acc == DG_ACC_POWER ? pw : sqrtf(pw);
+}
+
+// Lag, fractional delay and bin coordinate of one node in one snapshot, from
+// the double-float geometry (the lag by the FP64 expression where D lies
+// within 1e-6 of a rounding boundary); false when |D| is out of range.
+template <bool FRAC>
+__device__ __forceinline__ bool map_node(const MapArgs &a, const MapSnap &ms, int s, int64_t p, const dfl (&xyz)[3],
+                                         int &L, float &mu, float &u)
+{
+    dfl ed[12], D, nu;
+#pragma unroll
+    for (int t = 0; t < 12; ++t) ed[t] = {__ldg(a.ephf + 24 * (size_t)s + 2 * t), __ldg(a.ephf + 24 * (size_t)s + 2 * t + 1)};
+    geometry_dfl(xyz[0], xyz[1], xyz[2], ed, {a.fsc_hi, a.fsc_lo}, {a.ilf_hi, a.ilf_lo}, D, nu);
+    u = ((nu.hi - ms.nu0_hi) + (nu.lo - ms.nu0_lo)) * ms.inv_delta;
+    mu = 0.f;
+    if (!(fabsf(D.hi) < 1.0e9f)) return false;
+    if (FRAC ? floor_df(D, L, mu) : round_df(D, L)) return true;
+    double e[12], D64, nu64;
+    for (int t = 0; t < 12; ++t) e[t] = a.eph[12 * (size_t)s + t];
+    geometry(a.xyz[p], a.xyz[a.G + p], a.xyz[2 * a.G + p], e, a.fs, a.lambda, D64, nu64);
+    if (!(fabs(D64) < 1.0e9)) return false;
+    L = lag_of(D64, FRAC ? DG_DELAY_LAGRANGE4 : DG_DELAY_INTEGER);
+    mu = (float)(D64 - (double)L);
+    return true;
+}
+
+// One thread per node (32 consecutive nodes of a grid row per warp); WK warps
+// of a CTA share the nodes and split the snapshots, 8 / WK take their own
+// rows. WK = 8 serves small grids, which would leave the chip idle otherwise:
+// the partial values meet in shared memory and are added in snapshot order.
+template <bool FRAC, int WK> __global__ void __launch_bounds__(256) k_map_lookup(MapArgs a)
+{
+    constexpr int WN = 8 / WK;
+    __shared__ float s_val[WK > 1 ? WK : 1][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tiles_j = (a.nlon + 31) / 32;
+    const int tj = blockIdx.x % tiles_j, ti = blockIdx.x / tiles_j;
+    const int i = ti * WN + (WK > 1 ? warp / WK : warp), j = tj * 32 + lane;
+    const int wk = WK > 1 ? warp % WK : 0;
+    const bool ok = i < a.nrows && j < a.nlon;
+    const int64_t p = (int64_t)min(i, a.nrows - 1) * a.nlon + min(j, a.nlon - 1);
+    dfl xyz[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) xyz[d] = df_from(a.xyz[d * a.G + p]);
+    float sum = a.first ? 0.f : a.out[p];
+    bool any = !a.first;
+    for (int k = 0; k < a.S; k += WK) {
+        const int s = k + wk;
+        float v = 0.f;
+        if (s < a.S) {
+            const MapSnap ms = a.snap[s];
+            int L;
+            float mu, u;
+            if (map_node<FRAC>(a, ms, s, p, xyz, L, mu, u)) v = map_value<FRAC>(a, ms, s, L, mu, u);
+            else if (ok) atomicOr(a.err, ERR_LAG_RANGE);
+        }
+        if (WK == 1) {
+            sum = any ? sum + v : v;
+            any = true;
+        } else {
+            s_val[wk][lane] = v;
+            __syncthreads();
+            if (wk == 0)
+                for (int w = 0; w < WK && k + w < a.S; ++w) {
+                    sum = any ? sum + s_val[w][lane] : s_val[w][lane];
+                    any = true;
+                }
+            __syncthreads();
+        }
+    }
+    if (ok && wk == 0) a.out[p] = sum;
+}
+
+// ---------------------------------------------------------------------------
+// launchers
+// ---------------------------------------------------------------------------
+template <int LOGN> static cudaError_t launch_tables(const MapArgs &a, cudaStream_t st)
+{
+    constexpr int n = 1 << LOGN;
+    const size_t smem = sizeof(float2) * (size_t)(n + n / 16);
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(k_map_spec<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_map_corr<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    const dim3 gs((unsigned)a.Cmax, (unsigned)a.ntile, (unsigned)a.S);
+    k_map_spec<LOGN><<<gs, n / 16, smem, st>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const dim3 gc((unsigned)(a.Cmax * a.P), (unsigned)a.ntile, (unsigned)a.S);
+    k_map_corr<LOGN><<<gc, n / 16, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_map_twiddles(float2 *tw, int logn, cudaStream_t st)
+{
+    const int n = 1 << logn;
+    k_map_twiddles<<<(n + 255) / 256, 256, 0, st>>>(tw, n);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_map_tables(const MapArgs &a, cudaStream_t st, int *launches)
+{
+    cudaError_t e = cudaSuccess;
+    if (a.bad) {
+        k_map_bad_init<<<1, 256, 0, st>>>(a.bad, a.S);
+        k_map_bad<<<dim3(16, (unsigned)a.S, 2), 256, 0, st>>>(a);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        *launches += 2;
+    }
+    switch (a.logn) {
+    case 10: e = launch_tables<10>(a, st); break;
+    case 11: e = launch_tables<11>(a, st); break;
+    case 12: e = launch_tables<12>(a, st); break;
+    case 13: e = launch_tables<13>(a, st); break;
+    case 14: e = launch_tables<14>(a, st); break;
+    default: return cudaErrorInvalidValue;
+    }
+    *launches += 2;
+    return e;
+}
+
+cudaError_t launch_map_expand(const MapArgs &a, cudaStream_t st)
+{
+    const dim3 ge((unsigned)(a.NLpad / 32), (unsigned)((a.Q + kExpBins - 1) / kExpBins), (unsigned)a.S);
+    k_map_expand<<<ge, 32 * kExpWarps, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_map_lookup(const MapArgs &a, cudaStream_t st)
+{
+    const int64_t tiles_j = (a.nlon + 31) / 32;
+    const bool frac = a.delay != DG_DELAY_INTEGER;
+    // under about four CTAs per SM of one-row warps, the warps split the snapshots
+    const bool split = tiles_j * ((a.nrows + 7) / 8) < 152 * 4;
+    const int64_t blocks = tiles_j * (split ? a.nrows : (a.nrows + 7) / 8);
+    if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
+    const unsigned g = (unsigned)blocks;
+    if (split) {
+        if (frac) k_map_lookup<true, 8><<<g, 256, 0, st>>>(a);
+        else k_map_lookup<false, 8><<<g, 256, 0, st>>>(a);
+    } else {
+        if (frac) k_map_lookup<true, 1><<<g, 256, 0, st>>>(a);
+        else k_map_lookup<false, 1><<<g, 256, 0, st>>>(a);
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace dg
