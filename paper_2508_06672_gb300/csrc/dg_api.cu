@@ -65,6 +65,8 @@ struct CdftRun {  // one chunked-DFT surface, phase by phase (run_surface_cdft)
 struct GridRange {  // what a grid's nodes can take in one snapshot
     double d_lo, d_hi;    // D (samples)
     double nu_lo, nu_hi;  // FDOA (cycles per sample)
+    double rho, sep, vel; // least range (0: none), receivers' separation and speed
+    double row_m, col_m;  // longest step between neighbouring rows and columns
 };
 
 struct MapPlan {  // shapes of the delay-Doppler maps of the main grid (dg_map.cu)
@@ -75,12 +77,15 @@ struct MapPlan {  // shapes of the delay-Doppler maps of the main grid (dg_map.c
     int chunk_min = 0, chunk_max = 0;  // what dg_cdft_chunks reports
     int64_t rows = 0;                  // (lag, block) pairs of one surface
     double xnode[kMapMaxNodes] = {};
+    PolyShape poly{};
 };
 
 struct MapBufs {  // their device tables and scratch, grown on demand
     MapSnap *snap = nullptr;
     float2 *tw = nullptr, *F2 = nullptr, *U = nullptr, *X = nullptr, *phase = nullptr;
-    float *T = nullptr;
+    float *T = nullptr, *fit = nullptr, *coef = nullptr;
+    int fit_rows = 0;  // tile shape fit is for
+    size_t fit_cap = 0, coef_cap = 0;
     int *bad = nullptr;
     size_t snap_cap = 0, tw_cap = 0, F2_cap = 0, U_cap = 0, X_cap = 0, phase_cap = 0, T_cap = 0, bad_cap = 0;
     int tw_logn = 0, T_P = 0, T_Q = 0;  // what tw and T hold
@@ -501,7 +506,10 @@ static void fdoa_spans(const dg_ctx *c, const GridDev &g, std::vector<double> &s
                 if (b + 1 < nj) hj = std::max(hj, dist2(q, q + 1));
             }
         h = 0.5 * 1.05 * std::sqrt(hi + hj);
-        range->assign(c->K, GridRange{});
+        GridRange R0{};  // the steps, with 2 % for their change within a cell
+        R0.row_m = ni > 1 ? 1.02 * std::sqrt(hi) / std::floor((double)(g.nrows - 1) / (ni - 1)) : 0.0;
+        R0.col_m = nj > 1 ? 1.02 * std::sqrt(hj) / std::floor((double)(g.nlon - 1) / (nj - 1)) : 0.0;
+        range->assign(c->K, R0);
     }
     span.assign(c->K, 0.0);
     if (lags) lags->assign(c->K, 1.0);
@@ -539,10 +547,17 @@ static void fdoa_spans(const dg_ctx *c, const GridDev &g, std::vector<double> &s
             if (rho > 0.0) {
                 const double md = sep / rho * c->fs / kC * h;
                 const double mn = (dv / rho + 3.0 * v * sep / (rho * rho)) / (c->lambda * c->fs) * h;
-                R = GridRange{dlo - md, dhi + md, lo - mn, hi + mn};
+                R.d_lo = dlo - md;
+                R.d_hi = dhi + md;
+                R.nu_lo = lo - mn;
+                R.nu_hi = hi + mn;
+                R.rho = rho;
             } else {
-                R = GridRange{-1e300, 1e300, -1e300, 1e300};
+                R.d_lo = R.nu_lo = -1e300;
+                R.d_hi = R.nu_hi = 1e300;
             }
+            R.sep = sep;
+            R.vel = v;
         }
     }
 }
@@ -999,6 +1014,89 @@ static int map_nodes(double halfw, int Mb)
     return 0;
 }
 
+// Polynomial geometry (k_map_poly): the sample nodes of a tile of `rows`
+// rows, and the least-squares matrix [kPolyTerms][kPolyPts] from their values
+// to the coefficients of x^e y^b, e + b <= 5, of the offsets normalised to
+// [-1, 1] (x rows, y columns).
+static PolyShape poly_shape(int rows)
+{
+    static const int at64[6] = {1, 9, 23, 40, 54, 62}, at32[6] = {0, 4, 11, 20, 27, 31};
+    PolyShape s{};
+    s.rows = rows;
+    int n = 0;
+    for (int i = 0; i < 6; ++i)
+        for (int j = 0; j < 6; ++j) {
+            if ((i == 0 || i == 5) && (j == 0 || j == 5)) continue;
+            s.pr[n] = (rows == 64 ? at64 : at32)[i];
+            s.pc[n++] = at32[j];
+        }
+    return s;
+}
+
+static std::vector<float> poly_fit(const PolyShape &s)
+{
+    double A[kPolyPts][kPolyTerms], N[kPolyTerms][kPolyTerms + kPolyPts];
+    for (int i = 0; i < kPolyPts; ++i) {
+        const double x = (s.pr[i] - 0.5 * (s.rows - 1)) / (0.5 * (s.rows - 1));
+        const double y = (s.pc[i] - 0.5 * (kPolyCols - 1)) / (0.5 * (kPolyCols - 1));
+        int t = 0;
+        for (int e = 0; e < 6; ++e)
+            for (int b = 0; b + e < 6; ++b) A[i][t++] = std::pow(x, e) * std::pow(y, b);
+    }
+    for (int t = 0; t < kPolyTerms; ++t) {
+        for (int u = 0; u < kPolyTerms; ++u) {
+            N[t][u] = 0.0;
+            for (int i = 0; i < kPolyPts; ++i) N[t][u] += A[i][t] * A[i][u];
+        }
+        for (int i = 0; i < kPolyPts; ++i) N[t][kPolyTerms + i] = A[i][t];
+    }
+    // normal equations N X = A^T by Gauss-Jordan elimination with pivoting
+    for (int t = 0; t < kPolyTerms; ++t) {
+        int piv = t;
+        for (int u = t + 1; u < kPolyTerms; ++u)
+            if (std::fabs(N[u][t]) > std::fabs(N[piv][t])) piv = u;
+        for (int k = 0; k < kPolyTerms + kPolyPts; ++k) std::swap(N[t][k], N[piv][k]);
+        const double d = 1.0 / N[t][t];
+        for (int k = 0; k < kPolyTerms + kPolyPts; ++k) N[t][k] *= d;
+        for (int u = 0; u < kPolyTerms; ++u) {
+            if (u == t) continue;
+            const double f = N[u][t];
+            for (int k = 0; k < kPolyTerms + kPolyPts; ++k) N[u][k] -= f * N[t][k];
+        }
+    }
+    std::vector<float> fit((size_t)kPolyTerms * kPolyPts);
+    for (int t = 0; t < kPolyTerms; ++t)
+        for (int i = 0; i < kPolyPts; ++i) fit[(size_t)t * kPolyPts + i] = (float)N[t][kPolyTerms + i];
+    return fit;
+}
+
+// Tile rows of the polynomial geometry, or 0 (geometry per node): the grid
+// must fill the chip with tiles, its slopes stay under 8 samples per node
+// (exact linear part), and the bound on the first dropped terms, with a factor
+// 4 for the fit and 2^5 for the Chebyshev-like samples, under 2e-6 samples and
+// bins (1e-7 samples with the fractional delay, which uses D's fraction).
+static int poly_rows(const dg_ctx *c, const std::vector<MapSnap> &snap)
+{
+    const bool frac = c->opt.delay != DG_DELAY_INTEGER;
+    const int64_t tj = (c->gd.nlon + kPolyCols - 1) / kPolyCols;
+    for (int rows : {64, 32}) {
+        if (c->gd.nrows < rows || c->gd.nlon < kPolyCols) continue;
+        if (tj * ((c->gd.nrows + rows - 1) / rows) < (int64_t)c->sm_count * (rows == 64 ? 8 : 2)) continue;
+        bool ok = true;
+        for (int k = 0; k < c->K && ok; ++k) {
+            const GridRange &R = c->cd.main_range[k];
+            const double B = R.sep * c->fs / kC;
+            const double h = std::hypot(0.5 * rows * R.row_m, 0.5 * kPolyCols * R.col_m) / R.rho;
+            const double h6 = h * h * h * h * h * h;
+            const double u = R.vel * R.sep / (R.rho * c->lambda * c->fs * snap[k].delta);
+            ok = B / R.rho * std::max(R.row_m, R.col_m) < 8.0 && B * 6.0 * h6 / 8.0 < (frac ? 1e-7 : 2e-6) &&
+                 u * 36.0 * h6 / 8.0 < 2e-6;
+        }
+        if (ok) return rows;
+    }
+    return 0;
+}
+
 // Shapes: the FFT length n = 2^logn, the lag tile LT and the block
 // Mb = n - LT + 1 that take the fewest SM cycles by a model of the kernels
 // (FFT butterflies at 0.35 of the FP32 rate, expansion at 0.5, a floor for the
@@ -1045,6 +1143,7 @@ static dg_status map_plan(dg_ctx *c)
         s.nu0_hi = (float)s.nu0;
         s.nu0_lo = (float)(s.nu0 - (double)s.nu0_hi);
         s.inv_delta = (float)(1.0 / s.delta);
+        s.inv_delta_lo = (float)(1.0 / s.delta - (double)s.inv_delta);
         halfw = std::max(halfw, s.halfw);
     }
     double best = 1e300;
@@ -1099,8 +1198,11 @@ static dg_status map_plan(dg_ctx *c)
         if ((double)L.nbt_max * (double)B * 512.0 > (double)((size_t)64 << 30)) return DG_OK;
     }
     const size_t n = (size_t)1 << m.logn;
+    const int pr = poly_rows(c, snap);
+    if (pr) m.poly = poly_shape(pr);
+    const double ptiles = pr ? std::ceil((double)c->gd.nrows / pr) * std::ceil((double)c->gd.nlon / kPolyCols) : 0.0;
     const double per = 8.0 * ((double)m.ntile * m.Cmax * n + (double)m.Cmax * m.P * m.NLpad + (double)m.Q * m.NLpad +
-                              (double)m.Cmax * m.Q);
+                              (double)m.Cmax * m.Q) + 4.0 * kPolyStride * ptiles;
     const double budget = (double)(c->opt.scratch_mib ? c->opt.scratch_mib : 12288) * 1048576.0;
     m.S = (int)std::max(1.0, std::min((double)c->K, std::floor(budget / per)));
     // device tables and scratch (never inside a captured graph: a graph is
@@ -1116,6 +1218,17 @@ static dg_status map_plan(dg_ctx *c)
     if ((st = ensure(c, (void **)&d.X, &d.X_cap, sizeof(float2) * S * m.Q * m.NLpad)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&d.phase, &d.phase_cap, sizeof(float2) * S * m.Cmax * m.Q)) != DG_OK) return st;
     if (m.c64 && (st = ensure(c, (void **)&d.bad, &d.bad_cap, sizeof(int) * 4 * S)) != DG_OK) return st;
+    if (pr) {
+        const size_t fb = sizeof(float) * kPolyTerms * kPolyPts;
+        if ((st = ensure(c, (void **)&d.fit, &d.fit_cap, fb)) != DG_OK) return st;
+        if ((st = ensure(c, (void **)&d.coef, &d.coef_cap, sizeof(float) * kPolyStride * (size_t)ptiles * S)) != DG_OK)
+            return st;
+        if (d.fit_rows != pr) {
+            const std::vector<float> fit = poly_fit(m.poly);
+            CK(c, cudaMemcpyAsync(d.fit, fit.data(), fb, cudaMemcpyHostToDevice, c->stream));
+            d.fit_rows = pr;
+        }
+    }
     if ((st = ensure_ephf(c)) != DG_OK) return st;
     // pageable sources: staged before the calls return
     CK(c, cudaMemcpyAsync(d.snap, snap.data(), sizeof(MapSnap) * snap.size(), cudaMemcpyHostToDevice, c->stream));
@@ -1192,6 +1305,14 @@ static dg_status run_surface_map(dg_ctx *c, void *out)
         a.bad = m.c64 ? d.bad : nullptr;
         a.out = (float *)out;
         a.err = c->err_d;
+        a.poly = m.poly;
+        a.fit = d.fit;
+        a.coef = d.coef;
+        if (m.poly.rows) {
+            Timed t(c, DG_K_CDFT_COMBINE);
+            CK(c, launch_map_poly(a, c->stream));
+            t.done(1);
+        }
         {
             Timed t(c, DG_K_CDFT_CONTRACT);
             int n = 1;
@@ -2363,6 +2484,8 @@ dg_status dg_destroy(dg_ctx *c)
     fr(c->mb.X);
     fr(c->mb.phase);
     fr(c->mb.bad);
+    fr(c->mb.fit);
+    fr(c->mb.coef);
     fr(c->co.lag);
     fr(c->co.nu);
     fr(c->co.lmm);

@@ -493,8 +493,17 @@ constexpr double kMapNDelta = 7.5e-2;
 struct MapSnap {                  // one snapshot's table
     double nu0, delta;            // bins nu0 + q delta, q < Q (cycles per sample)
     double nuc, halfw;            // the bins' centre and half width: nodes nuc + halfw xnode[p]
-    float nu0_hi, nu0_lo, inv_delta;
+    float nu0_hi, nu0_lo, inv_delta, inv_delta_lo;
     int L0, NL;                   // lags L0 .. L0 + NL - 1
+};
+// Polynomial geometry of large grids: per (node tile, snapshot) D and the bin
+// coordinate as polynomials of total degree 5 in the node offsets, fitted to
+// the double-float geometry at kPolyPts nodes of the tile.
+constexpr int kPolyPts = 32, kPolyTerms = 21, kPolyCols = 32;
+constexpr int kPolyStride = 48;   // floats per (tile, snapshot): head 4, then 21 (D, bin) pairs
+struct PolyShape {                // of a tile of `rows` x kPolyCols nodes
+    int rows;                     // 64 or 32; 0: geometry per node
+    int pr[kPolyPts], pc[kPolyPts];  // the sample nodes' offsets in the tile
 };
 struct MapArgs {
     const StepDesc *sd;           // [S] captures
@@ -516,7 +525,11 @@ struct MapArgs {
     int *bad;                     // [S][4] first / last sample of y1, y2 that is not finite (NULL: no c64 capture)
     float *out;                   // [G]
     unsigned *err;
+    PolyShape poly;
+    const float *fit;             // [kPolyTerms][kPolyPts] samples -> coefficients
+    float *coef;                  // [tiles][S][kPolyStride]
 };
+cudaError_t launch_map_poly(const MapArgs &a, cudaStream_t s);
 cudaError_t launch_map_twiddles(float2 *tw, int logn, cudaStream_t s);
 cudaError_t launch_map_tables(const MapArgs &a, cudaStream_t s, int *launches);
 cudaError_t launch_map_expand(const MapArgs &a, cudaStream_t s);

@@ -47,6 +47,20 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b)
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 
+// Two FP32 FMAs in one instruction (Blackwell's packed form): half the issue
+// slots of the same arithmetic.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    unsigned long long r, x, y, z;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(c.x), "f"(c.y));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(r));
+    return d;
+}
+
 // e^{j 2 pi f x} for a frequency f = hi + lo (cycles per sample) and an
 // integer-valued x, |x| < 2^24.
 __device__ __forceinline__ float2 cis_df(float hi, float lo, float x)
@@ -329,64 +343,95 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN == 14 ? 1 : LOGN == 13 
     }
 }
 
-// X[q][l]: a warp takes 32 lags and kExpQ bins; 8 warps share the lags (their
-// U loads hit L1) and take 8 kExpQ consecutive bins.
-constexpr int kExpQ = 8;
+// X[q][l]: a warp takes 32 lags and NQ bins (in pairs: the packed FMAs run
+// over two bins, whose node weights lie side by side in shared memory); the
+// CTA's warps share the lags (their U loads hit L1). Per block and node a
+// warp loads 256 bytes of U and 4 NQ bytes of weights for 2 NQ x 32 FMAs.
 constexpr int kExpWarps = 8;
-constexpr int kExpBins = kExpQ * kExpWarps;
 
-__global__ void __launch_bounds__(32 * kExpWarps) k_map_expand(MapArgs a)
+__device__ __forceinline__ void cp_async8(void *dst, const void *src)
 {
-    __shared__ __align__(16) float sT[kMapMaxNodes][kExpBins];
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+template <int NQ> __global__ void __launch_bounds__(32 * kExpWarps) k_map_expand(MapArgs a)
+{
+    constexpr int NB = NQ * kExpWarps, H = NQ / 2, T = 32 * kExpWarps;
+    extern __shared__ __align__(16) float sm_f[];
     const int s = blockIdx.z, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const StepDesc sd = a.sd[s];
     const MapSnap ms = a.snap[s];
-    const int qb = blockIdx.y * kExpBins, P = a.P;
+    const int qb = blockIdx.y * NB, P = a.P;
     if (blockIdx.x * 32 >= ms.NL) return;
-    for (int i = threadIdx.x; i < P * kExpBins; i += 32 * kExpWarps) {
-        const int q = qb + i % kExpBins;
-        sT[i / kExpBins][i % kExpBins] = q < a.Q ? __ldg(a.T + (i / kExpBins) * a.Q + q) : 0.f;
-    }
-    __syncthreads();
-    const int q0 = qb + kExpQ * warp;
-    if (q0 >= a.Q) return;
-    const int l = blockIdx.x * 32 + lane;
+    float *sT = sm_f;                                              // [P][NB]
+    float2 *sE = reinterpret_cast<float2 *>(sT + P * NB);          // [3][NB]
+    float2 *sU = sE + 3 * NB;                                      // [3][P][32]
+    const int l0 = blockIdx.x * 32;
     const int C = (sd.n + a.Mb - 1) / a.Mb;
-    const float2 *U = a.U + (size_t)s * a.Cmax * P * a.NLpad + l;
+    const float2 *U = a.U + (size_t)s * a.Cmax * P * a.NLpad + l0;
     const float2 *E = a.phase + (size_t)s * a.Cmax * a.Q;
-    float2 x[kExpQ];
+    auto stage = [&](int c) {  // block c's U rows and phases, asynchronously
+        if (c < C) {
+            float2 *u = sU + (c % 3) * P * 32;
+            for (int i = threadIdx.x; i < P * 32; i += T)
+                cp_async8(u + i, U + ((size_t)c * P + (i >> 5)) * a.NLpad + (i & 31));
+            for (int i = threadIdx.x; i < NB; i += T)
+                cp_async8(sE + (c % 3) * NB + i, E + (size_t)c * a.Q + min(qb + i, a.Q - 1));
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    stage(0);
+    stage(1);
+    for (int i = threadIdx.x; i < P * NB; i += T) {
+        const int q = qb + i % NB;
+        sT[i] = q < a.Q ? __ldg(a.T + (i / NB) * a.Q + q) : 0.f;
+    }
+    float2 xr[H], xi[H];  // real and imaginary parts of bin pairs
 #pragma unroll
-    for (int i = 0; i < kExpQ; ++i) x[i] = make_float2(0.f, 0.f);
+    for (int i = 0; i < H; ++i) xr[i] = xi[i] = make_float2(0.f, 0.f);
     for (int c = 0; c < C; ++c) {
-        float2 y[kExpQ];
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();  // block c staged; every warp is done with block c - 1, whose slot takes c + 2
+        stage(c + 2);
+        const float2 *u_s = sU + (c % 3) * P * 32 + lane;
+        const float *t_s = sT + NQ * warp;
+        float2 yr[H], yi[H];
 #pragma unroll
-        for (int i = 0; i < kExpQ; ++i) y[i] = make_float2(0.f, 0.f);
-#pragma unroll 4
+        for (int i = 0; i < H; ++i) yr[i] = yi[i] = make_float2(0.f, 0.f);
+#pragma unroll 2
         for (int p = 0; p < P; ++p) {
-            const float2 u = U[((size_t)c * P + p) * a.NLpad];
-            const float4 ta = *reinterpret_cast<const float4 *>(&sT[p][kExpQ * warp]);
-            const float4 tb = *reinterpret_cast<const float4 *>(&sT[p][kExpQ * warp + 4]);
-            const float w[kExpQ] = {ta.x, ta.y, ta.z, ta.w, tb.x, tb.y, tb.z, tb.w};
+            const float2 u = u_s[32 * p];
+            const float2 ur = make_float2(u.x, u.x), ui = make_float2(u.y, u.y);
 #pragma unroll
-            for (int i = 0; i < kExpQ; ++i) {
-                y[i].x = fmaf(w[i], u.x, y[i].x);
-                y[i].y = fmaf(w[i], u.y, y[i].y);
+            for (int i = 0; i < H; i += 2) {
+                const float4 t = *reinterpret_cast<const float4 *>(t_s + NB * p + 2 * i);
+                const float2 ta = make_float2(t.x, t.y), tb = make_float2(t.z, t.w);
+                yr[i] = fma2(ta, ur, yr[i]);
+                yi[i] = fma2(ta, ui, yi[i]);
+                yr[i + 1] = fma2(tb, ur, yr[i + 1]);
+                yi[i + 1] = fma2(tb, ui, yi[i + 1]);
             }
         }
+        const float4 *e_s = reinterpret_cast<const float4 *>(sE + (c % 3) * NB + NQ * warp);
 #pragma unroll
-        for (int i = 0; i < kExpQ; ++i) {
-            const float2 e = __ldg(E + (size_t)c * a.Q + min(q0 + i, a.Q - 1));
-            x[i].x = fmaf(e.x, y[i].x, fmaf(-e.y, y[i].y, x[i].x));
-            x[i].y = fmaf(e.x, y[i].y, fmaf(e.y, y[i].x, x[i].y));
+        for (int i = 0; i < H; ++i) {
+            const float4 e = e_s[i];  // two bins' phases
+            const float2 er = make_float2(e.x, e.z), ei = make_float2(e.y, e.w);
+            xr[i] = fma2(er, yr[i], fma2(make_float2(-ei.x, -ei.y), yi[i], xr[i]));
+            xi[i] = fma2(er, yi[i], fma2(ei, yr[i], xi[i]));
         }
     }
+    const int l = l0 + lane, q0 = qb + NQ * warp;
     if (l >= ms.NL) return;
     const int L = ms.L0 + l;
     const bool none = L >= sd.n || L <= -sd.n;  // no overlap: exactly zero
 #pragma unroll
-    for (int i = 0; i < kExpQ; ++i)
-        if (q0 + i < a.Q)
-            a.X[((size_t)s * a.Q + q0 + i) * a.NLpad + l] = none ? make_float2(0.f, 0.f) : x[i];
+    for (int i = 0; i < NQ; ++i)
+        if (q0 + i < a.Q) {
+            const float2 v = i & 1 ? make_float2(xr[i / 2].y, xi[i / 2].y) : make_float2(xr[i / 2].x, xi[i / 2].x);
+            a.X[((size_t)s * a.Q + q0 + i) * a.NLpad + l] = none ? make_float2(0.f, 0.f) : v;
+        }
 }
 
 // Whether lag L's overlap touches a sample that is not finite: n runs over
@@ -397,26 +442,65 @@ __device__ __forceinline__ bool lag_bad(int4 b, int L, int N)
     return L >= 0 ? (b.x < N - L || b.w >= L) : (b.y >= -L || b.z < N + L);
 }
 
-// One candidate and snapshot: |C|^2 or |C|.
-template <bool FRAC>
-__device__ __forceinline__ float map_value(const MapArgs &a, const MapSnap &ms, int s, int L, float mu, float u)
+// Nearest integer of |x| < 2^22, as a float and as an integer, by the
+// round-off of 1.5 x 2^23 (two additions on the FP32 pipe where the
+// conversion instructions run at a fraction of its rate).
+__device__ __forceinline__ float round_magic(float x, int &n)
 {
-    // 6-point Lagrange interpolation on bins q0 - 2 .. q0 + 3 (see the
-    // combine of dg_cdft.cu); the host pads the bins so that q0 is inside
-    const int q0 = max(2, min(a.Q - 4, __float2int_rd(u)));
-    const float t = u - (float)q0;
-    const float a2 = t + 2.f, a1 = t + 1.f, b1 = t - 1.f, b2 = t - 2.f, b3 = t - 3.f;
-    const float t01 = t * b1, t23 = b2 * b3, s21 = a2 * a1;
-    const float w[6] = {-(a1 * t01 * t23) * (1.f / 120.f), (a2 * t01 * t23) * (1.f / 24.f),
-                        -(s21 * b1 * t23) * (1.f / 12.f),  (s21 * t * t23) * (1.f / 12.f),
-                        -(s21 * t01 * b3) * (1.f / 24.f),  (s21 * t01 * b2) * (1.f / 120.f)};
-    const int l = max(FRAC ? 1 : 0, min(ms.NL - (FRAC ? 3 : 1), L - ms.L0));
-    const float2 *X = a.X + ((size_t)s * a.Q + q0 - 2) * a.NLpad + l;
+    constexpr float magic = 12582912.f;
+    const float y = __fadd_rn(x, magic);
+    n = __float_as_int(y) - 0x4b400000;
+    return __fsub_rn(y, magic);
+}
+
+// The 6-point Lagrange weights of nodes at -2.5, -1.5, ..., 2.5 at s in
+// [-0.5, 0.5]: the pair +-n has E(s^2) (1 +- s / n), E the quadratic through
+// the other nodes' squares; E and E / n as one packed polynomial.
+__device__ __forceinline__ void weights6(float s, float (&w)[6])
+{
+    const float s2 = s * s;
+    const float2 q = make_float2(s2, s2);
+    auto pair = [&](float d, float inv_n, float b, float c) {
+        const float2 k2 = make_float2(d, d * inv_n), k1 = make_float2(d * b, d * b * inv_n),
+                     k0 = make_float2(d * c, d * c * inv_n);
+        return fma2(fma2(k2, q, k1), q, k0);
+    };
+    const float2 a = pair(1.f / 24.f, 2.f, -8.5f, 14.0625f);
+    const float2 b = pair(-1.f / 16.f, 1.f / 1.5f, -6.5f, 1.5625f);
+    const float2 c = pair(1.f / 48.f, 0.4f, -2.5f, 0.5625f);
+    w[0] = fmaf(-s, c.y, c.x);
+    w[1] = fmaf(-s, b.y, b.x);
+    w[2] = fmaf(-s, a.y, a.x);
+    w[3] = fmaf(s, a.y, a.x);
+    w[4] = fmaf(s, b.y, b.x);
+    w[5] = fmaf(s, c.y, c.x);
+}
+
+// One candidate and snapshot, at bin coordinate U0 + u: |C|^2 or |C|. BAD:
+// some capture may hold samples that are not finite. The host's bounds keep
+// lag and bins inside the table; an index that still falls outside reads its
+// start.
+template <bool FRAC, bool BAD>
+__device__ __forceinline__ float map_value(const MapArgs &a, const float2 *__restrict__ X, int s, int L0, int L,
+                                           float mu, int U0, float u)
+{
+    // bins q0 - 2 .. q0 + 3, q0 <= U0 + u <= q0 + 1, at its middle plus t
+    int k;
+    const float t = (u - 0.5f) - round_magic(u - 0.5f, k);
+    float w[6];
+    weights6(t, w);
+    int idx = (U0 + k - 2) * a.NLpad + (L - L0);
+    if (FRAC) {
+        if ((unsigned)(idx - 1) > (unsigned)((a.Q - 5) * a.NLpad - 4)) idx = 1;
+    } else {
+        if ((unsigned)idx >= (unsigned)((a.Q - 5) * a.NLpad)) idx = 0;
+    }
+    const float2 *R = X + idx;
     float cx = 0.f, cy = 0.f;
     if (!FRAC) {
 #pragma unroll
         for (int e = 0; e < 6; ++e) {
-            const float2 v = __ldg(X + (size_t)e * a.NLpad);
+            const float2 v = __ldg(R + (size_t)e * a.NLpad);
             cx = fmaf(w[e], v.x, cx);
             cy = fmaf(w[e], v.y, cy);
         }
@@ -425,11 +509,10 @@ __device__ __forceinline__ float map_value(const MapArgs &a, const MapSnap &ms, 
                              -(mu + 1.f) * mu * (mu - 2.f) * 0.5f, (mu + 1.f) * mu * (mu - 1.f) * (1.f / 6.f)};
 #pragma unroll
         for (int e = 0; e < 6; ++e) {
-            const float2 *R = X + (size_t)e * a.NLpad;
             float zx = 0.f, zy = 0.f;
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
-                const float2 v = __ldg(R + m - 1);
+                const float2 v = __ldg(R + (size_t)e * a.NLpad + m - 1);
                 zx = fmaf(lw[m], v.x, zx);
                 zy = fmaf(lw[m], v.y, zy);
             }
@@ -437,7 +520,7 @@ __device__ __forceinline__ float map_value(const MapArgs &a, const MapSnap &ms, 
             cy = fmaf(w[e], zy, cy);
         }
     }
-    if (a.bad) {
+    if (BAD) {
         const int4 b = __ldg(reinterpret_cast<const int4 *>(a.bad) + s);
         const int N = a.sd[s].n;
         bool bad = lag_bad(b, L, N);
@@ -472,11 +555,171 @@ __device__ __forceinline__ bool map_node(const MapArgs &a, const MapSnap &ms, in
     return true;
 }
 
+// Polynomial geometry. On a tile whose radius h is small against the range
+// rho to the receivers, D and the FDOA are smooth: the m-th Taylor term of
+// D is at most m |p2 - p1| fs / c (h / rho)^m. A warp evaluates the
+// double-float geometry at kPolyPts nodes of the tile (a 6 x 6 Chebyshev-like
+// lattice without its corners) and fits polynomials of total degree 5 in the
+// normalised offsets by a constant least-squares matrix; the host takes a
+// tile only where the bound on the truncation stays below 2e-6 samples.
+// Precision: D = I0 + gu r + gv c + P(r, c) with an integer I0 and slopes
+// that are multiples of 2^-13, so the linear part is exact in FP32 at every
+// node (|offset| <= 31.5, |slope| < 8: 23 bits), and only P, a few samples at
+// most, is rounded (about 5e-7).
+__device__ __forceinline__ float2 poly_offset(const MapArgs &a, int r, int c)  // from the tile's centre
+{
+    return make_float2((float)r - 0.5f * (float)(a.poly.rows - 1), (float)c - 0.5f * (float)(kPolyCols - 1));
+}
+
+constexpr int kPolyWarps = 8;
+__global__ void __launch_bounds__(32 * kPolyWarps) k_map_poly(MapArgs a, int tiles_j, int64_t pairs)
+{
+    __shared__ float s_fit[kPolyTerms][kPolyPts + 1];
+    __shared__ float2 s_val[kPolyWarps][kPolyPts];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i = threadIdx.x; i < kPolyTerms * kPolyPts; i += 32 * kPolyWarps)
+        s_fit[i / kPolyPts][i % kPolyPts] = __ldg(a.fit + i);
+    __syncthreads();
+    const int64_t w = blockIdx.x * (int64_t)kPolyWarps + warp;
+    if (w >= pairs) return;
+    const int s = (int)(w % a.S);
+    const int64_t tile = w / a.S;
+    const int r0 = min((int)(tile / tiles_j) * a.poly.rows, a.nrows - a.poly.rows);
+    const int c0 = min((int)(tile % tiles_j) * kPolyCols, a.nlon - kPolyCols);
+    const MapSnap ms = a.snap[s];
+    const int pr = a.poly.pr[lane], pc = a.poly.pc[lane];
+    const int64_t p = (int64_t)(r0 + pr) * a.nlon + c0 + pc;
+    dfl ed[12], D, nu;
+#pragma unroll
+    for (int t = 0; t < 12; ++t) ed[t] = {__ldg(a.ephf + 24 * (size_t)s + 2 * t), __ldg(a.ephf + 24 * (size_t)s + 2 * t + 1)};
+    geometry_dfl(df_from(a.xyz[p]), df_from(a.xyz[a.G + p]), df_from(a.xyz[2 * a.G + p]), ed, {a.fsc_hi, a.fsc_lo},
+                 {a.ilf_hi, a.ilf_lo}, D, nu);
+    constexpr unsigned all = 0xffffffffu;
+    constexpr int mid = 18;  // a sample near the centre anchors both
+    float I0 = rintf(__shfl_sync(all, D.hi, mid));
+    const dfl nr = {__shfl_sync(all, nu.hi, mid), __shfl_sync(all, nu.lo, mid)};
+    const dfl ur = df_mul(df_sub(nr, {ms.nu0_hi, ms.nu0_lo}), {ms.inv_delta, ms.inv_delta_lo});
+    const float U0 = rintf(ur.hi);
+    const float du = ((nu.hi - nr.hi) + (nu.lo - nr.lo)) * ms.inv_delta + ((ur.hi - U0) + ur.lo);
+    const float dD = (D.hi - I0) + D.lo;
+    // slopes per node from the linear terms (c^1: term 1, r^1: term 6)
+    const float hr = 0.5f * (float)(a.poly.rows - 1), hc = 0.5f * (float)(kPolyCols - 1);
+    float g0 = s_fit[0][lane] * dD, gc = s_fit[1][lane] * dD, gr = s_fit[6][lane] * dD;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        g0 += __shfl_xor_sync(all, g0, d);
+        gc += __shfl_xor_sync(all, gc, d);
+        gr += __shfl_xor_sync(all, gr, d);
+    }
+    I0 += rintf(g0);  // the centre's
+    gr = rintf(gr / hr * 8192.f) * (1.f / 8192.f);
+    gc = rintf(gc / hc * 8192.f) * (1.f / 8192.f);
+    const float2 o = poly_offset(a, pr, pc);
+    // D.hi - I0 and the linear part are multiples of 2^-14 or finer parts of D.hi: exact difference
+    s_val[warp][lane] = make_float2(((D.hi - I0) - fmaf(gr, o.x, gc * o.y)) + D.lo, du);
+    __syncwarp();
+    float *out = a.coef + (size_t)w * kPolyStride;
+    if (lane < kPolyTerms) {
+        float2 c = make_float2(0.f, 0.f);
+#pragma unroll 8
+        for (int i = 0; i < kPolyPts; ++i) {
+            const float2 v = s_val[warp][i];
+            c.x = fmaf(s_fit[lane][i], v.x, c.x);
+            c.y = fmaf(s_fit[lane][i], v.y, c.y);
+        }
+        *reinterpret_cast<float2 *>(out + 4 + 2 * lane) = c;
+    } else if (lane == kPolyTerms) {
+        *reinterpret_cast<float4 *>(out) = make_float4(I0, U0, gr, gc);
+    }
+}
+
+// The lookup of a tile of poly.rows x 32 nodes by one CTA: a warp takes a
+// compact 4-row x 8-column patch per step (their lags, and so their table
+// addresses, lie close together), R = rows / 8 steps of 4 rows; a thread's
+// column is fixed, so the polynomials collapse to one variable per snapshot.
+template <bool FRAC, bool BAD, int R>
+__global__ void __launch_bounds__(256, 4) k_map_lookup_poly(MapArgs a, int tiles_j)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tile = blockIdx.x, ti = tile / tiles_j, tj = tile % tiles_j;
+    constexpr int TR = 8 * R;
+    const int r0 = min(ti * TR, a.nrows - TR), c0 = min(tj * kPolyCols, a.nlon - kPolyCols);
+    const int j = tj * kPolyCols + (warp & 3) * 8 + (lane & 7);
+    const int i0 = ti * TR + (warp >> 2) * (4 * R) + (lane >> 3);
+    const float2 o = poly_offset(a, i0 - r0, j - c0);
+    const float vn = o.y * (2.f / (float)(kPolyCols - 1));
+    float sum[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = i0 + 4 * r;
+        sum[r] = (!a.first && i < a.nrows && j < a.nlon) ? a.out[(int64_t)i * a.nlon + j] : 0.f;
+    }
+    const float4 *cf = reinterpret_cast<const float4 *>(a.coef + (size_t)tile * a.S * kPolyStride);
+    const float2 vn2 = make_float2(vn, vn);
+    const float2 *X = a.X;
+    for (int s = 0; s < a.S; ++s, cf += kPolyStride / 4, X += (size_t)a.Q * a.NLpad) {
+        const int L0 = a.snap[s].L0;
+        const float4 head = __ldg(cf);
+        // polynomials in the row offset: x D, y bin coordinate; terms of
+        // r^0 (c^0..5), r^1 (c^0..4), r^2 (c^0..3), ...
+        float2 cr[6];
+        {
+            float2 m[22];
+#pragma unroll
+            for (int t = 0; t < 11; ++t) {
+                const float4 f = __ldg(cf + 1 + t);
+                m[2 * t] = make_float2(f.x, f.y);
+                m[2 * t + 1] = make_float2(f.z, f.w);
+            }
+            int at = 0;
+#pragma unroll
+            for (int e = 0; e < 6; ++e) {
+                float2 h = m[at + 5 - e];
+#pragma unroll
+                for (int b = 4 - e; b >= 0; --b) h = fma2(h, vn2, m[at + b]);
+                cr[e] = h;
+                at += 6 - e;
+            }
+        }
+        const float lin_c = head.w * o.y;
+        const int I0 = (int)head.x, U0 = (int)head.y;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float rr = o.x + 4.f * r;
+            const float un = rr * (2.f / (float)(TR - 1));
+            const float2 un2 = make_float2(un, un);
+            float2 h = cr[5];
+#pragma unroll
+            for (int e = 4; e >= 0; --e) h = fma2(h, un2, cr[e]);
+            const float lin = fmaf(head.z, rr, lin_c);  // exact
+            int n1, n2;
+            const float t = (lin - round_magic(lin, n1)) + h.x;  // D = I0 + n1 + t
+            const float mu = t - round_magic(FRAC ? t - 0.5f : t, n2);
+            int L = I0 + n1 + n2;  // Lagrange4: floor, or one less with mu = 1 at an integer
+            if (!FRAC && fabsf(mu) > 0.5f - 1e-5f) {  // within 1e-5 of a rounding boundary: the FP64 expression
+                const int i = min(i0 + 4 * r, a.nrows - 1);
+                double e[12], D64, nu64;
+                for (int q = 0; q < 12; ++q) e[q] = a.eph[12 * (size_t)s + q];
+                const int64_t p = (int64_t)i * a.nlon + min(j, a.nlon - 1);
+                geometry(a.xyz[p], a.xyz[a.G + p], a.xyz[2 * a.G + p], e, a.fs, a.lambda, D64, nu64);
+                L = lag_of(D64, DG_DELAY_INTEGER);
+            }
+            const float v = map_value<FRAC, BAD>(a, X, s, L0, L, mu, U0, h.y);
+            sum[r] = (s == 0 && a.first) ? v : sum[r] + v;
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = i0 + 4 * r;
+        if (i < a.nrows && j < a.nlon) a.out[(int64_t)i * a.nlon + j] = sum[r];
+    }
+}
+
 // One thread per node (32 consecutive nodes of a grid row per warp); WK warps
 // of a CTA share the nodes and split the snapshots, 8 / WK take their own
 // rows. WK = 8 serves small grids, which would leave the chip idle otherwise:
 // the partial values meet in shared memory and are added in snapshot order.
-template <bool FRAC, int WK> __global__ void __launch_bounds__(256) k_map_lookup(MapArgs a)
+template <bool FRAC, bool BAD, int WK> __global__ void __launch_bounds__(256) k_map_lookup(MapArgs a)
 {
     constexpr int WN = 8 / WK;
     __shared__ float s_val[WK > 1 ? WK : 1][32];
@@ -499,8 +742,13 @@ template <bool FRAC, int WK> __global__ void __launch_bounds__(256) k_map_lookup
             const MapSnap ms = a.snap[s];
             int L;
             float mu, u;
-            if (map_node<FRAC>(a, ms, s, p, xyz, L, mu, u)) v = map_value<FRAC>(a, ms, s, L, mu, u);
-            else if (ok) atomicOr(a.err, ERR_LAG_RANGE);
+            if (map_node<FRAC>(a, ms, s, p, xyz, L, mu, u)) {
+                int U0;
+                const float uf = round_magic(u, U0);
+                v = map_value<FRAC, BAD>(a, a.X + (size_t)s * a.Q * a.NLpad, s, ms.L0, L, mu, U0, u - uf);
+            } else if (ok) {
+                atomicOr(a.err, ERR_LAG_RANGE);
+            }
         }
         if (WK == 1) {
             sum = any ? sum + v : v;
@@ -565,30 +813,53 @@ cudaError_t launch_map_tables(const MapArgs &a, cudaStream_t st, int *launches)
     return e;
 }
 
+template <int NQ> static cudaError_t launch_expand(const MapArgs &a, cudaStream_t st)
+{
+    constexpr int NB = NQ * kExpWarps;
+    const size_t smem = sizeof(float) * (size_t)a.P * NB + sizeof(float2) * 3 * (size_t)(NB + a.P * 32);
+    const cudaError_t e = cudaFuncSetAttribute(k_map_expand<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const dim3 ge((unsigned)(a.NLpad / 32), (unsigned)((a.Q + NB - 1) / NB), (unsigned)a.S);
+    k_map_expand<NQ><<<ge, 32 * kExpWarps, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_map_expand(const MapArgs &a, cudaStream_t st)
 {
-    const dim3 ge((unsigned)(a.NLpad / 32), (unsigned)((a.Q + kExpBins - 1) / kExpBins), (unsigned)a.S);
-    k_map_expand<<<ge, 32 * kExpWarps, 0, st>>>(a);
+    // 16 bins per warp where the table is wide enough to fill the chip, 8 otherwise
+    return a.Q >= 128 ? launch_expand<16>(a, st) : launch_expand<8>(a, st);
+}
+
+cudaError_t launch_map_poly(const MapArgs &a, cudaStream_t st)
+{
+    const int64_t tiles_j = (a.nlon + kPolyCols - 1) / kPolyCols;
+    const int64_t pairs = tiles_j * ((a.nrows + a.poly.rows - 1) / a.poly.rows) * a.S;
+    const int64_t blocks = (pairs + kPolyWarps - 1) / kPolyWarps;
+    if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
+    k_map_poly<<<(unsigned)blocks, 32 * kPolyWarps, 0, st>>>(a, (int)tiles_j, pairs);
+    return cudaGetLastError();
+}
+
+template <bool FRAC, bool BAD> static cudaError_t launch_lookup(const MapArgs &a, cudaStream_t st)
+{
+    const int64_t tiles_j = (a.nlon + 31) / 32;
+    // under about four CTAs per SM of one-row warps, the warps split the snapshots
+    const bool split = !a.poly.rows && tiles_j * ((a.nrows + 7) / 8) < 152 * 4;
+    const int rows = a.poly.rows ? a.poly.rows : split ? 1 : 8;  // of a CTA
+    const int64_t blocks = tiles_j * ((a.nrows + rows - 1) / rows);
+    if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
+    const unsigned g = (unsigned)blocks;
+    if (a.poly.rows == 64) k_map_lookup_poly<FRAC, BAD, 8><<<g, 256, 0, st>>>(a, (int)tiles_j);
+    else if (a.poly.rows) k_map_lookup_poly<FRAC, BAD, 4><<<g, 256, 0, st>>>(a, (int)tiles_j);
+    else if (split) k_map_lookup<FRAC, BAD, 8><<<g, 256, 0, st>>>(a);
+    else k_map_lookup<FRAC, BAD, 1><<<g, 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_map_lookup(const MapArgs &a, cudaStream_t st)
 {
-    const int64_t tiles_j = (a.nlon + 31) / 32;
-    const bool frac = a.delay != DG_DELAY_INTEGER;
-    // under about four CTAs per SM of one-row warps, the warps split the snapshots
-    const bool split = tiles_j * ((a.nrows + 7) / 8) < 152 * 4;
-    const int64_t blocks = tiles_j * (split ? a.nrows : (a.nrows + 7) / 8);
-    if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
-    const unsigned g = (unsigned)blocks;
-    if (split) {
-        if (frac) k_map_lookup<true, 8><<<g, 256, 0, st>>>(a);
-        else k_map_lookup<false, 8><<<g, 256, 0, st>>>(a);
-    } else {
-        if (frac) k_map_lookup<true, 1><<<g, 256, 0, st>>>(a);
-        else k_map_lookup<false, 1><<<g, 256, 0, st>>>(a);
-    }
-    return cudaGetLastError();
+    if (a.delay == DG_DELAY_INTEGER) return a.bad ? launch_lookup<false, true>(a, st) : launch_lookup<false, false>(a, st);
+    return a.bad ? launch_lookup<true, true>(a, st) : launch_lookup<true, false>(a, st);
 }
 
 }  // namespace dg
