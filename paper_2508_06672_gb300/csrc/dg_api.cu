@@ -164,6 +164,7 @@ struct dg_ctx {
     ArgmaxResult *reg_host = nullptr;   // pinned mirror
     size_t reg_cap = 0;
     double *xyz = nullptr;
+    GridStep *gstep = nullptr;          // angular steps of the grid, of the refinement grid (device)
     double *eph = nullptr;
     std::vector<dg_ephem> eph_host;
     std::vector<Step> steps;
@@ -184,7 +185,11 @@ struct dg_ctx {
     LocalGrid loc;
     CdftBufs cd;
     MapPlan mp;
-    MapBufs mb;
+    MapBufs mb, mr;         // main surface; refinement
+    double *reg_xyz = nullptr;          // dg_search_regions: ECEF of the regions searched together
+    GridDev *reg_grids = nullptr;
+    GridStep *reg_steps = nullptr;
+    size_t reg_xyz_cap = 0, reg_grids_cap = 0, reg_steps_cap = 0;
     bool last_map = false;  // the last CDFT surface came from the maps
     CoarseBufs co;
     int cd_chunk_min = 0, cd_chunk_max = 0;              // chunks it used
@@ -192,10 +197,13 @@ struct dg_ctx {
     ArgmaxResult *amax_fine = nullptr;  // refinement argmax (device)
     dg_fix *fix_dev = nullptr;
     dg_fix *fix_host = nullptr;         // pinned
+    dg_fix *fix_dev_sync = nullptr, *fix_host_sync = nullptr;  // the same of dg_argmax_refine
     cudaGraphExec_t graph = nullptr;
     int64_t graph_launches = 0;         // kernels per replay
     uint64_t steps_gen = 1, graph_gen = 0;  // capture buffers / formats / lengths generation
     std::string err;
+    bool captured = false;              // a graph or a batch holds pointers into this context's buffers
+    std::vector<void *> retired;        // buffers replaced since: freed with the context
     int64_t launches = 0;
     std::vector<TimedLaunch> pending;
     double ms[DG_K_NCLASS] = {};
@@ -291,10 +299,24 @@ dg_status check_latched(dg_ctx *c)
     return DG_OK;
 }
 
+// Give a buffer back, or keep it until the context goes when a captured step
+// may still replay on it.
+dg_status release(dg_ctx *c, void *p)
+{
+    if (!p) return DG_OK;
+    if (c->captured) {
+        c->retired.push_back(p);
+        return DG_OK;
+    }
+    CK(c, cudaFreeAsync(p, c->stream));
+    return DG_OK;
+}
+
 dg_status ensure(dg_ctx *c, void **p, size_t *cap, size_t bytes)
 {
     if (*cap >= bytes && *p) return DG_OK;
-    if (*p) CK(c, cudaFreeAsync(*p, c->stream));
+    const dg_status st = release(c, *p);
+    if (st != DG_OK) return st;
     *p = nullptr;
     *cap = 0;
     CK(c, cudaMallocAsync(p, bytes, c->stream));
@@ -331,6 +353,7 @@ dg_status run_surface_cdft(dg_ctx *c, const GridDev &gd, const double *xyz, int6
                            bool refine);
 static dg_status map_plan(dg_ctx *c);
 static dg_status run_surface_map(dg_ctx *c, void *out);
+static dg_status refine_map(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *out, bool *done);
 
 // Surfaces whose candidates look their correlations up in delay-Doppler maps
 // (dg_map.cu) instead of the per-lag DFT rows of the contraction: the main
@@ -338,11 +361,12 @@ static dg_status run_surface_map(dg_ctx *c, void *out);
 // DG_TILES_AUTO) with an arithmetic that is FP32 or claims its accuracy (the
 // split forms). The single 16-bit forms keep the tensor-core products the
 // caller asked for.
-static bool map_eligible(const dg_ctx *c)
+static bool map_options(const dg_ctx *c)
 {
     return c->opt.algo == DG_ALGO_CDFT && c->opt.chunk == 0 && c->opt.tiles == DG_TILES_AUTO &&
-           c->opt.contract != DG_CONTRACT_BF16 && c->opt.contract != DG_CONTRACT_FP16 && c->G >= kMapMinNodes;
+           c->opt.contract != DG_CONTRACT_BF16 && c->opt.contract != DG_CONTRACT_FP16;
 }
+static bool map_eligible(const dg_ctx *c) { return map_options(c) && c->G >= kMapMinNodes; }
 
 dg_status run_surface(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *surf, void *out,
                       bool refine)
@@ -351,6 +375,10 @@ dg_status run_surface(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G
     if (!refine && map_eligible(c)) {
         if ((st = map_plan(c)) != DG_OK) return st;
         if (c->mp.ok) return run_surface_map(c, out);
+    }
+    if (refine && map_options(c)) {
+        bool done = false;
+        if ((st = refine_map(c, gd, xyz, G, out, &done)) != DG_OK || done) return st;
     }
     if (c->opt.algo == DG_ALGO_CDFT) return run_surface_cdft(c, gd, xyz, G, surf, out, refine);
     st = push_steps(c);
@@ -406,7 +434,8 @@ dg_status run_surface(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G
 template <typename P>
 dg_status grow(dg_ctx *c, P **p, size_t n)
 {
-    if (*p) CK(c, cudaFreeAsync(*p, c->stream));
+    const dg_status st = release(c, *p);
+    if (st != DG_OK) return st;
     *p = nullptr;
     CK(c, cudaMallocAsync((void **)p, sizeof(P) * (n ? n : 1), c->stream));
     return DG_OK;
@@ -465,20 +494,34 @@ static double grid_diameter(const GridDev &g)
     return 1.1 * d + 1.0;
 }
 
+// Curvature bounds of D (samples) and the FDOA (cycles per sample) at
+// distances >= rho from receivers `sep` apart with speeds <= v and relative
+// motion dv. Over a lattice cell a field stays within half its second
+// derivative times the squared half diagonal h of its bilinear interpolant,
+// and so of the cell's corner values. Order m of a range's Taylor series is at
+// most (2m - 3)!! / rho^(m-1); over the receivers' separation the second
+// derivatives of D then differ by at most 3 sep / rho^2 and those of u . v (a
+// third derivative of the range) by 15 v sep / rho^3 + 3 dv / rho^2. The
+// lattice's own curvature (the parallels' up to 80 degrees, 6 / Earth radius)
+// adds that much of the gradients, sep / rho and 3 v sep / rho^2 + dv / rho.
+struct Curvature {
+    double d, nu;
+};
+static Curvature field_curvature(const dg_ctx *c, double rho, double sep, double v, double dv)
+{
+    constexpr double kLattice = 6.0 / 6.3e6;
+    const double d2 = 3.0 * sep / (rho * rho) + kLattice * sep / rho;
+    const double n2 = 15.0 * v * sep / (rho * rho * rho) + 3.0 * dv / (rho * rho) +
+                      kLattice * (3.0 * v * sep / (rho * rho) + dv / rho);
+    return {d2 * c->fs / kC, n2 / (c->lambda * c->fs)};
+}
+
 // FDOA span of every snapshot over the shard, from a lattice of nodes (its
 // corners, edges and interior; the FDOA field is smooth at these scales): up
 // to 65 x 65 nodes, fewer on small shards (at least 9 x 9, about one lattice
 // node per 8 grid nodes), the node positions computed once for all
 // snapshots. lags: the lattice's lag counts. range: bounds of D and the FDOA
-// that hold at every node of the shard: the lattice's extremes widened by the
-// fields' Lipschitz bounds times the largest distance h of a node from the
-// lattice (half a cell's diagonal). With unit vectors u_i to the receivers at
-// distances >= rho, |grad D| = |u_2 - u_1| fs / c <= (|p2 - p1| / rho) fs / c;
-// the gradient of u . v is (v - u (u . v)) / rho, whose change over the
-// receivers' separation is at most 3 |v| |p2 - p1| / rho^2, so |grad nu| <=
-// (|v2 - v1| / rho + 3 |v| |p2 - p1| / rho^2) / (lambda fs). An infinite range
-// marks a snapshot whose receivers come within a cell or each other's
-// distance of the nodes.
+// that hold at every node of the shard (range_bounds).
 static void fdoa_spans(const dg_ctx *c, const GridDev &g, std::vector<double> &span,
                        std::vector<double> *lags = nullptr, std::vector<GridRange> *range = nullptr)
 {
@@ -493,6 +536,7 @@ static void fdoa_spans(const dg_ctx *c, const GridDev &g, std::vector<double> &s
             host_node_ecef(g, std::round(i), std::round(j), &p[3 * ((size_t)a * nj + b)]);
         }
     double h = 0.0;  // half the longest cell diagonal, with 5 % for the curvature within a cell
+    const bool low = std::fabs(g.lat0_rad) + 0.5 * g.nlat * g.dlat_m / 6.33e6 < 1.39;  // within 80 degrees
     if (range) {
         auto dist2 = [&](size_t q, size_t r) {
             const double *x = &p[3 * q], *y = &p[3 * r];
@@ -544,9 +588,9 @@ static void fdoa_spans(const dg_ctx *c, const GridDev &g, std::vector<double> &s
             const double v = std::max(norm(e.v1[0], e.v1[1], e.v1[2]), norm(e.v2[0], e.v2[1], e.v2[2]));
             const double rho = rmin - h - 0.5 * sep;  // also along the receivers' segment
             GridRange &R = (*range)[k];
-            if (rho > 0.0) {
-                const double md = sep / rho * c->fs / kC * h;
-                const double mn = (dv / rho + 3.0 * v * sep / (rho * rho)) / (c->lambda * c->fs) * h;
+            if (rho > 0.0 && low) {
+                const Curvature q = field_curvature(c, rho, sep, v, dv);
+                const double md = 0.5 * q.d * h * h, mn = 0.5 * q.nu * h * h;
                 R.d_lo = dlo - md;
                 R.d_hi = dhi + md;
                 R.nu_lo = lo - mn;
@@ -1097,45 +1141,41 @@ static int poly_rows(const dg_ctx *c, const std::vector<MapSnap> &snap)
     return 0;
 }
 
-// Shapes: the FFT length n = 2^logn, the lag tile LT and the block
-// Mb = n - LT + 1 that take the fewest SM cycles by a model of the kernels
-// (FFT butterflies at 0.35 of the FP32 rate, expansion at 0.5, a floor for the
-// chain of one CTA).
-static dg_status map_plan(dg_ctx *c)
+// The tables of `snap` (table s of capture s % K over lag and FDOA bounds
+// range[s]) share one shape. Sets L0, NL and the bins of every table and
+// Q, P, n = 2^logn, the lag tile LT and the block Mb = n - LT of m: those that
+// take the fewest SM cycles by a model of the kernels (FFT butterflies at
+// 0.35 of the FP32 rate, expansion at 0.5, a floor for the chain of one
+// CTA). False where the captures or the ranges do not suit the maps.
+static bool map_shape(const dg_ctx *c, const std::vector<GridRange> &range, std::vector<MapSnap> &snap, MapPlan &m)
 {
-    MapPlan &m = c->mp;
-    if (m.gen == c->steps_gen) return DG_OK;
-    m = MapPlan{};
-    CdftBufs &b = c->cd;
-    if (b.main_span.size() != (size_t)c->K || b.main_lags.size() != (size_t)c->K ||
-        b.main_range.size() != (size_t)c->K)
-        fdoa_spans(c, c->gd, b.main_span, &b.main_lags, &b.main_range);
     const bool frac = c->opt.delay != DG_DELAY_INTEGER;
-    std::vector<MapSnap> snap((size_t)c->K);
+    snap.assign(range.size(), MapSnap{});
     int nmax = 1, nlmax = 1;
     double Qd = 8.0;
-    m.gen = c->steps_gen;  // whatever the outcome, it holds until the shapes change
     for (int k = 0; k < c->K; ++k) {
-        const GridRange &R = b.main_range[k];
-        if (c->steps[k].n > (1 << 24)) return DG_OK;
-        // 0.01 samples absorb the rounding of D; Lagrange4 reaches L - 1 .. L + 2
-        if (!(std::fabs(R.d_lo) < 4e6 && std::fabs(R.d_hi) < 4e6)) return DG_OK;
-        const int lo = (int)std::floor(R.d_lo - 0.51) - (frac ? 1 : 0), hi = (int)std::ceil(R.d_hi + 0.51) + (frac ? 2 : 0);
-        snap[k].L0 = lo;
-        snap[k].NL = hi - lo + 1;
-        nlmax = std::max(nlmax, snap[k].NL);
+        if (c->steps[k].n > (1 << 24)) return false;
         nmax = std::max(nmax, (int)c->steps[k].n);
-        const double w = (R.nu_hi - R.nu_lo) * (1.0 + 1e-5) + 1e-13;
-        if (!(w < 0.046)) return DG_OK;  // wider than the 64 bins of the contraction's shortest chunk take: refused there
-        Qd = std::max(Qd, 6.0 + std::ceil(w * (double)c->steps[k].n / kMapNDelta));
         m.c64 |= c->steps[k].fmt == DG_IQ_C64;
     }
-    if (Qd > 8192.0 || nlmax > 65536) return DG_OK;
+    for (size_t s = 0; s < range.size(); ++s) {
+        const GridRange &R = range[s];
+        // 0.01 samples absorb the rounding of D; Lagrange4 reaches L - 1 .. L + 2
+        if (!(std::fabs(R.d_lo) < 4e6 && std::fabs(R.d_hi) < 4e6)) return false;
+        const int lo = (int)std::floor(R.d_lo - 0.51) - (frac ? 1 : 0), hi = (int)std::ceil(R.d_hi + 0.51) + (frac ? 2 : 0);
+        snap[s].L0 = lo;
+        snap[s].NL = hi - lo + 1;
+        nlmax = std::max(nlmax, snap[s].NL);
+        const double w = (R.nu_hi - R.nu_lo) * (1.0 + 1e-5) + 1e-13;
+        if (!(w < 0.046)) return false;  // wider than the 64 bins of the contraction's shortest chunk take: refused there
+        Qd = std::max(Qd, 6.0 + std::ceil(w * (double)c->steps[s % c->K].n / kMapNDelta));
+    }
+    if (Qd > 8192.0 || nlmax > 65536) return false;
     m.Q = (int)Qd;
     double halfw = 0.0;
-    for (int k = 0; k < c->K; ++k) {
-        MapSnap &s = snap[k];
-        const GridRange &R = b.main_range[k];
+    for (size_t q = 0; q < range.size(); ++q) {
+        MapSnap &s = snap[q];
+        const GridRange &R = range[q];
         s.delta = ((R.nu_hi - R.nu_lo) * (1.0 + 1e-5) + 1e-13) / (m.Q - 6);
         s.nu0 = 0.5 * (R.nu_lo + R.nu_hi) - 0.5 * (m.Q - 1) * s.delta;
         s.nuc = 0.5 * (R.nu_lo + R.nu_hi);
@@ -1146,6 +1186,8 @@ static dg_status map_plan(dg_ctx *c)
         s.inv_delta_lo = (float)(1.0 / s.delta - (double)s.inv_delta);
         halfw = std::max(halfw, s.halfw);
     }
+    std::map<int64_t, int> lengths;  // tables of each capture length
+    for (int k = 0; k < c->K; ++k) lengths[c->steps[k].n] += (int)(range.size() / (size_t)c->K);
     double best = 1e300;
     for (int logn = 10; logn <= 14; ++logn) {
         const int n = 1 << logn;
@@ -1156,13 +1198,10 @@ static dg_status map_plan(dg_ctx *c)
             if (Mb < n / 8) continue;
             const int P = map_nodes(halfw, Mb);
             if (P == 0) continue;
-            double ffts = 0.0, exps = 0.0, cmax = 0.0;
-            for (int k = 0; k < c->K; ++k) {
-                const double C = std::ceil((double)c->steps[k].n / Mb);
-                ffts += C * std::ceil((double)snap[k].NL / LT) * (1 + 2 * P);
-                exps += (double)snap[k].NL * m.Q * C * (2 * P + 4);
-                cmax = std::max(cmax, C);
-            }
+            double blocks = 0.0;
+            for (const auto &l : lengths) blocks += std::ceil((double)l.first / Mb) * l.second;
+            const double cmax = std::ceil((double)nmax / Mb), ffts = blocks * nt * (1 + 2 * P);
+            const double exps = blocks * nlmax * m.Q * (2 * P + 4);
             const double t_fft = ffts * n * logn * 5.0 / (128 * 0.35) / c->sm_count;
             const double cost = std::max(t_fft, 3.0 * (4000.0 + 1.6 * n)) + exps / (128 * 0.5) / c->sm_count +
                                 cmax * P * 40.0;
@@ -1176,59 +1215,35 @@ static dg_status map_plan(dg_ctx *c)
             if (nt * 32 >= nlmax) break;
         }
     }
-    if (best == 1e300) return DG_OK;
+    if (best == 1e300) return false;
     m.ntile = (nlmax + m.LT - 1) / m.LT;
     m.NLpad = (nlmax + 31) / 32 * 32;
     m.Cmax = (nmax + m.Mb - 1) / m.Mb;
-    for (int k = 0; k < c->K; ++k) m.rows += (int64_t)snap[k].NL * ((c->steps[k].n + m.Mb - 1) / m.Mb);
-    // the chunk the contraction would take (dg_cdft_chunks), and its limit on the per-lag DFT buffer
-    {
-        CdftLayout L;
-        std::vector<int> bb, gb;
-        if (cdft_batches(c, c->G, grid_diameter(c->gd), L, bb, gb) != DG_OK) return DG_OK;
-        const bool tc = c->opt.contract != DG_CONTRACT_FP32;
-        m.chunk_min = INT_MAX;
-        int64_t B = 1;
-        for (const auto &t : L.batches) {
-            const int M = auto_chunk(c, b.main_span, b.main_lags, t.k0, t.S, tc);
-            m.chunk_min = std::min(m.chunk_min, M);
-            m.chunk_max = std::max(m.chunk_max, M);
-            for (int s = 0; s < t.S; ++s) B = std::max<int64_t>(B, (c->steps[t.k0 + s].n + M - 1) / M);
-        }
-        if ((double)L.nbt_max * (double)B * 512.0 > (double)((size_t)64 << 30)) return DG_OK;
-    }
-    const size_t n = (size_t)1 << m.logn;
-    const int pr = poly_rows(c, snap);
-    if (pr) m.poly = poly_shape(pr);
-    const double ptiles = pr ? std::ceil((double)c->gd.nrows / pr) * std::ceil((double)c->gd.nlon / kPolyCols) : 0.0;
-    const double per = 8.0 * ((double)m.ntile * m.Cmax * n + (double)m.Cmax * m.P * m.NLpad + (double)m.Q * m.NLpad +
-                              (double)m.Cmax * m.Q) + 4.0 * kPolyStride * ptiles;
-    const double budget = (double)(c->opt.scratch_mib ? c->opt.scratch_mib : 12288) * 1048576.0;
-    m.S = (int)std::max(1.0, std::min((double)c->K, std::floor(budget / per)));
-    // device tables and scratch (never inside a captured graph: a graph is
-    // captured after one uncaptured call of the same shape)
+    for (int p = 0; p < m.P; ++p) m.xnode[p] = std::cos(kPi * (p + 0.5) / m.P);
+    return true;
+}
+
+// Device memory of one table (bytes) and of S of them at a time; the captures'
+// tables `snap` and the node polynomials (never inside a captured graph: a
+// graph is captured after one uncaptured call of the same shape).
+static double map_bytes(const MapPlan &m)
+{
+    return 8.0 * ((double)m.ntile * m.Cmax * ((size_t)1 << m.logn) + (double)m.Cmax * m.P * m.NLpad +
+                  (double)m.Q * m.NLpad + (double)m.Cmax * m.Q);
+}
+static dg_status map_buffers(dg_ctx *c, const MapPlan &m, size_t S, const std::vector<MapSnap> &snap)
+{
     MapBufs &d = c->mb;
+    const size_t n = (size_t)1 << m.logn;
     dg_status st;
-    const size_t S = (size_t)m.S;
-    if ((st = ensure(c, (void **)&d.snap, &d.snap_cap, sizeof(MapSnap) * (size_t)c->K)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&d.snap, &d.snap_cap, sizeof(MapSnap) * snap.size())) != DG_OK) return st;
     if ((st = ensure(c, (void **)&d.tw, &d.tw_cap, sizeof(float2) * n)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&d.T, &d.T_cap, sizeof(float) * (size_t)m.P * m.Q)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&d.F2, &d.F2_cap, sizeof(float2) * S * m.ntile * m.Cmax * n)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&d.U, &d.U_cap, sizeof(float2) * S * m.Cmax * m.P * m.NLpad)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&d.X, &d.X_cap, sizeof(float2) * S * m.Q * m.NLpad)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&d.phase, &d.phase_cap, sizeof(float2) * S * m.Cmax * m.Q)) != DG_OK) return st;
-    if (m.c64 && (st = ensure(c, (void **)&d.bad, &d.bad_cap, sizeof(int) * 4 * S)) != DG_OK) return st;
-    if (pr) {
-        const size_t fb = sizeof(float) * kPolyTerms * kPolyPts;
-        if ((st = ensure(c, (void **)&d.fit, &d.fit_cap, fb)) != DG_OK) return st;
-        if ((st = ensure(c, (void **)&d.coef, &d.coef_cap, sizeof(float) * kPolyStride * (size_t)ptiles * S)) != DG_OK)
-            return st;
-        if (d.fit_rows != pr) {
-            const std::vector<float> fit = poly_fit(m.poly);
-            CK(c, cudaMemcpyAsync(d.fit, fit.data(), fb, cudaMemcpyHostToDevice, c->stream));
-            d.fit_rows = pr;
-        }
-    }
+    if (m.c64 && (st = ensure(c, (void **)&d.bad, &d.bad_cap, sizeof(int) * 4 * (size_t)c->K)) != DG_OK) return st;
     if ((st = ensure_ephf(c)) != DG_OK) return st;
     // pageable sources: staged before the calls return
     CK(c, cudaMemcpyAsync(d.snap, snap.data(), sizeof(MapSnap) * snap.size(), cudaMemcpyHostToDevice, c->stream));
@@ -1237,7 +1252,6 @@ static dg_status map_plan(dg_ctx *c)
         ++c->launches;
         d.tw_logn = m.logn;
     }
-    for (int p = 0; p < m.P; ++p) m.xnode[p] = std::cos(kPi * (p + 0.5) / m.P);
     if (d.T_P != m.P || d.T_Q != m.Q) {
         std::vector<float> T((size_t)m.P * m.Q);
         for (int p = 0; p < m.P; ++p)
@@ -1252,8 +1266,113 @@ static dg_status map_plan(dg_ctx *c)
         d.T_P = m.P;
         d.T_Q = m.Q;
     }
+    return DG_OK;
+}
+
+// The chunk the contraction would take for the context's grid (what
+// dg_cdft_chunks reports whichever way the surface is computed), and whether
+// its per-lag DFT buffer would stay within the limit of cdft_setup.
+static bool map_chunks(dg_ctx *c, int *lo, int *hi)
+{
+    CdftBufs &b = c->cd;
+    if (b.main_span.size() != (size_t)c->K || b.main_lags.size() != (size_t)c->K ||
+        b.main_range.size() != (size_t)c->K)
+        fdoa_spans(c, c->gd, b.main_span, &b.main_lags, &b.main_range);
+    CdftLayout L;
+    std::vector<int> bb, gb;
+    if (cdft_batches(c, c->G, grid_diameter(c->gd), L, bb, gb) != DG_OK) return false;
+    const bool tc = c->opt.contract != DG_CONTRACT_FP32;
+    *lo = INT_MAX;
+    *hi = 0;
+    int64_t B = 1;
+    for (const auto &t : L.batches) {
+        const int M = auto_chunk(c, b.main_span, b.main_lags, t.k0, t.S, tc);
+        *lo = std::min(*lo, M);
+        *hi = std::max(*hi, M);
+        for (int s = 0; s < t.S; ++s) B = std::max<int64_t>(B, (c->steps[t.k0 + s].n + M - 1) / M);
+    }
+    return (double)L.nbt_max * (double)B * 512.0 <= (double)((size_t)64 << 30);
+}
+
+static dg_status map_plan(dg_ctx *c)
+{
+    MapPlan &m = c->mp;
+    if (m.gen == c->steps_gen) return DG_OK;
+    m = MapPlan{};
+    m.gen = c->steps_gen;  // whatever the outcome, it holds until the shapes change
+    CdftBufs &b = c->cd;
+    if (!map_chunks(c, &m.chunk_min, &m.chunk_max)) return DG_OK;
+    std::vector<MapSnap> snap;
+    if (!map_shape(c, b.main_range, snap, m)) return DG_OK;
+    for (int k = 0; k < c->K; ++k) m.rows += (int64_t)snap[k].NL * ((c->steps[k].n + m.Mb - 1) / m.Mb);
+    const int pr = poly_rows(c, snap);
+    if (pr) m.poly = poly_shape(pr);
+    const double ptiles = pr ? std::ceil((double)c->gd.nrows / pr) * std::ceil((double)c->gd.nlon / kPolyCols) : 0.0;
+    const double per = map_bytes(m) + 4.0 * kPolyStride * ptiles;
+    const double budget = (double)(c->opt.scratch_mib ? c->opt.scratch_mib : 12288) * 1048576.0;
+    m.S = (int)std::max(1.0, std::min((double)c->K, std::floor(budget / per)));
+    dg_status st;
+    if (pr) {
+        MapBufs &d = c->mb;
+        const size_t fb = sizeof(float) * kPolyTerms * kPolyPts;
+        if ((st = ensure(c, (void **)&d.fit, &d.fit_cap, fb)) != DG_OK) return st;
+        if ((st = ensure(c, (void **)&d.coef, &d.coef_cap, sizeof(float) * kPolyStride * (size_t)ptiles * m.S)) != DG_OK)
+            return st;
+        if (d.fit_rows != pr) {
+            const std::vector<float> fit = poly_fit(m.poly);
+            CK(c, cudaMemcpyAsync(d.fit, fit.data(), fb, cudaMemcpyHostToDevice, c->stream));
+            d.fit_rows = pr;
+        }
+    }
+    if ((st = map_buffers(c, m, (size_t)m.S, snap)) != DG_OK) return st;
     m.ok = true;
     return DG_OK;
+}
+
+// The arguments every table shares: captures and ephemerides from snapshot k0
+// on, the grid, the geometry's constants.
+static void map_common(dg_ctx *c, int k0, const double *xyz, const GridDev &gd, int64_t G, MapArgs &a)
+{
+    auto split = [](double v, float &h, float &l) {
+        h = (float)v;
+        l = (float)(v - (double)h);
+    };
+    a.sd = c->steps_d + k0;
+    a.xyz = xyz;
+    a.eph = c->eph + 12 * (size_t)k0;
+    a.ephf = c->cd.ephf + 24 * (size_t)k0;
+    split(c->fs / kC, a.fsc_hi, a.fsc_lo);
+    split(1.0 / (c->lambda * c->fs), a.ilf_hi, a.ilf_lo);
+    a.fs = c->fs;
+    a.lambda = c->lambda;
+    a.G = G;
+    a.nrows = gd.nrows;
+    a.nlon = gd.nlon;
+    a.delay = c->opt.delay;
+    a.acc = c->opt.acc;
+    a.err = c->err_d;
+    a.nreg = 1;
+}
+
+// The shape and the scratch of a plan's tables.
+static void map_tables_args(const MapPlan &m, const MapBufs &d, MapArgs &a)
+{
+    a.logn = m.logn;
+    a.Mb = m.Mb;
+    a.Cmax = m.Cmax;
+    a.P = m.P;
+    a.Q = m.Q;
+    a.LT = m.LT;
+    a.ntile = m.ntile;
+    a.NLpad = m.NLpad;
+    a.tw = d.tw;
+    a.T = d.T;
+    std::memcpy(a.xnode, m.xnode, sizeof a.xnode);
+    a.F2 = d.F2;
+    a.U = d.U;
+    a.X = d.X;
+    a.phase = d.phase;
+    a.bad = m.c64 ? d.bad : nullptr;
 }
 
 static dg_status run_surface_map(dg_ctx *c, void *out)
@@ -1265,46 +1384,14 @@ static dg_status run_surface_map(dg_ctx *c, void *out)
     c->cd_chunk_min = m.chunk_min;
     c->cd_chunk_max = m.chunk_max;
     c->last_map = true;
-    auto split = [](double v, float &h, float &l) {
-        h = (float)v;
-        l = (float)(v - (double)h);
-    };
     for (int k0 = 0; k0 < c->K; k0 += m.S) {
         MapArgs a{};
-        a.S = std::min(m.S, c->K - k0);
-        a.sd = c->steps_d + k0;
+        map_common(c, k0, c->xyz, c->gd, c->G, a);
+        a.S = a.ksd = std::min(m.S, c->K - k0);
         a.snap = d.snap + k0;
-        a.xyz = c->xyz;
-        a.eph = c->eph + 12 * (size_t)k0;
-        a.ephf = c->cd.ephf + 24 * (size_t)k0;
-        split(c->fs / kC, a.fsc_hi, a.fsc_lo);
-        split(1.0 / (c->lambda * c->fs), a.ilf_hi, a.ilf_lo);
-        a.fs = c->fs;
-        a.lambda = c->lambda;
-        a.G = c->G;
-        a.nrows = c->gd.nrows;
-        a.nlon = c->gd.nlon;
-        a.logn = m.logn;
-        a.Mb = m.Mb;
-        a.Cmax = m.Cmax;
-        a.P = m.P;
-        a.Q = m.Q;
-        a.LT = m.LT;
-        a.ntile = m.ntile;
-        a.NLpad = m.NLpad;
-        a.delay = c->opt.delay;
-        a.acc = c->opt.acc;
+        map_tables_args(m, d, a);
         a.first = k0 == 0;
-        a.tw = d.tw;
-        a.T = d.T;
-        std::memcpy(a.xnode, m.xnode, sizeof a.xnode);
-        a.F2 = d.F2;
-        a.U = d.U;
-        a.X = d.X;
-        a.phase = d.phase;
-        a.bad = m.c64 ? d.bad : nullptr;
         a.out = (float *)out;
-        a.err = c->err_d;
         a.poly = m.poly;
         a.fit = d.fit;
         a.coef = d.coef;
@@ -1327,6 +1414,142 @@ static dg_status run_surface_map(dg_ctx *c, void *out)
         }
     }
     CK(c, cudaMemcpyAsync(c->err_h, c->err_d, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+    return DG_OK;
+}
+
+// The least distance between the grid's nodes and the receivers of any
+// snapshot, less half the receivers' separation (0: no bound), and the
+// largest separation and relative motion. From 3 x 3 nodes where the grid is
+// small against its range (half a cell off at most), else 17 x 17.
+struct RefineBound {
+    double rho = 1e300, sep = 0.0, vel = 0.0, dv = 0.0;
+};
+static RefineBound refine_bound(const dg_ctx *c)
+{
+    for (int side : {3, 17}) {
+        RefineBound b;
+        const GridDev &g = c->gd;
+        const int ni = std::min(side, g.nrows), nj = std::min(side, g.nlon);
+        std::vector<double> p(3 * (size_t)ni * nj);
+        for (int i = 0; i < ni; ++i)
+            for (int j = 0; j < nj; ++j)
+                host_node_ecef(g, g.row0 + (ni > 1 ? (double)i * (g.nrows - 1) / (ni - 1) : 0.0),
+                               nj > 1 ? (double)j * (g.nlon - 1) / (nj - 1) : 0.0, &p[3 * ((size_t)i * nj + j)]);
+        auto norm = [](double x, double y, double z) { return std::sqrt(x * x + y * y + z * z); };
+        double hi = 0.0, hj = 0.0, rmin = 1e300;
+        for (int i = 0; i < ni; ++i)
+            for (int j = 0; j < nj; ++j) {
+                const double *x = &p[3 * ((size_t)i * nj + j)];
+                if (i + 1 < ni) hi = std::max(hi, norm(x[0] - x[3 * nj], x[1] - x[3 * nj + 1], x[2] - x[3 * nj + 2]));
+                if (j + 1 < nj) hj = std::max(hj, norm(x[0] - x[3], x[1] - x[4], x[2] - x[5]));
+                for (int k = 0; k < c->K; ++k) {
+                    const dg_ephem &e = c->eph_host[k];
+                    rmin = std::min(rmin, std::min(norm(e.p1[0] - x[0], e.p1[1] - x[1], e.p1[2] - x[2]),
+                                                   norm(e.p2[0] - x[0], e.p2[1] - x[1], e.p2[2] - x[2])));
+                }
+            }
+        for (int k = 0; k < c->K; ++k) {
+            const dg_ephem &e = c->eph_host[k];
+            b.sep = std::max(b.sep, norm(e.p2[0] - e.p1[0], e.p2[1] - e.p1[1], e.p2[2] - e.p1[2]));
+            b.dv = std::max(b.dv, norm(e.v2[0] - e.v1[0], e.v2[1] - e.v1[1], e.v2[2] - e.v1[2]));
+            b.vel = std::max(b.vel, std::max(norm(e.v1[0], e.v1[1], e.v1[2]), norm(e.v2[0], e.v2[1], e.v2[2])));
+        }
+        const double h = 0.55 * std::hypot(hi, hj);
+        b.rho = rmin - h - 0.5 * b.sep;
+        if (b.rho > 0.75 * rmin || side == 17) return b;
+    }
+    return RefineBound{};
+}
+
+// A refinement surface from a table of few lags (k_map_few), planned from the
+// grid's shape and bounds that hold anywhere on the main grid (its centre is
+// known on the device only). *done = false where the shape does not suit it.
+static dg_status refine_map(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *out, bool *done)
+{
+    *done = false;
+    if (!(gd.nlat & 1) || gd.nlat != gd.nlon || gd.nrows != gd.nlat) return DG_OK;  // the centre is a node
+    int nmax = 1;
+    bool c64 = false;
+    for (int k = 0; k < c->K; ++k) {
+        if (c->steps[k].n > (1 << 24) || !c->steps[k].loaded) return DG_OK;
+        nmax = std::max(nmax, (int)c->steps[k].n);
+        c64 |= c->steps[k].fmt == DG_IQ_C64;
+    }
+    const RefineBound rb = refine_bound(c);
+    // the farthest node: half a diagonal of the lattice in metres, with 2 % for
+    // the parallels' change of radius over up to 20 km at 80 degrees
+    if (std::fabs(c->gd.lat0_rad) + 0.5 * c->gd.nlat * c->gd.dlat_m / 6.33e6 > 1.39) return DG_OK;
+    const double half = (gd.nlat - 1) / 2, r = 1.02 * half * std::hypot(gd.dlat_m, gd.dlon_m);
+    const double rho = rb.rho - r;
+    if (!(rho > 0.0) || r > 2e4) return DG_OK;
+    const double md = rb.sep / rho * c->fs / kC * r;
+    const double mn = (rb.dv / rho + 3.0 * rb.vel * rb.sep / (rho * rho)) / (c->lambda * c->fs) * r;
+    const bool frac = c->opt.delay != DG_DELAY_INTEGER;
+    const double nl = std::ceil(2.0 * md + 1.02) + 2.0 + (frac ? 3.0 : 0.0);
+    const double w = 2.0 * mn * (1.0 + 1e-5) + 1e-13;
+    // the most bins the tables hold: the six that pad the stencils then widen the
+    // band least (at 8 bins it would be 3.5 times the FDOAs' own)
+    if (nl > kFewMaxLags || 6.0 + std::ceil(w * nmax / kMapNDelta) > kFewMaxBins) return DG_OK;
+    MapArgs a{};
+    MapFew f{};
+    a.Q = kFewMaxBins;
+    a.LT = (int)nl;
+    f.delta = w / (a.Q - 6);
+    f.halfw = 0.5 * (a.Q - 1) * f.delta;
+    f.md = md;
+    f.centre = (G - 1) / 2;
+    // terms of the Chebyshev series over the longest capture (the tail is at
+    // most 2 |J_P(theta)|: map_nodes' bound, for capture = block)
+    const int need = map_nodes(f.halfw, nmax);
+    if (need == 0 || need > kFewMaxNodes) return DG_OK;
+    a.P = need <= 4 ? 4 : need <= 6 ? 6 : 8;
+    a.NLpad = 32;
+    a.S = a.ksd = c->K;
+    f.tscale = 2.0f / (float)(nmax + 1);
+    // CTAs per snapshot: four per SM over all snapshots, a block of samples each at least
+    a.Cmax = std::max(1, std::min((nmax + kFewBlock - 1) / kFewBlock, (4 * c->sm_count + c->K - 1) / c->K));
+    const size_t u = sizeof(float) * map_few_partials(a.P, a.LT) * (size_t)a.Cmax * c->K;
+    if (u > ((size_t)1 << 32) || (c->opt.scratch_mib && (double)u > c->opt.scratch_mib * 1048576.0)) return DG_OK;
+    dg_status st = push_steps(c);
+    if (st != DG_OK) return st;
+    MapBufs &d = c->mr;
+    if ((st = ensure(c, (void **)&d.snap, &d.snap_cap, sizeof(MapSnap) * (size_t)c->K)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&d.U, &d.U_cap, u)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&d.X, &d.X_cap, sizeof(float2) * (size_t)c->K * a.Q * a.NLpad)) != DG_OK) return st;
+    if (c64 && (st = ensure(c, (void **)&d.bad, &d.bad_cap, sizeof(int) * 4 * (size_t)c->K)) != DG_OK) return st;
+    if ((st = ensure_ephf(c)) != DG_OK) return st;
+    // e^{j theta_q t} = sum_m j^m T[m][q] T_m(t), theta_q the phase of bin q at
+    // t = 1: the series' real coefficients by a 32-point cosine sum
+    for (int q = 0; q < a.Q; ++q) {
+        const double theta = 2.0 * kPi * (q * f.delta - f.halfw) / f.tscale;
+        for (int m = 0; m < a.P; ++m) {
+            double re = 0.0, im = 0.0;
+            for (int i = 0; i < 32; ++i) {
+                const double phi = kPi * (i + 0.5) / 32.0;
+                re += std::cos(theta * std::cos(phi)) * std::cos(m * phi);
+                im += std::sin(theta * std::cos(phi)) * std::cos(m * phi);
+            }
+            const double w = (m ? 2.0 : 1.0) / 32.0;
+            f.T[m * a.Q + q] = (float)(w * (m % 4 == 0 ? re : m % 4 == 1 ? im : m % 4 == 2 ? -re : -im));
+        }
+    }
+    map_common(c, 0, xyz, gd, G, a);
+    f.snap = d.snap;
+    a.snap = d.snap;
+    a.first = 1;
+    a.U = d.U;
+    a.X = d.X;
+    a.bad = c64 ? d.bad : nullptr;
+    a.out = (float *)out;
+    {
+        Timed t(c, DG_K_REFINE);
+        int n = 1;
+        CK(c, launch_map_few(a, f, c->stream, &n));
+        CK(c, launch_map_lookup(a, c->stream));
+        t.done(n);
+    }
+    CK(c, cudaMemcpyAsync(c->err_h, c->err_d, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+    *done = true;
     return DG_OK;
 }
 
@@ -1372,7 +1595,7 @@ dg_status run_argmax(dg_ctx *c, const void *v, int64_t n, const GridDev &gd, Arg
     int nlaunch = 0;
     {
         Timed t(c, DG_K_ARGMAX);
-        CK(c, launch_argmax(v, n, c->opt.prec, gd, c->amax_tmp, c->amax_res, &nlaunch, c->stream));
+        CK(c, launch_argmax(v, n, c->opt.prec, gd, c->gstep, c->amax_tmp, c->amax_res, &nlaunch, c->stream));
         t.done(nlaunch);
     }
     CK(c, cudaMemcpyAsync(c->amax_host, c->amax_res, sizeof(ArgmaxResult), cudaMemcpyDeviceToHost,
@@ -1503,6 +1726,7 @@ dg_status dg_create(const dg_grid *grid, const dg_ephem *eph, int32_t K, double 
     CKC(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device));
     CKC(cudaMallocAsync((void **)&c->xyz, sizeof(double) * 3 * (size_t)c->G, c->stream));
     c->xyz_cap = c->G;
+    CKC(cudaMallocAsync((void **)&c->gstep, 2 * sizeof(GridStep), c->stream));
     CKC(cudaMallocAsync((void **)&c->eph, sizeof(double) * 12 * (size_t)K, c->stream));
     CKC(cudaMallocAsync((void **)&c->steps_d, sizeof(StepDesc) * (size_t)K, c->stream));
     CKC(cudaMallocAsync((void **)&c->amax_res, sizeof(ArgmaxResult), c->stream));
@@ -1515,7 +1739,7 @@ dg_status dg_create(const dg_grid *grid, const dg_ephem *eph, int32_t K, double 
                         c->stream));
     {
         Timed t(c, DG_K_GRID);
-        CKC(launch_grid_ecef(c->gd, c->xyz, c->stream));
+        CKC(launch_grid_ecef(c->gd, c->xyz, c->stream, nullptr, nullptr, 1, c->gstep));
         t.done(1);
     }
     CKC(cudaStreamSynchronize(c->stream));  // eph_host may not move before the copy ran
@@ -1551,7 +1775,7 @@ dg_status dg_set_grid(dg_ctx *c, const dg_grid *grid)
     ++c->steps_gen;           // graphs and batches recorded on the old grid are stale
     {
         Timed t(c, DG_K_GRID);
-        CK(c, launch_grid_ecef(c->gd, c->xyz, c->stream));
+        CK(c, launch_grid_ecef(c->gd, c->xyz, c->stream, nullptr, nullptr, 1, c->gstep));
         t.done(1);
     }
     return DG_OK;
@@ -1619,9 +1843,10 @@ static dg_status ensure_local(dg_ctx *c, int64_t G)
 {
     const size_t esz = c->opt.prec == DG_PREC_FP64 ? 8 : 4;
     if (c->loc.g_cap < (size_t)G) {
-        if (c->loc.xyz) CK(c, cudaFreeAsync(c->loc.xyz, c->stream));
-        if (c->loc.surf) CK(c, cudaFreeAsync(c->loc.surf, c->stream));
-        if (c->loc.cost) CK(c, cudaFreeAsync(c->loc.cost, c->stream));
+        dg_status st;
+        if ((st = release(c, c->loc.xyz)) != DG_OK || (st = release(c, c->loc.surf)) != DG_OK ||
+            (st = release(c, c->loc.cost)) != DG_OK)
+            return st;
         c->loc = LocalGrid{};
         CK(c, cudaMallocAsync((void **)&c->loc.xyz, sizeof(double) * 3 * G, c->stream));
         CK(c, cudaMallocAsync(&c->loc.surf, esz * G * c->K + 8, c->stream));
@@ -1644,72 +1869,25 @@ static dg_status refine_half(dg_ctx *c, double spacing_m, double window_m, int *
     return DG_OK;
 }
 
+static dg_status ensure_post(dg_ctx *c, int half, dg_fix **fix_dev, dg_fix **fix_host);
+static dg_status step_device_post(dg_ctx *c, const void *cost, double spacing_m, int half, dg_fix *fix_dev,
+                                  dg_fix *fix_host);
+static dg_status read_fix(dg_ctx *c, const dg_fix *fix_host, dg_fix *out);
+
 dg_status dg_argmax_refine(dg_ctx *c, const void *cost, double spacing_m, double window_m, dg_fix *out)
 {
     if (!c) return fail(nullptr, DG_EINVAL, "ctx is NULL");
     c->err.clear();
     if (!cost || !out) return fail(c, DG_EINVAL, "cost and out must not be NULL");
-    const bool refine = spacing_m > 0 && window_m >= spacing_m;
     int half = 0;
-    if (refine) {
-        if (!(std::isfinite(spacing_m) && std::isfinite(window_m)))
-            return fail(c, DG_EINVAL, "refinement spacing and window must be finite");
-        const double h = std::floor(window_m / spacing_m + 0.5);
-        if (h > 2000) return fail(c, DG_EINVAL, "refinement grid wider than 4001 nodes");
-        half = (int)h;
-    }
-    CK(c, cudaStreamSynchronize(c->stream));
-    dg_status st = check_latched(c);
+    dg_status st = refine_half(c, spacing_m, window_m, &half);
     if (st != DG_OK) return st;
-    ArgmaxResult r;
-    st = run_argmax(c, cost, c->G, c->gd, &r);
-    if (st != DG_OK) return st;
-    if (r.idx < 0) return fail(c, DG_EINVAL, "the surface holds no finite value");
+    // the step of a captured graph, uncaptured: the refinement grid is centred
+    // on the argmax on the device and one synchronisation reads the fix
+    if ((st = ensure_post(c, half, &c->fix_dev_sync, &c->fix_host_sync)) != DG_OK) return st;
+    if ((st = step_device_post(c, cost, spacing_m, half, c->fix_dev_sync, c->fix_host_sync)) != DG_OK) return st;
     dg_fix f;
-    std::memset(&f, 0, sizeof f);
-    f.index = r.idx;
-    f.i = c->gd.row0 + (int)(r.idx / c->gd.nlon);
-    f.j = (int)(r.idx % c->gd.nlon);
-    f.lat_deg = r.lat_rad * (180.0 / kPi);
-    f.lon_deg = r.lon_rad * (180.0 / kPi);
-    f.cost = r.val;
-    f.sub_lat_deg = r.sub_lat_rad * (180.0 / kPi);
-    f.sub_lon_deg = r.sub_lon_rad * (180.0 / kPi);
-    if (refine) {
-        const int n = 2 * half + 1;
-        dg_grid lg;
-        lg.lat0_deg = f.lat_deg;
-        lg.lon0_deg = f.lon_deg;
-        lg.dlat_m = spacing_m;
-        lg.dlon_m = spacing_m;
-        lg.nlat = n;
-        lg.nlon = n;
-        const GridDev lgd = make_griddev(lg, 0, n);
-        const int64_t G = (int64_t)n * n;
-        if ((st = ensure_local(c, G)) != DG_OK) return st;
-        {
-            Timed t(c, DG_K_REFINE);
-            CK(c, launch_grid_ecef(lgd, c->loc.xyz, c->stream));
-            t.done(1);
-        }
-        st = run_surface(c, lgd, c->loc.xyz, G, c->loc.surf, c->loc.cost, true);
-        if (st != DG_OK) return st;
-        CK(c, cudaStreamSynchronize(c->stream));
-        st = check_latched(c);
-        if (st != DG_OK) return st;
-        ArgmaxResult q;
-        st = run_argmax(c, c->loc.cost, G, lgd, &q);
-        if (st != DG_OK) return st;
-        if (q.idx < 0) return fail(c, DG_EINVAL, "the refinement surface holds no finite value");
-        f.refine_n = n;
-        f.ri = (int)(q.idx / n);
-        f.rj = (int)(q.idx % n);
-        f.refined_lat_deg = q.lat_rad * (180.0 / kPi);
-        f.refined_lon_deg = q.lon_rad * (180.0 / kPi);
-        f.refined_cost = q.val;
-        f.sub_lat_deg = q.sub_lat_rad * (180.0 / kPi);
-        f.sub_lon_deg = q.sub_lon_rad * (180.0 / kPi);
-    }
+    if ((st = read_fix(c, c->fix_host_sync, &f)) != DG_OK) return st;
     *out = f;
     return DG_OK;
 }
@@ -1780,6 +1958,21 @@ dg_status dg_detect(dg_ctx *c, const void *cost, double threshold, int32_t relat
 // Whole steps as CUDA graphs
 // ---------------------------------------------------------------------------
 
+// Buffers of a step after its surface (allocated outside any capture).
+static dg_status ensure_post(dg_ctx *c, int half, dg_fix **fix_dev, dg_fix **fix_host)
+{
+    const int n = 2 * half + 1;
+    const int64_t Gl = half > 0 ? (int64_t)n * n : 0;
+    dg_status st;
+    if ((st = ensure(c, &c->amax_tmp, &c->amax_tmp_bytes, argmax_tmp_bytes(std::max<int64_t>(c->G, Gl)))) != DG_OK)
+        return st;
+    if (half > 0 && (st = ensure_local(c, Gl)) != DG_OK) return st;
+    if (!c->amax_fine) CK(c, cudaMallocAsync((void **)&c->amax_fine, sizeof(ArgmaxResult), c->stream));
+    if (!*fix_dev) CK(c, cudaMallocAsync((void **)fix_dev, sizeof(dg_fix), c->stream));
+    if (!*fix_host) CK(c, cudaMallocHost((void **)fix_host, sizeof(dg_fix)));
+    return DG_OK;
+}
+
 // Buffers a device-only step needs (allocated outside any capture).
 static dg_status prepare_step(dg_ctx *c, int half)
 {
@@ -1787,14 +1980,7 @@ static dg_status prepare_step(dg_ctx *c, int half)
         if (!c->steps[k].loaded) return fail(c, DG_ESTATE, "snapshot %d has not been loaded", k);
     dg_status st = ensure_surf(c);
     if (st != DG_OK) return st;
-    const int n = 2 * half + 1;
-    const int64_t Gl = half > 0 ? (int64_t)n * n : 0;
-    if ((st = ensure(c, &c->amax_tmp, &c->amax_tmp_bytes, argmax_tmp_bytes(std::max<int64_t>(c->G, Gl)))) != DG_OK)
-        return st;
-    if (half > 0 && (st = ensure_local(c, Gl)) != DG_OK) return st;
-    if (!c->amax_fine) CK(c, cudaMallocAsync((void **)&c->amax_fine, sizeof(ArgmaxResult), c->stream));
-    if (!c->fix_dev) CK(c, cudaMallocAsync((void **)&c->fix_dev, sizeof(dg_fix), c->stream));
-    if (!c->fix_host) CK(c, cudaMallocHost((void **)&c->fix_host, sizeof(dg_fix)));
+    if ((st = ensure_post(c, half, &c->fix_dev, &c->fix_host)) != DG_OK) return st;
     return push_steps(c);
 }
 
@@ -1802,23 +1988,26 @@ static dg_status prepare_step(dg_ctx *c, int half)
 // refinement grid centred on it (built on the device), the refinement
 // surface and argmax, and the fix record copied to the pinned fix_host. No
 // host synchronisation and no allocation (prepare_step ran before).
-static dg_status step_device_post(dg_ctx *c, void *cost, double spacing_m, int half);
-
 static dg_status step_device(dg_ctx *c, void *cost, double spacing_m, int half)
 {
     dg_status st = run_surface(c, c->gd, c->xyz, c->G, c->surf, cost, false);
     if (st != DG_OK) return st;
-    return step_device_post(c, cost, spacing_m, half);
+    return step_device_post(c, cost, spacing_m, half, c->fix_dev, c->fix_host);
 }
 
 // The rest of a step once the surface is enqueued: its argmax, the
 // refinement, the fix record.
-static dg_status step_device_post(dg_ctx *c, void *cost, double spacing_m, int half)
+static dg_status step_device_post(dg_ctx *c, const void *cost, double spacing_m, int half, dg_fix *fix_dev,
+                                  dg_fix *fix_host)
 {
     dg_status st = DG_OK;
-    int nl = 0;
-    CK(c, launch_argmax(cost, c->G, c->opt.prec, c->gd, c->amax_tmp, c->amax_res, &nl, c->stream));
-    const ArgmaxResult *fine = nullptr;
+    {
+        Timed t(c, DG_K_ARGMAX);
+        int nl = 0;
+        CK(c, launch_argmax(cost, c->G, c->opt.prec, c->gd, c->gstep, c->amax_tmp, c->amax_res, &nl, c->stream, nullptr,
+                            nullptr, 1, FixOut{half > 0 ? nullptr : fix_dev, nullptr, c->gd, 0}));
+        t.done(nl);
+    }
     const int n = 2 * half + 1;
     if (half > 0) {
         dg_grid lg;
@@ -1828,30 +2017,34 @@ static dg_status step_device_post(dg_ctx *c, void *cost, double spacing_m, int h
         lg.nlat = lg.nlon = n;
         const GridDev lgd = make_griddev(lg, 0, n);
         const int64_t Gl = (int64_t)n * n;
-        CK(c, launch_grid_ecef(lgd, c->loc.xyz, c->stream, c->amax_res));
-        ++nl;
+        {
+            Timed t(c, DG_K_REFINE);
+            CK(c, launch_grid_ecef(lgd, c->loc.xyz, c->stream, c->amax_res, nullptr, 1, c->gstep + 1));
+            t.done(1);
+        }
         st = run_surface(c, lgd, c->loc.xyz, Gl, c->loc.surf, c->loc.cost, true);
         if (st != DG_OK) return st;
-        CK(c, launch_argmax(c->loc.cost, Gl, c->opt.prec, lgd, c->amax_tmp, c->amax_fine, &nl, c->stream,
-                            c->amax_res));
-        fine = c->amax_fine;
+        {
+            Timed t(c, DG_K_ARGMAX);
+            int nl = 0;
+            CK(c, launch_argmax(c->loc.cost, Gl, c->opt.prec, lgd, c->gstep + 1, c->amax_tmp, c->amax_fine, &nl, c->stream,
+                                c->amax_res, nullptr, 1, FixOut{fix_dev, c->amax_res, c->gd, n}));
+            t.done(nl);
+        }
     }
-    CK(c, launch_make_fix(c->amax_res, fine, c->gd, half > 0 ? n : 0, c->fix_dev, c->stream));
-    ++nl;
-    c->launches += nl;
-    CK(c, cudaMemcpyAsync(c->fix_host, c->fix_dev, sizeof(dg_fix), cudaMemcpyDeviceToHost, c->stream));
+    CK(c, cudaMemcpyAsync(fix_host, fix_dev, sizeof(dg_fix), cudaMemcpyDeviceToHost, c->stream));
     return DG_OK;
 }
 
-static dg_status read_fix(dg_ctx *c, dg_fix *out)
+static dg_status read_fix(dg_ctx *c, const dg_fix *fix_host, dg_fix *out)
 {
     CK(c, cudaStreamSynchronize(c->stream));
     dg_status st = check_latched(c);
     if (st != DG_OK) return st;
-    if (c->fix_host->index < 0) return fail(c, DG_EINVAL, "the surface holds no finite value");
-    if (c->fix_host->refine_n > 0 && c->fix_host->ri < 0)
+    if (fix_host->index < 0) return fail(c, DG_EINVAL, "the surface holds no finite value");
+    if (fix_host->refine_n > 0 && fix_host->ri < 0)
         return fail(c, DG_EINVAL, "the refinement surface holds no finite value");
-    *out = *c->fix_host;
+    *out = *fix_host;
     return DG_OK;
 }
 
@@ -2016,7 +2209,8 @@ static dg_status capture_steps(dg_ctx *const *ctxs, int n, void *const *costs, d
     if (rounds && e == cudaSuccess) st = shared_surfaces(ctxs, n, costs, *rounds, stream, &shared);
     for (int i = 0; i < n && e == cudaSuccess && st == DG_OK; ++i) {
         dg_ctx *c = ctxs[i];
-        st = rounds ? step_device_post(c, costs[i], spacing_m, half[i]) : step_device(c, costs[i], spacing_m, half[i]);
+        st = rounds ? step_device_post(c, costs[i], spacing_m, half[i], c->fix_dev, c->fix_host)
+                    : step_device(c, costs[i], spacing_m, half[i]);
         if (st == DG_OK) e = cudaEventRecord(join[i], c->stream);
         if (e == cudaSuccess && st == DG_OK) e = cudaStreamWaitEvent(stream, join[i], 0);
     }
@@ -2058,12 +2252,13 @@ dg_status dg_graph_capture(dg_ctx *c, void *cost, double spacing_m, double windo
     if ((st = prepare_step(c, half)) != DG_OK) return st;
     if ((st = step_device(c, cost, spacing_m, half)) != DG_OK) return st;
     dg_fix f;
-    if ((st = read_fix(c, &f)) != DG_OK) return st;
+    if ((st = read_fix(c, c->fix_host, &f)) != DG_OK) return st;
     dg_ctx *const cs[1] = {c};
     void *const costs[1] = {cost};
     if ((st = capture_steps(cs, 1, costs, spacing_m, &half, c->stream, &c->graph, &c->graph_launches)) != DG_OK)
         return st;
     c->graph_gen = c->steps_gen;
+    c->captured = true;
     return DG_OK;
 }
 
@@ -2085,7 +2280,7 @@ dg_status dg_graph_fix(dg_ctx *c, dg_fix *out)
     c->err.clear();
     if (!out) return fail(c, DG_EINVAL, "out is NULL");
     if (!c->fix_host) return fail(c, DG_ESTATE, "no step has run");
-    return read_fix(c, out);
+    return read_fix(c, c->fix_host, out);
 }
 
 }  // extern "C" (reopened below)
@@ -2125,7 +2320,7 @@ dg_status dg_batch_capture(dg_ctx *const *ctxs, int32_t n, void *const *costs, d
         if (st == DG_OK) st = prepare_step(c, half[i]);
         if (st == DG_OK) st = step_device(c, costs[i], spacing_m, half[i]);
         dg_fix f;
-        if (st == DG_OK) st = read_fix(c, &f);
+        if (st == DG_OK) st = read_fix(c, c->fix_host, &f);
         if (st != DG_OK) return fail(nullptr, st, "context %d: %s", i, c->err.c_str());
     }
     dg_batch *b = new (std::nothrow) dg_batch();
@@ -2152,6 +2347,7 @@ dg_status dg_batch_capture(dg_ctx *const *ctxs, int32_t n, void *const *costs, d
         delete b;
         return fail(nullptr, st, "%s", m.c_str());
     }
+    for (int i = 0; i < n; ++i) ctxs[i]->captured = true;
     *out = b;
     return DG_OK;
 }
@@ -2181,7 +2377,7 @@ dg_status dg_batch_fixes(dg_batch *b, dg_fix *out)
     if (e != cudaSuccess) return fail(nullptr, DG_ECUDA, "cudaStreamSynchronize: %s", cudaGetErrorString(e));
     dg_status worst = DG_OK;
     for (size_t i = 0; i < b->ctxs.size(); ++i) {
-        dg_status st = read_fix(b->ctxs[i], &out[i]);
+        dg_status st = read_fix(b->ctxs[i], b->ctxs[i]->fix_host, &out[i]);
         if (st != DG_OK) {
             std::memset(&out[i], 0, sizeof(dg_fix));
             out[i].index = -1;
@@ -2424,6 +2620,10 @@ int64_t dg_launch_count(const dg_ctx *c) { return c ? c->launches : -1; }
 dg_status dg_cdft_chunks(const dg_ctx *c, int32_t *min_chunk, int32_t *max_chunk)
 {
     if (!c) return DG_EINVAL;
+    if (c->cd_chunk_max < 0) {  // the last surfaces were regions': the grid the context was left on
+        dg_ctx *m = const_cast<dg_ctx *>(c);
+        if (!map_chunks(m, &m->cd_chunk_min, &m->cd_chunk_max)) m->cd_chunk_min = m->cd_chunk_max = 0;
+    }
     const bool any = c->cd_chunk_max > 0;
     if (min_chunk) *min_chunk = any ? c->cd_chunk_min : 0;
     if (max_chunk) *max_chunk = any ? c->cd_chunk_max : 0;
@@ -2458,7 +2658,10 @@ dg_status dg_destroy(dg_ctx *c)
     auto fr = [&](void *p) {
         if (p) cudaFreeAsync(p, s);
     };
+    for (void *p : c->retired) fr(p);
     fr(c->xyz);
+    fr(c->gstep);
+    fr(c->reg_steps);
     fr(c->eph);
     fr(c->steps_d);
     fr(c->surf);
@@ -2466,6 +2669,7 @@ dg_status dg_destroy(dg_ctx *c)
     fr(c->amax_res);
     fr(c->amax_fine);
     fr(c->fix_dev);
+    fr(c->fix_dev_sync);
     if (c->graph) cudaGraphExecDestroy(c->graph);
     fr(c->err_d);
     fr(c->det_count);
@@ -2484,6 +2688,12 @@ dg_status dg_destroy(dg_ctx *c)
     fr(c->mb.X);
     fr(c->mb.phase);
     fr(c->mb.bad);
+    fr(c->reg_xyz);
+    fr(c->reg_grids);
+    fr(c->mr.snap);
+    fr(c->mr.U);
+    fr(c->mr.X);
+    fr(c->mr.bad);
     fr(c->mb.fit);
     fr(c->mb.coef);
     fr(c->co.lag);
@@ -2530,6 +2740,7 @@ dg_status dg_destroy(dg_ctx *c)
     if (c->amax_host) cudaFreeHost(c->amax_host);
     if (c->reg_host) cudaFreeHost(c->reg_host);
     if (c->fix_host) cudaFreeHost(c->fix_host);
+    if (c->fix_host_sync) cudaFreeHost(c->fix_host_sync);
     if (c->err_h) cudaFreeHost(c->err_h);
     delete c;
     if (e != cudaSuccess) return fail(nullptr, DG_ECUDA, "dg_destroy: %s", cudaGetErrorString(e));
@@ -2673,6 +2884,133 @@ dg_status dg_coarse_inspect(dg_ctx *c, float *caf, dg_coarse_step *steps, int32_
 // ---------------------------------------------------------------------------
 // Search of several regions with one host synchronisation.
 // ---------------------------------------------------------------------------
+
+// Bounds of D and the FDOA over a region in every snapshot from 3 x 3 nodes of
+// it (field_curvature); false where none hold.
+static bool region_range(const dg_ctx *c, const GridDev &g, GridRange *out)
+{
+    if (std::fabs(g.lat0_rad) + 0.5 * g.nlat * g.dlat_m / 6.33e6 > 1.39) return false;
+    double p[9][3], hi = 0.0, hj = 0.0;
+    auto norm = [](double x, double y, double z) { return std::sqrt(x * x + y * y + z * z); };
+    auto dist = [&](int a, int b) { return norm(p[a][0] - p[b][0], p[a][1] - p[b][1], p[a][2] - p[b][2]); };
+    for (int q = 0; q < 9; ++q) host_node_ecef(g, 0.5 * (q / 3) * (g.nlat - 1), 0.5 * (q % 3) * (g.nlon - 1), p[q]);
+    for (int q = 0; q < 9; ++q) {
+        if (q < 6) hi = std::max(hi, dist(q, q + 3));
+        if (q % 3 < 2) hj = std::max(hj, dist(q, q + 1));
+    }
+    const double h = 0.5 * 1.05 * std::hypot(hi, hj) + 1.0;
+    const double fc = c->fs / kC, lf = c->lambda * c->fs;
+    for (int k = 0; k < c->K; ++k) {
+        const dg_ephem &e = c->eph_host[k];
+        GridRange R{};
+        R.d_lo = R.nu_lo = 1e300;
+        R.d_hi = R.nu_hi = -1e300;
+        double rmin = 1e300;
+        for (int q = 0; q < 9; ++q) {
+            double rho[2], uv[2];
+            for (int t = 0; t < 2; ++t) {
+                const double *pp = t ? e.p2 : e.p1, *vv = t ? e.v2 : e.v1;
+                const double x = pp[0] - p[q][0], y = pp[1] - p[q][1], z = pp[2] - p[q][2];
+                rho[t] = norm(x, y, z);
+                uv[t] = (x * vv[0] + y * vv[1] + z * vv[2]) / rho[t];
+            }
+            const double D = (rho[1] - rho[0]) * fc, nu = (uv[0] - uv[1]) / lf;
+            R.d_lo = std::min(R.d_lo, D);
+            R.d_hi = std::max(R.d_hi, D);
+            R.nu_lo = std::min(R.nu_lo, nu);
+            R.nu_hi = std::max(R.nu_hi, nu);
+            rmin = std::min(rmin, std::min(rho[0], rho[1]));
+        }
+        const double sep = norm(e.p2[0] - e.p1[0], e.p2[1] - e.p1[1], e.p2[2] - e.p1[2]);
+        const double dv = norm(e.v2[0] - e.v1[0], e.v2[1] - e.v1[1], e.v2[2] - e.v1[2]);
+        const double v = std::max(norm(e.v1[0], e.v1[1], e.v1[2]), norm(e.v2[0], e.v2[1], e.v2[2]));
+        const double m = rmin - h - 0.5 * sep;
+        if (!(m > 0.0)) return false;
+        const Curvature q = field_curvature(c, m, sep, v, dv);
+        R.d_lo -= 0.5 * q.d * h * h;
+        R.d_hi += 0.5 * q.d * h * h;
+        R.nu_lo -= 0.5 * q.nu * h * h;
+        R.nu_hi += 0.5 * q.nu * h * h;
+        out[k] = R;
+    }
+    return true;
+}
+
+// The surfaces and argmax records of all regions through shared launches:
+// table s of the batch is of capture s % K and region s / K. *done = false
+// where the maps do not serve these regions.
+static dg_status regions_map(dg_ctx *c, const dg_grid *regions, int n, float *costs, bool *done)
+{
+    *done = false;
+    const int64_t G = (int64_t)regions[0].nlat * regions[0].nlon;
+    if (!map_options(c) || G < kMapMinNodes || c->gd.row0 != 0 || c->gd.nrows != c->grid.nlat) return DG_OK;
+    const size_t K = (size_t)c->K;
+    std::vector<GridDev> grids((size_t)n);
+    std::vector<GridRange> range(K * (size_t)n);
+    for (int r = 0; r < n; ++r) {
+        grids[(size_t)r] = make_griddev(regions[r], 0, regions[r].nlat);
+        if (!region_range(c, grids[(size_t)r], &range[K * (size_t)r])) return DG_OK;
+    }
+    MapPlan m;
+    std::vector<MapSnap> snap;
+    if (!map_shape(c, range, snap, m)) return DG_OK;
+    const double budget = (double)(c->opt.scratch_mib ? c->opt.scratch_mib : 12288) * 1048576.0;
+    const int nr = (int)std::min((double)std::min(n, (int)(65535 / K)), std::floor(budget / ((double)K * map_bytes(m))));
+    if (nr < 1) return DG_OK;
+    dg_status st;
+    c->mp.gen = 0;  // the tables of the main grid's plan are replaced
+    if ((st = map_buffers(c, m, K * (size_t)nr, snap)) != DG_OK) return st;
+    if ((st = push_steps(c)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&c->reg_xyz, &c->reg_xyz_cap, sizeof(double) * 3 * (size_t)G * nr)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&c->reg_grids, &c->reg_grids_cap, sizeof(GridDev) * (size_t)n)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&c->reg_steps, &c->reg_steps_cap, sizeof(GridStep) * (size_t)nr)) != DG_OK) return st;
+    if ((st = ensure(c, &c->amax_tmp, &c->amax_tmp_bytes, argmax_tmp_bytes(G) * (size_t)nr)) != DG_OK) return st;
+    CK(c, cudaMemcpyAsync(c->reg_grids, grids.data(), sizeof(GridDev) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
+    for (int r0 = 0; r0 < n; r0 += nr) {
+        const int R = std::min(nr, n - r0);
+        {
+            Timed t(c, DG_K_GRID);
+            CK(c, launch_grid_ecef(grids[0], c->reg_xyz, c->stream, nullptr, c->reg_grids + r0, R, c->reg_steps));
+            t.done(1);
+        }
+        MapArgs a{};
+        map_common(c, 0, c->reg_xyz, grids[0], G, a);
+        map_tables_args(m, c->mb, a);
+        a.ksd = c->K;
+        a.nreg = R;
+        a.S = c->K * R;
+        a.snap = c->mb.snap + K * (size_t)r0;
+        a.first = 1;
+        a.out = costs + G * r0;
+        {
+            Timed t(c, DG_K_CDFT_CONTRACT);
+            int nl = 1;
+            CK(c, launch_map_tables(a, c->stream, &nl));
+            CK(c, launch_map_expand(a, c->stream));
+            t.done(nl);
+        }
+        {
+            Timed t(c, DG_K_CDFT_COMBINE);
+            CK(c, launch_map_lookup(a, c->stream));
+            t.done(1);
+        }
+        {
+            Timed t(c, DG_K_ARGMAX);
+            int nl = 0;
+            CK(c, launch_argmax(a.out, G, DG_PREC_FP32, grids[0], c->reg_steps, c->amax_tmp, c->reg_res + r0, &nl, c->stream,
+                                nullptr, c->reg_grids + r0, R));
+            t.done(nl);
+        }
+    }
+    CK(c, cudaMemcpyAsync(c->err_h, c->err_d, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+    c->last_map = true;
+    c->cd_chunk_min = c->cd_chunk_max = -1;
+    c->mp.rows = 0;
+    for (size_t k = 0; k < K; ++k) c->mp.rows += (int64_t)snap[k].NL * ((c->steps[k].n + m.Mb - 1) / m.Mb);
+    *done = true;
+    return DG_OK;
+}
+
 dg_status dg_search_regions(dg_ctx *c, const dg_grid *regions, int32_t n, void *costs, double spacing_m,
                             double window_m, dg_fix *out, int32_t *best)
 {
@@ -2704,7 +3042,9 @@ dg_status dg_search_regions(dg_ctx *c, const dg_grid *regions, int32_t n, void *
         c->reg_cap = (size_t)n;
     }
     dg_status st;
-    for (int r = 0; r < n; ++r) {
+    bool done = false;
+    if ((st = regions_map(c, regions, n, (float *)costs, &done)) != DG_OK) return st;
+    for (int r = 0; r < n && !done; ++r) {
         if ((st = dg_set_grid(c, &regions[r])) != DG_OK) return st;
         if ((st = ensure_surf(c)) != DG_OK) return st;
         if ((st = ensure(c, &c->amax_tmp, &c->amax_tmp_bytes, argmax_tmp_bytes(G))) != DG_OK) return st;
@@ -2713,7 +3053,7 @@ dg_status dg_search_regions(dg_ctx *c, const dg_grid *regions, int32_t n, void *
         int nl = 0;
         {
             Timed t(c, DG_K_ARGMAX);
-            CK(c, launch_argmax(cr, G, c->opt.prec, c->gd, c->amax_tmp, c->reg_res + r, &nl, c->stream));
+            CK(c, launch_argmax(cr, G, c->opt.prec, c->gd, c->gstep, c->amax_tmp, c->reg_res + r, &nl, c->stream));
             t.done(nl);
         }
     }

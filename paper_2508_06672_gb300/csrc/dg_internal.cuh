@@ -291,7 +291,9 @@ struct ArgmaxResult;
 // centre (device, optional): take the grid's centre from an argmax record, as
 // the refinement grid does (its latitude / longitude rounded through degrees
 // exactly as the host would pass them)
-cudaError_t launch_grid_ecef(const GridDev &g, double *xyz, cudaStream_t s, const ArgmaxResult *centre = nullptr);
+// grids (device, optional): ngrids grids of g's size, xyz [ngrids][3][G]
+cudaError_t launch_grid_ecef(const GridDev &g, double *xyz, cudaStream_t s, const ArgmaxResult *centre = nullptr,
+                             const GridDev *grids = nullptr, int ngrids = 1, GridStep *step_out = nullptr);
 
 cudaError_t launch_step_geometry(const GridDev &g, const double *xyz, const double *eph_k,
                                  double fs, double lambda, int delay_mode, int *lag, double *D,
@@ -506,15 +508,16 @@ struct PolyShape {                // of a tile of `rows` x kPolyCols nodes
     int pr[kPolyPts], pc[kPolyPts];  // the sample nodes' offsets in the tile
 };
 struct MapArgs {
-    const StepDesc *sd;           // [S] captures
+    const StepDesc *sd;           // [ksd] captures
     const MapSnap *snap;          // [S]
-    const double *xyz, *eph;      // [3][G] node ECEF, [S][12]
-    const float *ephf;            // [S][24]
+    const double *xyz, *eph;      // [nreg][3][G] node ECEF, [ksd][12]
+    const float *ephf;            // [ksd][24]
     float fsc_hi, fsc_lo, ilf_hi, ilf_lo;  // as in CdftBatch
     double fs, lambda;
     int64_t G;
     int nrows, nlon;
     int S, logn, Mb, Cmax;        // FFT points 2^logn; block of samples; most blocks of a snapshot
+    int ksd, nreg;                // captures: table s is of capture s % ksd; regions: table s is of grid s / ksd
     int P, Q;                     // Doppler nodes per block, bins
     int LT, ntile, NLpad;         // lags per tile, tiles, lag stride (a multiple of 32)
     int delay, acc, first;        // first: the sum starts here (else it continues out)
@@ -522,14 +525,28 @@ struct MapArgs {
     const float *T;               // [P][Q] node polynomials at the bins
     double xnode[kMapMaxNodes];   // Chebyshev nodes on [-1, 1]
     float2 *F2, *U, *X, *phase;   // [S][ntile][Cmax][n], [S][Cmax][P][NLpad], [S][Q][NLpad], [S][Cmax][Q]
-    int *bad;                     // [S][4] first / last sample of y1, y2 that is not finite (NULL: no c64 capture)
-    float *out;                   // [G]
+    int *bad;                     // [ksd][4] first / last sample of y1, y2 that is not finite (NULL: no c64 capture)
+    float *out;                   // [nreg][G]
     unsigned *err;
     PolyShape poly;
     const float *fit;             // [kPolyTerms][kPolyPts] samples -> coefficients
     float *coef;                  // [tiles][S][kPolyStride]
 };
 cudaError_t launch_map_poly(const MapArgs &a, cudaStream_t s);
+
+// Tables of a few lags (a refinement grid) by direct sums over whole
+// captures, centred on one node of the grid on the device. Every node lies
+// within md samples and halfw - 2.5 delta cycles per sample of the centre.
+constexpr int kFewMaxLags = 32, kFewMaxNodes = 8, kFewMaxBins = 16, kFewBlock = 1024;
+struct MapFew {
+    int64_t centre;               // the node
+    double md, halfw, delta;      // bins: centre's FDOA - halfw + q delta
+    float tscale;                 // t = (n - N / 2) tscale in [-1, 1]
+    MapSnap *snap;                // [S], written here
+    float T[kFewMaxNodes * kFewMaxBins];  // [P][Q] Chebyshev series of the bins' phases
+};
+cudaError_t launch_map_few(const MapArgs &a, const MapFew &f, cudaStream_t s, int *launches);
+size_t map_few_partials(int P, int NL);   // floats of U per (snapshot, block)
 cudaError_t launch_map_twiddles(float2 *tw, int logn, cudaStream_t s);
 cudaError_t launch_map_tables(const MapArgs &a, cudaStream_t s, int *launches);
 cudaError_t launch_map_expand(const MapArgs &a, cudaStream_t s);
@@ -558,20 +575,31 @@ struct ArgmaxResult {
 // argmax_tmp_bytes(n) bytes; writes *res (device).
 size_t argmax_tmp_bytes(int64_t n);
 // The refinement grid centred on an argmax record (device): the same
-// degrees round trip as the host's dg_grid of the local grid.
+// degrees round trip as the host's dg_grid of the local grid. A record
+// without a node (every value NaN) leaves the grid's own centre.
 __device__ __forceinline__ void centre_on(GridDev &g, const ArgmaxResult *c)
 {
+    if (c->idx < 0) return;
     g.lat0_rad = (c->lat_rad * (180.0 / kPi)) * (kPi / 180.0);
     g.lon0_rad = (c->lon_rad * (180.0 / kPi)) * (kPi / 180.0);
 }
 
-// The fix of a step from its argmax records (device), as dg_argmax_refine
-// assembles it on the host; fine may be NULL (no refinement, n = 0).
-cudaError_t launch_make_fix(const ArgmaxResult *coarse, const ArgmaxResult *fine, const GridDev &g, int n,
-                            dg_fix *out, cudaStream_t s);
+// Where the last argmax of a step writes the fix of the step (NULL: no fix):
+// with coarse, the record is the refinement's (side n) and coarse the main
+// surface's over grid g; without, the record is the main surface's.
+struct FixOut {
+    dg_fix *fix;
+    const ArgmaxResult *coarse;
+    GridDev g;
+    int n;
+};
 
-cudaError_t launch_argmax(const void *v, int64_t n, int prec, const GridDev &g, void *tmp,
-                          ArgmaxResult *res, int *launches, cudaStream_t s, const ArgmaxResult *centre = nullptr);
+// step (device): the grid's angular steps as launch_grid_ecef wrote them;
+// grids (device, optional): ngrids surfaces of n values, with steps, tmp and
+// res for each
+cudaError_t launch_argmax(const void *v, int64_t n, int prec, const GridDev &g, const GridStep *step, void *tmp,
+                          ArgmaxResult *res, int *launches, cudaStream_t s, const ArgmaxResult *centre = nullptr,
+                          const GridDev *grids = nullptr, int ngrids = 1, FixOut fin = FixOut{});  // grids: ngrids surfaces, tmp and res for each
 
 // ---------------------------------------------------------------------------
 // Coarse delay-Doppler maps back-projected onto the grid's cells (the input

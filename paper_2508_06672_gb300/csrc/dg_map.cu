@@ -261,7 +261,7 @@ template <int LOGN> __global__ void __launch_bounds__((1 << LOGN) / 16) k_map_sp
     constexpr int n = 1 << LOGN, T = n / 16;
     extern __shared__ __align__(16) float2 sm[];
     const int t = threadIdx.x, c = blockIdx.x, tile = blockIdx.y, s = blockIdx.z;
-    const StepDesc sd = a.sd[s];
+    const StepDesc sd = a.sd[s % a.ksd];
     const MapSnap ms = a.snap[s];
     if ((int64_t)c * a.Mb >= sd.n || tile * a.LT >= ms.NL) return;
     if (tile == 0) {  // the block's phases at the bins
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN == 14 ? 1 : LOGN == 13 
     __shared__ float2 s_step[16];
     __shared__ float s_nu[2];
     const int t = threadIdx.x, p = blockIdx.x % a.P, c = blockIdx.x / a.P, tile = blockIdx.y, s = blockIdx.z;
-    const StepDesc sd = a.sd[s];
+    const StepDesc sd = a.sd[s % a.ksd];
     const MapSnap ms = a.snap[s];
     const int64_t n0 = (int64_t)c * a.Mb;
     if (n0 >= sd.n || tile * a.LT >= ms.NL) return;
@@ -355,29 +355,36 @@ __device__ __forceinline__ void cp_async8(void *dst, const void *src)
                  : "memory");
 }
 
-template <int NQ> __global__ void __launch_bounds__(32 * kExpWarps) k_map_expand(MapArgs a)
+// LW of the CTA's warps lie along the lags (32 each), 8 / LW along the bins:
+// narrow tables (few bins) take more lags per CTA. U and the phases are staged
+// kExpRows (block, node) rows at a time, so a stage's barrier is paid once for
+// several blocks where a block has few nodes.
+constexpr int kExpRows = 24;
+template <int NQ, int LW> __global__ void __launch_bounds__(32 * kExpWarps) k_map_expand(MapArgs a)
 {
-    constexpr int NB = NQ * kExpWarps, H = NQ / 2, T = 32 * kExpWarps;
+    constexpr int QW = kExpWarps / LW, NB = NQ * QW, H = NQ / 2, T = 32 * kExpWarps, NLC = 32 * LW;
     extern __shared__ __align__(16) float sm_f[];
     const int s = blockIdx.z, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const StepDesc sd = a.sd[s];
+    const StepDesc sd = a.sd[s % a.ksd];
     const MapSnap ms = a.snap[s];
-    const int qb = blockIdx.y * NB, P = a.P;
-    if (blockIdx.x * 32 >= ms.NL) return;
+    const int qb = blockIdx.y * NB, P = a.P, CS = max(1, kExpRows / P);  // blocks per stage
+    const int l0 = blockIdx.x * NLC;
+    if (l0 >= ms.NL) return;
     float *sT = sm_f;                                              // [P][NB]
-    float2 *sE = reinterpret_cast<float2 *>(sT + P * NB);          // [3][NB]
-    float2 *sU = sE + 3 * NB;                                      // [3][P][32]
-    const int l0 = blockIdx.x * 32;
-    const int C = (sd.n + a.Mb - 1) / a.Mb;
+    float2 *sE = reinterpret_cast<float2 *>(sT + P * NB);          // [3][CS][NB]
+    float2 *sU = sE + 3 * CS * NB;                                 // [3][CS P][NLC]
+    const int C = (sd.n + a.Mb - 1) / a.Mb, NS = (C + CS - 1) / CS;
     const float2 *U = a.U + (size_t)s * a.Cmax * P * a.NLpad + l0;
     const float2 *E = a.phase + (size_t)s * a.Cmax * a.Q;
-    auto stage = [&](int c) {  // block c's U rows and phases, asynchronously
-        if (c < C) {
-            float2 *u = sU + (c % 3) * P * 32;
-            for (int i = threadIdx.x; i < P * 32; i += T)
-                cp_async8(u + i, U + ((size_t)c * P + (i >> 5)) * a.NLpad + (i & 31));
-            for (int i = threadIdx.x; i < NB; i += T)
-                cp_async8(sE + (c % 3) * NB + i, E + (size_t)c * a.Q + min(qb + i, a.Q - 1));
+    const int lw = min(NLC, a.NLpad - l0);  // lags of the tile that exist in U (a multiple of 32)
+    auto stage = [&](int g) {  // the U rows and phases of blocks g CS .. , asynchronously
+        if (g < NS) {
+            const int nc = min(CS, C - g * CS);
+            float2 *u = sU + (g % 3) * CS * P * NLC;
+            for (int i = threadIdx.x; i < nc * P * NLC; i += T)
+                if (i % NLC < lw) cp_async8(u + i, U + ((size_t)g * CS * P + i / NLC) * a.NLpad + i % NLC);
+            for (int i = threadIdx.x; i < nc * NB; i += T)
+                cp_async8(sE + (g % 3) * CS * NB + i, E + (size_t)(g * CS + i / NB) * a.Q + min(qb + i % NB, a.Q - 1));
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -387,43 +394,49 @@ template <int NQ> __global__ void __launch_bounds__(32 * kExpWarps) k_map_expand
         const int q = qb + i % NB;
         sT[i] = q < a.Q ? __ldg(a.T + (i / NB) * a.Q + q) : 0.f;
     }
+    const int wq = warp % QW, wl = warp / QW, q0 = qb + NQ * wq;
     float2 xr[H], xi[H];  // real and imaginary parts of bin pairs
 #pragma unroll
     for (int i = 0; i < H; ++i) xr[i] = xi[i] = make_float2(0.f, 0.f);
-    for (int c = 0; c < C; ++c) {
+    for (int g = 0; g < NS; ++g) {
         asm volatile("cp.async.wait_group 1;" ::: "memory");
-        __syncthreads();  // block c staged; every warp is done with block c - 1, whose slot takes c + 2
-        stage(c + 2);
-        const float2 *u_s = sU + (c % 3) * P * 32 + lane;
-        const float *t_s = sT + NQ * warp;
-        float2 yr[H], yi[H];
+        __syncthreads();  // stage g in place; every warp is done with stage g - 1, whose slot takes g + 2
+        stage(g + 2);
+        if (q0 >= a.Q) continue;
+        const int nc = min(CS, C - g * CS);
+        const float2 *u_s = sU + (g % 3) * CS * P * NLC + 32 * wl + lane;
+        for (int cc = 0; cc < nc; ++cc) {
+            const float *t_s = sT + NQ * wq;
+            float2 yr[H], yi[H];
 #pragma unroll
-        for (int i = 0; i < H; ++i) yr[i] = yi[i] = make_float2(0.f, 0.f);
+            for (int i = 0; i < H; ++i) yr[i] = yi[i] = make_float2(0.f, 0.f);
 #pragma unroll 2
-        for (int p = 0; p < P; ++p) {
-            const float2 u = u_s[32 * p];
-            const float2 ur = make_float2(u.x, u.x), ui = make_float2(u.y, u.y);
+            for (int p = 0; p < P; ++p) {
+                const float2 u = *u_s;
+                u_s += NLC;
+                const float2 ur = make_float2(u.x, u.x), ui = make_float2(u.y, u.y);
 #pragma unroll
-            for (int i = 0; i < H; i += 2) {
-                const float4 t = *reinterpret_cast<const float4 *>(t_s + NB * p + 2 * i);
-                const float2 ta = make_float2(t.x, t.y), tb = make_float2(t.z, t.w);
-                yr[i] = fma2(ta, ur, yr[i]);
-                yi[i] = fma2(ta, ui, yi[i]);
-                yr[i + 1] = fma2(tb, ur, yr[i + 1]);
-                yi[i + 1] = fma2(tb, ui, yi[i + 1]);
+                for (int i = 0; i < H; i += 2) {
+                    const float4 t = *reinterpret_cast<const float4 *>(t_s + NB * p + 2 * i);
+                    const float2 ta = make_float2(t.x, t.y), tb = make_float2(t.z, t.w);
+                    yr[i] = fma2(ta, ur, yr[i]);
+                    yi[i] = fma2(ta, ui, yi[i]);
+                    yr[i + 1] = fma2(tb, ur, yr[i + 1]);
+                    yi[i + 1] = fma2(tb, ui, yi[i + 1]);
+                }
+            }
+            const float4 *e_s = reinterpret_cast<const float4 *>(sE + ((g % 3) * CS + cc) * NB + NQ * wq);
+#pragma unroll
+            for (int i = 0; i < H; ++i) {
+                const float4 e = e_s[i];  // two bins' phases
+                const float2 er = make_float2(e.x, e.z), ei = make_float2(e.y, e.w);
+                xr[i] = fma2(er, yr[i], fma2(make_float2(-ei.x, -ei.y), yi[i], xr[i]));
+                xi[i] = fma2(er, yi[i], fma2(ei, yr[i], xi[i]));
             }
         }
-        const float4 *e_s = reinterpret_cast<const float4 *>(sE + (c % 3) * NB + NQ * warp);
-#pragma unroll
-        for (int i = 0; i < H; ++i) {
-            const float4 e = e_s[i];  // two bins' phases
-            const float2 er = make_float2(e.x, e.z), ei = make_float2(e.y, e.w);
-            xr[i] = fma2(er, yr[i], fma2(make_float2(-ei.x, -ei.y), yi[i], xr[i]));
-            xi[i] = fma2(er, yi[i], fma2(ei, yr[i], xi[i]));
-        }
     }
-    const int l = l0 + lane, q0 = qb + NQ * warp;
-    if (l >= ms.NL) return;
+    const int l = l0 + 32 * wl + lane;
+    if (l >= ms.NL || q0 >= a.Q) return;
     const int L = ms.L0 + l;
     const bool none = L >= sd.n || L <= -sd.n;  // no overlap: exactly zero
 #pragma unroll
@@ -535,7 +548,7 @@ __device__ __forceinline__ float map_value(const MapArgs &a, const float2 *__res
 // the double-float geometry (the lag by the FP64 expression where D lies
 // within 1e-6 of a rounding boundary); false when |D| is out of range.
 template <bool FRAC>
-__device__ __forceinline__ bool map_node(const MapArgs &a, const MapSnap &ms, int s, int64_t p, const dfl (&xyz)[3],
+__device__ __forceinline__ bool map_node(const MapArgs &a, const MapSnap &ms, int s, const double *node, const dfl (&xyz)[3],
                                          int &L, float &mu, float &u)
 {
     dfl ed[12], D, nu;
@@ -548,7 +561,7 @@ __device__ __forceinline__ bool map_node(const MapArgs &a, const MapSnap &ms, in
     if (FRAC ? floor_df(D, L, mu) : round_df(D, L)) return true;
     double e[12], D64, nu64;
     for (int t = 0; t < 12; ++t) e[t] = a.eph[12 * (size_t)s + t];
-    geometry(a.xyz[p], a.xyz[a.G + p], a.xyz[2 * a.G + p], e, a.fs, a.lambda, D64, nu64);
+    geometry(node[0], node[a.G], node[2 * a.G], e, a.fs, a.lambda, D64, nu64);
     if (!(fabs(D64) < 1.0e9)) return false;
     L = lag_of(D64, FRAC ? DG_DELAY_LAGRANGE4 : DG_DELAY_INTEGER);
     mu = (float)(D64 - (double)L);
@@ -724,7 +737,11 @@ template <bool FRAC, bool BAD, int WK> __global__ void __launch_bounds__(256) k_
     constexpr int WN = 8 / WK;
     __shared__ float s_val[WK > 1 ? WK : 1][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tiles_j = (a.nlon + 31) / 32;
+    const int tiles_j = (a.nlon + 31) / 32, reg = blockIdx.y;
+    const double *xyz_r = a.xyz + 3 * a.G * reg;
+    float *out = a.out + a.G * reg;
+    const float2 *X = a.X + (size_t)reg * a.ksd * a.Q * a.NLpad;
+    const MapSnap *snap = a.snap + (size_t)reg * a.ksd;
     const int tj = blockIdx.x % tiles_j, ti = blockIdx.x / tiles_j;
     const int i = ti * WN + (WK > 1 ? warp / WK : warp), j = tj * 32 + lane;
     const int wk = WK > 1 ? warp % WK : 0;
@@ -732,20 +749,20 @@ template <bool FRAC, bool BAD, int WK> __global__ void __launch_bounds__(256) k_
     const int64_t p = (int64_t)min(i, a.nrows - 1) * a.nlon + min(j, a.nlon - 1);
     dfl xyz[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) xyz[d] = df_from(a.xyz[d * a.G + p]);
-    float sum = a.first ? 0.f : a.out[p];
+    for (int d = 0; d < 3; ++d) xyz[d] = df_from(xyz_r[d * a.G + p]);
+    float sum = a.first ? 0.f : out[p];
     bool any = !a.first;
-    for (int k = 0; k < a.S; k += WK) {
+    for (int k = 0; k < a.ksd; k += WK) {
         const int s = k + wk;
         float v = 0.f;
-        if (s < a.S) {
-            const MapSnap ms = a.snap[s];
+        if (s < a.ksd) {
+            const MapSnap ms = snap[s];
             int L;
             float mu, u;
-            if (map_node<FRAC>(a, ms, s, p, xyz, L, mu, u)) {
+            if (map_node<FRAC>(a, ms, s, xyz_r + p, xyz, L, mu, u)) {
                 int U0;
                 const float uf = round_magic(u, U0);
-                v = map_value<FRAC, BAD>(a, a.X + (size_t)s * a.Q * a.NLpad, s, ms.L0, L, mu, U0, u - uf);
+                v = map_value<FRAC, BAD>(a, X + (size_t)s * a.Q * a.NLpad, s, ms.L0, L, mu, U0, u - uf);
             } else if (ok) {
                 atomicOr(a.err, ERR_LAG_RANGE);
             }
@@ -757,14 +774,193 @@ template <bool FRAC, bool BAD, int WK> __global__ void __launch_bounds__(256) k_
             s_val[wk][lane] = v;
             __syncthreads();
             if (wk == 0)
-                for (int w = 0; w < WK && k + w < a.S; ++w) {
+                for (int w = 0; w < WK && k + w < a.ksd; ++w) {
                     sum = any ? sum + s_val[w][lane] : s_val[w][lane];
                     any = true;
                 }
             __syncthreads();
         }
     }
-    if (ok && wk == 0) a.out[p] = sum;
+    if (ok && wk == 0) out[p] = sum;
+}
+
+// Tables of a grid of a few lags (the refinement around a node). Its band is
+// so narrow that the phase turns by a fraction of a cycle over a capture:
+// with nu_c the centre's FDOA and t = (n - N/2) tscale in [-1, 1],
+//     X(l, nu) = sum_m j^m c_m(nu) S[m][l],
+//     S[m][l] = sum_n y1[n] e^{j 2 pi nu_c (n - N/2)} conj(y2[n + l]) T_m(t),
+// the Chebyshev series of e^{j 2 pi (nu - nu_c)(n - N/2)} cut after P terms (real
+// weights: 2 FMAs per term where a turned copy of y1 per Doppler node takes
+// 4 and a shared load). A CTA walks blocks of samples of one snapshot: y1
+// turned to nu_c and the window of y2 in shared memory; a warp takes 4 lags of
+// a share of the samples (5 shared loads for 16 + 8 P FMAs). The CTAs' sums are
+// added in a fixed order by k_map_few_x, which also expands the terms to the
+// table's bins.
+constexpr int kFewLags = 4;  // lags per warp
+
+// v[i] summed over the warp's lanes: halves are exchanged while the count is
+// even, so each lane ends with N / 32 of the sums (or a pair of lanes with
+// the same 3 for N = 48); returns this lane's first index.
+template <int N> __device__ __forceinline__ int warp_scatter_sum(float *v, int lane)
+{
+    int first = 0, n = N;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        if (n % 2 == 0) {
+            n /= 2;
+            const bool up = lane & d;
+#pragma unroll
+            for (int i = 0; i < N / 2; ++i) {
+                if (i >= n) break;
+                const float send = up ? v[i] : v[i + n];
+                const float keep = up ? v[i + n] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, d);
+            }
+            if (up) first += n;
+        } else {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                if (i >= n) break;
+                v[i] += __shfl_xor_sync(0xffffffffu, v[i], d);
+            }
+        }
+    }
+    return first;
+}
+
+template <int P> __global__ void __launch_bounds__(256) k_map_few(MapArgs a, MapFew f)
+{
+    constexpr int NV = 2 * kFewLags * P;  // floats per lag group
+    __shared__ __align__(16) float2 y1t[kFewBlock], y2w[kFewBlock + kFewMaxLags];
+    __shared__ float s_red[8][NV];
+    __shared__ float s_nu[2];
+    __shared__ int s_L0;
+    const int s = blockIdx.y, t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const StepDesc sd = a.sd[s];
+    const int N = sd.n;
+    if (t == 0) {  // the centre's geometry
+        dfl ed[12], D, nu;
+        for (int q = 0; q < 12; ++q) ed[q] = {__ldg(a.ephf + 24 * (size_t)s + 2 * q), __ldg(a.ephf + 24 * (size_t)s + 2 * q + 1)};
+        geometry_dfl(df_from(a.xyz[f.centre]), df_from(a.xyz[a.G + f.centre]), df_from(a.xyz[2 * a.G + f.centre]), ed,
+                     {a.fsc_hi, a.fsc_lo}, {a.ilf_hi, a.ilf_lo}, D, nu);
+        const int L0 = (int)floor((double)D.hi + (double)D.lo - f.md - 0.51) - (a.delay != DG_DELAY_INTEGER ? 1 : 0);
+        s_L0 = L0;
+        s_nu[0] = nu.hi;
+        s_nu[1] = nu.lo;
+        if (blockIdx.x == 0) {
+            MapSnap ms;
+            ms.nuc = (double)nu.hi + (double)nu.lo;
+            ms.nu0 = ms.nuc - f.halfw;
+            ms.delta = f.delta;
+            ms.halfw = f.halfw;
+            ms.nu0_hi = (float)ms.nu0;
+            ms.nu0_lo = (float)(ms.nu0 - (double)ms.nu0_hi);
+            ms.inv_delta = (float)(1.0 / f.delta);
+            ms.inv_delta_lo = (float)(1.0 / f.delta - (double)ms.inv_delta);
+            ms.L0 = L0;
+            ms.NL = a.LT;
+            f.snap[s] = ms;
+        }
+    }
+    __syncthreads();
+    const int L0 = s_L0, NG = (a.LT + kFewLags - 1) / kFewLags;
+    const float nh = s_nu[0], nl = s_nu[1];
+    const int NS = 8 / NG, g = warp % NG, sg = warp / NG;  // lag group, share of the samples
+    float v[NV];  // [lag][term][re, im]
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = 0.f;
+    for (int64_t n0 = (int64_t)blockIdx.x * kFewBlock; n0 < N; n0 += (int64_t)gridDim.x * kFewBlock) {
+        __syncthreads();
+        for (int i = t; i < kFewBlock + kFewLags * NG; i += 256) {
+            const int64_t q = n0 + L0 + i;
+            y2w[i] = q >= 0 && q < N ? load_sample(sd.y2, sd.fmt, (int)q) : make_float2(0.f, 0.f);
+        }
+        for (int i = t; i < kFewBlock; i += 256) {
+            const int64_t n = n0 + i;
+            const float2 y = n < N ? load_sample(sd.y1, sd.fmt, (int)n) : make_float2(0.f, 0.f);
+            y1t[i] = cmul(y, cis_df(nh, nl, (float)((int)n - N / 2)));
+        }
+        __syncthreads();
+        if (sg < NS) {
+            const float2 *b = y2w + kFewLags * g;
+            const float t0 = (float)((int)n0 - N / 2) * f.tscale;
+            for (int m = 32 * sg + lane; m < kFewBlock; m += 32 * NS) {
+                const float2 y = y1t[m];
+                const float x = fmaf((float)m, f.tscale, t0), x2 = 2.f * x;
+#pragma unroll
+                for (int l = 0; l < kFewLags; ++l) {
+                    const float2 w = b[m + l];
+                    const float zx = fmaf(y.x, w.x, y.y * w.y), zy = fmaf(y.y, w.x, -y.x * w.y);
+                    float *o = v + 2 * l * P;
+                    float tp = 1.f, tq = x;  // T_{m}, T_{m + 1}
+                    o[0] += zx;
+                    o[1] += zy;
+#pragma unroll
+                    for (int p = 1; p < P; ++p) {
+                        o[2 * p] = fmaf(tq, zx, o[2 * p]);
+                        o[2 * p + 1] = fmaf(tq, zy, o[2 * p + 1]);
+                        const float tn = fmaf(x2, tq, -tp);
+                        tp = tq;
+                        tq = tn;
+                    }
+                }
+            }
+        }
+    }
+    if (sg < NS) {
+        const int first = warp_scatter_sum<NV>(v, lane);
+        constexpr int per = NV % 32 == 0 ? NV / 32 : NV / 16;
+#pragma unroll
+        for (int i = 0; i < per; ++i) s_red[warp][first + i] = v[i];
+    }
+    __syncthreads();
+    float *out = reinterpret_cast<float *>(a.U) + ((size_t)s * a.Cmax + blockIdx.x) * (size_t)(NG * NV);
+    for (int i = t; i < NG * NV; i += 256) {
+        float x = 0.f;
+        for (int w = 0; w < NS; ++w) x += s_red[i / NV + w * NG][i % NV];
+        out[i] = x;
+    }
+}
+
+template <int P> __global__ void __launch_bounds__(256) k_map_few_x(MapArgs a, MapFew f)
+{
+    constexpr int NV = 2 * kFewLags * P;
+    __shared__ float s_sum[kFewMaxLags / kFewLags * NV];
+    const int s = blockIdx.x, t = threadIdx.x;
+    const int N = a.sd[s].n, n = (a.LT + kFewLags - 1) / kFewLags * NV;
+    const float *U = reinterpret_cast<const float *>(a.U) + (size_t)s * a.Cmax * n;
+    for (int i = t; i < n; i += 256) {
+        float x = 0.f;
+#pragma unroll 8
+        for (int c = 0; c < a.Cmax; ++c) x += __ldg(U + (size_t)c * n + i);
+        s_sum[i] = x;
+    }
+    __syncthreads();
+    const int L0 = f.snap[s].L0;
+    for (int i = t; i < a.Q * a.LT; i += 256) {
+        const int q = i / a.LT, l = i % a.LT, L = L0 + l;
+        float2 x = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const float *v = s_sum + (l / kFewLags) * NV + 2 * ((l % kFewLags) * P + p);
+            const float c = f.T[p * a.Q + q];
+            if (p % 4 == 0) {  // times j^p
+                x.x = fmaf(c, v[0], x.x);
+                x.y = fmaf(c, v[1], x.y);
+            } else if (p % 4 == 1) {
+                x.x = fmaf(-c, v[1], x.x);
+                x.y = fmaf(c, v[0], x.y);
+            } else if (p % 4 == 2) {
+                x.x = fmaf(-c, v[0], x.x);
+                x.y = fmaf(-c, v[1], x.y);
+            } else {
+                x.x = fmaf(c, v[1], x.x);
+                x.y = fmaf(-c, v[0], x.y);
+            }
+        }
+        if (L >= N || L <= -N) x = make_float2(0.f, 0.f);
+        a.X[((size_t)s * a.Q + q) * a.NLpad + l] = x;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -792,15 +988,43 @@ cudaError_t launch_map_twiddles(float2 *tw, int logn, cudaStream_t st)
     return cudaGetLastError();
 }
 
+static cudaError_t launch_bad(const MapArgs &a, cudaStream_t st, int *launches)
+{
+    if (!a.bad) return cudaSuccess;
+    k_map_bad_init<<<1, 256, 0, st>>>(a.bad, a.ksd);
+    k_map_bad<<<dim3(16, (unsigned)a.ksd, 2), 256, 0, st>>>(a);
+    *launches += 2;
+    return cudaGetLastError();
+}
+
+size_t map_few_partials(int P, int NL) { return (size_t)((NL + kFewLags - 1) / kFewLags) * 2 * kFewLags * P; }
+
+template <int P> static cudaError_t launch_few(const MapArgs &a, const MapFew &f, cudaStream_t st)
+{
+    k_map_few<P><<<dim3((unsigned)a.Cmax, (unsigned)a.S), 256, 0, st>>>(a, f);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_map_few_x<P><<<(unsigned)a.S, 256, 0, st>>>(a, f);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_map_few(const MapArgs &a, const MapFew &f, cudaStream_t st, int *launches)
+{
+    const cudaError_t e = launch_bad(a, st, launches);
+    if (e != cudaSuccess) return e;
+    *launches += 2;
+    switch (a.P) {
+    case 4: return launch_few<4>(a, f, st);
+    case 6: return launch_few<6>(a, f, st);
+    case 8: return launch_few<8>(a, f, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 cudaError_t launch_map_tables(const MapArgs &a, cudaStream_t st, int *launches)
 {
-    cudaError_t e = cudaSuccess;
-    if (a.bad) {
-        k_map_bad_init<<<1, 256, 0, st>>>(a.bad, a.S);
-        k_map_bad<<<dim3(16, (unsigned)a.S, 2), 256, 0, st>>>(a);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        *launches += 2;
-    }
+    cudaError_t e = launch_bad(a, st, launches);
+    if (e != cudaSuccess) return e;
     switch (a.logn) {
     case 10: e = launch_tables<10>(a, st); break;
     case 11: e = launch_tables<11>(a, st); break;
@@ -813,21 +1037,24 @@ cudaError_t launch_map_tables(const MapArgs &a, cudaStream_t st, int *launches)
     return e;
 }
 
-template <int NQ> static cudaError_t launch_expand(const MapArgs &a, cudaStream_t st)
+template <int NQ, int LW> static cudaError_t launch_expand(const MapArgs &a, cudaStream_t st)
 {
-    constexpr int NB = NQ * kExpWarps;
-    const size_t smem = sizeof(float) * (size_t)a.P * NB + sizeof(float2) * 3 * (size_t)(NB + a.P * 32);
-    const cudaError_t e = cudaFuncSetAttribute(k_map_expand<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr int NB = NQ * kExpWarps / LW, NLC = 32 * LW;
+    const int CS = a.P < kExpRows ? kExpRows / a.P : 1;
+    const size_t smem = sizeof(float) * (size_t)a.P * NB + sizeof(float2) * 3 * (size_t)CS * (NB + a.P * NLC);
+    const cudaError_t e = cudaFuncSetAttribute(k_map_expand<NQ, LW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const dim3 ge((unsigned)(a.NLpad / 32), (unsigned)((a.Q + NB - 1) / NB), (unsigned)a.S);
-    k_map_expand<NQ><<<ge, 32 * kExpWarps, smem, st>>>(a);
+    const dim3 ge((unsigned)((a.NLpad + NLC - 1) / NLC), (unsigned)((a.Q + NB - 1) / NB), (unsigned)a.S);
+    k_map_expand<NQ, LW><<<ge, 32 * kExpWarps, smem, st>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_map_expand(const MapArgs &a, cudaStream_t st)
 {
     // 16 bins per warp where the table is wide enough to fill the chip, 8 otherwise
-    return a.Q >= 128 ? launch_expand<16>(a, st) : launch_expand<8>(a, st);
+    if (a.Q >= 128) return launch_expand<16, 1>(a, st);
+    if (a.Q > 32) return launch_expand<8, 1>(a, st);
+    return a.Q > 16 ? launch_expand<8, 2>(a, st) : launch_expand<8, 4>(a, st);
 }
 
 cudaError_t launch_map_poly(const MapArgs &a, cudaStream_t st)
@@ -844,15 +1071,15 @@ template <bool FRAC, bool BAD> static cudaError_t launch_lookup(const MapArgs &a
 {
     const int64_t tiles_j = (a.nlon + 31) / 32;
     // under about four CTAs per SM of one-row warps, the warps split the snapshots
-    const bool split = !a.poly.rows && tiles_j * ((a.nrows + 7) / 8) < 152 * 4;
+    const bool split = !a.poly.rows && tiles_j * ((a.nrows + 7) / 8) * a.nreg < 152 * 4;
     const int rows = a.poly.rows ? a.poly.rows : split ? 1 : 8;  // of a CTA
     const int64_t blocks = tiles_j * ((a.nrows + rows - 1) / rows);
     if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
     const unsigned g = (unsigned)blocks;
     if (a.poly.rows == 64) k_map_lookup_poly<FRAC, BAD, 8><<<g, 256, 0, st>>>(a, (int)tiles_j);
     else if (a.poly.rows) k_map_lookup_poly<FRAC, BAD, 4><<<g, 256, 0, st>>>(a, (int)tiles_j);
-    else if (split) k_map_lookup<FRAC, BAD, 8><<<g, 256, 0, st>>>(a);
-    else k_map_lookup<FRAC, BAD, 1><<<g, 256, 0, st>>>(a);
+    else if (split) k_map_lookup<FRAC, BAD, 8><<<dim3(g, (unsigned)a.nreg), 256, 0, st>>>(a);
+    else k_map_lookup<FRAC, BAD, 1><<<dim3(g, (unsigned)a.nreg), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 

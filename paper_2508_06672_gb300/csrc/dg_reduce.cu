@@ -76,17 +76,25 @@ __device__ __forceinline__ VI block_best(VI v)
     return v;  // valid in thread 0
 }
 
+// Surface blockIdx.y of n values each (one for a single argmax). The scan
+// compares in the surface's own type: on FP32 values the FP64 comparison
+// would run at 1/64 of the rate.
 template <typename T>
 __global__ void __launch_bounds__(1024) k_argmax_partial(const T *__restrict__ v, int64_t n, VI *part)
 {
-    VI best{0.0, -1};
+    v += n * blockIdx.y;
+    T val = (T)0;
+    int64_t idx = -1;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
          p += (int64_t)gridDim.x * blockDim.x) {
-        const double x = (double)v[p];
-        if (x == x && (best.idx < 0 || x > best.val)) best = VI{x, p};  // p increases per thread
+        const T x = v[p];
+        if (x == x && (idx < 0 || x > val)) {  // p increases per thread
+            val = x;
+            idx = p;
+        }
     }
-    best = block_best(best);
-    if (threadIdx.x == 0) part[blockIdx.x] = best;
+    const VI best = block_best(VI{(double)val, idx});
+    if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = best;
 }
 
 // Offset (in nodes, within [-0.5, 0.5]) of the vertex of the parabola
@@ -104,76 +112,11 @@ __device__ __forceinline__ double parabola_offset(const T *v, int64_t c, int64_t
     return x != x ? 0.0 : fmin(0.5, fmax(-0.5, x));
 }
 
-__global__ void __launch_bounds__(1024) k_argmax_final(const VI *part, int nparts, GridDev g,
-                                                       ArgmaxResult *res, const ArgmaxResult *centre,
-                                                       const void *v, int prec)
+// The fields of dg_fix as dg_argmax_refine fills them (one thread); fine may
+// be NULL (no refinement, n = 0).
+__device__ __forceinline__ void make_fix(const ArgmaxResult *coarse, const ArgmaxResult *fine, const GridDev &g, int n,
+                                         dg_fix *out)
 {
-    if (centre) centre_on(g, centre);
-    VI best{0.0, -1};
-    for (int p = threadIdx.x; p < nparts; p += blockDim.x)
-        if (beats(part[p], best)) best = part[p];
-    best = block_best(best);
-    if (threadIdx.x == 0) {
-        res->val = best.val;
-        res->idx = best.idx;
-        res->lat_rad = 0.0;
-        res->lon_rad = 0.0;
-        res->sub_lat_rad = 0.0;
-        res->sub_lon_rad = 0.0;
-        if (best.idx >= 0) {
-            const GridStep st = grid_step(g);
-            const int il = (int)(best.idx / g.nlon), j = (int)(best.idx % g.nlon);
-            double lat, lon;
-            grid_node(g, st, g.row0 + il, j, lat, lon);
-            res->lat_rad = lat;
-            res->lon_rad = lon;
-            // neighbours within the surface (the shard's rows, the grid's columns)
-            double di, dj;
-            if (prec == DG_PREC_FP64) {
-                const double *d = (const double *)v;
-                di = parabola_offset(d, best.idx, g.nlon, il > 0, il < g.nrows - 1);
-                dj = parabola_offset(d, best.idx, 1, j > 0, j < g.nlon - 1);
-            } else {
-                const float *f = (const float *)v;
-                di = parabola_offset(f, best.idx, g.nlon, il > 0, il < g.nrows - 1);
-                dj = parabola_offset(f, best.idx, 1, j > 0, j < g.nlon - 1);
-            }
-            res->sub_lat_rad = __dadd_rn(lat, __dmul_rn(di, st.dlat));
-            res->sub_lon_rad = __dadd_rn(lon, __dmul_rn(dj, st.dlon));
-        }
-    }
-}
-
-static int argmax_blocks(int64_t n)
-{
-    int64_t b = (n + 1023) / 1024;
-    if (b > 152 * 2) b = 152 * 2;
-    if (b < 1) b = 1;
-    return (int)b;
-}
-
-size_t argmax_tmp_bytes(int64_t n) { return sizeof(VI) * (size_t)argmax_blocks(n); }
-
-cudaError_t launch_argmax(const void *v, int64_t n, int prec, const GridDev &g, void *tmp,
-                          ArgmaxResult *res, int *launches, cudaStream_t s, const ArgmaxResult *centre)
-{
-    const int nb = argmax_blocks(n);
-    VI *part = reinterpret_cast<VI *>(tmp);
-    if (prec == DG_PREC_FP64)
-        k_argmax_partial<double><<<nb, 1024, 0, s>>>((const double *)v, n, part);
-    else
-        k_argmax_partial<float><<<nb, 1024, 0, s>>>((const float *)v, n, part);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_argmax_final<<<1, 1024, 0, s>>>(part, nb, g, res, centre, v, prec);
-    if (launches) *launches += 2;
-    return cudaGetLastError();
-}
-
-// One thread: the fields of dg_fix as dg_argmax_refine fills them.
-__global__ void k_make_fix(const ArgmaxResult *coarse, const ArgmaxResult *fine, GridDev g, int n, dg_fix *out)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
     dg_fix f;
     memset(&f, 0, sizeof f);
     f.index = coarse->idx;
@@ -204,10 +147,87 @@ __global__ void k_make_fix(const ArgmaxResult *coarse, const ArgmaxResult *fine,
     *out = f;
 }
 
-cudaError_t launch_make_fix(const ArgmaxResult *coarse, const ArgmaxResult *fine, const GridDev &g, int n,
-                            dg_fix *out, cudaStream_t s)
+// The last pass: the record of surface blockIdx.x, its node placed by the
+// grid's stored angular steps (a single thread would need about 5 us for their
+// FP64 sines and divisions), and where fin.fix is given the step's fix record.
+__global__ void __launch_bounds__(1024) k_argmax_final(const VI *part, int nparts, GridDev g, const GridStep *step,
+                                                       ArgmaxResult *res, const ArgmaxResult *centre,
+                                                       const void *v, int prec, const GridDev *grids, int64_t n,
+                                                       FixOut fin)
 {
-    k_make_fix<<<1, 32, 0, s>>>(coarse, fine, g, n, out);
+    if (grids) {  // surface and grid blockIdx.x of several
+        g = grids[blockIdx.x];
+        step += blockIdx.x;
+        part += (int64_t)nparts * blockIdx.x;
+        res += blockIdx.x;
+        v = (const char *)v + (prec == DG_PREC_FP64 ? 8 : 4) * n * blockIdx.x;
+    }
+    if (centre) centre_on(g, centre);
+    VI best{0.0, -1};
+    for (int p = threadIdx.x; p < nparts; p += blockDim.x)
+        if (beats(part[p], best)) best = part[p];
+    best = block_best(best);
+    if (threadIdx.x == 0) {
+        ArgmaxResult r;
+        r.val = best.val;
+        r.idx = best.idx;
+        r.lat_rad = 0.0;
+        r.lon_rad = 0.0;
+        r.sub_lat_rad = 0.0;
+        r.sub_lon_rad = 0.0;
+        if (best.idx >= 0) {
+            const GridStep st = *step;
+            const int il = (int)(best.idx / g.nlon), j = (int)(best.idx % g.nlon);
+            double lat, lon;
+            grid_node(g, st, g.row0 + il, j, lat, lon);
+            r.lat_rad = lat;
+            r.lon_rad = lon;
+            // neighbours within the surface (the shard's rows, the grid's columns)
+            double di, dj;
+            if (prec == DG_PREC_FP64) {
+                const double *d = (const double *)v;
+                di = parabola_offset(d, best.idx, g.nlon, il > 0, il < g.nrows - 1);
+                dj = parabola_offset(d, best.idx, 1, j > 0, j < g.nlon - 1);
+            } else {
+                const float *f = (const float *)v;
+                di = parabola_offset(f, best.idx, g.nlon, il > 0, il < g.nrows - 1);
+                dj = parabola_offset(f, best.idx, 1, j > 0, j < g.nlon - 1);
+            }
+            r.sub_lat_rad = __dadd_rn(lat, __dmul_rn(di, st.dlat));
+            r.sub_lon_rad = __dadd_rn(lon, __dmul_rn(dj, st.dlon));
+        }
+        *res = r;
+        if (fin.fix) {
+            if (fin.coarse) make_fix(fin.coarse, &r, fin.g, fin.n, fin.fix);
+            else make_fix(&r, nullptr, fin.g, 0, fin.fix);
+        }
+    }
+}
+
+static int argmax_blocks(int64_t n)
+{
+    int64_t b = (n + 1023) / 1024;
+    if (b > 152 * 2) b = 152 * 2;
+    if (b < 1) b = 1;
+    return (int)b;
+}
+
+size_t argmax_tmp_bytes(int64_t n) { return sizeof(VI) * (size_t)argmax_blocks(n); }
+
+cudaError_t launch_argmax(const void *v, int64_t n, int prec, const GridDev &g, const GridStep *step, void *tmp,
+                          ArgmaxResult *res, int *launches, cudaStream_t s, const ArgmaxResult *centre,
+                          const GridDev *grids, int ngrids, FixOut fin)
+{
+    const int nb = argmax_blocks(n);
+    VI *part = reinterpret_cast<VI *>(tmp);
+    if (prec == DG_PREC_FP64)
+        k_argmax_partial<double><<<dim3(nb, ngrids), 1024, 0, s>>>((const double *)v, n, part);
+    else
+        k_argmax_partial<float><<<dim3(nb, ngrids), 1024, 0, s>>>((const float *)v, n, part);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_argmax_final<<<ngrids, 1024, 0, s>>>(part, nb, g, step, res, centre, v, prec, grids, n, fin);
+    if (launches) *launches += 2;
     return cudaGetLastError();
 }
 

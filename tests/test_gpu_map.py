@@ -119,3 +119,65 @@ def test_map_lags_without_overlap_and_samples_that_are_not_finite(delay):
         assert bad.any() and not bad.all()
         assert np.array_equal(np.isnan(a2), bad)
         assert rel_err(a2[~bad], b2[~bad], 0.01) < 2 * FP32_TOL
+
+
+@pytest.mark.parametrize("window", [(10.0, 200.0), (50.0, 4000.0), (100.0, 15000.0)])
+@pytest.mark.parametrize("delay", ["integer", "lagrange4"])
+def test_refinement_from_a_table_of_few_lags(window, delay):
+    """The refinement around a node (a few lags, summed directly) and windows
+    too wide for it: its maximum is the oracle's maximum of the same local grid
+    within the bound, and the synchronising call equals the captured step."""
+    torch = torch_cuda()
+    P = package()
+    s = _scene(44, 500.0, 7001, k=3, fmt="c64", fs=12.5e6, grid=(91, 93))
+    stream = torch.cuda.Stream()
+    g = P.Geolocator(s.grid, s.ephem, s.fs_hz, s.fc_hz, algo="cdft", contract="fp16x3", delay=delay, stream=stream)
+    g.load_captures(s.fmt, torch.from_numpy(s.y1).cuda(), torch.from_numpy(s.y2).cuda())
+    with torch.cuda.stream(stream):
+        cost = g.cost_surface()
+        fix = g.argmax_refine(cost, *window)
+    lg = oracle.refine_grid(s.grid, fix["index"], *window)
+    rows = None if lg["nlat"] < 200 else [fix["ri"]]
+    mode = 0 if delay == "integer" else 1
+    idx = np.unique(np.r_[fix["ri"] * lg["nlon"] + fix["rj"],
+                          np.random.default_rng(3).integers(0, lg["nlat"] * lg["nlon"], 800)])
+    ref = oracle.cost_points(lg, s.ephem, s.fs_hz, s.fc_hz, oracle.iq_to_f64(s.y1), oracle.iq_to_f64(s.y2), idx=idx,
+                             delay_mode=mode)
+    at = ref[np.searchsorted(idx, fix["ri"] * lg["nlon"] + fix["rj"])]
+    assert rows is None or fix["refine_n"] == lg["nlat"]
+    assert abs(fix["refined_cost"] - at) <= FP32_TOL * at
+    assert at >= ref.max() * (1 - 2 * FP32_TOL)
+    c2 = torch.empty_like(cost)
+    g.graph_capture(c2, *window)
+    g.graph_launch()
+    assert g.graph_fix() == fix
+    g.close()
+
+
+def test_regions_searched_together_match_fresh_contexts():
+    """Regions of many nodes share their launches: every region's surface is
+    a fresh context's within twice the bound, the fix its own maximum's."""
+    torch = torch_cuda()
+    P = package()
+    s = _scene(45, 400.0, 6001, k=3, fs=12.5e6, grid=(95, 91))
+    offs = [(0.0, 0.0), (0.4, -0.3), (-1.1, 0.8), (2.0, 2.0), (0.05, 0.02)]
+    regions = [dict(s.grid, lat0_deg=s.grid["lat0_deg"] + a, lon0_deg=s.grid["lon0_deg"] + b) for a, b in offs]
+    g = P.Geolocator(s.grid, s.ephem, s.fs_hz, s.fc_hz, algo="cdft", contract="bf16x3")
+    g.load_captures(s.fmt, torch.from_numpy(s.y1).cuda(), torch.from_numpy(s.y2).cuda())
+    before = g.cost_surface().clone()
+    fix, best, costs = g.search_regions(regions, 20.0, 300.0)
+    vals = []
+    for r, reg in enumerate(regions):
+        f = P.Geolocator(reg, s.ephem, s.fs_hz, s.fc_hz, algo="cdft", contract="bf16x3")
+        f.load_captures(s.fmt, torch.from_numpy(s.y1).cuda(), torch.from_numpy(s.y2).cuda())
+        c = f.cost_surface()
+        assert rel_err(costs[r].cpu().numpy(), c.cpu().numpy(), 0.01) < 2 * FP32_TOL
+        vals.append(float(c.max()))
+        f.close()
+    assert best == int(np.argmax(vals)) and fix["cost"] == float(costs[best].max())
+    assert g.grid["lat0_deg"] == regions[best]["lat0_deg"]
+    lo, hi = g.cdft_chunks()
+    assert 64 <= lo <= hi <= 2048
+    g.set_grid(s.grid)  # the context goes on on its own grid
+    assert torch.equal(g.cost_surface(), before)
+    g.close()
