@@ -94,6 +94,9 @@ struct MapBufs {  // their device tables and scratch, grown on demand
 struct CdftBufs {  // chunked-DFT scratch, grown on demand
     int *lr = nullptr;
     CdftLayout main_layout, loc_layout;
+    CdftLayout dmain_layout, dloc_layout;  // the direct path's lag groups
+    float2 *part = nullptr;                // and its segments' sums
+    size_t part_cap = 0;
     std::vector<double> main_span;  // FDOA span estimates per snapshot (main grid)
     std::vector<double> main_lags;  // and lag-count estimates
     std::vector<GridRange> main_range;  // and lag / FDOA bounds
@@ -353,6 +356,8 @@ dg_status run_surface_cdft(dg_ctx *c, const GridDev &gd, const double *xyz, int6
                            bool refine);
 static dg_status map_plan(dg_ctx *c);
 static dg_status run_surface_map(dg_ctx *c, void *out);
+static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *surf, void *out,
+                                 bool refine, bool *done);
 static dg_status refine_map(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *out, bool *done);
 
 // Surfaces whose candidates look their correlations up in delay-Doppler maps
@@ -381,6 +386,10 @@ dg_status run_surface(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G
         if ((st = refine_map(c, gd, xyz, G, out, &done)) != DG_OK || done) return st;
     }
     if (c->opt.algo == DG_ALGO_CDFT) return run_surface_cdft(c, gd, xyz, G, surf, out, refine);
+    if (c->opt.prec == DG_PREC_FP32 && c->opt.delay == DG_DELAY_INTEGER) {
+        bool done = false;
+        if ((st = run_surface_lag(c, gd, xyz, G, surf, out, refine, &done)) != DG_OK || done) return st;
+    }
     st = push_steps(c);
     if (st != DG_OK) return st;
     bool same_fmt = true;
@@ -730,6 +739,211 @@ static dg_status ensure_ephf(dg_ctx *c)
     return DG_OK;
 }
 
+// Scratch of the lag sort, grown on demand (never inside a captured graph: a
+// graph is captured after one uncaptured call of the same shape): S snapshots,
+// SG (snapshot, candidate) pairs, nbt lag slots, groups combine groups.
+static dg_status ensure_sort(dg_ctx *c, size_t S, size_t SG, size_t nbt, size_t groups)
+{
+    CdftBufs &b = c->cd;
+    dg_status st;
+    if (b.s_cap < S) {
+        if ((st = grow(c, &b.lr, 2 * S)) != DG_OK) return st;
+        if ((st = grow(c, &b.delta, S)) != DG_OK) return st;
+        if ((st = grow(c, &b.nubase, S)) != DG_OK) return st;
+        if ((st = grow(c, &b.nur, 2 * S)) != DG_OK) return st;
+        if ((st = grow(c, &b.tbase, S + 1)) != DG_OK) return st;
+        if ((st = grow(c, &b.hbase, S + 1)) != DG_OK) return st;
+        if ((st = grow(c, &b.layout, S)) != DG_OK) return st;
+        if ((st = grow(c, &b.Mcs, S)) != DG_OK) return st;
+        b.s_cap = S;
+    }
+    if (b.sg_cap < SG) {
+        if ((st = grow(c, &b.candL, SG)) != DG_OK) return st;
+        if ((st = grow(c, &b.candNu, SG)) != DG_OK) return st;
+        if ((st = grow(c, &b.order, SG)) != DG_OK) return st;
+        if ((st = grow(c, &b.nuS, SG)) != DG_OK) return st;
+        b.sg_cap = SG;
+    }
+    if (b.nb_cap < nbt) {
+        if ((st = grow(c, &b.count, nbt)) != DG_OK) return st;
+        if ((st = grow(c, &b.need, nbt)) != DG_OK) return st;
+        if ((st = grow(c, &b.offs, nbt)) != DG_OK) return st;
+        if ((st = grow(c, &b.subcnt, nbt)) != DG_OK) return st;
+        b.nb_cap = nbt;
+    }
+    if (b.g2b_cap < groups) {
+        if ((st = grow(c, &b.g2b, groups)) != DG_OK) return st;
+        b.g2b_cap = groups;
+    }
+    return DG_OK;
+}
+
+// The arguments of the geometry and the lag sort of one batch.
+static void sort_args(dg_ctx *c, const CdftLayout::Batch &bt, const CdftLayout &L, const GridDev &gd, const double *xyz,
+                      int64_t G, CdftBatch &a)
+{
+    CdftBufs &b = c->cd;
+    auto split = [](double d, float &h, float &l) {  // constants as double-float (hi, lo) pairs
+        h = (float)d;
+        l = (float)(d - (double)h);
+    };
+    a.xyz = xyz;
+    a.xyzf = b.xyzf;
+    a.ephf = b.ephf + 24 * (size_t)bt.k0;
+    split(c->fs / kC, a.fsc_hi, a.fsc_lo);
+    split(1.0 / (c->lambda * c->fs), a.ilf_hi, a.ilf_lo);
+    a.eph = c->eph + 12 * (size_t)bt.k0;
+    a.sd = c->steps_d + bt.k0;
+    a.S = bt.S;
+    a.k0 = bt.k0;
+    a.G = G;
+    a.nrows = gd.nrows;
+    a.nlon = gd.nlon;
+    a.fs = c->fs;
+    a.lambda = c->lambda;
+    a.acc = c->opt.acc;
+    a.err = c->err_d;
+    a.lr = b.lr;
+    a.nur = b.nur;
+    a.nubase = b.nubase;
+    a.delta = b.delta;
+    a.bbase = L.bbase + bt.base;
+    a.gbase = L.gbase + bt.base;
+    a.candL = b.candL;
+    a.candNu = b.candNu;
+    a.order = b.order;
+    a.nuS = b.nuS;
+    a.g2b = b.g2b;
+    a.count = b.count;
+    a.need = b.need;
+    a.offs = b.offs;
+    a.subcnt = b.subcnt;
+    a.delay = c->opt.delay;
+    a.candMu = b.candMu;
+    a.muS = b.muS;
+    a.ngroups = (int)bt.groups;
+}
+
+// The direct FP32 surface with the candidates grouped by lag (k_corr_lag):
+// per batch of snapshots (within 4 GiB of sort arrays) the chunked-DFT path's
+// geometry and lag sort, then the correlation. *done = false where the lag
+// slots or the captures are out of its range (the tile kernel serves those).
+static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *surf, void *out,
+                                 bool refine, bool *done)
+{
+    *done = false;
+    CdftBufs &b = c->cd;
+    CdftLayout &L = refine ? b.dloc_layout : b.dmain_layout;
+    for (int k = 0; k < c->K; ++k)
+        if (c->steps[k].n > (1 << 24) || !c->steps[k].loaded) return DG_OK;
+    GridDev shape = gd;  // as in cdft_setup: a captured refinement's centre is known on the device only
+    if (refine) {
+        shape.lat0_rad = c->gd.lat0_rad;
+        shape.lon0_rad = c->gd.lon0_rad;
+    }
+    const double diam = grid_diameter(shape);
+    dg_status st;
+    if (!(L.G == G && L.diam >= diam && !L.batches.empty())) {
+        CdftLayout n;
+        n.G = G;
+        n.diam = diam;
+        const int s_max = (int)std::max(1.0, std::min((double)std::min(c->K, 65535), std::floor(4294967296.0 / (16.0 * (double)G))));
+        std::vector<int> bb, gb;
+        for (int k0 = 0; k0 < c->K; k0 += s_max) {
+            const int S = std::min(s_max, c->K - k0);
+            CdftLayout::Batch t{k0, S, (int)bb.size(), 0, 0};
+            for (int s = 0; s <= S; ++s) {
+                if (t.nbt > (1 << 26) || t.groups > (1 << 30)) return DG_OK;
+                bb.push_back((int)t.nbt);
+                gb.push_back((int)t.groups);
+                if (s == S) break;
+                const int slots = lag_slots(c->eph_host[k0 + s], c->fs, diam);
+                t.nbt += slots;
+                t.groups += G / kDirectGroup + slots + 1;
+            }
+            n.batches.push_back(t);
+            n.s_max = std::max(n.s_max, S);
+            n.nbt_max = std::max(n.nbt_max, t.nbt);
+            n.groups_max = std::max(n.groups_max, t.groups);
+        }
+        n.bbase = L.bbase;
+        n.gbase = L.gbase;
+        L = n;
+        L.G = -1;  // until its tables are in place
+        if ((st = grow(c, &L.bbase, bb.size())) != DG_OK) return st;
+        if ((st = grow(c, &L.gbase, gb.size())) != DG_OK) return st;
+        // pageable sources: staged before the calls return
+        CK(c, cudaMemcpyAsync(L.bbase, bb.data(), sizeof(int) * bb.size(), cudaMemcpyHostToDevice, c->stream));
+        CK(c, cudaMemcpyAsync(L.gbase, gb.data(), sizeof(int) * gb.size(), cudaMemcpyHostToDevice, c->stream));
+        L.G = G;
+    }
+    // segments of samples: enough warps for about 8 rounds of the chip at 48
+    // warps per SM, from the whole grid's size (a row shard sums alike), in
+    // multiples of 256 samples
+    int nmax = 1;
+    for (int k = 0; k < c->K; ++k) nmax = std::max(nmax, (int)c->steps[k].n);
+    const double warps = (double)gd.nlat * gd.nlon / 32.0 * c->K;
+    const int want = (int)std::min(64.0, std::ceil(8.0 * 48.0 * 152.0 / std::max(warps, 1.0)));
+    const int seg_len = std::max(1, (nmax + 256 * want - 1) / (256 * want)) * 256;
+    const int nseg = (nmax + seg_len - 1) / seg_len;
+    if ((st = push_steps(c)) != DG_OK) return st;
+    const size_t S = (size_t)L.s_max, SG = S * (size_t)G;
+    if ((st = ensure_sort(c, S, SG, (size_t)L.nbt_max, (size_t)L.groups_max)) != DG_OK) return st;
+    if (nseg > 1 && (st = ensure(c, (void **)&b.part, &b.part_cap, sizeof(float2) * SG * nseg)) != DG_OK) return st;
+    if ((st = ensure_ephf(c)) != DG_OK) return st;
+    if (b.xyzf_cap < (size_t)G) {
+        if ((st = grow(c, &b.xyzf, 6 * (size_t)G)) != DG_OK) return st;
+        b.xyzf_cap = (size_t)G;
+    }
+    const bool one = L.batches.size() == 1;
+    {
+        Timed t(c, refine ? DG_K_REFINE : DG_K_CORR);
+        CK(c, launch_ecef_split(xyz, G, b.xyzf, c->stream, one ? b.lr : nullptr, b.nur, one ? L.s_max : 0));
+        t.done(1);
+    }
+    int slots = 0;
+    for (int k = 0; k < c->K; ++k) slots = std::max(slots, lag_slots(c->eph_host[k], c->fs, L.diam));
+    // one CTA sorts a snapshot where that is shorter than the three launches
+    const bool small = G <= kSortNodes && slots <= kSortSlots;
+    const bool fused = one && nseg > 1;  // the segments' sums go straight into the sum over snapshots
+    for (const auto &bt : L.batches) {
+        CdftBatch a{};
+        sort_args(c, bt, L, gd, xyz, G, a);
+        a.group = kDirectGroup;
+        a.nu_max = 0.2f;
+        a.mma = 1;  // no FP32 DFT table
+        a.lr_ready = one;
+        Timed t(c, refine ? DG_K_REFINE : DG_K_CORR);
+        CK(c, launch_cdft_geo(a, c->stream));
+        int n = one ? 1 : 2;
+        if (small) {
+            CK(c, launch_sort_small(a, c->stream));
+            n += 1;
+        } else {
+            CK(c, cudaMemsetAsync(b.g2b, 0xff, sizeof(int4) * (size_t)bt.groups, c->stream));
+            CK(c, launch_cdft_plan(a, (int)bt.nbt, c->stream));
+            n += 3;
+        }
+        float *sf = (float *)surf;
+        CK(c, launch_corr_lag(a, nseg, seg_len, sf, nseg > 1 ? b.part : nullptr, c->stream));
+        ++n;
+        if (nseg > 1) {
+            CK(c, launch_corr_segments(b.part, bt.S, nseg, G, c->opt.acc, sf + (size_t)bt.k0 * G,
+                                       fused ? (float *)out : nullptr, c->stream));
+            ++n;
+        }
+        t.done(n);
+    }
+    if (!fused) {
+        Timed t(c, refine ? DG_K_REFINE : DG_K_ACCUM);
+        CK(c, launch_accumulate(surf, c->K, G, DG_PREC_FP32, out, c->stream));
+        t.done(1);
+    }
+    CK(c, cudaMemcpyAsync(c->err_h, c->err_d, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+    *done = true;
+    return DG_OK;
+}
+
 // The phases of one chunked-DFT surface: setup (layout, chunks, buffers,
 // the candidates' double-float split), then per batch of snapshots its
 // arguments, plan, contraction and combine, then the ordered accumulation.
@@ -781,26 +995,10 @@ static dg_status cdft_setup(dg_ctx *c, CdftRun &r)
     }
     // scratch, grown on demand (never inside a captured graph: a graph is
     // captured after one uncaptured call of the same shape)
-    if (b.s_cap < (size_t)s_max) {
-        if ((st = grow(c, &b.lr, 2 * (size_t)s_max)) != DG_OK) return st;
-        if ((st = grow(c, &b.delta, (size_t)s_max)) != DG_OK) return st;
-        if ((st = grow(c, &b.nubase, (size_t)s_max)) != DG_OK) return st;
-        if ((st = grow(c, &b.nur, 2 * (size_t)s_max)) != DG_OK) return st;
-        if ((st = grow(c, &b.tbase, (size_t)s_max + 1)) != DG_OK) return st;
-        if ((st = grow(c, &b.hbase, (size_t)s_max + 1)) != DG_OK) return st;
-        if ((st = grow(c, &b.layout, (size_t)s_max)) != DG_OK) return st;
-        if ((st = grow(c, &b.Mcs, (size_t)s_max)) != DG_OK) return st;
-        b.s_cap = (size_t)s_max;
-    }
+    if ((st = ensure_sort(c, (size_t)s_max, (size_t)s_max * G, (size_t)L.nbt_max, (size_t)L.groups_max)) != DG_OK)
+        return st;
     if (!b.work) {
         if ((st = grow(c, &b.work, 2)) != DG_OK) return st;
-    }
-    if (b.sg_cap < (size_t)s_max * G) {
-        if ((st = grow(c, &b.candL, (size_t)s_max * G)) != DG_OK) return st;
-        if ((st = grow(c, &b.candNu, (size_t)s_max * G)) != DG_OK) return st;
-        if ((st = grow(c, &b.order, (size_t)s_max * G)) != DG_OK) return st;
-        if ((st = grow(c, &b.nuS, (size_t)s_max * G)) != DG_OK) return st;
-        b.sg_cap = (size_t)s_max * G;
     }
     if (c->opt.delay != DG_DELAY_INTEGER && b.mu_cap < (size_t)s_max * G) {
         if ((st = grow(c, &b.candMu, (size_t)s_max * G)) != DG_OK) return st;
@@ -811,14 +1009,6 @@ static dg_status cdft_setup(dg_ctx *c, CdftRun &r)
         if ((st = grow(c, &b.V, (size_t)s_max * M_max * 64)) != DG_OK) return st;
         b.v_cap = (size_t)s_max * M_max * 64;
     }
-    if (b.nb_cap < (size_t)L.nbt_max) {
-        const size_t n = (size_t)L.nbt_max;
-        if ((st = grow(c, &b.count, n)) != DG_OK) return st;
-        if ((st = grow(c, &b.need, n)) != DG_OK) return st;
-        if ((st = grow(c, &b.offs, n)) != DG_OK) return st;
-        if ((st = grow(c, &b.subcnt, n)) != DG_OK) return st;
-        b.nb_cap = n;
-    }
     const size_t w_elems = (size_t)L.nbt_max * (size_t)B_max * 128;
     if (w_elems * sizeof(float) > ((size_t)64 << 30))
         return fail(c, DG_EUNSUPPORTED, "CDFT: the per-lag DFT buffer would exceed 64 GiB (%lld lag slots x %d chunks); "
@@ -826,10 +1016,6 @@ static dg_status cdft_setup(dg_ctx *c, CdftRun &r)
     if (b.w_cap < w_elems) {
         if ((st = grow(c, &b.W, w_elems)) != DG_OK) return st;
         b.w_cap = w_elems;
-    }
-    if (b.g2b_cap < (size_t)L.groups_max) {
-        if ((st = grow(c, &b.g2b, (size_t)L.groups_max)) != DG_OK) return st;
-        b.g2b_cap = (size_t)L.groups_max;
     }
     if (mma) {
         const size_t bt = (size_t)s_max * cdft_btab_bytes(c->opt.contract, M_max);
@@ -869,11 +1055,6 @@ static void cdft_args(dg_ctx *c, const CdftRun &r, size_t bi, CdftBatch &a)
     const double *xyz = r.xyz;
     const GridDev &gd = r.gd;
     const int64_t G = r.G;
-    // constants of the geometry as double-float (hi, lo) pairs
-    auto split = [](double d, float &h, float &l) {
-        h = (float)d;
-        l = (float)(d - (double)h);
-    };
     const auto &bt = L.batches[bi];
     const int k0 = bt.k0, S = bt.S, M = Ms[bi];
     int Bmax = 1;
@@ -882,52 +1063,19 @@ static void cdft_args(dg_ctx *c, const CdftRun &r, size_t bi, CdftBatch &a)
         c->cd_chunk_min = std::min(c->cd_chunk_min, M);
         c->cd_chunk_max = std::max(c->cd_chunk_max, M);
     }
-    a.xyz = xyz;
-    a.xyzf = b.xyzf;
-    a.ephf = b.ephf + 24 * (size_t)k0;
-    split(c->fs / kC, a.fsc_hi, a.fsc_lo);
-    split(1.0 / (c->lambda * c->fs), a.ilf_hi, a.ilf_lo);
-    a.eph = c->eph + 12 * (size_t)k0;
-    a.sd = c->steps_d + k0;
-    a.S = S;
-    a.k0 = k0;
-    a.G = G;
-    a.nrows = gd.nrows;
-    a.nlon = gd.nlon;
-    a.fs = c->fs;
-    a.lambda = c->lambda;
+    sort_args(c, bt, L, gd, xyz, G, a);
     a.M = M;
     a.Bmax = Bmax;
-    a.acc = c->opt.acc;
-    a.err = c->err_d;
-    a.lr = b.lr;
-    a.nur = b.nur;
-    a.nubase = b.nubase;
-    a.bbase = L.bbase + bt.base;
-    a.gbase = L.gbase + bt.base;
-    a.candL = b.candL;
-    a.candNu = b.candNu;
-    a.order = b.order;
-    a.nuS = b.nuS;
-    a.g2b = b.g2b;
-    a.delta = b.delta;
     a.V = b.V;
-    a.count = b.count;
-    a.need = b.need;
-    a.delay = c->opt.delay;
-    a.candMu = b.candMu;
-    a.muS = b.muS;
-    a.offs = b.offs;
-    a.subcnt = b.subcnt;
     a.W = b.W;
     a.tbase = b.tbase;
     a.hbase = b.hbase;
     a.layout = b.layout;
     a.Mcs = b.Mcs;
     a.work = refine ? nullptr : b.work;
+    a.group = kCdftCombineGroup;
     a.tiles_mode = c->opt.tiles;
     a.mma = mma ? 1 : 0;
-    a.ngroups = (int)bt.groups;
     a.btab = b.btab;
     // FP16 needs the lag products inside its range: int16 products reach 2^31
     const int f = c->steps[k0].fmt;
@@ -2704,6 +2852,11 @@ dg_status dg_destroy(dg_ctx *c)
     fr(c->co.P);
     fr(c->co.A);
     fr(c->co.part);
+    fr(c->cd.part);
+    fr(c->cd.dmain_layout.bbase);
+    fr(c->cd.dmain_layout.gbase);
+    fr(c->cd.dloc_layout.bbase);
+    fr(c->cd.dloc_layout.gbase);
     fr(c->cd.main_layout.bbase);
     fr(c->cd.main_layout.gbase);
     fr(c->cd.loc_layout.bbase);

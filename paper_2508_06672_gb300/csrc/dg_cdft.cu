@@ -84,6 +84,11 @@ __global__ void __launch_bounds__(256, 4) k_cdft_geo(CdftBatch a)
         int L = INT_MIN;
         float mu = 0.f;
         bool ok = fabsf(D.hi) < 1.0e9f;
+        if (a.nu_max > 0.f && !(fabsf(nuf) <= a.nu_max)) {
+            atomicOr(a.err, ERR_NU_RANGE);
+            a.candL[(size_t)s * a.G + p] = INT_MIN;
+            continue;
+        }
         if (ok && !(a.delay == DG_DELAY_INTEGER ? round_df(D, L) : floor_df(D, L, mu))) {
             double e[12], D64, nu64;
             for (int t = 0; t < 12; ++t) e[t] = a.eph[12 * (size_t)s + t];
@@ -282,7 +287,7 @@ __global__ void __launch_bounds__(1024) k_cdft_scan(CdftBatch a)
     for (int i = b0; i < b1; ++i) {
         const int n = a.count[b_first + i];
         c += n;
-        g += (n + kCdftCombineGroup - 1) / kCdftCombineGroup;
+        g += (n + a.group - 1) / a.group;
     }
     s_c[t] = c;
     s_g[t] = g;
@@ -303,10 +308,10 @@ __global__ void __launch_bounds__(1024) k_cdft_scan(CdftBatch a)
         a.need[b] = nd ? 1 : 0;
         a.offs[b] = oc;
         const int n = a.count[b];
-        const int ng = (n + kCdftCombineGroup - 1) / kCdftCombineGroup;
+        const int ng = (n + a.group - 1) / a.group;
         for (int g = 0; g < ng; ++g)
             a.g2b[a.gbase[s] + og + g] =
-                make_int4(b, s, oc + g * kCdftCombineGroup, min(kCdftCombineGroup, n - g * kCdftCombineGroup));
+                make_int4(b, s, oc + g * a.group, min(a.group, n - g * a.group));
         oc += n;
         og += ng;
     }
@@ -491,6 +496,87 @@ __global__ void __launch_bounds__(256, 3) k_cdft_scatter(CdftBatch a)
         a.nuS[dst] = s_nu[p];
         if (frac) a.muS[dst] = s_mu[p];
     }
+}
+
+// ---------------------------------------------------------------------------
+// The sort of a small grid (at most kSortNodes candidates, kSortSlots lag
+// slots) in one launch: hist, scan and scatter of one snapshot by one CTA with
+// the buckets in shared memory. Three launches and four memsets cost more than
+// the work there (101^2 nodes, one snapshot: 27 us of kernels and as many
+// launch gaps).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(1024) k_sort_small(CdftBatch a)
+{
+    __shared__ int s_cnt[kSortSlots];
+    __shared__ int s_c[32], s_g[32];
+    const int s = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int lmin = a.lr[2 * s], bb = a.bbase[s], g0 = a.gbase[s], gcap = a.gbase[s + 1] - g0;
+    int NB = a.lr[2 * s + 1] >= lmin ? a.lr[2 * s + 1] - lmin + 1 : 0;
+    if (NB > a.bbase[s + 1] - bb || NB > kSortSlots) {
+        if (t == 0) atomicOr(a.err, ERR_LAG_RANGE);
+        NB = 0;
+    }
+    const int *Ls = a.candL + (size_t)s * a.G;
+    for (int i = t; i < NB; i += 1024) s_cnt[i] = 0;
+    __syncthreads();
+    const int G = (int)a.G;
+    for (int p = t; p < G && NB; p += 1024) {
+        const int l = Ls[p];
+        if (l != INT_MIN) atomicAdd(s_cnt + (l - lmin), 1);
+    }
+    __syncthreads();
+    // exclusive prefix sums of the candidates and of the groups per bucket;
+    // thread t owns buckets t * per ..
+    const int per = (NB + 1023) / 1024, b0 = min(NB, t * per), b1 = min(NB, b0 + per);
+    int c = 0, g = 0;
+    for (int b = b0; b < b1; ++b) {
+        c += s_cnt[b];
+        g += (s_cnt[b] + a.group - 1) / a.group;
+    }
+    int ci = c, gi = g;  // inclusive over the warp
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, ci, d), y = __shfl_up_sync(0xffffffffu, gi, d);
+        if (lane >= d) {
+            ci += x;
+            gi += y;
+        }
+    }
+    if (lane == 31) {
+        s_c[warp] = ci;
+        s_g[warp] = gi;
+    }
+    __syncthreads();
+    int oc = ci - c, og = gi - g, total = 0;
+    for (int w = 0; w < 32; ++w) {
+        if (w < warp) {
+            oc += s_c[w];
+            og += s_g[w];
+        }
+        total += s_g[w];
+    }
+    for (int b = b0; b < b1; ++b) {
+        const int n = s_cnt[b];
+        for (int i = 0; i < n; i += a.group) a.g2b[g0 + og++] = make_int4(bb + b, s, oc + i, min(a.group, n - i));
+        s_cnt[b] = oc;  // the bucket's fill cursor
+        oc += n;
+    }
+    for (int i = total + t; i < gcap; i += 1024) a.g2b[g0 + i] = make_int4(-1, -1, -1, -1);
+    __syncthreads();
+    const size_t so = (size_t)s * a.G;
+    for (int p = t; p < G && NB; p += 1024) {
+        const int l = Ls[p];
+        if (l == INT_MIN) continue;
+        const int at = atomicAdd(s_cnt + (l - lmin), 1);
+        a.order[so + at] = p;
+        a.nuS[so + at] = a.candNu[so + p];
+    }
+}
+
+cudaError_t launch_sort_small(const CdftBatch &a, cudaStream_t st)
+{
+    k_sort_small<<<a.S, 1024, 0, st>>>(a);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -860,8 +946,16 @@ static unsigned grid_for(int64_t n, int per, int cap = 152 * 16)
     return (unsigned)(b < 1 ? 1 : b);
 }
 
-__global__ void __launch_bounds__(256) k_ecef_split(const double *__restrict__ xyz, int64_t G, float *__restrict__ xf)
+__global__ void __launch_bounds__(256) k_ecef_split(const double *__restrict__ xyz, int64_t G, float *__restrict__ xf,
+                                                    int *lr, unsigned *nur, int S)
 {
+    if (blockIdx.x == 0)
+        for (int s = threadIdx.x; s < S; s += blockDim.x) {
+            lr[2 * s] = INT_MAX;
+            lr[2 * s + 1] = INT_MIN;
+            nur[2 * s] = 0xffffffffu;
+            nur[2 * s + 1] = 0u;
+        }
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < G; p += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -872,15 +966,15 @@ __global__ void __launch_bounds__(256) k_ecef_split(const double *__restrict__ x
     }
 }
 
-cudaError_t launch_ecef_split(const double *xyz, int64_t G, float *xyzf, cudaStream_t st)
+cudaError_t launch_ecef_split(const double *xyz, int64_t G, float *xyzf, cudaStream_t st, int *lr, unsigned *nur, int S)
 {
-    k_ecef_split<<<grid_for(G, 256), 256, 0, st>>>(xyz, G, xyzf);
+    k_ecef_split<<<grid_for(G, 256), 256, 0, st>>>(xyz, G, xyzf, lr, nur, S);
     return cudaGetLastError();
 }
 
 cudaError_t launch_cdft_geo(const CdftBatch &a, cudaStream_t st)
 {
-    k_cdft_lr_init<<<(a.S + 127) / 128, 128, 0, st>>>(a.lr, a.nur, a.S);
+    if (!a.lr_ready) k_cdft_lr_init<<<(a.S + 127) / 128, 128, 0, st>>>(a.lr, a.nur, a.S);
     dim3 grid(grid_for(a.G, 256 * 4, 152 * 8), (unsigned)a.S);
     k_cdft_geo<<<grid, 256, 0, st>>>(a);
     return cudaGetLastError();

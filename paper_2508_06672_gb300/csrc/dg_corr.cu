@@ -296,6 +296,200 @@ __global__ void __launch_bounds__(kThreads) k_corr_direct(CorrArgs a, int tiles_
     }
 }
 
+// ---------------------------------------------------------------------------
+// The same sum with the candidates grouped by lag (FP32, integer delay): all
+// candidates of a lag share z[n] = y1[n] conj(y2[n + L]), so a warp forms z
+// once (32 samples per instruction, into its slice of shared memory) and runs
+// the resonators of up to 32 candidates of that lag on broadcast reads of it:
+//     s[n] = (z[n] (-j)^n - s[n-2]) + 2 cos(theta) s[n-1];
+// with v[n] = s[n] times the signs +, +, -, - the subtraction is an addition,
+//     v[n] = (z[n] {1, -j}[n % 2] + v[n-2]) -/+ 2 cos(theta) v[n-1]  (n even / odd):
+// one packed addition and one packed FMA per candidate and sample where
+// the kernel above issues 6 FMAs and an 8-byte shared load of its own (2
+// cycles of the shared-memory port per warp, its bound). The FP32 pipe bounds
+// it: 4 operations per candidate-sample.
+// The lag sort (k_cdft_geo, hist, scan, scatter) gives the groups. Small
+// problems split the samples into segments (blockIdx.y) to fill the chip; a
+// segment's sum carries its absolute phase and k_corr_segments adds them in
+// order.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float2 add_x2(float2 a, float2 b)
+{
+    unsigned long long r, x, y;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(r));
+    return d;
+}
+__device__ __forceinline__ float2 fma_x2(float2 a, float2 b, float2 c)
+{
+    unsigned long long r, x, y, z;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(c.x), "f"(c.y));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(r));
+    return d;
+}
+
+constexpr int kLagChunk = 128;  // samples of z per warp and pass
+
+// One group's segment by one warp, R candidates per lane.
+template <int FMT, int R>
+__device__ __forceinline__ void corr_lag_group(const CdftBatch &a, const int4 &gr, const StepDesc &sd, int L, int n0,
+                                               int end, float2 *z, float *surf, float2 *part)
+{
+    const int lane = threadIdx.x & 31, s = gr.y, N = sd.n;
+    int cand[R];
+    float nu[R];
+    float2 cp[R], cn[R], v1[R], v2[R];  // +-2 cos(theta), v[n - 1], v[n - 2]
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const size_t at = (size_t)s * a.G + gr.z + min(lane + 32 * r, gr.w - 1);
+        cand[r] = a.order[at];
+        nu[r] = a.nuS[at];
+        const float c2 = -2.f * sinpif(2.f * nu[r]);
+        cp[r] = make_float2(c2, c2);
+        cn[r] = make_float2(-c2, -c2);
+        v1[r] = v2[r] = make_float2(0.f, 0.f);
+    }
+    // this lane's samples of the next pass: n0 + lane + 32 i, times -j where n
+    // (and so the lane) is odd
+    constexpr int E = kLagChunk / 32;
+    float2 x[E], y[E];
+    auto fetch = [&](int n) {
+        if (n + kLagChunk <= end && n + L >= 0 && n + L + kLagChunk <= N) {
+#pragma unroll
+            for (int i = 0; i < E; ++i) {
+                x[i] = IQ<FMT>::load(sd.y1, n + lane + 32 * i);
+                y[i] = IQ<FMT>::load(sd.y2, n + lane + 32 * i + L);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < E; ++i) {
+                const int q = n + lane + 32 * i, r = q + L;
+                x[i] = q < end ? IQ<FMT>::load(sd.y1, q) : make_float2(0.f, 0.f);
+                y[i] = q < end && r >= 0 && r < N ? IQ<FMT>::load(sd.y2, r) : make_float2(0.f, 0.f);
+            }
+        }
+    };
+    fetch(n0);
+    for (int n = n0; n < end; n += kLagChunk) {
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            const float zx = fmaf(x[i].x, y[i].x, x[i].y * y[i].y), zy = fmaf(x[i].y, y[i].x, -x[i].x * y[i].y);
+            z[lane + 32 * i] = lane & 1 ? make_float2(zy, -zx) : make_float2(zx, zy);
+        }
+        __syncwarp();
+        if (n + kLagChunk < end) fetch(n + kLagChunk);
+        const int len = min(kLagChunk, (end - n + 1) & ~1);  // zeros beyond the capture
+        const float4 *z4 = reinterpret_cast<const float4 *>(z);
+#pragma unroll 8
+        for (int m = 0; m < len / 2; ++m) {
+            const float4 q = z4[m];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v2[r] = fma_x2(cn[r], v1[r], add_x2(make_float2(q.x, q.y), v2[r]));
+#pragma unroll
+            for (int r = 0; r < R; ++r) v1[r] = fma_x2(cp[r], v2[r], add_x2(make_float2(q.z, q.w), v1[r]));
+        }
+    }
+    // the last pair's common sign: + for an even number of pairs before it
+    const float sg = (((end - n0 + 1) >> 1) - 1) & 1 ? -1.f : 1.f;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        if (lane + 32 * r >= gr.w) continue;
+        // close: e^{j theta (n_end - 1)} (s[n_end - 1] - e^{j theta} s[n_end - 2]), e^{j theta} = j e^{j 2 pi nu}
+        float st, ct;
+        sincospif(2.f * nu[r], &st, &ct);
+        const float2 s1 = make_float2(sg * v1[r].x, sg * v1[r].y), s2 = make_float2(sg * v2[r].x, sg * v2[r].y);
+        const float ux = s1.x + fmaf(st, s2.x, ct * s2.y), uy = s1.y + fmaf(st, s2.y, -ct * s2.x);
+        if (!part) {
+            const float pw = fmaf(ux, ux, uy * uy);
+            surf[(size_t)(a.k0 + s) * a.G + cand[r]] = a.acc == DG_ACC_POWER ? pw : sqrtf(pw);
+        } else {
+            const int e = n0 + ((end - n0 + 1) & ~1) - 1;
+            float se, ce;
+            sincospif(2.f * (frac_mul(nu[r], (float)e) + 0.25f * (float)(e & 3)), &se, &ce);
+            part[((size_t)s * gridDim.y + blockIdx.y) * a.G + cand[r]] =
+                make_float2(fmaf(ce, ux, -se * uy), fmaf(ce, uy, se * ux));
+        }
+    }
+}
+
+template <int FMT>
+__device__ __forceinline__ void corr_lag_fmt(const CdftBatch &a, const int4 &gr, const StepDesc &sd, int L, int n0,
+                                             int end, float2 *z, float *surf, float2 *part)
+{
+    if (gr.w > 32) corr_lag_group<FMT, 2>(a, gr, sd, L, n0, end, z, surf, part);
+    else corr_lag_group<FMT, 1>(a, gr, sd, L, n0, end, z, surf, part);
+}
+
+__global__ void __launch_bounds__(256) k_corr_lag(CdftBatch a, int seg_len, float *surf, float2 *part)
+{
+    __shared__ __align__(16) float2 s_z[8][kLagChunk];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t g = blockIdx.x * (int64_t)8 + warp;
+    if (g >= a.ngroups) return;
+    const int4 gr = a.g2b[g];
+    if (gr.x < 0) return;
+    const int s = gr.y;
+    const StepDesc sd = a.sd[s];
+    const int n0 = blockIdx.y * seg_len, N = sd.n;
+    if (n0 >= N) {  // a capture shorter than the longest: an empty segment
+        for (int i = lane; part && i < gr.w; i += 32)
+            part[((size_t)s * gridDim.y + blockIdx.y) * a.G + a.order[(size_t)s * a.G + gr.z + i]] = make_float2(0.f, 0.f);
+        return;
+    }
+    const int end = min(N, n0 + seg_len), L = a.lr[2 * s] + (gr.x - a.bbase[s]);
+    if (sd.fmt == DG_IQ_CI16) corr_lag_fmt<DG_IQ_CI16>(a, gr, sd, L, n0, end, s_z[warp], surf, part);
+    else if (sd.fmt == DG_IQ_CI8) corr_lag_fmt<DG_IQ_CI8>(a, gr, sd, L, n0, end, s_z[warp], surf, part);
+    else corr_lag_fmt<DG_IQ_C64>(a, gr, sd, L, n0, end, s_z[warp], surf, part);
+}
+
+// Segment sums to surface values: of each snapshot (surf), or summed over the
+// snapshots in order (out).
+__global__ void __launch_bounds__(256) k_corr_segments(const float2 *__restrict__ part, int S, int nseg, int64_t G,
+                                                       int acc, float *__restrict__ surf, float *__restrict__ out)
+{
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < G; p += (int64_t)gridDim.x * blockDim.x) {
+        float sum = 0.f;
+        for (int s = out ? 0 : blockIdx.y; s < (out ? S : blockIdx.y + 1); ++s) {
+            const float2 *q = part + (size_t)s * nseg * G + p;
+            float2 c = make_float2(0.f, 0.f);
+#pragma unroll 4
+            for (int i = 0; i < nseg; ++i) {
+                const float2 v = __ldg(q + (size_t)i * G);
+                c.x += v.x;
+                c.y += v.y;
+            }
+            float pw = fmaf(c.x, c.x, c.y * c.y);
+            if (acc != DG_ACC_POWER) pw = sqrtf(pw);
+            if (out) sum = s ? sum + pw : pw;
+            else surf[(size_t)s * G + p] = pw;
+        }
+        if (out) out[p] = sum;
+    }
+}
+
+cudaError_t launch_corr_lag(const CdftBatch &a, int nseg, int seg_len, float *surf, float2 *part, cudaStream_t s)
+{
+    k_corr_lag<<<dim3((unsigned)((a.ngroups + 7) / 8), (unsigned)nseg), 256, 0, s>>>(a, seg_len, surf, part);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_corr_segments(const float2 *part, int S, int nseg, int64_t G, int acc, float *surf, float *out,
+                                 cudaStream_t s)
+{
+    int64_t b = (G + 255) / 256;
+    if (b > 152 * 8) b = 152 * 8;
+    k_corr_segments<<<dim3((unsigned)b, out ? 1u : (unsigned)S), 256, 0, s>>>(part, S, nseg, G, acc, surf, out);
+    return cudaGetLastError();
+}
+
 template <typename T, int FMT, int DELAY, int R>
 static cudaError_t launch_one(const CorrArgs &a, cudaStream_t s)
 {

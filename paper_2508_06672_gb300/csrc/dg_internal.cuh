@@ -323,6 +323,17 @@ inline bool direct_rows_ok(int prec, int rows)
 // Launch the direct correlation for all K snapshots (one launch).
 cudaError_t launch_corr_direct(const CorrArgs &a, cudaStream_t s);
 
+// The direct correlation of candidates grouped by lag (dg_corr.cu): FP32,
+// integer delay. part: [S][nseg][G] complex sums of the segments of samples
+// (nseg > 1), else surf receives |C|^2 or |C| of the batch's snapshots.
+struct CdftBatch;
+constexpr int kDirectGroup = 64;  // candidates per warp
+cudaError_t launch_corr_lag(const CdftBatch &a, int nseg, int seg_len, float *surf, float2 *part, cudaStream_t s);
+// surf[s][p] of the segments' sums (out = NULL), or out[p] = their ordered sum
+// over the S snapshots
+cudaError_t launch_corr_segments(const float2 *part, int S, int nseg, int64_t G, int acc, float *surf, float *out,
+                                 cudaStream_t s);
+
 // out[p] = sum_k surf[k][p], k in order.
 cudaError_t launch_accumulate(const void *surf, int K, int64_t G, int prec, void *out,
                               cudaStream_t s);
@@ -387,6 +398,9 @@ struct CdftBatch {
     float *candMu;                // [S][G] fractional delay mu = D - floor(D) (Lagrange4 only)
     float *muS;                   // [S][G] mu in sorted order (Lagrange4 only)
     int *need;                    // [NBT] 1: the bucket's per-lag DFT rows are computed (scan)
+    int group;                    // candidates per combine group (scan's records)
+    float nu_max;                 // candidates beyond this FDOA are left out (ERR_NU_RANGE); 0: no limit
+    int lr_ready;                 // the ranges lr, nur are initialised (launch_ecef_split)
 };
 
 // Bucket b's rows are needed when a candidate's lag stencil reaches it: its
@@ -420,8 +434,15 @@ cudaError_t launch_cdft_contract_jobs(const TcJob *jobs, int n, const int *job_t
                                       unsigned wait_polls, cudaStream_t s);
 
 cudaError_t launch_cdft_geo(const CdftBatch &a, cudaStream_t s);
-// xyzf[6][G] = double-float split of xyz[3][G]
-cudaError_t launch_ecef_split(const double *xyz, int64_t G, float *xyzf, cudaStream_t s);
+// xyzf[6][G] = double-float split of xyz[3][G]; also initialises the lag and
+// FDOA ranges of S snapshots (lr != NULL)
+cudaError_t launch_ecef_split(const double *xyz, int64_t G, float *xyzf, cudaStream_t s, int *lr = nullptr,
+                              unsigned *nur = nullptr, int S = 0);
+// The lag sort of small grids in one launch (order, nuS and every group record
+// of the batch): one CTA per snapshot, at most kSortSlots lag slots each.
+constexpr int kSortSlots = 8192;
+constexpr int64_t kSortNodes = 32768;
+cudaError_t launch_sort_small(const CdftBatch &a, cudaStream_t s);
 cudaError_t launch_cdft_plan(const CdftBatch &a, int NBT, cudaStream_t s);
 cudaError_t launch_cdft_contract_fp32(const CdftBatch &a, int NBT, int fmt, cudaStream_t s);
 cudaError_t launch_cdft_combine(const CdftBatch &a, float *surf, cudaStream_t s);

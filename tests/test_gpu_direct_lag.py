@@ -1,0 +1,58 @@
+"""The direct FP32 correlation with the candidates grouped by lag: against
+the oracle over group sizes (under and over a warp's 32 and 64 candidates),
+both lag sorts, segments of samples that do not divide the capture, formats,
+and captures of different lengths in one launch."""
+import numpy as np
+import pytest
+
+import oracle
+import sim
+from gpu_common import gpu_surface, lag_boundary_mask, package, rel_err, torch_cuda
+
+pytestmark = pytest.mark.gpu
+FP32_TOL = 1e-4
+
+
+def _check(s, c, acc=0, npts=1200):
+    idx = np.unique(np.random.default_rng(1).integers(0, s.G, npts))
+    ref = oracle.cost_points(*oracle.scene_args(s), idx=idx, acc_mode=acc)
+    ok = ~lag_boundary_mask(s, idx)
+    assert rel_err(c.ravel()[idx][ok], ref[ok], 0.01) < FP32_TOL
+
+
+# (grid, spacing): one lag for many candidates, a few per lag, hundreds per
+# lag; grids below and above the one-launch sort's 32768 nodes
+@pytest.mark.parametrize("grid,spacing", [((33, 31), 5.0), ((41, 37), 2000.0), ((5, 3000), 100.0), ((190, 181), 150.0)])
+@pytest.mark.parametrize("n", [1, 255, 256, 1025, 7003])
+def test_lag_groups_match_oracle(grid, spacing, n):
+    s = sim.make_scene(seed=61, fs_hz=12.5e6, n_samples=n, k_steps=2, fmt="ci16", waveform="noise", snr_db=-3.0,
+                       grid_n=grid, grid_spacing_m=spacing, bw_hz=10e6)
+    g, c = gpu_surface(s)
+    _check(s, c)
+    g.close()
+
+
+@pytest.mark.parametrize("fmt", ["c64", "ci8"])
+def test_lag_groups_of_uneven_captures(fmt):
+    """Snapshots of other lengths than the longest (empty last segments) and of
+    another format in the same launch."""
+    torch = torch_cuda()
+    P = package()
+    s = sim.make_scene(seed=62, fs_hz=12.5e6, n_samples=5000, k_steps=3, fmt="ci16", waveform="noise", snr_db=-3.0,
+                       grid_n=(61, 67), grid_spacing_m=300.0, bw_hz=10e6)
+    g = P.Geolocator(s.grid, s.ephem, s.fs_hz, s.fc_hz, acc="mag")
+    g.load_captures(s.fmt, torch.from_numpy(s.y1).cuda(), torch.from_numpy(s.y2).cuda())
+    n = 300
+    dt = np.float32 if fmt == "c64" else np.int8
+    a, b = ((y[1][:n] / 100.0).astype(dt) for y in (s.y1, s.y2))
+    g.load_capture(1, fmt, torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda())
+    c = g.cost_surface().double().cpu().numpy().ravel()
+    g.close()
+    idx = np.unique(np.random.default_rng(2).integers(0, s.G, 600))
+    ref = np.zeros(idx.size)
+    for k in range(3):
+        y1, y2 = (a[None], b[None]) if k == 1 else (s.y1[k:k + 1], s.y2[k:k + 1])
+        ref += oracle.cost_points(s.grid, s.ephem[k:k + 1], s.fs_hz, s.fc_hz, oracle.iq_to_f64(y1), oracle.iq_to_f64(y2),
+                                  idx=idx, acc_mode=1)
+    ok = ~lag_boundary_mask(s, idx)
+    assert rel_err(c[idx][ok], ref[ok], 0.01) < FP32_TOL
