@@ -17,14 +17,13 @@
 //     each tap's A operand is that staging seen through a shifted
 //     descriptor (k_conv3x3_tc). The weights are converted to BF16 blocks
 //     once per call and stream in by bulk copy.
-//   weight gradient: rows = output channels, columns = (input channel, tap)
-//     pairs plus one column of ones (the bias gradient), K = pixels:
+//   weight gradient: rows = output channels, columns = input channels, one
+//     accumulator per tap, K = pixels:
 //       dw[o,c,u,v] = sum_{n,i,j} dy[n,o,i,j] x[n,c,i+u-1,j+v-1]
-//       db[o]       = sum_{n,i,j} dy[n,o,i,j]
-//     split over pixel ranges; the partial sums are added in a fixed order.
-//     128 threads gather a 32-pixel K block of both operands (rounded to
-//     BF16) into one of two shared-memory stages while one thread issues the
-//     MMAs of the previous block.
+//       db[o]       = sum_{n,i,j} dy[n,o,i,j]   (of the rounded dy, CUDA cores)
+//     split over image rows; the partial sums are added in a fixed order. The
+//     operands are read MN-major from the same staging of 8-channel pixels
+//     (k_conv3x3_dw_tc).
 // The FP32 kernels in dg_nn.cu stay as the reference.
 #include <cuda_bf16.h>
 
@@ -36,8 +35,6 @@ namespace dg {
 namespace {
 
 constexpr int kRowsTc = 128;                 // MMA M
-constexpr int kKB = 32;                      // K elements per staged block
-constexpr int kABytes = kRowsTc * kKB * 2;   // one 128 x 32 BF16 block
 constexpr uint32_t kNnWaitLimit = 1u << 24;  // polls before an mbarrier wait gives up
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -70,6 +67,27 @@ __device__ __forceinline__ void nn_mma(uint32_t d, uint64_t ad, uint64_t bd, uin
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
         "l"(ad), "l"(bd), "r"(id), "r"(acc)
+        : "memory");
+}
+
+// One lane of a converged warp. The issuing warp runs its loop with all lanes and
+// only the instruction itself is predicated: descriptors then stay in uniform
+// registers, where a branch on one lane moves each of them there first.
+__device__ __forceinline__ uint32_t nn_elect()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
+    return p;
+}
+
+__device__ __forceinline__ void nn_mma_if(uint32_t lead, uint32_t d, uint64_t ad, uint64_t bd, uint32_t id, uint32_t acc)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
+        "l"(ad), "l"(bd), "r"(id), "r"(acc), "r"(lead)
         : "memory");
 }
 
@@ -386,155 +404,302 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3x3_tc(const float *__rest
 }
 
 // ---------------------------------------------------------------------------
-// Weight and bias gradient. CTA: all output channels (rows, CO <= 128),
-// columns kc0 .. kc0 + NC - 1 of the CI * 9 + 1 (input channel, tap) columns
-// (the last is the bias: a column of ones), pixels p_lo .. p_hi of the
-// flattened B x H x W pixels (K). Writes its partial sums to
-// part[split][o][column].
+// Weight and bias gradient: K = pixels, rows = output channels (CO <= 128),
+// columns = 32 input channels, one accumulator per tap (9 x 32 of the 512
+// tensor-memory columns).
+//
+// Both operands are staged as the forward's halo is: 16-byte rows of 8
+// channels of one pixel, consecutive pixels 16 B apart. Read with the channel
+// dimension as M / N and the pixels as K that is the canonical MN-major
+// layout (core matrix: 8 pixels x 8 channels, 128 B along the pixels, the
+// channel groups a row of pixels apart), so the x operand of tap (u, v) is the
+// same staged row seen v pixels further, and u is one of three staged rows:
+// nothing is gathered per tap. (With pixels contiguous in each row, the K-major
+// layout, a shift by one pixel is no aligned start; the gathers it took, 9
+// loads per element, were 2.05 ms of the 2.33 ms of a 64 -> 128 channel
+// backward at 16 x 128 x 128.)
+// A CTA walks output rows of `tw` pixels (i fastest) of one block of 32 input
+// channels: dy in two buffers, x rows in a ring of four. 16 warps load the next
+// row's dy and its one new x row into registers a whole step ahead and store
+// them rounded, while one more warp issues the current row's 9 x tw / 16 MMAs.
+// That warp runs its loop with all lanes (nn_elect): issued from a branch on one
+// thread an MMA took 130 cycles, most of them moving descriptors into uniform
+// registers, and the kernel 155 us at that size; now 82 us, bound by the 80 KB a
+// row that each CTA loads and converts (8 staging warps: 125 us). Channel groups
+// are padded by one pixel against bank conflicts. Partial sums:
+// part[split][tap][c][o], then the bias [split][o].
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_conv3x3_dw_tc(const float *__restrict__ x, const float *__restrict__ dy,
-                                                        float *__restrict__ part, int CI, int CO, int H, int W,
-                                                        int64_t P, int64_t per_split, int NC, unsigned *err)
+constexpr int kDwThreads = 512;                // staging threads; one more warp issues the MMAs
+constexpr int kDwCB = 32;                      // input channels per CTA
+constexpr int kDwRing = 4;                     // staged x rows
+
+// bytes of one dy buffer, of one x row
+__host__ __device__ constexpr int dw_a_bytes(int tw) { return (kRowsTc / 8) * (tw + 1) * 16; }
+__host__ __device__ constexpr int dw_x_bytes(int tw) { return (kDwCB / 8) * (tw + 2) * 16; }
+__host__ __device__ constexpr int dw_smem(int tw) { return 2 * dw_a_bytes(tw) + kDwRing * dw_x_bytes(tw); }
+
+// MN-major, no swizzle: pixel groups (K) 128 B apart (leading byte offset),
+// channel groups (M / N) `group` B apart (stride byte offset)
+__device__ __forceinline__ uint64_t mn_desc(uint32_t saddr, uint32_t group)
+{
+    return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(group >> 4) << 32) |
+           (1ull << 46);
+}
+
+__device__ __forceinline__ uint4 pack8(const float (&v)[8])
+{
+    uint32_t pk[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) pk[e] = bf16_bits(v[2 * e]) | (bf16_bits(v[2 * e + 1]) << 16);
+    return make_uint4(pk[0], pk[1], pk[2], pk[3]);
+}
+
+__global__ void __launch_bounds__(kDwThreads + 32, 1)
+    k_conv3x3_dw_tc(const float *__restrict__ x, const float *__restrict__ dy, float *__restrict__ part, int CI, int CO,
+                    int H, int W, int tw, int nb, int64_t rows, int64_t per_split, int S, unsigned *err)
 {
     extern __shared__ __align__(1024) unsigned char nsm[];
-    __shared__ __align__(8) uint64_t done[2], fin;
+    __shared__ __align__(8) uint64_t done[2];
     __shared__ uint32_t tslot;
-    __shared__ int pn[kKB], pi[kKB], pj[kKB];
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int ncol = CI * 9 + 1, kc0 = blockIdx.x * NC, split = blockIdx.y;
-    const int64_t p_lo = (int64_t)split * per_split, p_hi = min(P, p_lo + per_split);
-    const int nblk = p_hi > p_lo ? (int)((p_hi - p_lo + kKB - 1) / kKB) : 0;
-    const int bbytes = NC * kKB * 2;
-    unsigned char *stage[2] = {nsm, nsm + kABytes + bbytes};
+    const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane = t & 31;
+    const bool mma_warp = warp == kDwThreads / 32;  // ng <= 16 groups: no bias there
+    const int c0 = blockIdx.x * kDwCB, split = blockIdx.y;
+    const int64_t r_lo = (int64_t)split * per_split, r_hi = min(rows, r_lo + per_split);
+    const int nrow = r_hi > r_lo ? (int)(r_hi - r_lo) : 0;
+    const int abytes = dw_a_bytes(tw), xbytes = dw_x_bytes(tw), xq = tw + 2;
+    unsigned char *sa = nsm, *sx = nsm + 2 * abytes;
+    const int64_t HW = (int64_t)H * W;
     if (t == 0) {
         nn_mbar_init(smem_addr(&done[0]), 1);
         nn_mbar_init(smem_addr(&done[1]), 1);
-        nn_mbar_init(smem_addr(&fin), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) nn_tmem_alloc(smem_addr(&tslot), (uint32_t)tmem_cols(NC));
+    if (warp == 0) nn_tmem_alloc(smem_addr(&tslot), 512u);
+    // rows of output channels past CO are zero in both dy buffers
+    for (int i = t; i < 2 * abytes / 16; i += kDwThreads + 32)
+        *reinterpret_cast<uint4 *>(sa + 16 * (size_t)i) = make_uint4(0, 0, 0, 0);
     nn_before_sync();
     __syncthreads();
     nn_after_sync();
     const uint32_t tmem = tslot;
-    const uint32_t id = nn_idesc(NC);
-    const int64_t HW = (int64_t)H * W;
-    bool ok = true;
-    for (int kb = 0; kb < nblk; ++kb) {
-        const int sg = kb & 1;
-        if (kb >= 2) ok = ok && nn_wait(smem_addr(&done[sg]), (uint32_t)((kb - 2) >> 1) & 1u);
-        // the block's 32 pixels (image, row, column; -1: past the range)
-        if (t < kKB) {
-            const int64_t p = p_lo + (int64_t)kb * kKB + t;
-            if (p < p_hi) {
-                const int64_t nimg = p / HW, r = p - nimg * HW;
-                pn[t] = (int)nimg;
-                pi[t] = (int)(r / W);
-                pj[t] = (int)(r - (r / W) * W);
+    // FP32 D, BF16 A and B, both MN-major, N = 32, M = 128
+    const uint32_t id = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(kDwCB >> 3) << 17) |
+                        ((uint32_t)(kRowsTc >> 4) << 24);
+    const int ng = (CO + 7) / 8;  // groups of 8 output channels
+    struct Row {  // image, first column, row of a step
+        int n, j0, i;
+    };
+    auto next = [&](Row &o) {
+        if (++o.i == H) {
+            o.i = 0;
+            o.j0 += tw;
+            if (o.j0 >= nb * tw) {
+                o.j0 = 0;
+                ++o.n;
+            }
+        }
+    };
+    Row cur;  // the only divisions
+    cur.i = (int)(r_lo % H);
+    cur.j0 = (int)((r_lo / H) % nb) * tw;
+    cur.n = (int)(r_lo / H / nb);
+    // x row `row` of the strip (zero outside the image): into registers, and
+    // into its ring slot
+    constexpr int kXi = ((kDwCB / 8) * (kRowsTc + 2) + kDwThreads - 1) / kDwThreads;
+    float xv[kXi][8];
+    int xo[kXi], xcol[kXi], xch[kXi];  // this thread's pixels: offset of 8 channels, column and first channel
+#pragma unroll
+    for (int k = 0; k < kXi; ++k) {
+        const int it = t + k * kDwThreads;
+        xcol[k] = it % xq - 1;
+        xch[k] = it / xq < kDwCB / 8 ? c0 + 8 * (it / xq) : CI;
+        xo[k] = 16 * it;
+    }
+    auto load_x = [&](const Row &o, int row) {
+        const bool in = row >= 0 && row < H;
+#pragma unroll
+        for (int k = 0; k < kXi; ++k) {
+            const int col = o.j0 + xcol[k], nc = in && col >= 0 && col < W ? CI - xch[k] : 0;
+            const float *src = x + ((int64_t)o.n * CI + xch[k]) * HW + (int64_t)row * W + col;
+            if (nc >= 8) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) xv[k][e] = __ldg(src + e * HW);
             } else {
-                pn[t] = -1;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) xv[k][e] = e < nc ? __ldg(src + e * HW) : 0.f;
             }
         }
-        __syncthreads();
-        unsigned char *sa = stage[sg], *sb = sa + kABytes;
-        // A: output channel t over the 32 pixels, 8 per 16-byte row
+    };
+    auto store_x = [&](int row) {
+        unsigned char *dst = sx + (size_t)(row & (kDwRing - 1)) * xbytes;
 #pragma unroll
-        for (int g = 0; g < kKB / 8; ++g) {
-            uint32_t pk[4];
+        for (int k = 0; k < kXi; ++k)
+            if (xo[k] < xbytes) *reinterpret_cast<uint4 *>(dst + xo[k]) = pack8(xv[k]);
+    };
+    // dy: item k of a warp is a group of 8 channels x 32 pixels, lanes along the pixels
+    constexpr int kDi = (kRowsTc / 8) * (kRowsTc / 32) / (kDwThreads / 32);
+    float v[kDi][8];
+    auto load_dy = [&](const Row &o) {
+        const int left = min(tw, W - o.j0);
+        const float *base = dy + (int64_t)o.n * CO * HW + (int64_t)o.i * W + o.j0;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int kk = 8 * g + e;
-                float v = 0.f;
-                if (t < CO && pn[kk] >= 0)
-                    v = __ldg(dy + (((size_t)pn[kk] * CO + t) * H + pi[kk]) * W + pj[kk]);
-                const uint32_t h = bf16_bits(v);
-                pk[e >> 1] = (e & 1) ? (pk[e >> 1] | (h << 16)) : h;
-            }
-            *reinterpret_cast<uint4 *>(sa + kmaj(t, 8 * g)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-        }
-        // B: columns kc0 + t and kc0 + t + 128 over the 32 pixels
-        for (int row = t; row < NC; row += 128) {
-            const int col = kc0 + row;
-            const int c = col / 9, uv = col - 9 * c, u = uv / 3, vv = uv - 3 * u;
+        for (int k = 0; k < kDi; ++k) {
+            const int it = warp + k * (kDwThreads / 32), q = 32 * (it & 3) + lane, g = it >> 2;
+            const int nc = q < left ? min(8, CO - 8 * g) : 0;
+            const float *src = base + (int64_t)8 * g * HW + q;
+            if (nc >= 8) {
 #pragma unroll
-            for (int g = 0; g < kKB / 8; ++g) {
-                uint32_t pk[4];
+                for (int e = 0; e < 8; ++e) v[k][e] = __ldg(src + e * HW);
+            } else {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int kk = 8 * g + e;
-                    float v = 0.f;
-                    if (pn[kk] >= 0 && col < ncol) {
-                        if (col == ncol - 1) {
-                            v = 1.f;  // the bias column
-                        } else {
-                            const int ii = pi[kk] + u - 1, jj = pj[kk] + vv - 1;
-                            if (ii >= 0 && ii < H && jj >= 0 && jj < W)
-                                v = __ldg(x + (((size_t)pn[kk] * CI + c) * H + ii) * W + jj);
-                        }
-                    }
-                    const uint32_t h = bf16_bits(v);
-                    pk[e >> 1] = (e & 1) ? (pk[e >> 1] | (h << 16)) : h;
-                }
-                *reinterpret_cast<uint4 *>(sb + kmaj(row, 8 * g)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                for (int e = 0; e < 8; ++e) v[k][e] = e < nc ? __ldg(src + e * HW) : 0.f;
             }
         }
+    };
+    auto store_dy = [&](int buf) {
+#pragma unroll
+        for (int k = 0; k < kDi; ++k) {
+            const int it = warp + k * (kDwThreads / 32), q = 32 * (it & 3) + lane, g = it >> 2;
+            if (g < ng && q < tw)
+                *reinterpret_cast<uint4 *>(sa + (size_t)buf * abytes + ((size_t)g * (tw + 1) + q) * 16) = pack8(v[k]);
+        }
+    };
+    // the registers hold the next row's dy and its one new x row, loaded a whole
+    // step before they are stored
+    Row pre = cur;  // the row in the registers
+    if (nrow > 1) next(pre);
+    if (nrow > 0 && !mma_warp) {
+        for (int u = -1; u <= 0; ++u) {
+            load_x(cur, cur.i + u);
+            store_x(cur.i + u);
+        }
+        load_dy(cur);
+        load_x(cur, cur.i + 1);
+        store_x(cur.i + 1);
+        store_dy(0);
         nn_fence_async();
-        nn_before_sync();
-        ok = __syncthreads_and(ok) != 0;  // every thread's stage was free
-        nn_after_sync();
-        if (t == 0 && ok) {
-#pragma unroll
-            for (int kk = 0; kk < kKB; kk += 16)
-                nn_mma(tmem, nn_sdesc(smem_addr(sa) + kk * 16), nn_sdesc(smem_addr(sb) + kk * 16), id,
-                       (kb > 0 || kk > 0) ? 1u : 0u);
-            nn_commit(smem_addr(&done[sg]));
+        if (nrow > 1) {
+            load_dy(pre);
+            load_x(pre, pre.i + 1);
         }
     }
-    if (nblk > 0) {
-        const int last = nblk - 1;
-        ok = ok && nn_wait(smem_addr(&done[last & 1]), (uint32_t)(last >> 1) & 1u);
+    float db8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // bias: warp w sums channels 8 w .. 8 w + 7
+    bool ok = __syncthreads_and(1) != 0;
+    int issued = 0;  // rows whose MMAs have been issued
+    for (int k = 0; k < nrow && ok; ++k) {
+        issued = k + 1;
+        if (mma_warp) {
+            nn_after_sync();
+            const uint32_t lead = nn_elect();
+            const uint64_t da = mn_desc(smem_addr(sa) + (uint32_t)((k & 1) * abytes), (uint32_t)(tw + 1) * 16);
+            const uint32_t xb = smem_addr(sx);
+            for (int ks = 0; ks < tw / 16; ++ks) {  // 256 bytes further per 16 pixels
+                const uint32_t acc = (k > 0 || ks > 0) ? 1u : 0u;
+#pragma unroll
+                for (int u = 0; u < 3; ++u) {
+                    const uint64_t db = mn_desc(xb + (uint32_t)(((cur.i + u - 1) & (kDwRing - 1)) * xbytes), (uint32_t)xq * 16);
+#pragma unroll
+                    for (int vv = 0; vv < 3; ++vv)
+                        nn_mma_if(lead, tmem + (uint32_t)((3 * u + vv) * kDwCB), da + (uint64_t)(16 * ks),
+                                  db + (uint64_t)(16 * ks + vv), id, acc);
+                }
+            }
+            if (lead) nn_commit(smem_addr(&done[k & 1]));
+            __syncwarp();
+        } else if (k + 1 < nrow) {
+            // the buffers written next were read by the MMAs of row k - 1; a new
+            // strip replaces rows that row k's MMAs read
+            const bool strip = pre.i == 0;
+            if (strip) ok = nn_wait(smem_addr(&done[k & 1]), (uint32_t)(k >> 1) & 1u);
+            else if (k > 0) ok = nn_wait(smem_addr(&done[(k - 1) & 1]), (uint32_t)((k - 1) >> 1) & 1u);
+            if (ok) {
+                store_x(pre.i + 1);
+                store_dy((k + 1) & 1);
+                if (strip)
+                    for (int u = -1; u <= 0; ++u) {
+                        load_x(pre, u);
+                        store_x(u);
+                    }
+                nn_fence_async();
+            }
+        }
+        cur = pre;
+        if (k + 2 < nrow) {
+            next(pre);
+            if (!mma_warp) {
+                load_dy(pre);
+                load_x(pre, pre.i + 1);
+            }
+        }
+        if (blockIdx.x == 0 && warp < ng)  // the staged (rounded) row, on the CUDA cores
+            for (int q = lane; q < tw; q += 32) {
+                const uint4 p = *reinterpret_cast<const uint4 *>(sa + (size_t)(k & 1) * abytes +
+                                                                 ((size_t)warp * (tw + 1) + q) * 16);
+                const uint32_t w4[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    db8[2 * e] += __uint_as_float(w4[e] << 16);
+                    db8[2 * e + 1] += __uint_as_float(w4[e] & 0xffff0000u);
+                }
+            }
+        nn_before_sync();
+        ok = __syncthreads_and(ok) != 0;
+    }
+    // the last commits cover every MMA issued (also after a wait gave up)
+    for (int k = max(0, issued - 2); k < issued; ++k) {
+        const bool fin = nn_wait(smem_addr(&done[k & 1]), (uint32_t)(k >> 1) & 1u);
+        ok = ok && fin;
     }
     ok = __syncthreads_and(ok) != 0;
     nn_after_sync();
     if (!ok) {
-        if (t == 0) {
-            nn_commit(smem_addr(&fin));
-            nn_wait(smem_addr(&fin), 0u);
-            atomicOr(err, 1u);
-        }
+        if (t == 0) atomicOr(err, 1u);
     } else {
-        // warp w holds output channels 32 w .. 32 w + 31
-        const int o = 32 * warp + lane;
-        const uint32_t tl = tmem + ((uint32_t)(32 * warp) << 16);
-        for (int c0 = 0; c0 < NC; c0 += 32) {
-            uint32_t r[32];
-            if (nblk > 0) nn_ld32(tl + (uint32_t)c0, r);
+        if (warp < 4) {  // warp w holds output channels 32 w .. 32 w + 31
+            const int o = 32 * warp + lane;
+            const uint32_t tl = tmem + ((uint32_t)(32 * warp) << 16);
+            for (int tap = 0; tap < 9; ++tap) {
+                uint32_t r[32];
+                nn_ld32(tl + (uint32_t)(tap * kDwCB), r);
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                const int col = kc0 + c0 + e;
-                if (o < CO && c0 + e < NC && col < ncol)
-                    part[((size_t)split * CO + o) * ncol + col] = nblk > 0 ? __uint_as_float(r[e]) : 0.f;
+                for (int e = 0; e < 32; ++e)
+                    if (o < CO && c0 + e < CI)
+                        part[(((size_t)split * 9 + tap) * CI + c0 + e) * CO + o] = nrow > 0 ? __uint_as_float(r[e]) : 0.f;
+            }
+        }
+        if (blockIdx.x == 0 && warp < ng) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                float b = db8[e];
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1) b += __shfl_xor_sync(0xffffffffu, b, d);
+                if (lane == 0 && 8 * warp + e < CO) part[(size_t)S * 9 * CI * CO + (size_t)split * CO + 8 * warp + e] = b;
             }
         }
     }
     nn_before_sync();
     __syncthreads();
     nn_after_sync();
-    if (warp == 0) nn_tmem_free(tmem, (uint32_t)tmem_cols(NC));
+    if (warp == 0) nn_tmem_free(tmem, 512u);
 }
 
 // dw[o][c][u][v] and db[o] = the splits' partial sums, added in split order.
 __global__ void k_conv3x3_dw_tc_sum(const float *__restrict__ part, float *__restrict__ dw, float *__restrict__ db,
                                     int CI, int CO, int S)
 {
-    const int ncol = CI * 9 + 1;
-    const int64_t n = (int64_t)CO * ncol;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t n = (int64_t)9 * CI * CO;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n + CO; e += (int64_t)gridDim.x * blockDim.x) {
+        const float *p = e < n ? part + e : part + (size_t)S * n + (e - n);
+        const int64_t stride = e < n ? n : CO;
         float acc = 0.f;
-        for (int s = 0; s < S; ++s) acc += part[(size_t)s * n + e];
-        const int o = (int)(e / ncol), col = (int)(e - (int64_t)o * ncol);
-        if (col < ncol - 1) dw[(size_t)o * (ncol - 1) + col] = acc;
-        else db[o] = acc;
+#pragma unroll 8
+        for (int s = 0; s < S; ++s) acc += __ldg(p + (size_t)s * stride);
+        if (e < n) {
+            const int o = (int)(e % CO), c = (int)((e / CO) % CI), tap = (int)(e / ((int64_t)CO * CI));
+            dw[((size_t)o * CI + c) * 9 + tap] = acc;
+        } else {
+            db[e - n] = acc;
+        }
     }
 }
 
@@ -543,15 +708,22 @@ __device__ unsigned g_nn_tc_err;  // a tensor-core layer's wait gave up (dg_nn_t
 namespace {
 
 int nt_of(int co) { return std::min(128, (co + 15) / 16 * 16); }
-int nc_of(int ci) { return std::min(256, (ci * 9 + 1 + 15) / 16 * 16); }
-
-int64_t dw_splits(int B, int Ci, int Co, int H, int W)
+// Pixels of an output row per step (a multiple of 16, at most 128, the row in
+// equal parts), parts per row, and splits: one CTA per SM over the blocks of
+// input channels, a row each at least.
+struct DwShape {
+    int tw, nb;
+    int64_t rows, S;
+};
+DwShape dw_shape(int B, int Ci, int H, int W)
 {
-    const int64_t P = (int64_t)B * H * W;
-    const int64_t tiles = (Ci * 9 + 1 + nc_of(Ci) - 1) / nc_of(Ci);
-    int64_t S = (152 * 4 + tiles - 1) / tiles;          // about four CTAs per SM
-    S = std::min<int64_t>(S, std::max<int64_t>(1, P / 1024));
-    return std::max<int64_t>(1, std::min<int64_t>(S, 4096));
+    DwShape d;
+    d.nb = (W + kRowsTc - 1) / kRowsTc;
+    d.tw = ((W + d.nb - 1) / d.nb + 15) / 16 * 16;
+    d.rows = (int64_t)B * H * d.nb;
+    const int64_t blocks = (Ci + kDwCB - 1) / kDwCB;
+    d.S = std::max<int64_t>(1, std::min<int64_t>(d.rows, std::max<int64_t>(1, 152 / blocks)));
+    return d;
 }
 
 bool tc_shape_ok(int B, int Ci, int Co, int H, int W)
@@ -595,7 +767,7 @@ int64_t bwd_wimg_floats(int Ci, int Co) { return (wimg_elems(Co, Ci, nt_of(Ci)) 
 
 int64_t nn_conv_tc_scratch(int B, int Ci, int Co, int H, int W)
 {
-    return std::max(fwd_scratch(Ci, Co), bwd_wimg_floats(Ci, Co) + dw_splits(B, Ci, Co, H, W) * (int64_t)Co * (Ci * 9 + 1));
+    return std::max(fwd_scratch(Ci, Co), bwd_wimg_floats(Ci, Co) + dw_shape(B, Ci, H, W).S * (int64_t)Co * (Ci * 9 + 1));
 }
 
 }  // namespace dg
@@ -641,19 +813,17 @@ dg_status dg_nn_conv3x3_backward_tc(const float *x, const float *w, const float 
     if (e != cudaSuccess) return dg::nn_done(e, "dg_nn_conv3x3_backward_tc");
     unsigned *err = dg::err_word();
     if (!err) return dg::nn_done(cudaErrorInvalidSymbol, "dg_nn_conv3x3_backward_tc");
-    const int NC = dg::nc_of(Ci);
-    const int64_t S = dg::dw_splits(B, Ci, Co, H, W);
-    const int64_t P = (int64_t)B * H * W;
-    const int64_t per = (P + S - 1) / S;
-    const int smem = 2 * (dg::kABytes + NC * dg::kKB * 2);
+    const dg::DwShape d = dg::dw_shape(B, Ci, H, W);
+    const int smem = dg::dw_smem(d.tw);
     if ((e = cudaFuncSetAttribute(dg::k_conv3x3_dw_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
         return dg::nn_done(e, "dg_nn_conv3x3_backward_tc");
-    const dim3 grid((unsigned)((Ci * 9 + 1 + NC - 1) / NC), (unsigned)S);
-    dg::k_conv3x3_dw_tc<<<grid, 128, smem, s>>>(x, dy, part, Ci, Co, H, W, P, per, NC, err);
+    const dim3 grid((unsigned)((Ci + dg::kDwCB - 1) / dg::kDwCB), (unsigned)d.S);
+    dg::k_conv3x3_dw_tc<<<grid, dg::kDwThreads + 32, smem, s>>>(x, dy, part, Ci, Co, H, W, d.tw, d.nb, d.rows,
+                                                                (d.rows + d.S - 1) / d.S, (int)d.S, err);
     if ((e = cudaGetLastError()) != cudaSuccess) return dg::nn_done(e, "dg_nn_conv3x3_backward_tc");
     const int64_t n = (int64_t)Co * (Ci * 9 + 1);
-    dg::k_conv3x3_dw_tc_sum<<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(part, dw, db, Ci,
-                                                                                                  Co, (int)S);
+    dg::k_conv3x3_dw_tc_sum<<<(unsigned)std::min<int64_t>((n + 127) / 128, 152 * 16), 128, 0, s>>>(part, dw, db, Ci, Co,
+                                                                                                   (int)d.S);
     return dg::nn_done(cudaGetLastError(), "dg_nn_conv3x3_backward_tc");
 }
 
