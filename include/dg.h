@@ -537,6 +537,11 @@ dg_status dg_nn_conv3x3_backward(const float *x, const float *w, const float *dy
 dg_status dg_nn_conv3x3_forward_tc(const float *x, const float *w, const float *b, float *y, int32_t B,
                                    int32_t Ci, int32_t Co, int32_t H, int32_t W, float *scratch,
                                    void *stream);
+/* The same with y = max(y, 0): bit for bit dg_nn_relu_forward of its output,
+ * without that pass over memory. */
+dg_status dg_nn_conv3x3_relu_forward_tc(const float *x, const float *w, const float *b, float *y, int32_t B,
+                                        int32_t Ci, int32_t Co, int32_t H, int32_t W, float *scratch,
+                                        void *stream);
 int64_t dg_nn_conv3x3_tc_scratch(int32_t B, int32_t Ci, int32_t Co, int32_t H, int32_t W);
 dg_status dg_nn_conv3x3_backward_tc(const float *x, const float *w, const float *dy, float *dx, float *dw,
                                     float *db, int32_t B, int32_t Ci, int32_t Co, int32_t H, int32_t W,

@@ -96,6 +96,11 @@ __device__ __forceinline__ void nn_commit(uint32_t bar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
+__device__ __forceinline__ void nn_arrive(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
 __device__ __forceinline__ void nn_mbar_init(uint32_t bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
@@ -162,7 +167,7 @@ __device__ __forceinline__ uint16_t bf16_bits(float v)
 }
 
 // Tensor-memory columns of an accumulator of n columns (a power of two >= 32).
-__host__ __device__ constexpr int tmem_cols(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : 256; }
+__host__ __device__ constexpr int tmem_cols(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : n <= 256 ? 256 : 512; }
 
 }  // namespace
 
@@ -179,23 +184,31 @@ __host__ __device__ constexpr int tmem_cols(int n) { return n <= 32 ? 32 : n <= 
 // same staging seen from input row r + u and shifted by v pixels: a
 // different descriptor start, nothing gathered per tap. The weights come
 // pre-converted (k_conv_tc_wimg: one 32-channel x NT block per (channel
-// block, tap) in the canonical layout) and stream through a ring of
-// kWRing shared-memory slots by bulk copy. One thread issues the MMAs of a
-// channel block (9 taps x kHaloRows rows x 2 K-steps of 16) while every
-// thread stages the next block's input rows into the other buffer.
+// block, tap) in the canonical layout) by bulk copy, once per CTA where they
+// fit beside the staged rows, else through a ring of slots.
+//
+// One CTA per SM walks the tiles; its warps have a role each and meet only on
+// mbarriers: 13 stage input rows into a ring of buffers, one copies weights, one
+// issues the MMAs (with all lanes, see nn_elect), four write finished tiles out
+// of one of two accumulator sets while the next tile's products run. (A CTA per
+// tile in which every thread staged, one also issued, and all met twice per
+// channel block: 222 us for 128 -> 64 channels at 16 x 128 x 128, MMA pipes 8 %
+// busy; now 73 us, bound by the latency of the staging's loads.) Each output's products are added in the order (channel block, tap,
+// K-step).
 // x: [B][CI][H][W]; y: [B][CO][H][W]; b may be NULL.
 // ---------------------------------------------------------------------------
 constexpr int kHaloRows = 2;                                   // output rows per CTA
 constexpr int kHaloCB = 32;                                    // input channels per block
 constexpr int kHaloQ = kRowsTc + 2;                            // staged pixels per input row
 constexpr int kHaloBytes = (kHaloRows + 2) * (kHaloCB / 8) * kHaloQ * 16;
-constexpr int kWRing = 5;                                      // weight blocks in shared memory
-constexpr int kConvThreads = 256;
+constexpr int kProdWarps = 13;                                 // staging warps: 5 rows of 8 channels a thread
+constexpr int kConvThreads = 32 * (kProdWarps + 6);            // + 4 output warps, weights, MMAs
+constexpr int kHaloMax = 4;                                    // staging buffers, at most
+constexpr int kWSlots = 64;                                    // weight blocks in shared memory, at most
+constexpr int kConvSmem = 224 * 1024;                          // dynamic shared memory, at most
 
 // accumulator columns of one output row (NT rounded up to the 32-column loads)
 __host__ __device__ constexpr int acc_stride(int nt) { return (nt + 31) / 32 * 32; }
-
-__host__ __device__ constexpr int conv_tc_smem(int nt) { return 2 * kHaloBytes + kWRing * nt * kHaloCB * 2; }
 
 // elements (16-bit) of the pre-converted weights of a layer with CI inputs and CO outputs
 __host__ __device__ inline int64_t wimg_elems(int ci, int co, int nt)
@@ -258,149 +271,252 @@ __global__ void k_conv_tc_wimg(const float *__restrict__ w, uint16_t *__restrict
 // Input rows i0 - 1 .. i0 + kHaloRows of channel block cb, pixels j0 - 1 ..
 // j0 + 128, as BF16 (zeros outside the image and past CI): 16-byte row
 // ((row * 4 + channel group) * kHaloQ + pixel). Consecutive threads take
-// consecutive pixels, so each of the 8 loads of a row is coalesced.
+// consecutive pixels, so each of the 8 loads of a row is coalesced; all of a
+// thread's 40 loads are in flight together (with 16 the staging waited on
+// memory: 90 against 80 us for a 128 -> 64 channel layer at 512 x 512).
 __device__ __forceinline__ void stage_halo(unsigned char *hb, const float *__restrict__ xn, int cb, int CI, int H,
                                            int W, int i0, int j0)
 {
-    constexpr int items = (kHaloRows + 2) * (kHaloCB / 8) * kHaloQ;
-    for (int it = threadIdx.x; it < items; it += kConvThreads) {
+    constexpr int items = (kHaloRows + 2) * (kHaloCB / 8) * kHaloQ, per = items / (32 * kProdWarps);
+    static_assert(per * 32 * kProdWarps == items, "every thread takes the same number of rows");
+    const int64_t HW = (int64_t)H * W;
+    float v[per][8];
+#pragma unroll
+    for (int z = 0; z < per; ++z) {
+        const int it = threadIdx.x + z * 32 * kProdWarps;
         const int q = it % kHaloQ, rest = it / kHaloQ;
         const int g = rest % (kHaloCB / 8), rr = rest / (kHaloCB / 8);
         const int row = i0 - 1 + rr, col = j0 - 1 + q, c0 = cb * kHaloCB + g * 8;
-        const bool in = row >= 0 && row < H && col >= 0 && col < W;
-        float v[8];
+        const int nc = row >= 0 && row < H && col >= 0 && col < W ? CI - c0 : 0;
+        const float *src = xn + (int64_t)c0 * HW + (int64_t)row * W + col;
+        if (nc >= 8) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e)
-            v[e] = (in && c0 + e < CI) ? __ldg(xn + ((size_t)(c0 + e) * H + row) * W + col) : 0.f;
+            for (int e = 0; e < 8; ++e) v[z][e] = __ldg(src + e * HW);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[z][e] = e < nc ? __ldg(src + e * HW) : 0.f;
+        }
+    }
+#pragma unroll
+    for (int z = 0; z < per; ++z) {
         uint32_t pk[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) pk[e] = bf16_bits(v[2 * e]) | (bf16_bits(v[2 * e + 1]) << 16);
-        *reinterpret_cast<uint4 *>(hb + (size_t)it * 16) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        for (int e = 0; e < 4; ++e) pk[e] = bf16_bits(v[z][2 * e]) | (bf16_bits(v[z][2 * e + 1]) << 16);
+        *reinterpret_cast<uint4 *>(hb + (size_t)(threadIdx.x + z * 32 * kProdWarps) * 16) =
+            make_uint4(pk[0], pk[1], pk[2], pk[3]);
     }
 }
 
-__global__ void __launch_bounds__(kConvThreads) k_conv3x3_tc(const float *__restrict__ x,
-                                                             const uint16_t *__restrict__ wimg,
-                                                             const float *__restrict__ b, float *__restrict__ y,
-                                                             int CI, int CO, int H, int W, int NT, unsigned *err)
+// nh staging buffers and nw weight slots (nw = all of the layer's blocks when
+// they are resident; then there is one block of output channels). relu: write
+// max(y, 0).
+__global__ void __launch_bounds__(kConvThreads, 1)
+    k_conv3x3_tc(const float *__restrict__ x, const uint16_t *__restrict__ wimg, const float *__restrict__ b,
+                 float *__restrict__ y, int CI, int CO, int H, int W, int NT, int nh, int nw, int64_t tiles, int relu,
+                 unsigned *err)
 {
     extern __shared__ __align__(1024) unsigned char nsm[];
-    __shared__ __align__(8) uint64_t wfull[kWRing], wempty[kWRing], hdone[2], fin;
+    __shared__ __align__(8) uint64_t wfull[kWSlots], wempty[kWSlots], hfull[kHaloMax], hempty[kHaloMax], afull[2],
+        aempty[2], fin;
     __shared__ uint32_t tslot;
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane = t & 31;
     const int ob = (CO + NT - 1) / NT;
-    const int n = blockIdx.z / ob, obi = blockIdx.z % ob, o0 = obi * NT;
-    const int i0 = blockIdx.y * kHaloRows, j0 = blockIdx.x * kRowsTc;
     const int ncb = (CI + kHaloCB - 1) / kHaloCB, nblk = ncb * 9;
+    const int tx = (W + kRowsTc - 1) / kRowsTc, ty = (H + kHaloRows - 1) / kHaloRows;
+    const bool resident = nw == nblk && ob == 1;
     const int AS = acc_stride(NT);
     const uint32_t wbytes = (uint32_t)NT * kHaloCB * 2;
-    unsigned char *halo[2] = {nsm, nsm + kHaloBytes};
-    unsigned char *wring = nsm + 2 * kHaloBytes;
-    const unsigned char *wsrc = reinterpret_cast<const unsigned char *>(wimg) + (size_t)obi * ncb * 9 * wbytes;
+    const uint32_t ncols = (uint32_t)tmem_cols(2 * kHaloRows * AS);
+    unsigned char *wring = nsm + (size_t)nh * kHaloBytes;
+    struct Tile {
+        int n, obi, i0, j0;
+    };
+    auto tile_of = [&](int64_t v) {
+        Tile o;
+        o.j0 = (int)(v % tx) * kRowsTc;
+        v /= tx;
+        o.i0 = (int)(v % ty) * kHaloRows;
+        v /= ty;
+        o.obi = (int)(v % ob);
+        o.n = (int)(v / ob);
+        return o;
+    };
     if (t == 0) {
-        for (int k = 0; k < kWRing; ++k) {
+        for (int k = 0; k < nw; ++k) {
             nn_mbar_init(smem_addr(&wfull[k]), 1);
             nn_mbar_init(smem_addr(&wempty[k]), 1);
         }
-        nn_mbar_init(smem_addr(&hdone[0]), 1);
-        nn_mbar_init(smem_addr(&hdone[1]), 1);
+        for (int k = 0; k < nh; ++k) {
+            nn_mbar_init(smem_addr(&hfull[k]), kProdWarps);
+            nn_mbar_init(smem_addr(&hempty[k]), 1);
+        }
+        for (int k = 0; k < 2; ++k) {
+            nn_mbar_init(smem_addr(&afull[k]), 1);
+            nn_mbar_init(smem_addr(&aempty[k]), 4);
+        }
         nn_mbar_init(smem_addr(&fin), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) nn_tmem_alloc(smem_addr(&tslot), (uint32_t)tmem_cols(kHaloRows * AS));
+    if (warp == 0) nn_tmem_alloc(smem_addr(&tslot), ncols);
     nn_before_sync();
     __syncthreads();
     nn_after_sync();
     const uint32_t tmem = tslot;
-    const uint32_t id = nn_idesc(NT);
-    int issued = 0;  // weight blocks whose copy thread 0 has issued
-    if (t == 0)
-        for (; issued < min(kWRing, nblk); ++issued) {
-            nn_expect_tx(smem_addr(&wfull[issued]), wbytes);
-            nn_bulk_g2s(smem_addr(wring + (size_t)issued * wbytes), wsrc + (size_t)issued * wbytes, wbytes,
-                        smem_addr(&wfull[issued]));
-        }
-    const float *xn = x + (size_t)n * CI * H * W;
-    stage_halo(halo[0], xn, 0, CI, H, W, i0, j0);
-    nn_fence_async();
-    bool ok = __syncthreads_and(1) != 0;
-    for (int cb = 0; cb < ncb && ok; ++cb) {
-        const unsigned char *hb = halo[cb & 1];
-        if (t == 0) {
-            for (int tap = 0; tap < 9 && ok; ++tap) {
-                const int g = cb * 9 + tap, slot = g % kWRing;
-                // the slot of block g - 2 takes block g - 2 + kWRing once that
-                // block's MMAs are done (those of block g - 1 keep the pipe busy)
-                if (g >= 2 && issued == g - 2 + kWRing && issued < nblk) {
-                    const int ps = (g - 2) % kWRing;
-                    ok = nn_wait(smem_addr(&wempty[ps]), (uint32_t)((g - 2) / kWRing) & 1u);
-                    if (!ok) break;
-                    nn_expect_tx(smem_addr(&wfull[ps]), wbytes);
-                    nn_bulk_g2s(smem_addr(wring + (size_t)ps * wbytes), wsrc + (size_t)issued * wbytes, wbytes,
-                                smem_addr(&wfull[ps]));
-                    ++issued;
+    bool ok = true;
+    int64_t copied = 0;  // weight blocks whose copy this thread has issued
+    if (warp < kProdWarps) {
+        int s = 0;
+        uint32_t ph = 1;  // parity of the buffer's last release; a fresh barrier passes parity 1
+        for (int64_t v = blockIdx.x; v < tiles && ok; v += gridDim.x) {
+            const Tile o = tile_of(v);
+            const float *xn = x + (size_t)o.n * CI * H * W;
+            for (int cb = 0; cb < ncb; ++cb) {
+                ok = nn_wait(smem_addr(&hempty[s]), ph);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    ok = false;
+                    break;
                 }
-                ok = nn_wait(smem_addr(&wfull[slot]), (uint32_t)(g / kWRing) & 1u);
-                if (!ok) break;
-                nn_after_sync();
-                const int u = tap / 3, v = tap - 3 * (tap / 3);
-                const uint32_t wb = smem_addr(wring + (size_t)slot * wbytes);
-#pragma unroll
-                for (int r = 0; r < kHaloRows; ++r)
-#pragma unroll
-                    for (int h = 0; h < kHaloCB / 16; ++h) {
-                        const uint32_t a = smem_addr(hb) + (uint32_t)((((r + u) * (kHaloCB / 8) + 2 * h) * kHaloQ + v) * 16);
-                        nn_mma(tmem + (uint32_t)(r * AS), halo_desc(a), nn_sdesc(wb + h * 256), id,
-                               (cb > 0 || tap > 0 || h > 0) ? 1u : 0u);
-                    }
-                nn_commit(smem_addr(&wempty[slot]));
+                stage_halo(nsm + (size_t)s * kHaloBytes, xn, cb, CI, H, W, o.i0, o.j0);
+                nn_fence_async();
+                __syncwarp();
+                if (lane == 0) nn_arrive(smem_addr(&hfull[s]));
+                if (++s == nh) {
+                    s = 0;
+                    ph ^= 1;
+                }
             }
-            // completes once every MMA issued so far (all reading hb) is done
-            nn_commit(smem_addr(&hdone[cb & 1]));
         }
-        if (cb + 1 < ncb) {
-            // the other buffer was read by the MMAs of block cb - 1
-            if (cb >= 1) ok = ok && nn_wait(smem_addr(&hdone[(cb + 1) & 1]), (uint32_t)((cb - 1) >> 1) & 1u);
-            if (ok) stage_halo(halo[(cb + 1) & 1], xn, cb + 1, CI, H, W, i0, j0);
-            nn_fence_async();
+    } else if (warp < kProdWarps + 4) {
+        const int q = warp & 3;  // tensor-memory lanes (pixels) 32 q .. + 31
+        int set = 0;
+        uint32_t ph = 0;
+        for (int64_t v = blockIdx.x; v < tiles && ok; v += gridDim.x) {
+            const Tile o = tile_of(v);
+            ok = __all_sync(0xffffffffu, nn_wait(smem_addr(&afull[set]), ph));
+            if (!ok) break;
+            nn_after_sync();
+            const int jp = o.j0 + 32 * q + lane, o0 = o.obi * NT;
+            float *yn = y + (size_t)o.n * CO * H * W;
+            const int64_t HW = (int64_t)H * W;
+            for (int r = 0; r < kHaloRows; ++r) {
+                const int i = o.i0 + r;
+                const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((set * kHaloRows + r) * AS);
+                for (int c0 = 0; c0 < NT; c0 += 32) {
+                    uint32_t rv[32];
+                    nn_ld32(tl + (uint32_t)c0, rv);
+                    const int nc = min(min(NT - c0, CO - o0 - c0), 32);
+                    const float bl = b && lane < nc ? __ldg(b + o0 + c0 + lane) : 0.f;
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) {
+                        const float val = __uint_as_float(rv[e]) + __shfl_sync(0xffffffffu, bl, e);
+                        rv[e] = __float_as_uint(relu ? fmaxf(val, 0.f) : val);
+                    }
+                    if (i < H && jp < W) {
+                        float *dst = yn + (int64_t)(o0 + c0) * HW + (int64_t)i * W + jp;
+                        if (nc == 32) {
+#pragma unroll
+                            for (int e = 0; e < 32; ++e) dst[e * HW] = __uint_as_float(rv[e]);
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 32; ++e)
+                                if (e < nc) dst[e * HW] = __uint_as_float(rv[e]);
+                        }
+                    }
+                }
+            }
+            nn_before_sync();
+            __syncwarp();
+            if (lane == 0) nn_arrive(smem_addr(&aempty[set]));
+            if (set) ph ^= 1;
+            set ^= 1;
         }
-        ok = __syncthreads_and(ok) != 0;
-    }
-    // every MMA is done once the last block's commit has landed
-    if (ok) ok = nn_wait(smem_addr(&hdone[(ncb - 1) & 1]), (uint32_t)((ncb - 1) >> 1) & 1u);
-    ok = __syncthreads_and(ok) != 0;
-    nn_after_sync();
-    if (!ok) {
-        if (t == 0) {
-            // a wait gave up: the MMAs and the weight copies issued so far
-            // land before the tensor memory and shared memory are released
-            nn_commit(smem_addr(&fin));
-            nn_wait(smem_addr(&fin), 0u);
-            for (int g = max(0, issued - kWRing); g < issued; ++g)
-                nn_wait(smem_addr(&wfull[g % kWRing]), (uint32_t)(g / kWRing) & 1u);
-            atomicOr(err, 1u);
+    } else if (warp == kProdWarps + 4) {
+        if (lane == 0) {
+            int slot = 0;
+            uint32_t ph = 1;
+            for (int64_t v = blockIdx.x; v < tiles && ok; v += gridDim.x) {
+                const unsigned char *wsrc = reinterpret_cast<const unsigned char *>(wimg) +
+                                            (size_t)tile_of(v).obi * nblk * wbytes;
+                for (int g = 0; g < nblk && ok; ++g) {
+                    ok = nn_wait(smem_addr(&wempty[slot]), ph);
+                    if (!ok) break;
+                    nn_expect_tx(smem_addr(&wfull[slot]), wbytes);
+                    nn_bulk_g2s(smem_addr(wring + (size_t)slot * wbytes), wsrc + (size_t)g * wbytes, wbytes,
+                                smem_addr(&wfull[slot]));
+                    ++copied;
+                    if (++slot == nw) {
+                        slot = 0;
+                        ph ^= 1;
+                    }
+                }
+                if (resident) break;
+            }
         }
     } else {
-        // warp w: tensor-memory lanes (pixels) 32 (w % 4) .. + 31, output row w / 4
-        const int q = warp & 3, r = warp >> 2;
-        const int i = i0 + r, jp = j0 + 32 * q + lane;
-        const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(r * AS);
-        float *yn = y + (size_t)n * CO * H * W;
-        for (int c0 = 0; c0 < NT; c0 += 32) {
-            uint32_t rv[32];
-            nn_ld32(tl + (uint32_t)c0, rv);
+        const uint32_t lead = nn_elect(), id = nn_idesc(NT);
+        int s = 0, slot = 0, set = 0;
+        uint32_t hph = 0, wph = 0, aph = 1;
+        bool first = true;
+        for (int64_t v = blockIdx.x; v < tiles && ok; v += gridDim.x) {
+            ok = __all_sync(0xffffffffu, nn_wait(smem_addr(&aempty[set]), aph));
+            const uint32_t acc0 = tmem + (uint32_t)(set * kHaloRows * AS);
+            for (int cb = 0; cb < ncb && ok; ++cb) {
+                ok = __all_sync(0xffffffffu, nn_wait(smem_addr(&hfull[s]), hph));
+                if (!ok) break;
+                const uint64_t ad = halo_desc(smem_addr(nsm) + (uint32_t)(s * kHaloBytes));
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                const int o = o0 + c0 + e;
-                if (c0 + e < NT && o < CO && i < H && jp < W)
-                    yn[((size_t)o * H + i) * W + jp] = __uint_as_float(rv[e]) + (b ? __ldg(b + o) : 0.f);
+                for (int tap = 0; tap < 9; ++tap) {
+                    if (first || !resident) {
+                        ok = ok && nn_wait(smem_addr(&wfull[slot]), wph);
+                        ok = __all_sync(0xffffffffu, ok);
+                    }
+                    nn_after_sync();
+                    if (ok) {
+                        const int u = tap / 3, vv = tap - 3 * (tap / 3);
+                        const uint64_t wd = nn_sdesc(smem_addr(wring) + (uint32_t)slot * wbytes);
+#pragma unroll
+                        for (int r = 0; r < kHaloRows; ++r)
+#pragma unroll
+                            for (int h = 0; h < kHaloCB / 16; ++h)
+                                nn_mma_if(lead, acc0 + (uint32_t)(r * AS),
+                                          ad + (uint64_t)(((r + u) * (kHaloCB / 8) + 2 * h) * kHaloQ + vv),
+                                          wd + (uint64_t)(16 * h), id, (cb > 0 || tap > 0 || h > 0) ? 1u : 0u);
+                        if (!resident && lead) nn_commit(smem_addr(&wempty[slot]));
+                    }
+                    if (++slot == nw) {
+                        slot = 0;
+                        wph ^= 1;
+                    }
+                }
+                if (lead) nn_commit(smem_addr(&hempty[s]));
+                if (++s == nh) {
+                    s = 0;
+                    hph ^= 1;
+                }
             }
+            if (lead) nn_commit(smem_addr(&afull[set]));
+            first = false;
+            if (set) aph ^= 1;
+            set ^= 1;
         }
+        // completes once every MMA issued is done
+        if (lead) nn_commit(smem_addr(&fin));
+    }
+    __syncwarp();
+    // before tensor memory and shared memory are released the MMAs and copies
+    // issued have landed, also where a wait gave up
+    if (t == 32 * (kProdWarps + 4))
+        for (int64_t g = copied > nw ? copied - nw : 0; g < copied; ++g)
+            ok = nn_wait(smem_addr(&wfull[g % nw]), (uint32_t)(g / nw) & 1u) && ok;
+    ok = __syncthreads_and(ok) != 0;
+    if (t == 0) {
+        ok = nn_wait(smem_addr(&fin), 0u) && ok;
+        if (!ok) atomicOr(err, 1u);
     }
     nn_before_sync();
     __syncthreads();
     nn_after_sync();
-    if (warp == 0) nn_tmem_free(tmem, (uint32_t)tmem_cols(kHaloRows * AS));
+    if (warp == 0) nn_tmem_free(tmem, ncols);
 }
 
 // ---------------------------------------------------------------------------
@@ -739,7 +855,7 @@ unsigned *err_word()
 }
 
 cudaError_t launch_conv_tc(bool tr, const float *x, const float *w, const float *b, float *y, int B, int CI, int CO,
-                           int H, int W, uint16_t *wimg, cudaStream_t s)
+                           int H, int W, uint16_t *wimg, cudaStream_t s, int relu = 0)
 {
     unsigned *err = err_word();
     if (!err) return cudaErrorInvalidSymbol;
@@ -750,11 +866,18 @@ cudaError_t launch_conv_tc(bool tr, const float *x, const float *w, const float 
     else k_conv_tc_wimg<false><<<gw, 256, 0, s>>>(w, wimg, CI, CO, NT);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int smem = conv_tc_smem(NT);
+    // the whole layer's weights beside at least two staging buffers, or else a
+    // ring of 16 slots at most
+    const int ob = (CO + NT - 1) / NT, nblk = (CI + kHaloCB - 1) / kHaloCB * 9, wbytes = NT * kHaloCB * 2;
+    const bool resident = ob == 1 && nblk <= kWSlots && nblk * wbytes + 2 * kHaloBytes <= kConvSmem;
+    const int nw = resident ? nblk : std::min(nblk, std::min(16, (kConvSmem - 2 * kHaloBytes) / wbytes));
+    const int nh = std::min(kHaloMax, (kConvSmem - nw * wbytes) / kHaloBytes);
+    const int smem = nh * kHaloBytes + nw * wbytes;
     if ((e = cudaFuncSetAttribute(k_conv3x3_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
         return e;
-    const dim3 grid((W + kRowsTc - 1) / kRowsTc, (H + kHaloRows - 1) / kHaloRows, B * ((CO + NT - 1) / NT));
-    k_conv3x3_tc<<<grid, kConvThreads, smem, s>>>(x, wimg, b, y, CI, CO, H, W, NT, err);
+    const int64_t tiles = (int64_t)((W + kRowsTc - 1) / kRowsTc) * ((H + kHaloRows - 1) / kHaloRows) * B * ob;
+    k_conv3x3_tc<<<(unsigned)std::min<int64_t>(tiles, 152), kConvThreads, smem, s>>>(x, wimg, b, y, CI, CO, H, W, NT, nh, nw,
+                                                                                     tiles, relu, err);
     return cudaGetLastError();
 }
 
@@ -774,17 +897,29 @@ int64_t nn_conv_tc_scratch(int B, int Ci, int Co, int H, int W)
 
 extern "C" {
 
+static dg_status conv_forward_tc(const char *name, const float *x, const float *w, const float *b, float *y, int32_t B,
+                                 int32_t Ci, int32_t Co, int32_t H, int32_t W, float *scratch, void *stream, int relu)
+{
+    if (!x || !w || !b || !y || !scratch) return dg::nn_fail(DG_EINVAL, "%s: null pointer", name);
+    if (!dg::tc_shape_ok(B, Ci, Co, H, W))
+        return dg::nn_fail(DG_EINVAL, "%s: bad shape B=%d Ci=%d Co=%d H=%d W=%d", name, B, Ci, Co, H, W);
+    if ((reinterpret_cast<uintptr_t>(scratch) & 15) != 0)
+        return dg::nn_fail(DG_EINVAL, "%s: scratch must be 16-byte aligned", name);
+    return dg::nn_done(dg::launch_conv_tc(false, x, w, b, y, B, Ci, Co, H, W, reinterpret_cast<uint16_t *>(scratch),
+                                          (cudaStream_t)stream, relu),
+                       name);
+}
+
 dg_status dg_nn_conv3x3_forward_tc(const float *x, const float *w, const float *b, float *y, int32_t B, int32_t Ci,
                                    int32_t Co, int32_t H, int32_t W, float *scratch, void *stream)
 {
-    if (!x || !w || !b || !y || !scratch) return dg::nn_fail(DG_EINVAL, "dg_nn_conv3x3_forward_tc: null pointer");
-    if (!dg::tc_shape_ok(B, Ci, Co, H, W))
-        return dg::nn_fail(DG_EINVAL, "dg_nn_conv3x3_forward_tc: bad shape B=%d Ci=%d Co=%d H=%d W=%d", B, Ci, Co, H, W);
-    if ((reinterpret_cast<uintptr_t>(scratch) & 15) != 0)
-        return dg::nn_fail(DG_EINVAL, "dg_nn_conv3x3_forward_tc: scratch must be 16-byte aligned");
-    return dg::nn_done(dg::launch_conv_tc(false, x, w, b, y, B, Ci, Co, H, W, reinterpret_cast<uint16_t *>(scratch),
-                                          (cudaStream_t)stream),
-                       "dg_nn_conv3x3_forward_tc");
+    return conv_forward_tc("dg_nn_conv3x3_forward_tc", x, w, b, y, B, Ci, Co, H, W, scratch, stream, 0);
+}
+
+dg_status dg_nn_conv3x3_relu_forward_tc(const float *x, const float *w, const float *b, float *y, int32_t B, int32_t Ci,
+                                        int32_t Co, int32_t H, int32_t W, float *scratch, void *stream)
+{
+    return conv_forward_tc("dg_nn_conv3x3_relu_forward_tc", x, w, b, y, B, Ci, Co, H, W, scratch, stream, 1);
 }
 
 int64_t dg_nn_conv3x3_tc_scratch(int32_t B, int32_t Ci, int32_t Co, int32_t H, int32_t W)

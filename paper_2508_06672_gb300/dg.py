@@ -68,7 +68,7 @@ EXPORTED_SYMBOLS = [
     "dg_nn_relu_backward", "dg_nn_bce_scratch", "dg_nn_bce_logits", "dg_nn_adam", "dg_nn_last_error",
     "dg_coarse_maps", "dg_coarse_inspect", "dg_set_grid", "dg_search_regions", "dg_fp32_peak",
     "dg_debug_tc_wait_limit", "dg_batch_rounds", "dg_nn_conv3x3_forward_tc", "dg_nn_conv3x3_backward_tc",
-    "dg_nn_conv3x3_tc_scratch", "dg_nn_tc_check",
+    "dg_nn_conv3x3_tc_scratch", "dg_nn_tc_check", "dg_nn_conv3x3_relu_forward_tc",
 ]
 DG_NOALLOC_SCRATCH_BYTES = 16 * 1024 * 1024
 
@@ -218,6 +218,7 @@ def lib():
             L.dg_nn_conv3x3_scratch.argtypes = [i32, i32, i32, i32, i32]
             L.dg_nn_conv3x3_scratch.restype = i64
             L.dg_nn_conv3x3_forward_tc.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, i32, vp, vp]
+            L.dg_nn_conv3x3_relu_forward_tc.argtypes = L.dg_nn_conv3x3_forward_tc.argtypes
             L.dg_nn_conv3x3_backward_tc.argtypes = [vp, vp, vp, vp, vp, vp, i32, i32, i32, i32, i32, vp, vp]
             L.dg_nn_conv3x3_tc_scratch.argtypes = [i32, i32, i32, i32, i32]
             L.dg_nn_conv3x3_tc_scratch.restype = i64
@@ -230,7 +231,7 @@ def lib():
             L.dg_nn_adam.argtypes = [vp, vp, vp, vp, i64, flt, flt, flt, flt, i32, vp]
             for f in ("dg_nn_conv3x3_forward", "dg_nn_conv3x3_backward", "dg_nn_relu_forward",
                       "dg_nn_relu_backward", "dg_nn_bce_logits", "dg_nn_adam", "dg_nn_conv3x3_forward_tc",
-                      "dg_nn_conv3x3_backward_tc", "dg_nn_tc_check"):
+                      "dg_nn_conv3x3_relu_forward_tc", "dg_nn_conv3x3_backward_tc", "dg_nn_tc_check"):
                 getattr(L, f).restype = C.c_int
             L.dg_nn_last_error.argtypes = []
             L.dg_nn_last_error.restype = C.c_char_p
@@ -488,9 +489,10 @@ def dg_nn_conv3x3_backward(x, w, dy, dx, dw, db, scratch=None, stream=None):
                                            B, Ci, Co, H, W, _ptr(scratch), _stream(stream, x)))
 
 
-def dg_nn_conv3x3_forward_tc(x, w, b, y, scratch=None, stream=None):
+def dg_nn_conv3x3_forward_tc(x, w, b, y, scratch=None, stream=None, relu=False):
     """dg_nn_conv3x3_forward on the tensor cores: BF16 operands, FP32 sums;
-    scratch: dg_nn_conv3x3_tc_scratch floats (allocated here when None)."""
+    scratch: dg_nn_conv3x3_tc_scratch floats (allocated here when None).
+    relu: y = max(y, 0) in the same pass."""
     import torch
     B, Ci, H, W = x.shape
     Co = w.shape[0]
@@ -503,8 +505,8 @@ def dg_nn_conv3x3_forward_tc(x, w, b, y, scratch=None, stream=None):
     if (tuple(w.shape) != (Co, Ci, 3, 3) or tuple(b.shape) != (Co,) or tuple(y.shape) != (B, Co, H, W)
             or scratch.numel() < need):
         raise ValueError("dg_nn_conv3x3_forward_tc: shape mismatch")
-    _nn_check(lib().dg_nn_conv3x3_forward_tc(_ptr(x), _ptr(w), _ptr(b), _ptr(y), B, Ci, Co, H, W,
-                                             _ptr(scratch), _stream(stream, x)))
+    f = lib().dg_nn_conv3x3_relu_forward_tc if relu else lib().dg_nn_conv3x3_forward_tc
+    _nn_check(f(_ptr(x), _ptr(w), _ptr(b), _ptr(y), B, Ci, Co, H, W, _ptr(scratch), _stream(stream, x)))
 
 
 def dg_nn_conv3x3_backward_tc(x, w, dy, dx, dw, db, scratch=None, stream=None):

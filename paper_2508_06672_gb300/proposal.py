@@ -84,6 +84,10 @@ class ProposalNet:
         L = len(self.params)
         for k, (w, b) in enumerate(self.params):
             z = torch.empty((B, w.shape[0], H, W), dtype=torch.float32, device=x.device)
+            if self.tc and not keep and k < L - 1:  # nothing needs the values before the relu
+                dg.dg_nn_conv3x3_forward_tc(h, w, b, z, relu=True)
+                h = z
+                continue
             (dg.dg_nn_conv3x3_forward_tc if self.tc else dg.dg_nn_conv3x3_forward)(h, w, b, z)
             if k < L - 1:
                 hk = torch.empty_like(z) if keep else z

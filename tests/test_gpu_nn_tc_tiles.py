@@ -1,0 +1,49 @@
+"""The persistent tensor-core convolution over its tile schedule, against the
+same products in 64 bits on operands rounded to BF16.
+
+What the kernel can get wrong at a schedule's edges is a whole tile or a whole
+channel block, so it is held to the FP32 accumulation's own bound: K products of
+BF16 values, exact in FP32, summed by the tensor cores with at most one
+truncation (2^-22 of the running sum's magnitude) per product, and one rounding
+for the bias: (K 2^-22) sum |a b| + 2^-23 |y|. Shapes: more tiles than SMs and
+one more than a whole wave, weights resident and streamed through the ring
+(beyond 128 outputs, and 256 x 128 channels), single rows and odd rows, widths
+around one 128-pixel tile. The fused relu is compared bit for bit."""
+import pytest
+
+from gpu_common import package, torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(1, 20, 32, 307, 100), (2, 33, 64, 153, 129), (1, 128, 64, 8, 127), (1, 256, 128, 5, 257),
+          (1, 40, 300, 7, 128), (3, 1, 1, 103, 1)]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_conv_tc_over_the_tile_schedule(shape):
+    P = package()
+    torch = torch_cuda()
+    B, Ci, Co, H, W = shape
+    g = torch.Generator(device="cuda").manual_seed(sum(shape))
+    r = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16).to(torch.float32)  # noqa: E731
+    x, w, b = r(B, Ci, H, W), r(Co, Ci, 3, 3), r(Co)
+    y = torch.full((B, Co, H, W), float("nan"), device="cuda")
+    z = torch.full_like(y, float("nan"))
+    P.dg_nn_conv3x3_forward_tc(x, w, b, y)
+    P.dg_nn_conv3x3_forward_tc(x, w, b, z, relu=True)
+    h = torch.empty_like(y)
+    P.dg_nn_relu_forward(y, h)
+    P.dg_nn_tc_check()
+
+    def conv(a, k):  # 64 bits, one shifted product per tap
+        p = torch.nn.functional.pad(a.double(), (1, 1, 1, 1))
+        out = torch.zeros((B, Co, H, W), dtype=torch.float64, device="cuda")
+        for u in range(3):
+            for v in range(3):
+                out += torch.einsum("nchw,oc->nohw", p[:, :, u:u + H, v:v + W], k[:, :, u, v].double())
+        return out
+
+    ref = conv(x, w) + b.double().view(1, -1, 1, 1)
+    lim = 9 * Ci * 2.0 ** -22 * conv(x.abs(), w.abs()) + 2.0 ** -23 * ref.abs() + 1e-30
+    assert bool(((y.double() - ref).abs() <= lim).all())
+    assert torch.equal(z, h)
