@@ -143,16 +143,28 @@ struct CoarseBufs {  // coarse delay-Doppler maps (dg_coarse_maps), grown on dem
     int *lmm = nullptr;
     unsigned long long *nmm = nullptr;
     CoarseStep *st = nullptr;
-    float2 *P = nullptr;
-    float *A = nullptr;
+    float2 *P = nullptr, *tw = nullptr, *F2 = nullptr;
+    float *A = nullptr, *pool = nullptr;
+    float4 *turn = nullptr;
+    MapSnap *snap = nullptr;
+    int *bad = nullptr;
     double *part = nullptr;
     size_t lag_cap = 0, nu_cap = 0, lmm_cap = 0, nmm_cap = 0, st_cap = 0, P_cap = 0, A_cap = 0, part_cap = 0;
+    size_t tw_cap = 0, F2_cap = 0, pool_cap = 0, turn_cap = 0, snap_cap = 0, bad_cap = 0;
+    int tw_logn = 0;  // what tw holds
     int Q = 0, M = 0, nlag_cap = 0, nb_max = 0;  // shape of the last maps (Q = 0: none yet)
+};
+
+struct PastGrid {  // host bounds of a grid the context had (grid_bounds_switch)
+    dg_grid grid;
+    std::vector<double> span, lags;
+    std::vector<GridRange> range;
 };
 
 }  // namespace
 
 struct dg_ctx {
+    std::vector<PastGrid> past;  // at most four
     dg_grid grid{};
     dg_options opt{};
     int K = 0;
@@ -578,7 +590,7 @@ static void fdoa_spans(const dg_ctx *c, const GridDev &g, std::vector<double> &s
                 r[t] = std::sqrt(dx * dx + dy * dy + dz * dz);
                 f[t] = -(dx * vv[0] + dy * vv[1] + dz * vv[2]) / (r[t] * c->lambda);
             }
-            const double nu = (f[1] - f[0]) / c->fs;
+            const double nu = f[1] - f[0];  // times fs
             lo = std::min(lo, nu);
             hi = std::max(hi, nu);
             if (lags) {  // Eq. 7 and 9: the lattice's lag range
@@ -588,6 +600,8 @@ static void fdoa_spans(const dg_ctx *c, const GridDev &g, std::vector<double> &s
                 rmin = std::min(rmin, std::min(r[0], r[1]));
             }
         }
+        lo /= c->fs;
+        hi /= c->fs;
         span[k] = hi - lo;
         if (lags) (*lags)[k] = std::floor(dhi + 0.5) - std::floor(dlo + 0.5) + 1.0;
         if (lags && range) {
@@ -1896,6 +1910,35 @@ dg_status dg_create(const dg_grid *grid, const dg_ephem *eph, int32_t K, double 
     return DG_OK;
 }
 
+// The host's bounds of the current grid (fdoa_spans: 0.7 ms for a 65 x 65
+// lattice and 20 snapshots) go to a list of the last few grids, by their values,
+// and those of the next one come back from it: a search that alternates between a
+// footprint and its regions computes each once.
+static bool same_grid(const dg_grid &a, const dg_grid &b)
+{
+    return a.lat0_deg == b.lat0_deg && a.lon0_deg == b.lon0_deg && a.dlat_m == b.dlat_m && a.dlon_m == b.dlon_m &&
+           a.nlat == b.nlat && a.nlon == b.nlon;
+}
+static void grid_bounds_switch(dg_ctx *c, const dg_grid &next)
+{
+    CdftBufs &b = c->cd;
+    if (!b.main_span.empty()) {
+        if (c->past.size() >= 4) c->past.erase(c->past.begin());
+        c->past.push_back({c->grid, std::move(b.main_span), std::move(b.main_lags), std::move(b.main_range)});
+    }
+    b.main_span.clear();
+    b.main_lags.clear();
+    b.main_range.clear();
+    for (size_t i = 0; i < c->past.size(); ++i) {
+        if (!same_grid(c->past[i].grid, next)) continue;
+        b.main_span = std::move(c->past[i].span);
+        b.main_lags = std::move(c->past[i].lags);
+        b.main_range = std::move(c->past[i].range);
+        c->past.erase(c->past.begin() + (long)i);
+        break;
+    }
+}
+
 dg_status dg_set_grid(dg_ctx *c, const dg_grid *grid)
 {
     if (!c) return fail(nullptr, DG_EINVAL, "ctx is NULL");
@@ -1912,14 +1955,13 @@ dg_status dg_set_grid(dg_ctx *c, const dg_grid *grid)
         CK(c, cudaMallocAsync((void **)&c->xyz, sizeof(double) * 3 * (size_t)G, c->stream));
         c->xyz_cap = G;
     }
+    const bool same = same_grid(c->grid, *grid);
+    if (!same) grid_bounds_switch(c, *grid);
     c->grid = *grid;
     c->opt.row0 = 0;
     c->opt.nrows = 0;
     c->gd = make_griddev(*grid, 0, grid->nlat);
     c->G = G;
-    c->cd.main_span.clear();  // FDOA spans and lag counts of the old grid
-    c->cd.main_lags.clear();
-    c->cd.main_range.clear();
     ++c->steps_gen;           // graphs and batches recorded on the old grid are stale
     {
         Timed t(c, DG_K_GRID);
@@ -2850,6 +2892,12 @@ dg_status dg_destroy(dg_ctx *c)
     fr(c->co.nmm);
     fr(c->co.st);
     fr(c->co.P);
+    fr(c->co.tw);
+    fr(c->co.F2);
+    fr(c->co.pool);
+    fr(c->co.turn);
+    fr(c->co.snap);
+    fr(c->co.bad);
     fr(c->co.A);
     fr(c->co.part);
     fr(c->cd.part);
@@ -2903,6 +2951,34 @@ dg_status dg_destroy(dg_ctx *c)
 // ---------------------------------------------------------------------------
 // Coarse delay-Doppler maps back-projected onto the grid's cells.
 // ---------------------------------------------------------------------------
+
+// Whether the chunk sums go through FFT correlations (launch_chunk_sums: LT = n -
+// M lags a tile), and the transform's size and tiles: the cheaper by a model of
+// both, the transforms at 18 TFLOP/s against 8 M flop per lag at k_caf_lags' 64.
+// Measured on 20 captures of 65536 samples, 4192 lags and chunks of 512: 732 us
+// direct, 73 through the FFTs (the model: 730 and 90).
+static bool coarse_fft(const dg_ctx *c, int nmax, int M, int nb_max, int nlag_cap, MapArgs &f)
+{
+    if (nmax > (1 << 24) || M < 32) return false;  // tiles of a multiple of 32 lags
+    double best = (double)((nlag_cap + 895) / 896 * 896) * nb_max * 8.0 * M / 64.0;
+    bool fft = false;
+    const double budget = (double)(c->opt.scratch_mib ? c->opt.scratch_mib : 12288) * 1048576.0;
+    for (int logn = 10; logn <= 14; ++logn) {
+        const int n = 1 << logn, lt = n - M;
+        if (lt < M) continue;
+        const int nt = (nlag_cap + lt - 1) / lt, nwin = nb_max + (nt - 1) * (lt / M);
+        const double cost = 5.0 * n * logn * ((double)nb_max + nwin + (double)nb_max * nt) / 18.0;
+        if (nt > 65535 || cost >= best || 8.0 * c->K * ((double)nb_max + nwin) * n > budget) continue;
+        best = cost;
+        fft = true;
+        f.logn = logn;
+        f.LT = lt;
+        f.ntile = nt;
+        f.nwin = nwin;
+    }
+    return fft;
+}
+
 dg_status dg_coarse_maps(dg_ctx *c, int32_t bins, int32_t chunk, float *maps)
 {
     if (!c) return fail(nullptr, DG_EINVAL, "ctx is NULL");
@@ -2919,27 +2995,6 @@ dg_status dg_coarse_maps(dg_ctx *c, int32_t bins, int32_t chunk, float *maps)
         if (!c->steps[k].loaded) return fail(c, DG_ESTATE, "snapshot %d has not been loaded", k);
         nmax = std::max(nmax, (int)c->steps[k].n);
     }
-    // planning from the host's lattice estimate of the FDOA span (25 % margin)
-    std::vector<double> &spans = c->cd.main_span;  // cached until the grid changes
-    if (spans.size() != (size_t)c->K) fdoa_spans(c, c->gd, spans);
-    double span = 0.0;
-    for (int k = 0; k < c->K; ++k) span = std::max(span, spans[k]);
-    span *= 1.25;
-    int M = chunk;
-    if (M == 0) {  // the chunk's phase error (nu_q - nu_c) m stays below 1/8 cycle
-        M = 1024;
-        while (M > 1 && 0.5 * span * M > 0.125) M >>= 1;
-    }
-    int Q = bins;
-    if (Q == 0) {  // two bins per Doppler resolution cell 1 / N
-        Q = (int)std::ceil(2.0 * nmax * span) + 1;
-        Q = std::min(256, std::max(16, (Q + 7) / 8 * 8));
-    }
-    const int nb_max = (nmax + M - 1) / M;
-    if (nb_max > 65535) return fail(c, DG_EUNSUPPORTED, "chunk %d leaves %d chunks (at most 65535)", M, nb_max);
-    const double diam = grid_diameter(c->gd);
-    int nlag_cap = 0;
-    for (int k = 0; k < c->K; ++k) nlag_cap = std::max(nlag_cap, lag_slots(c->eph_host[k], c->fs, diam));
     const size_t KG = (size_t)c->K * (size_t)c->G, K = (size_t)c->K;
     CoarseBufs &b = c->co;
     dg_status st;
@@ -2948,10 +3003,6 @@ dg_status dg_coarse_maps(dg_ctx *c, int32_t bins, int32_t chunk, float *maps)
     if ((st = ensure(c, (void **)&b.lmm, &b.lmm_cap, sizeof(int) * 2 * K)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&b.nmm, &b.nmm_cap, sizeof(unsigned long long) * 2 * K)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&b.st, &b.st_cap, sizeof(CoarseStep) * K)) != DG_OK) return st;
-    if ((st = ensure(c, (void **)&b.P, &b.P_cap, sizeof(float2) * K * nb_max * (size_t)nlag_cap)) != DG_OK) return st;
-    if ((st = ensure(c, (void **)&b.A, &b.A_cap, sizeof(float) * K * (size_t)nlag_cap * Q)) != DG_OK) return st;
-    if ((st = ensure(c, (void **)&b.part, &b.part_cap, sizeof(double) * K * coarse_bin_tiles(nlag_cap))) != DG_OK)
-        return st;
     if ((st = push_steps(c)) != DG_OK) return st;
     if ((st = ensure_ephf(c)) != DG_OK) return st;
     if (c->cd.xyzf_cap < (size_t)c->G) {
@@ -2974,25 +3025,91 @@ dg_status dg_coarse_maps(dg_ctx *c, int32_t bins, int32_t chunk, float *maps)
     a.K = c->K;
     a.fs = c->fs;
     a.lambda = c->lambda;
-    a.Q = Q;
-    a.M = M;
-    a.nlag_cap = nlag_cap;
-    a.nb_max = nb_max;
     a.lag = b.lag;
     a.nu = b.nu;
     a.lmm = b.lmm;
     a.nmm = b.nmm;
     a.st = b.st;
-    a.P = b.P;
-    a.A = b.A;
-    a.part = b.part;
     a.maps = maps;
     a.err = c->err_d;
-    {
+    {  // under way while the host plans (its lattice takes longer on a new grid)
         Timed t(c, DG_K_COARSE);
         int n = 1;
         CK(c, launch_ecef_split(c->xyz, c->G, c->cd.xyzf, c->stream));
-        CK(c, launch_coarse(a, c->stream, &n));
+        CK(c, launch_coarse_geo(a, c->stream, &n));
+        t.done(n);
+    }
+    // planning from the host's lattice estimate of the FDOA span (25 % margin)
+    std::vector<double> &spans = c->cd.main_span;  // cached until the grid changes
+    if (spans.size() != K) fdoa_spans(c, c->gd, spans);
+    double span = 0.0;
+    for (int k = 0; k < c->K; ++k) span = std::max(span, spans[k]);
+    span *= 1.25;
+    int M = chunk;
+    if (M == 0) {  // the chunk's phase error (nu_q - nu_c) m stays below 1/8 cycle
+        M = 1024;
+        while (M > 1 && 0.5 * span * M > 0.125) M >>= 1;
+    }
+    int Q = bins;
+    if (Q == 0) {  // two bins per Doppler resolution cell 1 / N
+        Q = (int)std::ceil(2.0 * nmax * span) + 1;
+        Q = std::min(256, std::max(16, (Q + 7) / 8 * 8));
+    }
+    const int nb_max = (nmax + M - 1) / M;
+    if (nb_max > 65535) return fail(c, DG_EUNSUPPORTED, "chunk %d leaves %d chunks (at most 65535)", M, nb_max);
+    const double diam = grid_diameter(c->gd);
+    int nlag_cap = 0;
+    for (int k = 0; k < c->K; ++k) nlag_cap = std::max(nlag_cap, lag_slots(c->eph_host[k], c->fs, diam));
+    MapArgs f{};
+    const bool fft = coarse_fft(c, nmax, M, nb_max, nlag_cap, f);
+    a.Q = Q;
+    a.M = M;
+    a.nlag_cap = nlag_cap;
+    a.nb_max = nb_max;
+    a.nh_max = (nb_max + 1) / 2;
+    a.Dpad = coarse_dpad(Q);
+    if ((st = ensure(c, (void **)&b.P, &b.P_cap, sizeof(float2) * K * nb_max * (size_t)nlag_cap)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&b.A, &b.A_cap, sizeof(float) * K * (size_t)nlag_cap * Q)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&b.pool, &b.pool_cap, sizeof(float) * K * (size_t)nlag_cap * Q)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&b.turn, &b.turn_cap, sizeof(float4) * K * a.nh_max * (size_t)(a.Dpad / 2))) != DG_OK)
+        return st;
+    if ((st = ensure(c, (void **)&b.part, &b.part_cap, sizeof(double) * K * coarse_parts(nlag_cap, Q))) != DG_OK)
+        return st;
+    a.P = b.P;
+    a.A = b.A;
+    a.pool = b.pool;
+    a.turn = b.turn;
+    a.part = b.part;
+    if (fft) {
+        const size_t n = (size_t)1 << f.logn;
+        bool c64 = false;
+        for (int k = 0; k < c->K; ++k) c64 |= c->steps[k].fmt == DG_IQ_C64;
+        if ((st = ensure(c, (void **)&b.snap, &b.snap_cap, sizeof(MapSnap) * K)) != DG_OK) return st;
+        if ((st = ensure(c, (void **)&b.F2, &b.F2_cap, sizeof(float2) * K * ((size_t)nb_max + f.nwin) * n)) != DG_OK) return st;
+        if (c64 && (st = ensure(c, (void **)&b.bad, &b.bad_cap, sizeof(int) * 4 * K)) != DG_OK) return st;
+        if (b.tw_logn != f.logn) {
+            if ((st = ensure(c, (void **)&b.tw, &b.tw_cap, sizeof(float2) * n)) != DG_OK) return st;
+            CK(c, launch_map_twiddles(b.tw, f.logn, c->stream));
+            ++c->launches;
+            b.tw_logn = f.logn;
+        }
+        a.snap = b.snap;
+        a.bad = c64 ? b.bad : nullptr;
+        f.sd = c->steps_d;
+        f.snap = b.snap;
+        f.S = f.ksd = c->K;
+        f.Cmax = nb_max;
+        f.Mb = M;
+        f.NLpad = nlag_cap;
+        f.tw = b.tw;
+        f.F2 = b.F2;
+        f.U = b.P;
+        f.bad = c64 ? b.bad : nullptr;
+    }
+    {
+        Timed t(c, DG_K_COARSE);
+        int n = 0;
+        CK(c, launch_coarse(a, fft ? &f : nullptr, c->stream, &n));
         t.done(n);
     }
     CK(c, cudaMemcpyAsync(c->err_h, c->err_d, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
@@ -3014,9 +3131,10 @@ dg_status dg_coarse_inspect(dg_ctx *c, float *caf, dg_coarse_step *steps, int32_
         shape[1] = b.M;
         shape[2] = b.nlag_cap;
     }
-    if (caf)
-        CK(c, cudaMemcpyAsync(caf, b.A, sizeof(float) * (size_t)c->K * b.nlag_cap * b.Q, cudaMemcpyDeviceToDevice,
-                              c->stream));
+    if (caf) {
+        CK(c, launch_coarse_transpose(b.A, caf, c->K, b.Q, b.nlag_cap, c->stream));
+        ++c->launches;
+    }
     if (steps) {
         std::vector<CoarseStep> h(c->K);
         CK(c, cudaMemcpyAsync(h.data(), b.st, sizeof(CoarseStep) * c->K, cudaMemcpyDeviceToHost, c->stream));

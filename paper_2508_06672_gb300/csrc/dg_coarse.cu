@@ -21,14 +21,18 @@
 //   k_coarse_init / k_coarse_geo / k_coarse_params   node lags and FDOAs
 //       (double-float geometry, Eq. 3-10), their ranges per snapshot, the
 //       map parameters;
-//   k_caf_lags   the chunk sums: for one chunk and a tile of 896 lags, both
-//       sample windows sit in shared memory; each thread slides a register
-//       window of y2 across 7 consecutive lags (7 is odd, so the lanes'
-//       strided reads hit distinct banks): 7 x 7 complex FMAs per 14 loads;
-//   k_caf_bins   the chunk DFT at the Q bins and |.|^2, with the twiddles of
-//       32 chunks staged in shared memory; deterministic partial sums of A;
-//   k_caf_mean   mu per snapshot (fixed-order sum);
+//   chunk sums   by FFT correlation (k_chunk_spec and k_chunk_corr of dg_map.cu),
+//       or for short chunks directly:
+//   k_caf_lags   for one chunk and a tile of 896 lags, both sample windows sit in
+//       shared memory; each thread slides a register window of y2 across 7
+//       consecutive lags (7 is odd, so the lanes' strided reads hit distinct
+//       banks): 7 x 7 complex FMAs per 14 loads;
+//   k_caf_fold   the chunk DFT at the Q bins and |.|^2; deterministic partial
+//       sums of A;
+//   k_caf_pool   maxima of A over 8 consecutive lags, and mu per snapshot
+//       (fixed-order sum);
 //   k_coarse_backproject   the max-pool per cell.
+#include <cfloat>
 #include <climits>
 
 #include "dg_internal.cuh"
@@ -39,8 +43,10 @@ namespace {
 constexpr int kCafR = 7;                          // lags per thread
 constexpr int kCafThreads = 128;
 constexpr int kCafTile = kCafR * kCafThreads;     // lags per k_caf_lags CTA
-constexpr int kBinLags = 32;                      // lags per k_caf_bins CTA
-constexpr int kBinChunks = 32;                    // chunks staged at a time
+constexpr int kFoldWarps = 4;                     // warps of a k_caf_fold CTA
+constexpr int kFoldBins = 16;                     // bin pairs per warp
+constexpr int kFoldRows = 16;                     // chunk pairs staged at a time
+constexpr int kPoolLags = 8;                      // lags per pooled maximum
 
 __device__ __forceinline__ float2 load_iq(const void *b, int fmt, int idx)
 {
@@ -71,7 +77,10 @@ __global__ void k_coarse_init(int *lmm, unsigned long long *nmm, int K)
     }
 }
 
-// One thread per (node, snapshot k = blockIdx.y): Eq. 3-10 in double-float
+// Nodes of snapshot k = blockIdx.y, about eight per thread, the next one loaded
+// while the current one is computed (228 -> 82 us for 20 snapshots of 513^2 nodes
+// with that and the minima kept in FP32; bound by instruction issue, about 520 a
+// node): Eq. 3-10 in double-float
 // arithmetic on the FP32 pipes (ranges to about 1e-7 m), the lag of Eq. 9
 // (round half away from zero; decided by the FP64 expression where D lies
 // within 1e-6 of a rounding boundary) and the FDOA rounded to FP32; block
@@ -84,14 +93,23 @@ __global__ void __launch_bounds__(256) k_coarse_geo(CoarseArgs a)
     for (int t = 0; t < 12; ++t) ed[t] = {__ldg(a.ephf + 24 * k + 2 * t), __ldg(a.ephf + 24 * k + 2 * t + 1)};
     const dfl fsc = {a.fsc_hi, a.fsc_lo}, ilf = {a.ilf_hi, a.ilf_lo};
     int lmin = INT_MAX, lmax = INT_MIN;
-    unsigned long long nmin = ~0ull, nmax = 0ull;
+    float nmin = FLT_MAX, nmax = -FLT_MAX;
     const int64_t G = a.G;
     const float *xf = a.xyzf;
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < G; p += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    float x[6];  // the next node, loaded one node ahead
+    if (p < G)
+#pragma unroll
+        for (int e = 0; e < 6; ++e) x[e] = __ldg(xf + e * G + p);
+    for (; p < G; p += step) {
         dfl D;
         float nu;
-        geometry_df({xf[p], xf[G + p]}, {xf[2 * G + p], xf[3 * G + p]}, {xf[4 * G + p], xf[5 * G + p]}, ed, fsc, ilf,
-                    D, nu);
+        const dfl nx = {x[0], x[1]}, ny = {x[2], x[3]}, nz = {x[4], x[5]};
+        const int64_t pn = p + step < G ? p + step : p;
+#pragma unroll
+        for (int e = 0; e < 6; ++e) x[e] = __ldg(xf + e * G + pn);
+        geometry_df(nx, ny, nz, ed, fsc, ilf, D, nu);
         int L;
         if (!round_df(D, L)) {
             double e[12], D64, nu64;
@@ -103,22 +121,21 @@ __global__ void __launch_bounds__(256) k_coarse_geo(CoarseArgs a)
         a.nu[k * G + p] = nu;
         lmin = min(lmin, L);
         lmax = max(lmax, L);
-        const unsigned long long key = dkey((double)nu);
-        nmin = min(nmin, key);
-        nmax = max(nmax, key);
+        nmin = fminf(nmin, nu);
+        nmax = fmaxf(nmax, nu);
     }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) {
         lmin = min(lmin, __shfl_xor_sync(0xffffffffu, lmin, d));
         lmax = max(lmax, __shfl_xor_sync(0xffffffffu, lmax, d));
-        nmin = min(nmin, __shfl_xor_sync(0xffffffffu, nmin, d));
-        nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, d));
+        nmin = fminf(nmin, __shfl_xor_sync(0xffffffffu, nmin, d));
+        nmax = fmaxf(nmax, __shfl_xor_sync(0xffffffffu, nmax, d));
     }
     if ((threadIdx.x & 31) == 0 && lmin <= lmax) {
         atomicMin(a.lmm + 2 * k, lmin);
         atomicMax(a.lmm + 2 * k + 1, lmax);
-        atomicMin(a.nmm + 2 * k, nmin);
-        atomicMax(a.nmm + 2 * k + 1, nmax);
+        atomicMin(a.nmm + 2 * k, dkey((double)nmin));
+        atomicMax(a.nmm + 2 * k + 1, dkey((double)nmax));
     }
 }
 
@@ -140,6 +157,35 @@ __global__ void k_coarse_params(CoarseArgs a)
         s.nu_c = __dmul_rn(0.5, __dadd_rn(lo, hi));
         s.mu = 0.0;
         a.st[k] = s;
+        if (a.snap) {  // the correlation's lags, and its one Doppler node
+            MapSnap m{};
+            m.nuc = s.nu_c;
+            m.L0 = l0;
+            m.NL = nlag;
+            a.snap[k] = m;
+        }
+    }
+}
+
+// The chunk DFT's factors: cos and sin of 2 pi d_j o_i M for the offset o_i =
+// (nb - 1) / 2 - i of chunk pair i from the middle and half the distance d_j of
+// bin pair j, two bin pairs a record (see k_caf_fold).
+__global__ void __launch_bounds__(256) k_caf_turns(CoarseArgs a)
+{
+    const int k = blockIdx.y, H = a.Dpad / 2;
+    const double delta = a.st[k].delta;
+    const int nb = (a.steps[k].n + a.M - 1) / a.M, nh = (nb + 1) / 2;
+    for (int64_t it = blockIdx.x * 256 + threadIdx.x; it < (int64_t)nh * H; it += gridDim.x * 256) {
+        const int i = (int)(it / H), j = 2 * (int)(it % H);
+        const double x = (0.5 * (nb - 1) - i) * (double)a.M;
+        float s[2], c[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            double ph = (0.5 * (a.Q - 1) - (j + e)) * delta * x;
+            ph = __dsub_rn(ph, floor(ph));
+            sincospif(2.0f * (float)ph, &s[e], &c[e]);
+        }
+        a.turn[((size_t)k * a.nh_max + i) * H + j / 2] = make_float4(c[0], c[1], s[0], s[1]);
     }
 }
 
@@ -220,137 +266,262 @@ __global__ void __launch_bounds__(kCafThreads) k_caf_lags(CoarseArgs a)
     }
 }
 
-// Xc at the Q bins for 32 lags of snapshot k = blockIdx.y; warp w takes the
-// bins w, w + 8, ..., at most UQ of them (UQ >= Q / 8); A = |Xc|^2 and the
-// block's sum of A (in a fixed order).
-template <int UQ>
-__global__ void __launch_bounds__(256) k_caf_bins(CoarseArgs a)
+// Whether lag L's sum reads a sample that is not finite. Every lag's does where
+// y1 holds one (zeros of y2 included: 0 x NaN); y2's index runs from L over the
+// nx samples that the direct kernel sums.
+__device__ __forceinline__ bool caf_bad(int4 b, int L, int nx)
 {
-    extern __shared__ float2 sm[];
-    __shared__ double red[8];
-    const int k = blockIdx.y;
+    if (b.y >= 0) return true;
+    return b.w >= 0 && (L >= 0 ? b.w >= L : b.z < nx + L);
+}
+
+// Xc at the Q bins for the CTA's lags of snapshot k = blockIdx.y: a warp takes
+// 32 lags and 16 bin pairs. The bins lie symmetrically around nu_c and the
+// chunks around their middle, and a unit phase per bin drops out of |.|^2: bins
+// nu_c +- d and chunks at offsets +- o share
+//     C = sum cos(2 pi d o M) (P_+ + P_-),   S = sum sin(2 pi d o M) (P_+ - P_-),
+//     Xc(nu_c +- d) = C +- j S,
+// 4 real FMAs for 2 bins x 2 chunks where the complex products take 16. FP32
+// pipe; the factors (k_caf_turns) and the chunk pairs' sums and differences come
+// from shared memory, two bin pairs per packed FMA. 20 snapshots of 4192 lags,
+// 128 chunks and 40 bins: 254 -> 42 us. A = |Xc|^2, lags fastest, and the CTA's
+// sum of A (in a fixed order). QW of the CTA's warps lie along the bins.
+__device__ __forceinline__ void fma2_to(float2 &c, float2 a, float2 b)
+{
+    unsigned long long r, x, y, z;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(c.x), "f"(c.y));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(c.x), "=f"(c.y) : "l"(r));
+}
+
+__device__ __forceinline__ void cp_async8z(void *dst, const void *src, bool in)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(in ? 8u : 0u)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+template <int QW> __global__ void __launch_bounds__(32 * kFoldWarps) k_caf_fold(CoarseArgs a)
+{
+    constexpr int LW = kFoldWarps / QW, NL = 32 * LW, H = kFoldBins / 2, T = 32 * kFoldWarps;
+    extern __shared__ __align__(16) unsigned char fold_sm[];
+    float4 *s_w = reinterpret_cast<float4 *>(fold_sm);                   // [2][rows][QW H] cos, sin of two bin pairs
+    float2 *s_p = reinterpret_cast<float2 *>(s_w + 2 * kFoldRows * QW * H);  // [2][rows][2][NL] the pair's chunks
+    __shared__ double red[kFoldWarps];
+    const int k = blockIdx.y, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const CoarseStep st = a.st[k];
-    const int lt0 = blockIdx.x * kBinLags;
-    const int ntb = gridDim.x;
+    const int lt0 = blockIdx.x * NL, part = blockIdx.z * gridDim.x + blockIdx.x, parts = gridDim.x * gridDim.z;
     if (lt0 >= st.nlag) {
-        if (threadIdx.x == 0) a.part[(size_t)k * ntb + blockIdx.x] = 0.0;
+        if (t == 0) a.part[(size_t)k * parts + part] = 0.0;
         return;
     }
-    const int Q = a.Q, M = a.M;
-    const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
-    const int nb = (a.steps[k].n + M - 1) / M;
-    float2 *tw = sm;                       // [Q][32]
-    float2 *ps = sm + Q * kBinChunks;      // [32 chunks][32 lags]
-    float xr[UQ], xi[UQ];
-#pragma unroll
-    for (int u = 0; u < UQ; ++u) xr[u] = xi[u] = 0.f;
-    for (int b0 = 0; b0 < nb; b0 += kBinChunks) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < Q * kBinChunks; i += blockDim.x) {
-            const int q = i / kBinChunks, b = b0 + i % kBinChunks;
-            const double nq = __dadd_rn(st.nu_lo, __dmul_rn((double)q, st.delta));
-            double ph = __dmul_rn(__dsub_rn(nq, st.nu_c), (double)b * (double)M);
-            ph = __dsub_rn(ph, floor(ph));
-            float sn, cn;
-            sincospif(2.0f * (float)ph, &sn, &cn);
-            tw[i] = make_float2(cn, sn);
+    const int N = a.steps[k].n, nb = (N + a.M - 1) / a.M, nh = (nb + 1) / 2, ns = (nh + kFoldRows - 1) / kFoldRows;
+    const int wq = warp % QW, wl = warp / QW;
+    const int j0 = (blockIdx.z * QW + wq) * kFoldBins, nq2 = (a.Q + 1) / 2;  // bin pairs, the middle bin one of them
+    const float2 *Pk = a.P + (size_t)k * a.nb_max * a.nlag_cap;
+    const float4 *W = a.turn + (size_t)k * a.nh_max * (a.Dpad / 2) + blockIdx.z * QW * H;
+    auto stage = [&](int g) {  // chunk pairs g kFoldRows .. , asynchronously
+        if (g < ns) {
+            const int i0 = g * kFoldRows, nr = min(kFoldRows, nh - i0);
+            for (int x = t; x < nr * 2 * NL; x += T) {
+                const int r = x / (2 * NL), h = x / NL & 1, l = lt0 + x % NL, b = i0 + r, bh = nb - 1 - b;
+                // the middle chunk of an odd number has no partner (and sin = 0)
+                const bool in = l < st.nlag && (h || bh != b);
+                cp_async8z(s_p + (g & 1) * kFoldRows * 2 * NL + x, in ? Pk + (size_t)(h ? bh : b) * a.nlag_cap + l : Pk, in);
+            }
+            for (int x = t; x < nr * QW * H; x += T)
+                cp_async16(s_w + (g & 1) * kFoldRows * QW * H + x,
+                           W + (size_t)(i0 + x / (QW * H)) * (a.Dpad / 2) + x % (QW * H));
         }
-        for (int i = threadIdx.x; i < kBinChunks * kBinLags; i += blockDim.x) {
-            const int b = b0 + i / kBinLags, t = lt0 + i % kBinLags;
-            ps[i] = (b < nb && t < st.nlag) ? a.P[((size_t)k * a.nb_max + b) * a.nlag_cap + t] : make_float2(0.f, 0.f);
-        }
-        __syncthreads();
-        for (int bb = 0; bb < kBinChunks; ++bb) {
-            const float2 p = ps[bb * kBinLags + lane];
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float2 cr[H], ci[H], sr[H], si[H];
 #pragma unroll
-            for (int u = 0; u < UQ; ++u) {
-                const int q = wq + 8 * u;
-                if (q < Q) {
-                    const float2 w = tw[q * kBinChunks + bb];
-                    xr[u] = fmaf(w.x, p.x, fmaf(-w.y, p.y, xr[u]));
-                    xi[u] = fmaf(w.x, p.y, fmaf(w.y, p.x, xi[u]));
+    for (int h = 0; h < H; ++h) cr[h] = ci[h] = sr[h] = si[h] = make_float2(0.f, 0.f);
+    stage(0);
+    for (int g = 0; g < ns; ++g) {
+        stage(g + 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        if (j0 < nq2) {
+            const int nr = min(kFoldRows, nh - g * kFoldRows);
+            const float2 *p_s = s_p + (g & 1) * kFoldRows * 2 * NL + 32 * wl + lane;
+            const float4 *w_s = s_w + (g & 1) * kFoldRows * QW * H + wq * H;
+            for (int r = 0; r < nr; ++r, p_s += 2 * NL, w_s += QW * H) {
+                const float2 lo = p_s[0], hi = p_s[NL];
+                const float2 ur = make_float2(hi.x + lo.x, hi.x + lo.x), ui = make_float2(hi.y + lo.y, hi.y + lo.y);
+                const float2 vr = make_float2(hi.x - lo.x, hi.x - lo.x), vi = make_float2(hi.y - lo.y, hi.y - lo.y);
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    const float4 w = w_s[h];
+                    const float2 c = make_float2(w.x, w.y), n = make_float2(w.z, w.w);
+                    fma2_to(cr[h], c, ur);
+                    fma2_to(ci[h], c, ui);
+                    fma2_to(sr[h], n, vr);
+                    fma2_to(si[h], n, vi);
                 }
             }
         }
+        __syncthreads();  // the buffer is free for stage g + 2
     }
-    const int t = lt0 + lane;
+    const int l = lt0 + 32 * wl + lane;
     double sum = 0.0;
-    if (t < st.nlag) {
-        float *Ak = a.A + ((size_t)k * a.nlag_cap + t) * Q;
+    if (l < st.nlag && j0 < nq2) {
+        const bool bad = a.bad && caf_bad(reinterpret_cast<const int4 *>(a.bad)[k], st.l0 + l,
+                                          (nb - 1) * a.M + (a.M + kCafR - 1) / kCafR * kCafR);
+        float *Ak = a.A + (size_t)k * a.Q * a.nlag_cap + l;
 #pragma unroll
-        for (int u = 0; u < UQ; ++u) {
-            const int q = wq + 8 * u;
-            if (q < Q) {
-                const float v = fmaf(xr[u], xr[u], xi[u] * xi[u]);
-                Ak[q] = v;
-                sum += (double)v;
+        for (int z = 0; z < kFoldBins; ++z) {
+            const int j = j0 + z;
+            if (j >= nq2) continue;
+            const float c0 = z & 1 ? cr[z / 2].y : cr[z / 2].x, c1 = z & 1 ? ci[z / 2].y : ci[z / 2].x;
+            const float s0 = z & 1 ? sr[z / 2].y : sr[z / 2].x, s1 = z & 1 ? si[z / 2].y : si[z / 2].x;
+            float up = fmaf(c0 - s1, c0 - s1, (c1 + s0) * (c1 + s0));
+            float dn = fmaf(c0 + s1, c0 + s1, (c1 - s0) * (c1 - s0));
+            if (bad) up = dn = __int_as_float(0x7fffffff);
+            Ak[(size_t)(a.Q - 1 - j) * a.nlag_cap] = up;
+            sum += (double)up;
+            if (2 * j != a.Q - 1) {
+                Ak[(size_t)j * a.nlag_cap] = dn;
+                sum += (double)dn;
             }
         }
     }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
-    if (lane == 0) red[wq] = sum;
+    if (lane == 0) red[warp] = sum;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (t == 0) {
         double s = 0.0;
-        for (int w = 0; w < 8; ++w) s += red[w];
-        a.part[(size_t)k * ntb + blockIdx.x] = s;
+        for (int w = 0; w < kFoldWarps; ++w) s += red[w];
+        a.part[(size_t)k * parts + part] = s;
     }
 }
 
-__global__ void __launch_bounds__(256) k_caf_mean(CoarseArgs a, int ntb)
+// Maxima over kPoolLags lags from each lag on (clipped at the last), per bin;
+// the first CTA of a snapshot also sums mu. A cell's box then takes one or two
+// loads per bin where its lags would take a dozen.
+__global__ void __launch_bounds__(256) k_caf_pool(CoarseArgs a, int parts)
 {
+    __shared__ float s_a[256 + kPoolLags];
     __shared__ double red[8];
-    const int k = blockIdx.x;
-    double s = 0.0;
-    for (int i = threadIdx.x; i < ntb; i += blockDim.x) s += a.part[(size_t)k * ntb + i];
+    const int k = blockIdx.z, q = blockIdx.y, l0 = blockIdx.x * 256, t = threadIdx.x;
+    const int nlag = a.st[k].nlag;
+    if (blockIdx.x == 0 && q == 0) {
+        double s = 0.0;
+        for (int i = t; i < parts; i += 256) s += a.part[(size_t)k * parts + i];
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < 8; ++w) t += red[w];
-        a.st[k].mu = t / ((double)a.st[k].nlag * (double)a.Q);
+        for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+        if ((t & 31) == 0) red[t >> 5] = s;
+        __syncthreads();
+        if (t == 0) {
+            double m = 0.0;
+            for (int w = 0; w < 8; ++w) m += red[w];
+            a.st[k].mu = m / ((double)nlag * (double)a.Q);
+        }
     }
+    if (l0 >= nlag) return;
+    const float *A = a.A + ((size_t)k * a.Q + q) * a.nlag_cap;
+    for (int x = t; x < 256 + kPoolLags; x += 256) s_a[x] = l0 + x < nlag ? A[l0 + x] : 0.f;
+    __syncthreads();
+    float m = s_a[t];
+#pragma unroll
+    for (int x = 1; x < kPoolLags; ++x) m = fmaxf(m, s_a[t + x]);
+    if (l0 + t < nlag) a.pool[((size_t)k * a.Q + q) * a.nlag_cap + l0 + t] = m;
 }
 
-// One thread per (cell, snapshot k = blockIdx.y).
-__global__ void __launch_bounds__(256) k_coarse_backproject(CoarseArgs a)
+// A with the bins fastest, [nlag_cap][Q] per snapshot (dg_coarse_inspect).
+__global__ void __launch_bounds__(256) k_caf_transpose(const float *__restrict__ A, float *__restrict__ out, int Q, int cap)
 {
-    const int k = blockIdx.y;
+    __shared__ float s[32][33];
+    const int k = blockIdx.z, l0 = blockIdx.x * 32, q0 = blockIdx.y * 32, x = threadIdx.x & 31;
+    for (int y = threadIdx.x >> 5; y < 32; y += 8)
+        if (q0 + y < Q && l0 + x < cap) s[y][x] = A[((size_t)k * Q + q0 + y) * cap + l0 + x];
+    __syncthreads();
+    for (int y = threadIdx.x >> 5; y < 32; y += 8)
+        if (l0 + y < cap && q0 + x < Q) out[((size_t)k * cap + l0 + y) * Q + q0 + x] = s[x][y];
+}
+
+// (v - lo) / delta of FP32 FDOAs v and lo in bins, rounded down or up. In FP32
+// the quotient is off by under 4 2^-24 of itself (Q <= 256 bins: 6.1e-5);
+// within 1e-4 of an integer the FP64 expression decides.
+__device__ __forceinline__ int bin_of(float v, const CoarseStep &st, float lo, float inv, bool up)
+{
+    const float x = (v - lo) * inv, r = rintf(x);
+    if (fabsf(x - r) < 1e-4f) {
+        const double d = __ddiv_rn(__dsub_rn((double)v, st.nu_lo), st.delta);
+        return (int)(up ? ceil(d) : floor(d));
+    }
+    return (int)(up ? ceilf(x) : floorf(x));
+}
+
+// Cells of column j (one thread) and kBackRows rows of snapshot k =
+// blockIdx.z: a cell's box of A through the pooled maxima, the corners of a row
+// kept for the next one. FP32 except next to a bin edge: the FP64 quotients and
+// the division by mu of every cell were bound by the FP64 units, the loads of a
+// box with the bins fastest by L1 (432 -> 65 us for 20 snapshots of 512^2 cells).
+constexpr int kBackRows = 8;
+__global__ void __launch_bounds__(128) k_coarse_backproject(CoarseArgs a)
+{
+    const int k = blockIdx.z;
     const CoarseStep st = a.st[k];
     const int Q = a.Q;
-    const int nlon = a.nlon, ncol = nlon - 1;
-    const int64_t ncell = (int64_t)(a.nlat - 1) * ncol;
+    const int nlon = a.nlon, ncol = nlon - 1, nrow = a.nlat - 1;
+    const int64_t ncell = (int64_t)nrow * ncol;
     const int *lag = a.lag + (size_t)k * a.G;
     const float *nu = a.nu + (size_t)k * a.G;
-    const float *Ak = a.A + (size_t)k * a.nlag_cap * Q;
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = c / ncol, j = c % ncol;
-        const int64_t p = i * nlon + j;
-        const int64_t pc[4] = {p, p + 1, p + nlon, p + nlon + 1};
-        int la = INT_MAX, lb = INT_MIN;
-        double vmin = 1e300, vmax = -1e300;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            la = min(la, lag[pc[u]]);
-            lb = max(lb, lag[pc[u]]);
-            vmin = fmin(vmin, (double)nu[pc[u]]);
-            vmax = fmax(vmax, (double)nu[pc[u]]);
+    const float *Ak = a.A + (size_t)k * a.nlag_cap * Q, *Bk = a.pool + (size_t)k * a.nlag_cap * Q;
+    const float lo = (float)st.nu_lo, inv = (float)(1.0 / st.delta);
+    const double im = 1.0 / st.mu;
+    const float im_hi = (float)im, im_lo = (float)(im - (double)im_hi);
+    const bool fast = im_hi > 1e-30f && im_hi < 1e30f;
+    for (int j = blockIdx.x * 128 + threadIdx.x; j < ncol; j += gridDim.x * 128)
+        for (int i0 = blockIdx.y * kBackRows; i0 < nrow; i0 += gridDim.y * kBackRows) {
+            const int64_t p0 = (int64_t)i0 * nlon + j;
+            int l0 = __ldg(lag + p0), l1 = __ldg(lag + p0 + 1);
+            float v0 = __ldg(nu + p0), v1 = __ldg(nu + p0 + 1);
+            int ll = min(l0, l1), lh = max(l0, l1);
+            float vl = fminf(v0, v1), vh = fmaxf(v0, v1);
+#pragma unroll 2
+            for (int r = 0; r < kBackRows && i0 + r < nrow; ++r) {
+                const int64_t p = p0 + (int64_t)(r + 1) * nlon;
+                l0 = __ldg(lag + p);
+                l1 = __ldg(lag + p + 1);
+                v0 = __ldg(nu + p);
+                v1 = __ldg(nu + p + 1);
+                const int la = max(0, min(ll, min(l0, l1)) - st.l0), lb = min(st.nlag - 1, max(lh, max(l0, l1)) - st.l0);
+                const float vmin = fminf(vl, fminf(v0, v1)), vmax = fmaxf(vh, fmaxf(v0, v1));
+                ll = min(l0, l1);
+                lh = max(l0, l1);
+                vl = fminf(v0, v1);
+                vh = fmaxf(v0, v1);
+                int qa = 0, qb = Q - 1;
+                if (st.delta > 0.0) {
+                    qa = max(0, bin_of(vmin, st, lo, inv, false));
+                    qb = min(Q - 1, bin_of(vmax, st, lo, inv, true));
+                }
+                float m = 0.f;
+                const int len = lb - la + 1;
+                const float *row = (len >= kPoolLags ? Bk : Ak) + (int64_t)qa * a.nlag_cap + la;
+                const int step = len >= kPoolLags ? kPoolLags : 1, last = len - step;
+                for (int q = qa; q <= qb; ++q, row += a.nlag_cap) {
+                    for (int t = 0; t < last; t += step) m = fmaxf(m, __ldg(row + t));
+                    if (last >= 0) m = fmaxf(m, __ldg(row + last));
+                }
+                // m / mu: m times the reciprocal in two words
+                const float h = m * im_hi;
+                const float v = h + fmaf(m, im_lo, fmaf(m, im_hi, -h));
+                a.maps[(size_t)k * ncell + (int64_t)(i0 + r) * ncol + j] =
+                    st.mu > 0.0 ? (fast && isfinite(h) ? v : (float)((double)m / st.mu)) : 0.f;
+            }
         }
-        la = max(0, la - st.l0);
-        lb = min(st.nlag - 1, lb - st.l0);
-        int qa = 0, qb = Q - 1;
-        if (st.delta > 0.0) {
-            qa = max(0, (int)floor(__ddiv_rn(__dsub_rn(vmin, st.nu_lo), st.delta)));
-            qb = min(Q - 1, (int)ceil(__ddiv_rn(__dsub_rn(vmax, st.nu_lo), st.delta)));
-        }
-        float m = 0.f;
-        for (int t = la; t <= lb; ++t)
-            for (int q = qa; q <= qb; ++q) m = fmaxf(m, Ak[(size_t)t * Q + q]);
-        a.maps[(size_t)k * ncell + c] = st.mu > 0.0 ? (float)((double)m / st.mu) : 0.f;
-    }
 }
 
 unsigned blocks_for(int64_t n, int per, int cap)
@@ -361,42 +532,75 @@ unsigned blocks_for(int64_t n, int per, int cap)
 
 }  // namespace
 
-int coarse_bin_tiles(int nlag_cap) { return (nlag_cap + kBinLags - 1) / kBinLags; }
+// bin pairs per CTA's warps along the bins, and the CTAs along lags and bins
+static int fold_qw(int Q) { return (Q + 1) / 2 <= kFoldBins ? 1 : (Q + 1) / 2 <= 2 * kFoldBins ? 2 : 4; }
+int coarse_parts(int nlag_cap, int Q)
+{
+    const int nl = 32 * (kFoldWarps / fold_qw(Q)), nj = kFoldBins * fold_qw(Q);
+    return (nlag_cap + nl - 1) / nl * (((Q + 1) / 2 + nj - 1) / nj);
+}
+int coarse_dpad(int Q)
+{
+    const int nj = kFoldBins * fold_qw(Q);
+    return ((Q + 1) / 2 + nj - 1) / nj * nj;
+}
 
-cudaError_t launch_coarse(const CoarseArgs &a, cudaStream_t s, int *launches)
+template <int QW> static cudaError_t launch_fold(const CoarseArgs &a, cudaStream_t s)
+{
+    const unsigned nl = 32 * (kFoldWarps / QW), nj = kFoldBins * QW;
+    const size_t smem = kFoldRows * (sizeof(float4) * 2 * nj / 2 + sizeof(float2) * 4 * nl);
+    const cudaError_t e = cudaFuncSetAttribute(k_caf_fold<QW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_caf_fold<QW><<<dim3((a.nlag_cap + nl - 1) / nl, a.K, ((a.Q + 1) / 2 + nj - 1) / nj), 32 * kFoldWarps, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_coarse(const CoarseArgs &a, const MapArgs *fft, cudaStream_t s, int *launches)
+{
+    cudaError_t e;
+    k_coarse_params<<<1, 64, 0, s>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_caf_turns<<<dim3(blocks_for((int64_t)a.nh_max * a.Dpad / 2, 256, 152 * 8), a.K), 256, 0, s>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (fft) {
+        if ((e = launch_chunk_sums(*fft, s, launches)) != cudaSuccess) return e;
+    } else {
+        const size_t lag_smem = sizeof(float2) * (2 * (size_t)a.M + kCafTile + 3 * kCafR);
+        if (lag_smem > 48 * 1024) {
+            e = cudaFuncSetAttribute(k_caf_lags, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lag_smem);
+            if (e != cudaSuccess) return e;
+        }
+        k_caf_lags<<<dim3((a.nlag_cap + kCafTile - 1) / kCafTile, a.nb_max, a.K), kCafThreads, lag_smem, s>>>(a);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        ++*launches;
+    }
+    const int qw = fold_qw(a.Q);
+    e = qw == 1 ? launch_fold<1>(a, s) : qw == 2 ? launch_fold<2>(a, s) : launch_fold<4>(a, s);
+    if (e != cudaSuccess) return e;
+    k_caf_pool<<<dim3((a.nlag_cap + 255) / 256, a.Q, a.K), 256, 0, s>>>(a, coarse_parts(a.nlag_cap, a.Q));
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_coarse_backproject<<<dim3(blocks_for(a.nlon - 1, 128, 65535), blocks_for(a.nlat - 1, kBackRows, 65535), a.K), 128, 0,
+                           s>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    *launches += 5;
+    return cudaSuccess;
+}
+
+// The nodes' lags and FDOAs and their ranges: needs no shape of the maps.
+cudaError_t launch_coarse_geo(const CoarseArgs &a, cudaStream_t s, int *launches)
 {
     cudaError_t e;
     k_coarse_init<<<1, 64, 0, s>>>(a.lmm, a.nmm, a.K);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_coarse_geo<<<dim3(blocks_for(a.G, 256, 152 * 4), a.K), 256, 0, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_coarse_params<<<1, 64, 0, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const size_t lag_smem = sizeof(float2) * (2 * (size_t)a.M + kCafTile + 3 * kCafR);
-    if (lag_smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(k_caf_lags, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lag_smem);
-        if (e != cudaSuccess) return e;
-    }
-    k_caf_lags<<<dim3((a.nlag_cap + kCafTile - 1) / kCafTile, a.nb_max, a.K), kCafThreads, lag_smem, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const int ntb = coarse_bin_tiles(a.nlag_cap);
-    const size_t bin_smem = sizeof(float2) * ((size_t)a.Q * kBinChunks + kBinChunks * kBinLags);
-    const int uq = (a.Q + 7) / 8;
-    auto bins = uq <= 1 ? k_caf_bins<1> : uq <= 2 ? k_caf_bins<2> : uq <= 4 ? k_caf_bins<4>
-              : uq <= 8 ? k_caf_bins<8> : uq <= 16 ? k_caf_bins<16> : k_caf_bins<32>;
-    if (bin_smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(bins, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bin_smem);
-        if (e != cudaSuccess) return e;
-    }
-    bins<<<dim3(ntb, a.K), 256, bin_smem, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_caf_mean<<<a.K, 256, 0, s>>>(a, ntb);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const int64_t ncell = (int64_t)(a.nlat - 1) * (a.nlon - 1);
-    k_coarse_backproject<<<dim3(blocks_for(ncell, 256, 152 * 8), a.K), 256, 0, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    *launches += 7;
-    return cudaSuccess;
+    k_coarse_geo<<<dim3(blocks_for(a.G, 256, 152 * 3 * 4 / a.K + 1), a.K), 256, 0, s>>>(a);
+    *launches += 2;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_coarse_transpose(const float *A, float *out, int K, int Q, int nlag_cap, cudaStream_t s)
+{
+    k_caf_transpose<<<dim3((nlag_cap + 31) / 32, (Q + 31) / 32, K), 256, 0, s>>>(A, out, Q, nlag_cap);
+    return cudaGetLastError();
 }
 
 }  // namespace dg

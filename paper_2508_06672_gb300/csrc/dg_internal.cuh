@@ -542,6 +542,7 @@ struct MapArgs {
     int P, Q;                     // Doppler nodes per block, bins
     int LT, ntile, NLpad;         // lags per tile, tiles, lag stride (a multiple of 32)
     int delay, acc, first;        // first: the sum starts here (else it continues out)
+    int nwin;                     // windows of y2 of a chunk sum (k_chunk_spec)
     const float2 *tw;             // [2^logn] e^{-j 2 pi i / n}
     const float *T;               // [P][Q] node polynomials at the bins
     double xnode[kMapMaxNodes];   // Chebyshev nodes on [-1, 1]
@@ -571,6 +572,7 @@ size_t map_few_partials(int P, int NL);   // floats of U per (snapshot, block)
 cudaError_t launch_map_twiddles(float2 *tw, int logn, cudaStream_t s);
 cudaError_t launch_map_tables(const MapArgs &a, cudaStream_t s, int *launches);
 cudaError_t launch_map_expand(const MapArgs &a, cudaStream_t s);
+cudaError_t launch_chunk_sums(const MapArgs &a, cudaStream_t s, int *launches);
 cudaError_t launch_map_lookup(const MapArgs &a, cudaStream_t s);
 
 // Threshold detection (dg_detect.cu). cap: power of two <= kDetectCap candidates
@@ -651,13 +653,22 @@ struct CoarseArgs {
     unsigned long long *nmm;      // [K][2] FDOA min / max (ordered keys)
     CoarseStep *st;               // [K]
     float2 *P;                    // [K][nb_max][nlag_cap] chunk sums
-    float *A;                     // [K][nlag_cap][Q] the maps |X|^2
-    double *part;                 // [K][ceil(nlag_cap / 32)] partial sums of A
+    float *A, *pool;              // [K][Q][nlag_cap] the maps |X|^2, and their maxima over a few lags
+    float4 *turn;                 // [K][nh_max][Dpad / 2] the chunk DFT's factors
+    int nh_max, Dpad;             // most chunk pairs; bin pairs, padded (coarse_dpad)
+    MapSnap *snap;                // [K] the FFT correlation's parameters (NULL: direct chunk sums)
+    const int *bad;               // [K][4] as MapArgs::bad, for c64 captures through the FFTs (else NULL)
+    double *part;                 // [K][coarse_parts] partial sums of A
     float *maps;                  // [K][nlat - 1][nlon - 1]
     unsigned *err;
 };
-int coarse_bin_tiles(int nlag_cap);
-// The whole coarse pipeline (7 launches; *launches += 7).
-cudaError_t launch_coarse(const CoarseArgs &a, cudaStream_t s, int *launches);
+int coarse_parts(int nlag_cap, int Q);
+int coarse_dpad(int Q);
+// The whole coarse pipeline: the nodes' lags and FDOAs (what does not depend on
+// the maps' shape), then the maps; fft: the chunk sums' correlation, NULL for
+// the direct kernel.
+cudaError_t launch_coarse_geo(const CoarseArgs &a, cudaStream_t s, int *launches);
+cudaError_t launch_coarse(const CoarseArgs &a, const MapArgs *fft, cudaStream_t s, int *launches);
+cudaError_t launch_coarse_transpose(const float *A, float *out, int K, int Q, int nlag_cap, cudaStream_t s);
 
 }  // namespace dg

@@ -44,8 +44,6 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b)
 {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 
 // Two FP32 FMAs in one instruction (Blackwell's packed form): half the issue
 // slots of the same arithmetic.
@@ -60,6 +58,26 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
     asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(r));
     return d;
 }
+
+__device__ __forceinline__ void cp_async8(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+// Sums and differences of complex pairs in one instruction (a - b as a + b (-1),
+// exact), where both parts take the same sign and place.
+__device__ __forceinline__ float2 cadd(float2 a, float2 b)
+{
+    unsigned long long r, x, y;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(r));
+    return d;
+}
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return fma2(b, make_float2(-1.f, -1.f), a); }
 
 // e^{j 2 pi f x} for a frequency f = hi + lo (cycles per sample) and an
 // integer-valued x, |x| < 2^24.
@@ -343,17 +361,81 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN == 14 ? 1 : LOGN == 13 
     }
 }
 
+// Chunk sums of the coarse maps (dg_coarse.cu): for each chunk c of Mb = M samples
+// and lag l, sum_m y1[cM + m] e^{j 2 pi nuc (cM + m)} conj(y2[cM + m + l]). The
+// windows of y2 start M samples apart and the lag tiles LT = n - M apart, a
+// multiple of M (both powers of two): window w = c + tile LT / M serves every
+// chunk and tile of that sum, so a snapshot takes Cmax + nwin forward transforms
+// and one inverse per (chunk, tile), where a window and a turned chunk per (chunk,
+// tile) took three. F2: [S][Cmax + nwin][n].
+template <int LOGN> __global__ void __launch_bounds__((1 << LOGN) / 16) k_chunk_spec(MapArgs a)
+{
+    constexpr int n = 1 << LOGN, T = n / 16;
+    extern __shared__ __align__(16) float2 sm[];
+    __shared__ float2 s_step[16];
+    const int t = threadIdx.x, s = blockIdx.y, c = blockIdx.x, w = c - a.Cmax, hop = a.LT / a.Mb;
+    const StepDesc sd = a.sd[s];
+    const MapSnap ms = a.snap[s];
+    const int nb = (sd.n + a.Mb - 1) / a.Mb, nt = (ms.NL + a.LT - 1) / a.LT;
+    if (w < 0 ? c >= nb : w >= nb + (nt - 1) * hop) return;
+    float2 v[16];
+    if (w < 0) {
+        const float nh = (float)ms.nuc, nl = (float)(ms.nuc - (double)nh);
+        if (t < 16) s_step[t] = cis_df(nh, nl, (float)(T * t));
+        __syncthreads();
+        const float2 base = cis_df(nh, nl, (float)(c * a.Mb + t));
+        const int len = min(a.Mb, sd.n - c * a.Mb);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const int m = t + T * e;
+            v[e] = m < len ? cmul(load_sample(sd.y1, sd.fmt, c * a.Mb + m), cmul(base, s_step[e])) : make_float2(0.f, 0.f);
+        }
+    } else {
+        const int64_t i0 = (int64_t)w * a.Mb + ms.L0;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const int64_t i = i0 + t + T * e;
+            v[e] = i >= 0 && i < sd.n ? load_sample(sd.y2, sd.fmt, (int)i) : make_float2(0.f, 0.f);
+        }
+    }
+    fft_cta<LOGN>(v, sm, a.tw);
+    float2 *F = a.F2 + ((size_t)s * (a.Cmax + a.nwin) + c) * n + t;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) F[T * e] = v[e];
+}
+
+template <int LOGN>
+__global__ void __launch_bounds__((1 << LOGN) / 16, LOGN == 14 ? 1 : LOGN == 13 ? 2 : 768 * 16 / (1 << LOGN)) k_chunk_corr(MapArgs a)
+{
+    constexpr int n = 1 << LOGN, T = n / 16;
+    extern __shared__ __align__(16) float2 sm[];
+    const int t = threadIdx.x, c = blockIdx.x, tile = blockIdx.y, s = blockIdx.z;
+    const MapSnap ms = a.snap[s];
+    if (c * a.Mb >= a.sd[s].n || tile * a.LT >= ms.NL) return;
+    const float2 *Fs = a.F2 + (size_t)s * (a.Cmax + a.nwin) * n + t;
+    const float2 *F1 = Fs + (size_t)c * n, *F2 = Fs + (size_t)(a.Cmax + c + tile * (a.LT / a.Mb)) * n;
+    constexpr float inv = 1.0f / (float)n;
+    float2 v[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        const float2 g = __ldg(F1 + T * e), f = __ldg(F2 + T * e);
+        v[e] = make_float2(fmaf(g.x, f.x, g.y * f.y) * inv, fmaf(g.y, f.x, -g.x * f.y) * inv);
+    }
+    fft_cta<LOGN>(v, sm, a.tw);
+    float2 *U = a.U + ((size_t)s * a.Cmax + c) * a.NLpad;
+    const int l0 = tile * a.LT, nl_t = min(a.LT, ms.NL - l0);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        const int l = t + T * e;
+        if (l < nl_t) U[l0 + l] = v[e];
+    }
+}
+
 // X[q][l]: a warp takes 32 lags and NQ bins (in pairs: the packed FMAs run
 // over two bins, whose node weights lie side by side in shared memory); the
 // CTA's warps share the lags (their U loads hit L1). Per block and node a
 // warp loads 256 bytes of U and 4 NQ bytes of weights for 2 NQ x 32 FMAs.
 constexpr int kExpWarps = 8;
-
-__device__ __forceinline__ void cp_async8(void *dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
 
 // LW of the CTA's warps lie along the lags (32 each), 8 / LW along the bins:
 // narrow tables (few bins) take more lags per CTA. U and the phases are staged
@@ -1035,6 +1117,34 @@ cudaError_t launch_map_tables(const MapArgs &a, cudaStream_t st, int *launches)
     }
     *launches += 2;
     return e;
+}
+
+template <int LOGN> static cudaError_t launch_chunks(const MapArgs &a, cudaStream_t st)
+{
+    constexpr int n = 1 << LOGN;
+    const size_t smem = sizeof(float2) * (size_t)(n + n / 16);
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(k_chunk_spec<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_chunk_corr<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    k_chunk_spec<LOGN><<<dim3((unsigned)(a.Cmax + a.nwin), (unsigned)a.S), n / 16, smem, st>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_chunk_corr<LOGN><<<dim3((unsigned)a.Cmax, (unsigned)a.ntile, (unsigned)a.S), n / 16, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_chunk_sums(const MapArgs &a, cudaStream_t st, int *launches)
+{
+    cudaError_t e = launch_bad(a, st, launches);
+    if (e != cudaSuccess) return e;
+    *launches += 2;
+    switch (a.logn) {
+    case 10: return launch_chunks<10>(a, st);
+    case 11: return launch_chunks<11>(a, st);
+    case 12: return launch_chunks<12>(a, st);
+    case 13: return launch_chunks<13>(a, st);
+    case 14: return launch_chunks<14>(a, st);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 template <int NQ, int LW> static cudaError_t launch_expand(const MapArgs &a, cudaStream_t st)
