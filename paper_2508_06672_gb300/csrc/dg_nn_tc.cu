@@ -166,6 +166,13 @@ __device__ __forceinline__ uint16_t bf16_bits(float v)
     return *reinterpret_cast<const uint16_t *>(&h);
 }
 
+// two values rounded as bf16_bits, the first in the low half
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
+{
+    const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+
 // Tensor-memory columns of an accumulator of n columns (a power of two >= 32).
 __host__ __device__ constexpr int tmem_cols(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : n <= 256 ? 256 : 512; }
 
@@ -189,11 +196,11 @@ __host__ __device__ constexpr int tmem_cols(int n) { return n <= 32 ? 32 : n <= 
 //
 // One CTA per SM walks the tiles; its warps have a role each and meet only on
 // mbarriers: 13 stage input rows into a ring of buffers, one copies weights, one
-// issues the MMAs (with all lanes, see nn_elect), four write finished tiles out
+// issues the MMAs (with all lanes, see nn_elect), eight write finished tiles out
 // of one of two accumulator sets while the next tile's products run. (A CTA per
 // tile in which every thread staged, one also issued, and all met twice per
 // channel block: 222 us for 128 -> 64 channels at 16 x 128 x 128, MMA pipes 8 %
-// busy; now 73 us, bound by the latency of the staging's loads.) Each output's products are added in the order (channel block, tap,
+// busy; now 69 us, bound by the staging's loads.) Each output's products are added in the order (channel block, tap,
 // K-step).
 // x: [B][CI][H][W]; y: [B][CO][H][W]; b may be NULL.
 // ---------------------------------------------------------------------------
@@ -202,7 +209,8 @@ constexpr int kHaloCB = 32;                                    // input channels
 constexpr int kHaloQ = kRowsTc + 2;                            // staged pixels per input row
 constexpr int kHaloBytes = (kHaloRows + 2) * (kHaloCB / 8) * kHaloQ * 16;
 constexpr int kProdWarps = 13;                                 // staging warps: 5 rows of 8 channels a thread
-constexpr int kConvThreads = 32 * (kProdWarps + 6);            // + 4 output warps, weights, MMAs
+constexpr int kOutWarps = 8;                                   // output warps: four per output row
+constexpr int kConvThreads = 32 * (kProdWarps + kOutWarps + 2);  // + weights, MMAs
 constexpr int kHaloMax = 4;                                    // staging buffers, at most
 constexpr int kWSlots = 64;                                    // weight blocks in shared memory, at most
 constexpr int kConvSmem = 224 * 1024;                          // dynamic shared memory, at most
@@ -272,36 +280,44 @@ __global__ void k_conv_tc_wimg(const float *__restrict__ w, uint16_t *__restrict
 // j0 + 128, as BF16 (zeros outside the image and past CI): 16-byte row
 // ((row * 4 + channel group) * kHaloQ + pixel). Consecutive threads take
 // consecutive pixels, so each of the 8 loads of a row is coalesced; all of a
-// thread's 40 loads are in flight together (with 16 the staging waited on
-// memory: 90 against 80 us for a 128 -> 64 channel layer at 512 x 512).
+// thread's 40 loads are in flight together. WIDE = false: a block's 32 planes
+// span less than 4 GB, so a load's address is a base shared by the CTA plus the
+// thread's 32-bit offset. At 4.8 TB/s from L2 (the halo rows are read twice over)
+// the staging bounds the kernel.
+template <bool WIDE>
 __device__ __forceinline__ void stage_halo(unsigned char *hb, const float *__restrict__ xn, int cb, int CI, int H,
                                            int W, int i0, int j0)
 {
     constexpr int items = (kHaloRows + 2) * (kHaloCB / 8) * kHaloQ, per = items / (32 * kProdWarps);
     static_assert(per * 32 * kProdWarps == items, "every thread takes the same number of rows");
     const int64_t HW = (int64_t)H * W;
+    const int c0 = cb * kHaloCB;
+    const char *base = reinterpret_cast<const char *>(xn + (int64_t)c0 * HW + (int64_t)(i0 - 1) * W + (j0 - 1));
     float v[per][8];
 #pragma unroll
     for (int z = 0; z < per; ++z) {
         const int it = threadIdx.x + z * 32 * kProdWarps;
         const int q = it % kHaloQ, rest = it / kHaloQ;
         const int g = rest % (kHaloCB / 8), rr = rest / (kHaloCB / 8);
-        const int row = i0 - 1 + rr, col = j0 - 1 + q, c0 = cb * kHaloCB + g * 8;
-        const int nc = row >= 0 && row < H && col >= 0 && col < W ? CI - c0 : 0;
-        const float *src = xn + (int64_t)c0 * HW + (int64_t)row * W + col;
+        const bool in = (unsigned)(i0 - 1 + rr) < (unsigned)H && (unsigned)(j0 - 1 + q) < (unsigned)W;
+        const int nc = in ? CI - c0 - 8 * g : 0;
+        const int64_t o64 = 4 * (8 * g * HW + (int64_t)rr * W + q);
+        const unsigned o32 = 4u * (8u * (unsigned)g * (unsigned)HW + (unsigned)(rr * W + q));
         if (nc >= 8) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[z][e] = __ldg(src + e * HW);
+            for (int e = 0; e < 8; ++e)
+                v[z][e] = __ldg(reinterpret_cast<const float *>(base + 4 * e * HW + (WIDE ? o64 : (int64_t)o32)));
         } else {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[z][e] = e < nc ? __ldg(src + e * HW) : 0.f;
+            for (int e = 0; e < 8; ++e)
+                v[z][e] = e < nc ? __ldg(reinterpret_cast<const float *>(base + 4 * e * HW + (WIDE ? o64 : (int64_t)o32))) : 0.f;
         }
     }
 #pragma unroll
     for (int z = 0; z < per; ++z) {
         uint32_t pk[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) pk[e] = bf16_bits(v[z][2 * e]) | (bf16_bits(v[z][2 * e + 1]) << 16);
+        for (int e = 0; e < 4; ++e) pk[e] = bf16_pair(v[z][2 * e], v[z][2 * e + 1]);
         *reinterpret_cast<uint4 *>(hb + (size_t)(threadIdx.x + z * 32 * kProdWarps) * 16) =
             make_uint4(pk[0], pk[1], pk[2], pk[3]);
     }
@@ -310,6 +326,7 @@ __device__ __forceinline__ void stage_halo(unsigned char *hb, const float *__res
 // nh staging buffers and nw weight slots (nw = all of the layer's blocks when
 // they are resident; then there is one block of output channels). relu: write
 // max(y, 0).
+template <bool WIDE>
 __global__ void __launch_bounds__(kConvThreads, 1)
     k_conv3x3_tc(const float *__restrict__ x, const uint16_t *__restrict__ wimg, const float *__restrict__ b,
                  float *__restrict__ y, int CI, int CO, int H, int W, int NT, int nh, int nw, int64_t tiles, int relu,
@@ -352,7 +369,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
         }
         for (int k = 0; k < 2; ++k) {
             nn_mbar_init(smem_addr(&afull[k]), 1);
-            nn_mbar_init(smem_addr(&aempty[k]), 4);
+            nn_mbar_init(smem_addr(&aempty[k]), kOutWarps);
         }
         nn_mbar_init(smem_addr(&fin), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -376,7 +393,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
                     ok = false;
                     break;
                 }
-                stage_halo(nsm + (size_t)s * kHaloBytes, xn, cb, CI, H, W, o.i0, o.j0);
+                stage_halo<WIDE>(nsm + (size_t)s * kHaloBytes, xn, cb, CI, H, W, o.i0, o.j0);
                 nn_fence_async();
                 __syncwarp();
                 if (lane == 0) nn_arrive(smem_addr(&hfull[s]));
@@ -386,8 +403,9 @@ __global__ void __launch_bounds__(kConvThreads, 1)
                 }
             }
         }
-    } else if (warp < kProdWarps + 4) {
-        const int q = warp & 3;  // tensor-memory lanes (pixels) 32 q .. + 31
+    } else if (warp < kProdWarps + kOutWarps) {
+        // tensor-memory lanes (pixels) 32 q .. + 31, output row r of the tile
+        const int q = warp & 3, r = (warp - kProdWarps) >> 2;
         int set = 0;
         uint32_t ph = 0;
         for (int64_t v = blockIdx.x; v < tiles && ok; v += gridDim.x) {
@@ -398,29 +416,29 @@ __global__ void __launch_bounds__(kConvThreads, 1)
             const int jp = o.j0 + 32 * q + lane, o0 = o.obi * NT;
             float *yn = y + (size_t)o.n * CO * H * W;
             const int64_t HW = (int64_t)H * W;
-            for (int r = 0; r < kHaloRows; ++r) {
-                const int i = o.i0 + r;
-                const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((set * kHaloRows + r) * AS);
-                for (int c0 = 0; c0 < NT; c0 += 32) {
-                    uint32_t rv[32];
-                    nn_ld32(tl + (uint32_t)c0, rv);
-                    const int nc = min(min(NT - c0, CO - o0 - c0), 32);
-                    const float bl = b && lane < nc ? __ldg(b + o0 + c0 + lane) : 0.f;
+            const int i = o.i0 + r;
+            const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((set * kHaloRows + r) * AS);
+            const unsigned o32 = 4u * (unsigned)(i * W + jp);
+            for (int c0 = 0; c0 < NT; c0 += 32) {
+                uint32_t rv[32];
+                nn_ld32(tl + (uint32_t)c0, rv);
+                const int nc = min(min(NT - c0, CO - o0 - c0), 32);
+                const float bl = b && lane < nc ? __ldg(b + o0 + c0 + lane) : 0.f;
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        const float val = __uint_as_float(rv[e]) + __shfl_sync(0xffffffffu, bl, e);
-                        rv[e] = __float_as_uint(relu ? fmaxf(val, 0.f) : val);
-                    }
-                    if (i < H && jp < W) {
-                        float *dst = yn + (int64_t)(o0 + c0) * HW + (int64_t)i * W + jp;
-                        if (nc == 32) {
+                for (int e = 0; e < 32; ++e) {
+                    const float val = __uint_as_float(rv[e]) + __shfl_sync(0xffffffffu, bl, e);
+                    rv[e] = __float_as_uint(relu ? fmaxf(val, 0.f) : val);
+                }
+                if (i < H && jp < W) {
+                    char *dst = reinterpret_cast<char *>(yn + (int64_t)(o0 + c0) * HW);
+                    const int64_t off = WIDE ? 4 * ((int64_t)i * W + jp) : (int64_t)o32;
+                    if (nc == 32) {
 #pragma unroll
-                            for (int e = 0; e < 32; ++e) dst[e * HW] = __uint_as_float(rv[e]);
-                        } else {
+                        for (int e = 0; e < 32; ++e) *reinterpret_cast<float *>(dst + 4 * e * HW + off) = __uint_as_float(rv[e]);
+                    } else {
 #pragma unroll
-                            for (int e = 0; e < 32; ++e)
-                                if (e < nc) dst[e * HW] = __uint_as_float(rv[e]);
-                        }
+                        for (int e = 0; e < 32; ++e)
+                            if (e < nc) *reinterpret_cast<float *>(dst + 4 * e * HW + off) = __uint_as_float(rv[e]);
                     }
                 }
             }
@@ -430,7 +448,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
             if (set) ph ^= 1;
             set ^= 1;
         }
-    } else if (warp == kProdWarps + 4) {
+    } else if (warp == kProdWarps + kOutWarps) {
         if (lane == 0) {
             int slot = 0;
             uint32_t ph = 1;
@@ -505,7 +523,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     __syncwarp();
     // before tensor memory and shared memory are released the MMAs and copies
     // issued have landed, also where a wait gave up
-    if (t == 32 * (kProdWarps + 4))
+    if (t == 32 * (kProdWarps + kOutWarps))
         for (int64_t g = copied > nw ? copied - nw : 0; g < copied; ++g)
             ok = nn_wait(smem_addr(&wfull[g % nw]), (uint32_t)(g / nw) & 1u) && ok;
     ok = __syncthreads_and(ok) != 0;
@@ -566,7 +584,7 @@ __device__ __forceinline__ uint4 pack8(const float (&v)[8])
 {
     uint32_t pk[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) pk[e] = bf16_bits(v[2 * e]) | (bf16_bits(v[2 * e + 1]) << 16);
+    for (int e = 0; e < 4; ++e) pk[e] = bf16_pair(v[2 * e], v[2 * e + 1]);
     return make_uint4(pk[0], pk[1], pk[2], pk[3]);
 }
 
@@ -873,11 +891,14 @@ cudaError_t launch_conv_tc(bool tr, const float *x, const float *w, const float 
     const int nw = resident ? nblk : std::min(nblk, std::min(16, (kConvSmem - 2 * kHaloBytes) / wbytes));
     const int nh = std::min(kHaloMax, (kConvSmem - nw * wbytes) / kHaloBytes);
     const int smem = nh * kHaloBytes + nw * wbytes;
-    if ((e = cudaFuncSetAttribute(k_conv3x3_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+    // 32 planes and a row of pixels each, in bytes, against the 32-bit offsets
+    const bool wide = 4.0 * (kHaloCB * (double)H * W + 8.0 * W + 4096.0) > 4294967295.0;
+    auto kernel = wide ? k_conv3x3_tc<true> : k_conv3x3_tc<false>;
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
         return e;
     const int64_t tiles = (int64_t)((W + kRowsTc - 1) / kRowsTc) * ((H + kHaloRows - 1) / kHaloRows) * B * ob;
-    k_conv3x3_tc<<<(unsigned)std::min<int64_t>(tiles, 152), kConvThreads, smem, s>>>(x, wimg, b, y, CI, CO, H, W, NT, nh, nw,
-                                                                                     tiles, relu, err);
+    kernel<<<(unsigned)std::min<int64_t>(tiles, 152), kConvThreads, smem, s>>>(x, wimg, b, y, CI, CO, H, W, NT, nh, nw, tiles,
+                                                                               relu, err);
     return cudaGetLastError();
 }
 
