@@ -247,6 +247,11 @@ dg_status dg_set_grid(dg_ctx *ctx, const dg_grid *grid);
 dg_status dg_search_regions(dg_ctx *ctx, const dg_grid *regions, int32_t n, void *costs,
                             double refine_spacing_m, double refine_window_m, dg_fix *out, int32_t *best);
 
+/* The largest cost of each of the n regions of the last dg_search_regions (NaN:
+ * a region without a finite value), from the records that search read; no
+ * launch and no synchronisation. DG_ESTATE: that search had fewer regions. */
+dg_status dg_region_maxima(dg_ctx *ctx, double *out, int32_t n);
+
 /* The cost surface of the shard (Eq. 11 summed over snapshots, Algorithm 1):
  * out[p] = sum_k |C_k(p)|^2 (or |C_k(p)|), p over the shard's nrows * nlon
  * nodes. out is a device pointer to float (FP32) or double (FP64) with room

@@ -192,9 +192,9 @@ struct dg_ctx {
     size_t amax_tmp_bytes = 0;
     ArgmaxResult *amax_res = nullptr;
     ArgmaxResult *amax_host = nullptr;  // pinned
-    int *det_count = nullptr;
     int64_t *det_cand = nullptr;
-    DetectPeak *det_out = nullptr;
+    DetectPeak *det_out = nullptr, *det_host = nullptr;
+    int reg_n = 0;  // regions of the last search, their records in reg_host
     unsigned *err_d = nullptr;
     unsigned *err_h = nullptr;          // pinned mirror
     LocalGrid loc;
@@ -1668,8 +1668,10 @@ static dg_status refine_map(dg_ctx *c, const GridDev &gd, const double *xyz, int
     a.NLpad = 32;
     a.S = a.ksd = c->K;
     f.tscale = 2.0f / (float)(nmax + 1);
-    // CTAs per snapshot: four per SM over all snapshots, a block of samples each at least
-    a.Cmax = std::max(1, std::min((nmax + kFewBlock - 1) / kFewBlock, (4 * c->sm_count + c->K - 1) / c->K));
+    // CTAs per snapshot: what fits on the chip over all snapshots (by the kernel's
+    // registers), a block of samples each at least
+    const int per_sm = a.P == 4 ? 4 : a.P == 6 ? 3 : 2;
+    a.Cmax = std::max(1, std::min((nmax + kFewBlock - 1) / kFewBlock, per_sm * c->sm_count / c->K));
     const size_t u = sizeof(float) * map_few_partials(a.P, a.LT) * (size_t)a.Cmax * c->K;
     if (u > ((size_t)1 << 32) || (c->opt.scratch_mib && (double)u > c->opt.scratch_mib * 1048576.0)) return DG_OK;
     dg_status st = push_steps(c);
@@ -1681,18 +1683,28 @@ static dg_status refine_map(dg_ctx *c, const GridDev &gd, const double *xyz, int
     if (c64 && (st = ensure(c, (void **)&d.bad, &d.bad_cap, sizeof(int) * 4 * (size_t)c->K)) != DG_OK) return st;
     if ((st = ensure_ephf(c)) != DG_OK) return st;
     // e^{j theta_q t} = sum_m j^m T[m][q] T_m(t), theta_q the phase of bin q at
-    // t = 1: the series' real coefficients by a 32-point cosine sum
-    for (int q = 0; q < a.Q; ++q) {
+    // t = 1: the series' real coefficients by a 32-point cosine sum, folded (the
+    // points lie symmetrically around 0, and so do the bins). 272 sines on the
+    // host; each coefficient's own sum took 12 thousand, 90 us.
+    double px[16], tm[kFewMaxNodes][16];  // points cos((i + 1/2) pi / 32), T_m there
+    for (int i = 0; i < 16; ++i) {
+        px[i] = std::cos(kPi * (i + 0.5) / 32.0);
+        for (int m = 0; m < a.P; ++m)
+            tm[m][i] = m == 0 ? 1.0 : m == 1 ? px[i] : 2.0 * px[i] * tm[m - 1][i] - tm[m - 2][i];
+    }
+    for (int q = 0; q < a.Q / 2; ++q) {
         const double theta = 2.0 * kPi * (q * f.delta - f.halfw) / f.tscale;
+        double cs[16], sn[16];
+        for (int i = 0; i < 16; ++i) {
+            cs[i] = std::cos(theta * px[i]);
+            sn[i] = std::sin(theta * px[i]);
+        }
         for (int m = 0; m < a.P; ++m) {
-            double re = 0.0, im = 0.0;
-            for (int i = 0; i < 32; ++i) {
-                const double phi = kPi * (i + 0.5) / 32.0;
-                re += std::cos(theta * std::cos(phi)) * std::cos(m * phi);
-                im += std::sin(theta * std::cos(phi)) * std::cos(m * phi);
-            }
-            const double w = (m ? 2.0 : 1.0) / 32.0;
-            f.T[m * a.Q + q] = (float)(w * (m % 4 == 0 ? re : m % 4 == 1 ? im : m % 4 == 2 ? -re : -im));
+            double x = 0.0;
+            for (int i = 0; i < 16; ++i) x += (m & 1 ? sn[i] : cs[i]) * tm[m][i];
+            x *= (m ? 4.0 : 2.0) / 32.0 * (m % 4 < 2 ? 1.0 : -1.0);
+            f.T[m * a.Q + q] = (float)x;
+            f.T[m * a.Q + a.Q - 1 - q] = (float)(m & 1 ? -x : x);
         }
     }
     map_common(c, 0, xyz, gd, G, a);
@@ -1939,7 +1951,8 @@ static void grid_bounds_switch(dg_ctx *c, const dg_grid &next)
     }
 }
 
-dg_status dg_set_grid(dg_ctx *c, const dg_grid *grid)
+// xyz, step: the grid's nodes and angular steps where they are on the device.
+static dg_status set_grid(dg_ctx *c, const dg_grid *grid, const double *xyz, const GridStep *step)
 {
     if (!c) return fail(nullptr, DG_EINVAL, "ctx is NULL");
     c->err.clear();
@@ -1963,6 +1976,11 @@ dg_status dg_set_grid(dg_ctx *c, const dg_grid *grid)
     c->gd = make_griddev(*grid, 0, grid->nlat);
     c->G = G;
     ++c->steps_gen;           // graphs and batches recorded on the old grid are stale
+    if (xyz) {
+        CK(c, cudaMemcpyAsync(c->xyz, xyz, sizeof(double) * 3 * (size_t)G, cudaMemcpyDeviceToDevice, c->stream));
+        CK(c, cudaMemcpyAsync(c->gstep, step, sizeof(GridStep), cudaMemcpyDeviceToDevice, c->stream));
+        return DG_OK;
+    }
     {
         Timed t(c, DG_K_GRID);
         CK(c, launch_grid_ecef(c->gd, c->xyz, c->stream, nullptr, nullptr, 1, c->gstep));
@@ -1970,6 +1988,8 @@ dg_status dg_set_grid(dg_ctx *c, const dg_grid *grid)
     }
     return DG_OK;
 }
+
+dg_status dg_set_grid(dg_ctx *c, const dg_grid *grid) { return set_grid(c, grid, nullptr, nullptr); }
 
 dg_status dg_load_capture(dg_ctx *c, int32_t step, int32_t fmt, const void *y1, const void *y2,
                           int64_t n, int32_t is_device_ptr)
@@ -2061,10 +2081,11 @@ static dg_status refine_half(dg_ctx *c, double spacing_m, double window_m, int *
 
 static dg_status ensure_post(dg_ctx *c, int half, dg_fix **fix_dev, dg_fix **fix_host);
 static dg_status step_device_post(dg_ctx *c, const void *cost, double spacing_m, int half, dg_fix *fix_dev,
-                                  dg_fix *fix_host);
+                                  dg_fix *fix_host, const ArgmaxResult *known);
 static dg_status read_fix(dg_ctx *c, const dg_fix *fix_host, dg_fix *out);
 
-dg_status dg_argmax_refine(dg_ctx *c, const void *cost, double spacing_m, double window_m, dg_fix *out)
+static dg_status argmax_refine(dg_ctx *c, const void *cost, double spacing_m, double window_m, dg_fix *out,
+                               const ArgmaxResult *known)
 {
     if (!c) return fail(nullptr, DG_EINVAL, "ctx is NULL");
     c->err.clear();
@@ -2075,11 +2096,16 @@ dg_status dg_argmax_refine(dg_ctx *c, const void *cost, double spacing_m, double
     // the step of a captured graph, uncaptured: the refinement grid is centred
     // on the argmax on the device and one synchronisation reads the fix
     if ((st = ensure_post(c, half, &c->fix_dev_sync, &c->fix_host_sync)) != DG_OK) return st;
-    if ((st = step_device_post(c, cost, spacing_m, half, c->fix_dev_sync, c->fix_host_sync)) != DG_OK) return st;
+    if ((st = step_device_post(c, cost, spacing_m, half, c->fix_dev_sync, c->fix_host_sync, known)) != DG_OK) return st;
     dg_fix f;
     if ((st = read_fix(c, c->fix_host_sync, &f)) != DG_OK) return st;
     *out = f;
     return DG_OK;
+}
+
+dg_status dg_argmax_refine(dg_ctx *c, const void *cost, double spacing_m, double window_m, dg_fix *out)
+{
+    return argmax_refine(c, cost, spacing_m, window_m, out, nullptr);
 }
 
 dg_status dg_detect(dg_ctx *c, const void *cost, double threshold, int32_t relative, int32_t radius,
@@ -2092,34 +2118,37 @@ dg_status dg_detect(dg_ctx *c, const void *cost, double threshold, int32_t relat
     if (max_peaks < 1 || max_peaks > kDetectCap) return fail(c, DG_EINVAL, "max_peaks must be in [1, %d]", kDetectCap);
     if (!std::isfinite(threshold)) return fail(c, DG_EINVAL, "threshold must be finite");
     constexpr int kCap = kDetectCap;
-    CK(c, cudaStreamSynchronize(c->stream));
-    dg_status st = check_latched(c);
-    if (st != DG_OK) return st;
+    dg_status st;
     double thr = threshold;
     if (relative) {
+        CK(c, cudaStreamSynchronize(c->stream));
+        if ((st = check_latched(c)) != DG_OK) return st;
         ArgmaxResult r;
         if ((st = run_argmax(c, cost, c->G, c->gd, &r)) != DG_OK) return st;
         if (r.idx < 0) return fail(c, DG_EINVAL, "the surface holds no finite value");
         thr = threshold * r.val;
     }
-    if (!c->det_count) {
-        CK(c, cudaMallocAsync((void **)&c->det_count, sizeof(int), c->stream));
+    const size_t out_bytes = sizeof(DetectPeak) * kCap + sizeof(int);  // records, then their count
+    if (!c->det_out) {
         CK(c, cudaMallocAsync((void **)&c->det_cand, sizeof(int64_t) * kCap, c->stream));
-        CK(c, cudaMallocAsync((void **)&c->det_out, sizeof(DetectPeak) * kCap, c->stream));
+        CK(c, cudaMallocAsync((void **)&c->det_out, out_bytes, c->stream));
     }
+    if (!c->det_host) CK(c, cudaMallocHost((void **)&c->det_host, out_bytes));
+    int *const count_d = reinterpret_cast<int *>(c->det_out + max_peaks);  // behind the records asked for
+    const DetectPeak *const pk = c->det_host;
     int count = 0;
-    std::vector<DetectPeak> pk((size_t)max_peaks);
     for (int round = 0;; ++round) {
         {
             Timed t(c, DG_K_ARGMAX);
-            CK(c, launch_detect(cost, c->opt.prec, c->gd, thr, radius, kCap, max_peaks, c->det_count, c->det_cand,
+            CK(c, launch_detect(cost, c->opt.prec, c->gd, c->gstep, thr, radius, kCap, max_peaks, count_d, c->det_cand,
                                 c->det_out, c->stream));
             t.done(2);
         }
-        CK(c, cudaMemcpyAsync(&count, c->det_count, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-        CK(c, cudaMemcpyAsync(pk.data(), c->det_out, sizeof(DetectPeak) * (size_t)max_peaks, cudaMemcpyDeviceToHost,
-                              c->stream));
+        CK(c, cudaMemcpyAsync(c->det_host, c->det_out, sizeof(DetectPeak) * (size_t)max_peaks + sizeof(int),
+                              cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaStreamSynchronize(c->stream));
+        if ((st = check_latched(c)) != DG_OK) return st;
+        count = *reinterpret_cast<const int *>(c->det_host + max_peaks);
         if (count <= kCap) break;
         // More peaks pass than the sort holds: it ordered kCap of them (an
         // arbitrary subset), so at least max_peaks peaks reach its
@@ -2182,16 +2211,18 @@ static dg_status step_device(dg_ctx *c, void *cost, double spacing_m, int half)
 {
     dg_status st = run_surface(c, c->gd, c->xyz, c->G, c->surf, cost, false);
     if (st != DG_OK) return st;
-    return step_device_post(c, cost, spacing_m, half, c->fix_dev, c->fix_host);
+    return step_device_post(c, cost, spacing_m, half, c->fix_dev, c->fix_host, nullptr);
 }
 
-// The rest of a step once the surface is enqueued: its argmax, the
-// refinement, the fix record.
+// The rest of a step once the surface is enqueued: its argmax (unless its record
+// is on the device: known), the refinement, the fix record.
 static dg_status step_device_post(dg_ctx *c, const void *cost, double spacing_m, int half, dg_fix *fix_dev,
-                                  dg_fix *fix_host)
+                                  dg_fix *fix_host, const ArgmaxResult *known)
 {
     dg_status st = DG_OK;
-    {
+    if (known && half > 0) {  // the surface's record is on the device already
+        CK(c, cudaMemcpyAsync(c->amax_res, known, sizeof(ArgmaxResult), cudaMemcpyDeviceToDevice, c->stream));
+    } else {
         Timed t(c, DG_K_ARGMAX);
         int nl = 0;
         CK(c, launch_argmax(cost, c->G, c->opt.prec, c->gd, c->gstep, c->amax_tmp, c->amax_res, &nl, c->stream, nullptr,
@@ -2399,7 +2430,7 @@ static dg_status capture_steps(dg_ctx *const *ctxs, int n, void *const *costs, d
     if (rounds && e == cudaSuccess) st = shared_surfaces(ctxs, n, costs, *rounds, stream, &shared);
     for (int i = 0; i < n && e == cudaSuccess && st == DG_OK; ++i) {
         dg_ctx *c = ctxs[i];
-        st = rounds ? step_device_post(c, costs[i], spacing_m, half[i], c->fix_dev, c->fix_host)
+        st = rounds ? step_device_post(c, costs[i], spacing_m, half[i], c->fix_dev, c->fix_host, nullptr)
                     : step_device(c, costs[i], spacing_m, half[i]);
         if (st == DG_OK) e = cudaEventRecord(join[i], c->stream);
         if (e == cudaSuccess && st == DG_OK) e = cudaStreamWaitEvent(stream, join[i], 0);
@@ -2862,7 +2893,6 @@ dg_status dg_destroy(dg_ctx *c)
     fr(c->fix_dev_sync);
     if (c->graph) cudaGraphExecDestroy(c->graph);
     fr(c->err_d);
-    fr(c->det_count);
     fr(c->det_cand);
     fr(c->det_out);
     fr(c->loc.xyz);
@@ -2940,6 +2970,7 @@ dg_status dg_destroy(dg_ctx *c)
     cudaError_t e = cudaStreamSynchronize(s);
     if (c->amax_host) cudaFreeHost(c->amax_host);
     if (c->reg_host) cudaFreeHost(c->reg_host);
+    if (c->det_host) cudaFreeHost(c->det_host);
     if (c->fix_host) cudaFreeHost(c->fix_host);
     if (c->fix_host_sync) cudaFreeHost(c->fix_host_sync);
     if (c->err_h) cudaFreeHost(c->err_h);
@@ -3210,42 +3241,54 @@ static bool region_range(const dg_ctx *c, const GridDev &g, GridRange *out)
 // The surfaces and argmax records of all regions through shared launches:
 // table s of the batch is of capture s % K and region s / K. *done = false
 // where the maps do not serve these regions.
-static dg_status regions_map(dg_ctx *c, const dg_grid *regions, int n, float *costs, bool *done)
+static dg_status regions_map(dg_ctx *c, const dg_grid *regions, int n, float *costs, bool *done, bool *nodes)
 {
-    *done = false;
+    *done = *nodes = false;
     const int64_t G = (int64_t)regions[0].nlat * regions[0].nlon;
     if (!map_options(c) || G < kMapMinNodes || c->gd.row0 != 0 || c->gd.nrows != c->grid.nlat) return DG_OK;
     const size_t K = (size_t)c->K;
     std::vector<GridDev> grids((size_t)n);
     std::vector<GridRange> range(K * (size_t)n);
-    for (int r = 0; r < n; ++r) {
-        grids[(size_t)r] = make_griddev(regions[r], 0, regions[r].nlat);
-        if (!region_range(c, grids[(size_t)r], &range[K * (size_t)r])) return DG_OK;
+    for (int r = 0; r < n; ++r) grids[(size_t)r] = make_griddev(regions[r], 0, regions[r].nlat);
+    dg_status st;
+    // every region's nodes at once, under way while the host plans
+    const bool all = n <= 64 && (double)n * G * 24.0 <= 256e6;
+    if ((st = ensure(c, (void **)&c->reg_grids, &c->reg_grids_cap, sizeof(GridDev) * (size_t)n)) != DG_OK) return st;
+    CK(c, cudaMemcpyAsync(c->reg_grids, grids.data(), sizeof(GridDev) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
+    if (all) {
+        if ((st = ensure(c, (void **)&c->reg_xyz, &c->reg_xyz_cap, sizeof(double) * 3 * (size_t)G * n)) != DG_OK) return st;
+        if ((st = ensure(c, (void **)&c->reg_steps, &c->reg_steps_cap, sizeof(GridStep) * (size_t)n)) != DG_OK) return st;
+        Timed t(c, DG_K_GRID);
+        CK(c, launch_grid_ecef(grids[0], c->reg_xyz, c->stream, nullptr, c->reg_grids, n, c->reg_steps));
+        t.done(1);
     }
+    for (int r = 0; r < n; ++r)
+        if (!region_range(c, grids[(size_t)r], &range[K * (size_t)r])) return DG_OK;
     MapPlan m;
     std::vector<MapSnap> snap;
     if (!map_shape(c, range, snap, m)) return DG_OK;
     const double budget = (double)(c->opt.scratch_mib ? c->opt.scratch_mib : 12288) * 1048576.0;
     const int nr = (int)std::min((double)std::min(n, (int)(65535 / K)), std::floor(budget / ((double)K * map_bytes(m))));
     if (nr < 1) return DG_OK;
-    dg_status st;
     c->mp.gen = 0;  // the tables of the main grid's plan are replaced
     if ((st = map_buffers(c, m, K * (size_t)nr, snap)) != DG_OK) return st;
     if ((st = push_steps(c)) != DG_OK) return st;
-    if ((st = ensure(c, (void **)&c->reg_xyz, &c->reg_xyz_cap, sizeof(double) * 3 * (size_t)G * nr)) != DG_OK) return st;
-    if ((st = ensure(c, (void **)&c->reg_grids, &c->reg_grids_cap, sizeof(GridDev) * (size_t)n)) != DG_OK) return st;
-    if ((st = ensure(c, (void **)&c->reg_steps, &c->reg_steps_cap, sizeof(GridStep) * (size_t)nr)) != DG_OK) return st;
+    if (!all) {
+        if ((st = ensure(c, (void **)&c->reg_xyz, &c->reg_xyz_cap, sizeof(double) * 3 * (size_t)G * nr)) != DG_OK) return st;
+        if ((st = ensure(c, (void **)&c->reg_steps, &c->reg_steps_cap, sizeof(GridStep) * (size_t)nr)) != DG_OK) return st;
+    }
     if ((st = ensure(c, &c->amax_tmp, &c->amax_tmp_bytes, argmax_tmp_bytes(G) * (size_t)nr)) != DG_OK) return st;
-    CK(c, cudaMemcpyAsync(c->reg_grids, grids.data(), sizeof(GridDev) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
     for (int r0 = 0; r0 < n; r0 += nr) {
         const int R = std::min(nr, n - r0);
-        {
+        const double *xyz = c->reg_xyz + (all ? 3 * G * r0 : 0);
+        const GridStep *steps = c->reg_steps + (all ? r0 : 0);
+        if (!all) {
             Timed t(c, DG_K_GRID);
             CK(c, launch_grid_ecef(grids[0], c->reg_xyz, c->stream, nullptr, c->reg_grids + r0, R, c->reg_steps));
             t.done(1);
         }
         MapArgs a{};
-        map_common(c, 0, c->reg_xyz, grids[0], G, a);
+        map_common(c, 0, xyz, grids[0], G, a);
         map_tables_args(m, c->mb, a);
         a.ksd = c->K;
         a.nreg = R;
@@ -3268,7 +3311,7 @@ static dg_status regions_map(dg_ctx *c, const dg_grid *regions, int n, float *co
         {
             Timed t(c, DG_K_ARGMAX);
             int nl = 0;
-            CK(c, launch_argmax(a.out, G, DG_PREC_FP32, grids[0], c->reg_steps, c->amax_tmp, c->reg_res + r0, &nl, c->stream,
+            CK(c, launch_argmax(a.out, G, DG_PREC_FP32, grids[0], steps, c->amax_tmp, c->reg_res + r0, &nl, c->stream,
                                 nullptr, c->reg_grids + r0, R));
             t.done(nl);
         }
@@ -3279,6 +3322,7 @@ static dg_status regions_map(dg_ctx *c, const dg_grid *regions, int n, float *co
     c->mp.rows = 0;
     for (size_t k = 0; k < K; ++k) c->mp.rows += (int64_t)snap[k].NL * ((c->steps[k].n + m.Mb - 1) / m.Mb);
     *done = true;
+    *nodes = all;
     return DG_OK;
 }
 
@@ -3313,8 +3357,9 @@ dg_status dg_search_regions(dg_ctx *c, const dg_grid *regions, int32_t n, void *
         c->reg_cap = (size_t)n;
     }
     dg_status st;
-    bool done = false;
-    if ((st = regions_map(c, regions, n, (float *)costs, &done)) != DG_OK) return st;
+    bool done = false, nodes = false;
+    c->reg_n = 0;
+    if ((st = regions_map(c, regions, n, (float *)costs, &done, &nodes)) != DG_OK) return st;
     for (int r = 0; r < n && !done; ++r) {
         if ((st = dg_set_grid(c, &regions[r])) != DG_OK) return st;
         if ((st = ensure_surf(c)) != DG_OK) return st;
@@ -3331,13 +3376,27 @@ dg_status dg_search_regions(dg_ctx *c, const dg_grid *regions, int32_t n, void *
     CK(c, cudaMemcpyAsync(c->reg_host, c->reg_res, sizeof(ArgmaxResult) * n, cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
     if ((st = check_latched(c)) != DG_OK) return st;
+    c->reg_n = n;
     int b = -1;
     for (int r = 0; r < n; ++r)
         if (c->reg_host[r].idx >= 0 && (b < 0 || c->reg_host[r].val > c->reg_host[b].val)) b = r;
     if (b < 0) return fail(c, DG_EINVAL, "no region holds a finite value");
-    if ((st = dg_set_grid(c, &regions[b])) != DG_OK) return st;
-    if ((st = dg_argmax_refine(c, (char *)costs + esz * (size_t)G * b, spacing_m, window_m, out)) != DG_OK) return st;
+    // the best region becomes the context's grid; its nodes are there already
+    if ((st = set_grid(c, &regions[b], nodes ? c->reg_xyz + 3 * G * b : nullptr, nodes ? c->reg_steps + b : nullptr)) != DG_OK)
+        return st;
+    if ((st = argmax_refine(c, (char *)costs + esz * (size_t)G * b, spacing_m, window_m, out, c->reg_res + b)) != DG_OK)
+        return st;
     if (best) *best = b;
+    return DG_OK;
+}
+
+dg_status dg_region_maxima(dg_ctx *c, double *out, int32_t n)
+{
+    if (!c) return fail(nullptr, DG_EINVAL, "ctx is NULL");
+    c->err.clear();
+    if (!out) return fail(c, DG_EINVAL, "out is NULL");
+    if (n < 1 || n > c->reg_n) return fail(c, DG_ESTATE, "the last search had %d regions, not %d", c->reg_n, n);
+    for (int r = 0; r < n; ++r) out[r] = c->reg_host[r].idx >= 0 ? c->reg_host[r].val : std::nan("");
     return DG_OK;
 }
 

@@ -32,6 +32,7 @@
 //   k_caf_pool   maxima of A over 8 consecutive lags, and mu per snapshot
 //       (fixed-order sum);
 //   k_coarse_backproject   the max-pool per cell.
+#include <algorithm>
 #include <cfloat>
 #include <climits>
 
@@ -44,7 +45,7 @@ constexpr int kCafR = 7;                          // lags per thread
 constexpr int kCafThreads = 128;
 constexpr int kCafTile = kCafR * kCafThreads;     // lags per k_caf_lags CTA
 constexpr int kFoldWarps = 4;                     // warps of a k_caf_fold CTA
-constexpr int kFoldBins = 16;                     // bin pairs per warp
+constexpr int kFoldBins = 16;                     // bin pairs per warp, at most
 constexpr int kFoldRows = 16;                     // chunk pairs staged at a time
 constexpr int kPoolLags = 8;                      // lags per pooled maximum
 
@@ -276,7 +277,7 @@ __device__ __forceinline__ bool caf_bad(int4 b, int L, int nx)
 }
 
 // Xc at the Q bins for the CTA's lags of snapshot k = blockIdx.y: a warp takes
-// 32 lags and 16 bin pairs. The bins lie symmetrically around nu_c and the
+// 32 lags and 2 H bin pairs. The bins lie symmetrically around nu_c and the
 // chunks around their middle, and a unit phase per bin drops out of |.|^2: bins
 // nu_c +- d and chunks at offsets +- o share
 //     C = sum cos(2 pi d o M) (P_+ + P_-),   S = sum sin(2 pi d o M) (P_+ - P_-),
@@ -284,7 +285,7 @@ __device__ __forceinline__ bool caf_bad(int4 b, int L, int nx)
 // 4 real FMAs for 2 bins x 2 chunks where the complex products take 16. FP32
 // pipe; the factors (k_caf_turns) and the chunk pairs' sums and differences come
 // from shared memory, two bin pairs per packed FMA. 20 snapshots of 4192 lags,
-// 128 chunks and 40 bins: 254 -> 42 us. A = |Xc|^2, lags fastest, and the CTA's
+// 128 chunks and 40 bins: 254 -> 34 us. A = |Xc|^2, lags fastest, and the CTA's
 // sum of A (in a fixed order). QW of the CTA's warps lie along the bins.
 __device__ __forceinline__ void fma2_to(float2 &c, float2 a, float2 b)
 {
@@ -308,9 +309,9 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src)
                  : "memory");
 }
 
-template <int QW> __global__ void __launch_bounds__(32 * kFoldWarps) k_caf_fold(CoarseArgs a)
+template <int QW, int H> __global__ void __launch_bounds__(32 * kFoldWarps) k_caf_fold(CoarseArgs a)
 {
-    constexpr int LW = kFoldWarps / QW, NL = 32 * LW, H = kFoldBins / 2, T = 32 * kFoldWarps;
+    constexpr int LW = kFoldWarps / QW, NL = 32 * LW, T = 32 * kFoldWarps;
     extern __shared__ __align__(16) unsigned char fold_sm[];
     float4 *s_w = reinterpret_cast<float4 *>(fold_sm);                   // [2][rows][QW H] cos, sin of two bin pairs
     float2 *s_p = reinterpret_cast<float2 *>(s_w + 2 * kFoldRows * QW * H);  // [2][rows][2][NL] the pair's chunks
@@ -324,7 +325,7 @@ template <int QW> __global__ void __launch_bounds__(32 * kFoldWarps) k_caf_fold(
     }
     const int N = a.steps[k].n, nb = (N + a.M - 1) / a.M, nh = (nb + 1) / 2, ns = (nh + kFoldRows - 1) / kFoldRows;
     const int wq = warp % QW, wl = warp / QW;
-    const int j0 = (blockIdx.z * QW + wq) * kFoldBins, nq2 = (a.Q + 1) / 2;  // bin pairs, the middle bin one of them
+    const int j0 = (blockIdx.z * QW + wq) * 2 * H, nq2 = (a.Q + 1) / 2;  // bin pairs, the middle bin one of them
     const float2 *Pk = a.P + (size_t)k * a.nb_max * a.nlag_cap;
     const float4 *W = a.turn + (size_t)k * a.nh_max * (a.Dpad / 2) + blockIdx.z * QW * H;
     auto stage = [&](int g) {  // chunk pairs g kFoldRows .. , asynchronously
@@ -378,7 +379,7 @@ template <int QW> __global__ void __launch_bounds__(32 * kFoldWarps) k_caf_fold(
                                           (nb - 1) * a.M + (a.M + kCafR - 1) / kCafR * kCafR);
         float *Ak = a.A + (size_t)k * a.Q * a.nlag_cap + l;
 #pragma unroll
-        for (int z = 0; z < kFoldBins; ++z) {
+        for (int z = 0; z < 2 * H; ++z) {
             const int j = j0 + z;
             if (j >= nq2) continue;
             const float c0 = z & 1 ? cr[z / 2].y : cr[z / 2].x, c1 = z & 1 ? ci[z / 2].y : ci[z / 2].x;
@@ -532,27 +533,42 @@ unsigned blocks_for(int64_t n, int per, int cap)
 
 }  // namespace
 
-// bin pairs per CTA's warps along the bins, and the CTAs along lags and bins
+// Warps of a CTA along the bins, and the bin pairs of one (an even number: the
+// pairs in equal parts, so that a map of 40 bins leaves none of them idle).
 static int fold_qw(int Q) { return (Q + 1) / 2 <= kFoldBins ? 1 : (Q + 1) / 2 <= 2 * kFoldBins ? 2 : 4; }
+static int fold_pairs(int Q)
+{
+    const int qw = fold_qw(Q), p = std::min(kFoldBins, ((Q + 1) / 2 + qw - 1) / qw);
+    return p <= 8 ? 8 : p <= 10 ? 10 : p <= 12 ? 12 : 16;
+}
 int coarse_parts(int nlag_cap, int Q)
 {
-    const int nl = 32 * (kFoldWarps / fold_qw(Q)), nj = kFoldBins * fold_qw(Q);
+    const int nl = 32 * (kFoldWarps / fold_qw(Q)), nj = fold_pairs(Q) * fold_qw(Q);
     return (nlag_cap + nl - 1) / nl * (((Q + 1) / 2 + nj - 1) / nj);
 }
 int coarse_dpad(int Q)
 {
-    const int nj = kFoldBins * fold_qw(Q);
+    const int nj = fold_pairs(Q) * fold_qw(Q);
     return ((Q + 1) / 2 + nj - 1) / nj * nj;
 }
 
+template <int QW, int H> static cudaError_t launch_fold_h(const CoarseArgs &a, cudaStream_t s)
+{
+    const unsigned nl = 32 * (kFoldWarps / QW), nj = 2 * H * QW;
+    const size_t smem = kFoldRows * (sizeof(float4) * 2 * nj / 2 + sizeof(float2) * 4 * nl);
+    const cudaError_t e = cudaFuncSetAttribute(k_caf_fold<QW, H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_caf_fold<QW, H><<<dim3((a.nlag_cap + nl - 1) / nl, a.K, ((a.Q + 1) / 2 + nj - 1) / nj), 32 * kFoldWarps, smem, s>>>(a);
+    return cudaGetLastError();
+}
 template <int QW> static cudaError_t launch_fold(const CoarseArgs &a, cudaStream_t s)
 {
-    const unsigned nl = 32 * (kFoldWarps / QW), nj = kFoldBins * QW;
-    const size_t smem = kFoldRows * (sizeof(float4) * 2 * nj / 2 + sizeof(float2) * 4 * nl);
-    const cudaError_t e = cudaFuncSetAttribute(k_caf_fold<QW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_caf_fold<QW><<<dim3((a.nlag_cap + nl - 1) / nl, a.K, ((a.Q + 1) / 2 + nj - 1) / nj), 32 * kFoldWarps, smem, s>>>(a);
-    return cudaGetLastError();
+    switch (fold_pairs(a.Q)) {
+    case 8: return launch_fold_h<QW, 4>(a, s);
+    case 10: return launch_fold_h<QW, 5>(a, s);
+    case 12: return launch_fold_h<QW, 6>(a, s);
+    default: return launch_fold_h<QW, 8>(a, s);
+    }
 }
 
 cudaError_t launch_coarse(const CoarseArgs &a, const MapArgs *fft, cudaStream_t s, int *launches)

@@ -72,10 +72,12 @@ __device__ __forceinline__ unsigned long long sort_key(double x)
 // kDetectCap) by (value desc, index asc), over the next power of two; the first
 // max_peaks become peak records. The values are compared as integers: FP64
 // comparisons at 1/64 of the rate took 1.5 us a stage (102 us for any number of
-// candidates, now 39 for about 1000).
+// candidates; for about 1000 of them now 39, and 16 where at most 16 peaks are
+// picked instead).
 template <typename T>
 __global__ void __launch_bounds__(1024) k_detect_sort(const T *__restrict__ v, const int *count, const int64_t *cand,
-                                                      int cap, int max_peaks, GridDev g, DetectPeak *out)
+                                                      int cap, int max_peaks, GridDev g, const GridStep *step,
+                                                      DetectPeak *out)
 {
     __shared__ unsigned long long sv[kDetectCap];
     __shared__ int64_t si[kDetectCap];
@@ -92,6 +94,55 @@ __global__ void __launch_bounds__(1024) k_detect_sort(const T *__restrict__ v, c
         }
     }
     __syncthreads();
+    if (max_peaks <= 16) {
+        // a few peaks are picked one by one: the sort's stages take longer
+        __shared__ unsigned long long wv[32];
+        __shared__ int64_t wi[32];
+        __shared__ int64_t pick[16];
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        for (int r = 0; r < min(n, max_peaks); ++r) {
+            unsigned long long bv = 0ull;
+            int64_t bi = INT64_MAX;
+            for (int t = threadIdx.x; t < n; t += blockDim.x) {
+                const unsigned long long v1 = sv[t];
+                const int64_t i1 = si[t];
+                if (v1 > bv || (v1 == bv && i1 < bi)) {
+                    bv = v1;
+                    bi = i1;
+                }
+            }
+            for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1) {
+                    const unsigned long long v1 = __shfl_xor_sync(0xffffffffu, bv, d);
+                    const int64_t i1 = __shfl_xor_sync(0xffffffffu, bi, d);
+                    if (v1 > bv || (v1 == bv && i1 < bi)) {
+                        bv = v1;
+                        bi = i1;
+                    }
+                }
+                if (pass == 0) {
+                    if (lane == 0) {
+                        wv[warp] = bv;
+                        wi[warp] = bi;
+                    }
+                    __syncthreads();
+                    bv = wv[lane];  // every warp reduces the 32 warps' bests
+                    bi = wi[lane];
+                }
+            }
+            if (threadIdx.x == 0) pick[r] = bi;
+            for (int t = threadIdx.x; t < n; t += blockDim.x)
+                if (si[t] == bi) {
+                    sv[t] = 0ull;  // out of the running
+                    si[t] = INT64_MAX;
+                }
+            __syncthreads();
+        }
+        if (threadIdx.x < min(n, max_peaks)) si[threadIdx.x] = pick[threadIdx.x];
+        __syncthreads();
+        size = 0;  // sorted
+    }
     for (int k = 2; k <= size && size <= cap; k <<= 1)
         for (int jj = k >> 1; jj > 0; jj >>= 1) {
             for (int w = threadIdx.x; w < size / 2; w += blockDim.x) {
@@ -109,7 +160,7 @@ __global__ void __launch_bounds__(1024) k_detect_sort(const T *__restrict__ v, c
             }
             __syncthreads();
         }
-    const GridStep st = grid_step(g);
+    const GridStep st = *step;
     for (int t = threadIdx.x; t < min(n, max_peaks); t += blockDim.x) {
         const int i = g.row0 + (int)(si[t] / g.nlon), j = (int)(si[t] % g.nlon);
         double lat, lon;
@@ -123,8 +174,8 @@ __global__ void __launch_bounds__(1024) k_detect_sort(const T *__restrict__ v, c
     }
 }
 
-cudaError_t launch_detect(const void *v, int prec, const GridDev &g, double thr, int r, int cap, int max_peaks,
-                          int *count, int64_t *cand, DetectPeak *out, cudaStream_t s)
+cudaError_t launch_detect(const void *v, int prec, const GridDev &g, const GridStep *step, double thr, int r, int cap,
+                          int max_peaks, int *count, int64_t *cand, DetectPeak *out, cudaStream_t s)
 {
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
@@ -135,11 +186,11 @@ cudaError_t launch_detect(const void *v, int prec, const GridDev &g, double thr,
     if (prec == DG_PREC_FP64) {
         k_detect_mark<double><<<(unsigned)blocks, 256, 0, s>>>((const double *)v, g.nrows, g.nlon, thr, r, cap, count, cand);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_detect_sort<double><<<1, 1024, 0, s>>>((const double *)v, count, cand, cap, max_peaks, g, out);
+        k_detect_sort<double><<<1, 1024, 0, s>>>((const double *)v, count, cand, cap, max_peaks, g, step, out);
     } else {
         k_detect_mark<float><<<(unsigned)blocks, 256, 0, s>>>((const float *)v, g.nrows, g.nlon, thr, r, cap, count, cand);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_detect_sort<float><<<1, 1024, 0, s>>>((const float *)v, count, cand, cap, max_peaks, g, out);
+        k_detect_sort<float><<<1, 1024, 0, s>>>((const float *)v, count, cand, cap, max_peaks, g, step, out);
     }
     return cudaGetLastError();
 }

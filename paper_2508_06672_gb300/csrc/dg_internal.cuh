@@ -154,17 +154,91 @@ __device__ __forceinline__ dfl df_div_fast(dfl a, dfl b)
 // of a cancelling sum, an error of 1e-9 cycles per sample already shows at
 // 1e-4 in |C|^2. So the range rates r_i . v_i / rho_i and their difference
 // are double-float too, and nu is rounded to FP32 once, at the end.
+//
+// Both receivers run through the same operations, so they share Blackwell's packed
+// FP32 instructions, one in each half: about 260 instructions a node for 520.
+__device__ __forceinline__ float2 pk_fma(float2 a, float2 b, float2 c)
+{
+    unsigned long long r, x, y, z;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(c.x), "f"(c.y));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(r));
+    return d;
+}
+__device__ __forceinline__ float2 pk_add(float2 a, float2 b)
+{
+    unsigned long long r, x, y;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(r));
+    return d;
+}
+__device__ __forceinline__ float2 pk_mul(float2 a, float2 b)
+{
+    unsigned long long r, x, y;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(r));
+    return d;
+}
+// a - b as a + b (-1): one rounding, as the subtraction
+__device__ __forceinline__ float2 pk_sub(float2 a, float2 b) { return pk_fma(b, make_float2(-1.f, -1.f), a); }
+
+struct dfl2 {  // two double-floats
+    float2 hi, lo;
+};
+__device__ __forceinline__ dfl2 df2_fast_two_sum(float2 a, float2 b)
+{
+    const float2 s = pk_add(a, b);
+    return {s, pk_sub(b, pk_sub(s, a))};
+}
+__device__ __forceinline__ dfl2 df2_add_fast(dfl2 a, dfl2 b)
+{
+    const float2 s = pk_add(a.hi, b.hi), bb = pk_sub(s, a.hi);
+    const float2 t = pk_add(pk_sub(a.hi, pk_sub(s, bb)), pk_sub(b.hi, bb));
+    return df2_fast_two_sum(s, pk_add(t, pk_add(a.lo, b.lo)));
+}
+__device__ __forceinline__ dfl2 df2_mul(dfl2 a, dfl2 b)
+{
+    const float2 p = pk_mul(a.hi, b.hi);
+    float2 e = pk_fma(a.hi, b.hi, pk_mul(p, make_float2(-1.f, -1.f)));
+    e = pk_fma(a.hi, b.lo, e);
+    e = pk_fma(a.lo, b.hi, e);
+    return df2_fast_two_sum(p, e);
+}
+__device__ __forceinline__ dfl2 df2_sqrt(dfl2 a)  // as df_sqrt
+{
+    const float2 y = make_float2(sqrtf(a.hi.x), sqrtf(a.hi.y));
+    const float2 r = pk_add(pk_fma(make_float2(-y.x, -y.y), y, a.hi), a.lo);
+    return df2_fast_two_sum(y, make_float2(__fdividef(r.x, 2.f * y.x), __fdividef(r.y, 2.f * y.y)));
+}
+__device__ __forceinline__ dfl2 df2_div_fast(dfl2 a, dfl2 b)  // as df_div_fast
+{
+    const float2 q = make_float2(__fdividef(a.hi.x, b.hi.x), __fdividef(a.hi.y, b.hi.y)), n = make_float2(-q.x, -q.y);
+    const float2 r = pk_add(pk_fma(n, b.hi, a.hi), pk_fma(n, b.lo, a.lo));
+    return df2_fast_two_sum(q, make_float2(__fdividef(r.x, b.hi.x), __fdividef(r.y, b.hi.y)));
+}
+
 __device__ __forceinline__ void geometry_dfl(dfl x, dfl y, dfl z, const dfl *e, dfl fs_over_c, dfl inv_lam_fs,
                                              dfl &D, dfl &nu)
 {
-    const dfl r1x = df_sub_fast(e[0], x), r1y = df_sub_fast(e[1], y), r1z = df_sub_fast(e[2], z);
-    const dfl r2x = df_sub_fast(e[6], x), r2y = df_sub_fast(e[7], y), r2z = df_sub_fast(e[8], z);
-    const dfl rho1 = df_sqrt(df_add_fast(df_add_fast(df_mul(r1x, r1x), df_mul(r1y, r1y)), df_mul(r1z, r1z)));
-    const dfl rho2 = df_sqrt(df_add_fast(df_add_fast(df_mul(r2x, r2x), df_mul(r2y, r2y)), df_mul(r2z, r2z)));
-    D = df_mul(df_sub_fast(rho2, rho1), fs_over_c);
-    const dfl q1 = df_div_fast(df_add_fast(df_add_fast(df_mul(r1x, e[3]), df_mul(r1y, e[4])), df_mul(r1z, e[5])), rho1);
-    const dfl q2 = df_div_fast(df_add_fast(df_add_fast(df_mul(r2x, e[9]), df_mul(r2y, e[10])), df_mul(r2z, e[11])), rho2);
-    nu = df_mul(df_sub_fast(q1, q2), inv_lam_fs);  // (f2 - f1) lambda / (lambda fs)
+    auto both = [](dfl a, dfl b) { return dfl2{make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)}; };
+    auto minus = [](dfl a) { return dfl2{make_float2(-a.hi, -a.hi), make_float2(-a.lo, -a.lo)}; };
+    const dfl2 rx = df2_add_fast(both(e[0], e[6]), minus(x)), ry = df2_add_fast(both(e[1], e[7]), minus(y)),
+               rz = df2_add_fast(both(e[2], e[8]), minus(z));
+    const dfl2 rho = df2_sqrt(df2_add_fast(df2_add_fast(df2_mul(rx, rx), df2_mul(ry, ry)), df2_mul(rz, rz)));
+    D = df_mul(df_sub_fast({rho.hi.y, rho.lo.y}, {rho.hi.x, rho.lo.x}), fs_over_c);
+    const dfl2 q = df2_div_fast(df2_add_fast(df2_add_fast(df2_mul(rx, both(e[3], e[9])), df2_mul(ry, both(e[4], e[10]))),
+                                             df2_mul(rz, both(e[5], e[11]))),
+                                rho);
+    nu = df_mul(df_sub_fast({q.hi.x, q.lo.x}, {q.hi.y, q.lo.y}), inv_lam_fs);  // (f2 - f1) lambda / (lambda fs)
 }
 __device__ __forceinline__ void geometry_df(dfl x, dfl y, dfl z, const dfl *e, dfl fs_over_c, dfl inv_lam_fs,
                                             dfl &D, float &nu)
@@ -583,8 +657,8 @@ struct DetectPeak {
     int i, j;
     double lat_rad, lon_rad, value;
 };
-cudaError_t launch_detect(const void *v, int prec, const GridDev &g, double thr, int r, int cap, int max_peaks,
-                          int *count, int64_t *cand, DetectPeak *out, cudaStream_t s);
+cudaError_t launch_detect(const void *v, int prec, const GridDev &g, const GridStep *step, double thr, int r, int cap,
+                          int max_peaks, int *count, int64_t *cand, DetectPeak *out, cudaStream_t s);
 
 // Argmax record written by launch_argmax.
 struct ArgmaxResult {

@@ -79,21 +79,25 @@ __device__ __forceinline__ VI block_best(VI v)
 // Surface blockIdx.y of n values each (one for a single argmax). The scan
 // compares in the surface's own type: on FP32 values the FP64 comparison
 // would run at 1/64 of the rate.
-template <typename T>
-__global__ void __launch_bounds__(1024) k_argmax_partial(const T *__restrict__ v, int64_t n, VI *part)
+template <typename T> __device__ __forceinline__ VI scan(const T *__restrict__ v, int64_t n, int64_t p, int64_t step)
 {
-    v += n * blockIdx.y;
     T val = (T)0;
     int64_t idx = -1;
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * blockDim.x) {
+    for (; p < n; p += step) {
         const T x = v[p];
         if (x == x && (idx < 0 || x > val)) {  // p increases per thread
             val = x;
             idx = p;
         }
     }
-    const VI best = block_best(VI{(double)val, idx});
+    return VI{(double)val, idx};
+}
+
+template <typename T>
+__global__ void __launch_bounds__(1024) k_argmax_partial(const T *__restrict__ v, int64_t n, VI *part)
+{
+    const VI best = block_best(scan(v + n * blockIdx.y, n, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+                                    (int64_t)gridDim.x * blockDim.x));
     if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = best;
 }
 
@@ -150,6 +154,8 @@ __device__ __forceinline__ void make_fix(const ArgmaxResult *coarse, const Argma
 // The last pass: the record of surface blockIdx.x, its node placed by the
 // grid's stored angular steps (a single thread would need about 5 us for their
 // FP64 sines and divisions), and where fin.fix is given the step's fix record.
+// With nparts = 0 it scans the surface itself: one launch for a few thousand
+// nodes (a refinement grid of 41 x 41: 14 us for the two, 11 for one).
 __global__ void __launch_bounds__(1024) k_argmax_final(const VI *part, int nparts, GridDev g, const GridStep *step,
                                                        ArgmaxResult *res, const ArgmaxResult *centre,
                                                        const void *v, int prec, const GridDev *grids, int64_t n,
@@ -166,6 +172,8 @@ __global__ void __launch_bounds__(1024) k_argmax_final(const VI *part, int npart
     VI best{0.0, -1};
     for (int p = threadIdx.x; p < nparts; p += blockDim.x)
         if (beats(part[p], best)) best = part[p];
+    if (nparts == 0) best = prec == DG_PREC_FP64 ? scan((const double *)v, n, threadIdx.x, blockDim.x)
+                                                 : scan((const float *)v, n, threadIdx.x, blockDim.x);
     best = block_best(best);
     if (threadIdx.x == 0) {
         ArgmaxResult r;
@@ -204,6 +212,10 @@ __global__ void __launch_bounds__(1024) k_argmax_final(const VI *part, int npart
     }
 }
 
+// Nodes that one CTA scans by itself: four loads a thread take less than a second
+// launch (about 5 us).
+constexpr int64_t kArgmaxOne = 4096;
+
 static int argmax_blocks(int64_t n)
 {
     int64_t b = (n + 1023) / 1024;
@@ -218,16 +230,18 @@ cudaError_t launch_argmax(const void *v, int64_t n, int prec, const GridDev &g, 
                           ArgmaxResult *res, int *launches, cudaStream_t s, const ArgmaxResult *centre,
                           const GridDev *grids, int ngrids, FixOut fin)
 {
-    const int nb = argmax_blocks(n);
+    const int nb = n <= kArgmaxOne ? 0 : argmax_blocks(n);
     VI *part = reinterpret_cast<VI *>(tmp);
-    if (prec == DG_PREC_FP64)
-        k_argmax_partial<double><<<dim3(nb, ngrids), 1024, 0, s>>>((const double *)v, n, part);
-    else
-        k_argmax_partial<float><<<dim3(nb, ngrids), 1024, 0, s>>>((const float *)v, n, part);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (nb) {
+        if (prec == DG_PREC_FP64)
+            k_argmax_partial<double><<<dim3(nb, ngrids), 1024, 0, s>>>((const double *)v, n, part);
+        else
+            k_argmax_partial<float><<<dim3(nb, ngrids), 1024, 0, s>>>((const float *)v, n, part);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     k_argmax_final<<<ngrids, 1024, 0, s>>>(part, nb, g, step, res, centre, v, prec, grids, n, fin);
-    if (launches) *launches += 2;
+    if (launches) *launches += nb ? 2 : 1;
     return cudaGetLastError();
 }
 

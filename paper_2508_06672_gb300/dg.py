@@ -69,6 +69,7 @@ EXPORTED_SYMBOLS = [
     "dg_coarse_maps", "dg_coarse_inspect", "dg_set_grid", "dg_search_regions", "dg_fp32_peak",
     "dg_debug_tc_wait_limit", "dg_batch_rounds", "dg_nn_conv3x3_forward_tc", "dg_nn_conv3x3_backward_tc",
     "dg_nn_conv3x3_tc_scratch", "dg_nn_tc_check", "dg_nn_conv3x3_relu_forward_tc",
+    "dg_region_maxima",
 ]
 DG_NOALLOC_SCRATCH_BYTES = 16 * 1024 * 1024
 
@@ -204,6 +205,8 @@ def lib():
             L.dg_noalloc_last_error.argtypes = []
             L.dg_noalloc_last_error.restype = C.c_char_p
             flt = C.c_float
+            L.dg_region_maxima.argtypes = [vp, C.POINTER(dbl), i32]
+            L.dg_region_maxima.restype = C.c_int
             L.dg_search_regions.argtypes = [vp, C.POINTER(dg_grid), i32, vp, dbl, dbl, C.POINTER(dg_fix),
                                             C.POINTER(i32)]
             L.dg_search_regions.restype = C.c_int
@@ -738,6 +741,13 @@ class Geolocator:
         self.grid = {k: getattr(g, k) for k, _ in dg_grid._fields_}
         self.nrows, self.nlon = int(g.nlat), int(g.nlon)
         return fix.as_dict(), best.value, costs
+
+    def region_maxima(self, n):
+        """The largest cost of each of the n regions of the last
+        search_regions (list of float; NaN: no finite value)."""
+        out = (C.c_double * n)()
+        _check(lib().dg_region_maxima(self.ctx, out, n), self.ctx)
+        return list(out)
 
     def coarse_maps(self, bins=0, chunk=0, out=None):
         """Coarse delay-Doppler maps back-projected onto the grid's cells:

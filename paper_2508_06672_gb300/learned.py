@@ -174,16 +174,22 @@ class LearnedSearch:
         n = 2 * self.half + 1
         return min(fix["i"], fix["j"], n - 1 - fix["i"], n - 1 - fix["j"]) < self.edge
 
-    def unsure(self, peaks, costs):
+    def unsure(self, peaks, costs, maxima=None):
         """True when the proposals do not single out a region: the best
         proposal's logit is under ``min_logit``, or the best region's
         maximum cost exceeds the runner-up's by less than ``min_region_gap``
-        of it. ``costs``: the regions' cost surfaces (device)."""
+        of it. ``costs``: the regions' cost surfaces (device); ``maxima``: their
+        largest values, where the caller has them."""
         if self.min_logit is not None and max(p["value"] for p in peaks) < self.min_logit:
             return True
         if self.min_region_gap is not None and len(peaks) > 1:
-            with self.torch.cuda.stream(self.geo.stream):
-                top = self.torch.topk(costs.flatten(1).amax(1), 2).values.tolist()
+            if maxima is not None:
+                if any(v != v for v in maxima):
+                    return False
+                top = sorted(maxima, reverse=True)[:2]
+            else:
+                with self.torch.cuda.stream(self.geo.stream):
+                    top = self.torch.topk(costs.flatten(1).amax(1), 2).values.tolist()
             return top[0] - top[1] < self.min_region_gap * top[0]
         return False
 
@@ -211,7 +217,8 @@ class LearnedSearch:
                 self.cost = self.torch.empty((self.regions, n, n), dtype=self.torch.float32, device=self.geo.device)
             regions = [self.region_grid(p["lat_deg"], p["lon_deg"]) for p in peaks]
             fix, best, costs = self.geo.search_regions(regions, *self.refine, costs=self.cost)
-            if not fallback or not (self.doubtful(fix) or self.unsure(peaks, costs[:len(regions)])):
+            if not fallback or not (self.doubtful(fix) or
+                                    self.unsure(peaks, costs[:len(regions)], self.geo.region_maxima(len(regions)))):
                 return fix, best, peaks
         elif not fallback:
             return None, -1, peaks
