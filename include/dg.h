@@ -542,7 +542,15 @@ dg_status dg_nn_conv3x3_backward(const float *x, const float *w, const float *dy
 dg_status dg_nn_conv3x3_forward_tc(const float *x, const float *w, const float *b, float *y, int32_t B,
                                    int32_t Ci, int32_t Co, int32_t H, int32_t W, float *scratch,
                                    void *stream);
-/* The same with y = max(y, 0): bit for bit dg_nn_relu_forward of its output,
+/* A network's forward pass in one call: layers convolutions as above (weights w[l]
+ * [channels[l + 1]][channels[l]][3][3] and biases b[l], host arrays of device
+ * pointers), relu between them; bit for bit the calls one by one, the weights of
+ * all layers converted in one launch. At most 16 layers; scratch:
+ * dg_nn_forward_tc_scratch floats (device, 16-byte aligned; -1: out of range). */
+int64_t dg_nn_forward_tc_scratch(const int32_t *channels, int32_t layers, int32_t B, int32_t H, int32_t W);
+dg_status dg_nn_forward_tc(const float *x, const float *const *w, const float *const *b, const int32_t *channels,
+                           int32_t layers, float *y, int32_t B, int32_t H, int32_t W, float *scratch, void *stream);
+/* dg_nn_conv3x3_forward_tc with y = max(y, 0): bit for bit dg_nn_relu_forward of its output,
  * without that pass over memory. */
 dg_status dg_nn_conv3x3_relu_forward_tc(const float *x, const float *w, const float *b, float *y, int32_t B,
                                         int32_t Ci, int32_t Co, int32_t H, int32_t W, float *scratch,

@@ -140,21 +140,27 @@ __global__ void __launch_bounds__(256) k_coarse_geo(CoarseArgs a)
     }
 }
 
-__global__ void k_coarse_params(CoarseArgs a)
+// The parameters of snapshot k = blockIdx.y (written by its first CTA), and the
+// chunk DFT's factors: cos and sin of 2 pi d_j o_i M for the offset o_i = (nb - 1)
+// / 2 - i of chunk pair i from the middle and half the distance d_j of bin pair j,
+// two bin pairs a record (see k_caf_fold).
+__global__ void __launch_bounds__(256) k_coarse_params(CoarseArgs a)
 {
-    for (int k = threadIdx.x; k < a.K; k += blockDim.x) {
+    const int k = blockIdx.y, H = a.Dpad / 2;
+    const double lo = undkey(a.nmm[2 * k]), hi = undkey(a.nmm[2 * k + 1]);
+    const double delta = a.Q > 1 ? __ddiv_rn(__dsub_rn(hi, lo), (double)(a.Q - 1)) : 0.0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         const int l0 = a.lmm[2 * k], l1 = a.lmm[2 * k + 1];
         int nlag = (l1 >= l0) ? l1 - l0 + 1 : 0;
         if (nlag < 1 || nlag > a.nlag_cap) {
             atomicOr(a.err, ERR_LAG_RANGE);
             nlag = max(1, min(nlag, a.nlag_cap));
         }
-        const double lo = undkey(a.nmm[2 * k]), hi = undkey(a.nmm[2 * k + 1]);
         CoarseStep s;
         s.l0 = l0;
         s.nlag = nlag;
         s.nu_lo = lo;
-        s.delta = a.Q > 1 ? __ddiv_rn(__dsub_rn(hi, lo), (double)(a.Q - 1)) : 0.0;
+        s.delta = delta;
         s.nu_c = __dmul_rn(0.5, __dadd_rn(lo, hi));
         s.mu = 0.0;
         a.st[k] = s;
@@ -166,15 +172,6 @@ __global__ void k_coarse_params(CoarseArgs a)
             a.snap[k] = m;
         }
     }
-}
-
-// The chunk DFT's factors: cos and sin of 2 pi d_j o_i M for the offset o_i =
-// (nb - 1) / 2 - i of chunk pair i from the middle and half the distance d_j of
-// bin pair j, two bin pairs a record (see k_caf_fold).
-__global__ void __launch_bounds__(256) k_caf_turns(CoarseArgs a)
-{
-    const int k = blockIdx.y, H = a.Dpad / 2;
-    const double delta = a.st[k].delta;
     const int nb = (a.steps[k].n + a.M - 1) / a.M, nh = (nb + 1) / 2;
     for (int64_t it = blockIdx.x * 256 + threadIdx.x; it < (int64_t)nh * H; it += gridDim.x * 256) {
         const int i = (int)(it / H), j = 2 * (int)(it % H);
@@ -283,7 +280,7 @@ __device__ __forceinline__ bool caf_bad(int4 b, int L, int nx)
 //     C = sum cos(2 pi d o M) (P_+ + P_-),   S = sum sin(2 pi d o M) (P_+ - P_-),
 //     Xc(nu_c +- d) = C +- j S,
 // 4 real FMAs for 2 bins x 2 chunks where the complex products take 16. FP32
-// pipe; the factors (k_caf_turns) and the chunk pairs' sums and differences come
+// pipe; the factors (k_coarse_params) and the chunk pairs' sums and differences come
 // from shared memory, two bin pairs per packed FMA. 20 snapshots of 4192 lags,
 // 128 chunks and 40 bins: 254 -> 34 us. A = |Xc|^2, lags fastest, and the CTA's
 // sum of A (in a fixed order). QW of the CTA's warps lie along the bins.
@@ -574,9 +571,7 @@ template <int QW> static cudaError_t launch_fold(const CoarseArgs &a, cudaStream
 cudaError_t launch_coarse(const CoarseArgs &a, const MapArgs *fft, cudaStream_t s, int *launches)
 {
     cudaError_t e;
-    k_coarse_params<<<1, 64, 0, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_caf_turns<<<dim3(blocks_for((int64_t)a.nh_max * a.Dpad / 2, 256, 152 * 8), a.K), 256, 0, s>>>(a);
+    k_coarse_params<<<dim3(blocks_for((int64_t)a.nh_max * a.Dpad / 2, 256, 152 * 8), a.K), 256, 0, s>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (fft) {
         if ((e = launch_chunk_sums(*fft, s, launches)) != cudaSuccess) return e;
@@ -598,7 +593,7 @@ cudaError_t launch_coarse(const CoarseArgs &a, const MapArgs *fft, cudaStream_t 
     k_coarse_backproject<<<dim3(blocks_for(a.nlon - 1, 128, 65535), blocks_for(a.nlat - 1, kBackRows, 65535), a.K), 128, 0,
                            s>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    *launches += 5;
+    *launches += 4;
     return cudaSuccess;
 }
 

@@ -305,7 +305,7 @@ template <int LOGN> __global__ void __launch_bounds__((1 << LOGN) / 16) k_map_sp
 }
 
 template <int LOGN>
-__global__ void __launch_bounds__((1 << LOGN) / 16, LOGN == 14 ? 1 : LOGN == 13 ? 2 : 768 * 16 / (1 << LOGN)) k_map_corr(MapArgs a)
+__global__ void __launch_bounds__((1 << LOGN) / 16, LOGN == 14 ? 1 : LOGN == 13 ? 2 : 1024 * 16 / (1 << LOGN)) k_map_corr(MapArgs a)
 {
     constexpr int n = 1 << LOGN, T = n / 16;
     extern __shared__ __align__(16) float2 sm[];
@@ -1164,7 +1164,7 @@ cudaError_t launch_map_expand(const MapArgs &a, cudaStream_t st)
     // 16 bins per warp where the table is wide enough to fill the chip, 8 otherwise
     if (a.Q >= 128) return launch_expand<16, 1>(a, st);
     if (a.Q > 32) return launch_expand<8, 1>(a, st);
-    return a.Q > 16 ? launch_expand<8, 2>(a, st) : launch_expand<8, 4>(a, st);
+    return a.Q > 16 ? launch_expand<4, 1>(a, st) : launch_expand<4, 2>(a, st);
 }
 
 cudaError_t launch_map_poly(const MapArgs &a, cudaStream_t st)

@@ -250,7 +250,7 @@ __device__ __forceinline__ void nn_bulk_g2s(uint32_t dst, const void *src, uint3
 // NT output channels x 32 input channels in the canonical K-major layout
 // (kmaj), zeros past CO and CI.
 template <bool TR>
-__global__ void k_conv_tc_wimg(const float *__restrict__ w, uint16_t *__restrict__ wimg, int CI, int CO, int NT)
+__device__ __forceinline__ void convert_weights(const float *__restrict__ w, uint16_t *__restrict__ wimg, int CI, int CO, int NT)
 {
     const int ncb = (CI + kHaloCB - 1) / kHaloCB, ob = (CO + NT - 1) / NT;
     const int64_t items = (int64_t)ob * ncb * 9 * NT * (kHaloCB / 8);
@@ -274,6 +274,26 @@ __global__ void k_conv_tc_wimg(const float *__restrict__ w, uint16_t *__restrict
         unsigned char *dst = reinterpret_cast<unsigned char *>(wimg) + (size_t)blk * NT * kHaloCB * 2 + kmaj(ol, kg * 8);
         *reinterpret_cast<uint4 *>(dst) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
     }
+}
+
+template <bool TR>
+__global__ void k_conv_tc_wimg(const float *__restrict__ w, uint16_t *__restrict__ wimg, int CI, int CO, int NT)
+{
+    convert_weights<TR>(w, wimg, CI, CO, NT);
+}
+
+// The forward weights of all layers of a network, layer blockIdx.y: a launch per
+// layer takes 4 us for a microsecond of work.
+constexpr int kNetLayers = 16;
+struct NetWeights {
+    const float *w[kNetLayers];
+    int64_t off[kNetLayers];  // of the layer's blocks in wimg (elements)
+    int CI[kNetLayers], CO[kNetLayers], NT[kNetLayers];
+};
+__global__ void k_net_tc_wimg(NetWeights n, uint16_t *__restrict__ wimg)
+{
+    const int l = blockIdx.y;
+    convert_weights<false>(n.w[l], wimg + n.off[l], n.CI[l], n.CO[l], n.NT[l]);
 }
 
 // Input rows i0 - 1 .. i0 + kHaloRows of channel block cb, pixels j0 - 1 ..
@@ -872,18 +892,14 @@ unsigned *err_word()
     return cudaGetSymbolAddress(&p, g_nn_tc_err) == cudaSuccess ? (unsigned *)p : nullptr;
 }
 
-cudaError_t launch_conv_tc(bool tr, const float *x, const float *w, const float *b, float *y, int B, int CI, int CO,
-                           int H, int W, uint16_t *wimg, cudaStream_t s, int relu = 0)
+// The convolution on converted weights.
+cudaError_t launch_conv_blocks(const float *x, const uint16_t *wimg, const float *b, float *y, int B, int CI, int CO, int H,
+                               int W, cudaStream_t s, int relu)
 {
     unsigned *err = err_word();
     if (!err) return cudaErrorInvalidSymbol;
     const int NT = nt_of(CO);
-    const int64_t items = wimg_elems(CI, CO, NT) / 8;
-    const unsigned gw = (unsigned)std::min<int64_t>((items + 255) / 256, 152 * 8);
-    if (tr) k_conv_tc_wimg<true><<<gw, 256, 0, s>>>(w, wimg, CI, CO, NT);
-    else k_conv_tc_wimg<false><<<gw, 256, 0, s>>>(w, wimg, CI, CO, NT);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     // the whole layer's weights beside at least two staging buffers, or else a
     // ring of 16 slots at most
     const int ob = (CO + NT - 1) / NT, nblk = (CI + kHaloCB - 1) / kHaloCB * 9, wbytes = NT * kHaloCB * 2;
@@ -900,6 +916,37 @@ cudaError_t launch_conv_tc(bool tr, const float *x, const float *w, const float 
     kernel<<<(unsigned)std::min<int64_t>(tiles, 152), kConvThreads, smem, s>>>(x, wimg, b, y, CI, CO, H, W, NT, nh, nw, tiles,
                                                                                relu, err);
     return cudaGetLastError();
+}
+
+cudaError_t launch_conv_tc(bool tr, const float *x, const float *w, const float *b, float *y, int B, int CI, int CO,
+                           int H, int W, uint16_t *wimg, cudaStream_t s, int relu = 0)
+{
+    const int NT = nt_of(CO);
+    const int64_t items = wimg_elems(CI, CO, NT) / 8;
+    const unsigned gw = (unsigned)std::min<int64_t>((items + 255) / 256, 152 * 8);
+    if (tr) k_conv_tc_wimg<true><<<gw, 256, 0, s>>>(w, wimg, CI, CO, NT);
+    else k_conv_tc_wimg<false><<<gw, 256, 0, s>>>(w, wimg, CI, CO, NT);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_conv_blocks(x, wimg, b, y, B, CI, CO, H, W, s, relu);
+}
+
+// Scratch of a whole network (floats): every layer's blocks, then two buffers of
+// the widest hidden layer; off: the layers' blocks (elements). -1: a shape out of
+// range.
+int64_t net_scratch(const int32_t *ch, int L, int B, int H, int W, int64_t *off, int64_t *act)
+{
+    if (!ch || L < 1 || L > kNetLayers) return -1;
+    int64_t e = 0;
+    int wide = 0;
+    for (int l = 0; l < L; ++l) {
+        if (!tc_shape_ok(B, ch[l], ch[l + 1], H, W)) return -1;
+        if (off) off[l] = e;
+        e += (wimg_elems(ch[l], ch[l + 1], nt_of(ch[l + 1])) + 7) / 8 * 8;
+        if (l > 0) wide = std::max(wide, ch[l]);
+    }
+    const int64_t a = ((int64_t)B * wide * H * W + 3) / 4 * 4;
+    if (act) *act = a;
+    return e / 2 + (L > 2 ? 2 : L > 1 ? 1 : 0) * a;
 }
 
 // floats of scratch: the forward's weight blocks, or the backward's (data
@@ -941,6 +988,46 @@ dg_status dg_nn_conv3x3_relu_forward_tc(const float *x, const float *w, const fl
                                         int32_t Co, int32_t H, int32_t W, float *scratch, void *stream)
 {
     return conv_forward_tc("dg_nn_conv3x3_relu_forward_tc", x, w, b, y, B, Ci, Co, H, W, scratch, stream, 1);
+}
+
+int64_t dg_nn_forward_tc_scratch(const int32_t *channels, int32_t layers, int32_t B, int32_t H, int32_t W)
+{
+    return dg::net_scratch(channels, layers, B, H, W, nullptr, nullptr);
+}
+
+dg_status dg_nn_forward_tc(const float *x, const float *const *w, const float *const *b, const int32_t *channels,
+                           int32_t layers, float *y, int32_t B, int32_t H, int32_t W, float *scratch, void *stream)
+{
+    if (!x || !w || !b || !channels || !y || !scratch) return dg::nn_fail(DG_EINVAL, "dg_nn_forward_tc: null pointer");
+    int64_t act = 0;
+    dg::NetWeights n{};
+    if (dg::net_scratch(channels, layers, B, H, W, n.off, &act) < 0)
+        return dg::nn_fail(DG_EINVAL, "dg_nn_forward_tc: bad shape (%d layers, B=%d H=%d W=%d)", layers, B, H, W);
+    if ((reinterpret_cast<uintptr_t>(scratch) & 15) != 0)
+        return dg::nn_fail(DG_EINVAL, "dg_nn_forward_tc: scratch must be 16-byte aligned");
+    int64_t elems = 0, most = 0;
+    for (int l = 0; l < layers; ++l) {
+        if (!w[l] || !b[l]) return dg::nn_fail(DG_EINVAL, "dg_nn_forward_tc: null pointer");
+        n.w[l] = w[l];
+        n.CI[l] = channels[l];
+        n.CO[l] = channels[l + 1];
+        n.NT[l] = dg::nt_of(channels[l + 1]);
+        const int64_t e = dg::wimg_elems(n.CI[l], n.CO[l], n.NT[l]);
+        elems = n.off[l] + (e + 7) / 8 * 8;
+        most = std::max(most, e / 8);
+    }
+    cudaStream_t s = (cudaStream_t)stream;
+    uint16_t *wimg = reinterpret_cast<uint16_t *>(scratch);
+    dg::k_net_tc_wimg<<<dim3((unsigned)std::min<int64_t>((most + 255) / 256, 152 * 8), (unsigned)layers), 256, 0, s>>>(n, wimg);
+    cudaError_t e = cudaGetLastError();
+    float *buf[2] = {scratch + elems / 2, scratch + elems / 2 + act};
+    const float *h = x;
+    for (int l = 0; l < layers && e == cudaSuccess; ++l) {
+        float *z = l + 1 == layers ? y : buf[l & 1];
+        e = dg::launch_conv_blocks(h, wimg + n.off[l], b[l], z, B, channels[l], channels[l + 1], H, W, s, l + 1 < layers);
+        h = z;
+    }
+    return dg::nn_done(e, "dg_nn_forward_tc");
 }
 
 int64_t dg_nn_conv3x3_tc_scratch(int32_t B, int32_t Ci, int32_t Co, int32_t H, int32_t W)

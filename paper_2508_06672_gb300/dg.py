@@ -69,7 +69,7 @@ EXPORTED_SYMBOLS = [
     "dg_coarse_maps", "dg_coarse_inspect", "dg_set_grid", "dg_search_regions", "dg_fp32_peak",
     "dg_debug_tc_wait_limit", "dg_batch_rounds", "dg_nn_conv3x3_forward_tc", "dg_nn_conv3x3_backward_tc",
     "dg_nn_conv3x3_tc_scratch", "dg_nn_tc_check", "dg_nn_conv3x3_relu_forward_tc",
-    "dg_region_maxima",
+    "dg_region_maxima", "dg_nn_forward_tc", "dg_nn_forward_tc_scratch",
 ]
 DG_NOALLOC_SCRATCH_BYTES = 16 * 1024 * 1024
 
@@ -221,6 +221,10 @@ def lib():
             L.dg_nn_conv3x3_scratch.argtypes = [i32, i32, i32, i32, i32]
             L.dg_nn_conv3x3_scratch.restype = i64
             L.dg_nn_conv3x3_forward_tc.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, i32, vp, vp]
+            L.dg_nn_forward_tc_scratch.argtypes = [C.POINTER(i32), i32, i32, i32, i32]
+            L.dg_nn_forward_tc_scratch.restype = i64
+            L.dg_nn_forward_tc.argtypes = [vp, C.POINTER(vp), C.POINTER(vp), C.POINTER(i32), i32, vp, i32, i32, i32, vp, vp]
+            L.dg_nn_forward_tc.restype = C.c_int
             L.dg_nn_conv3x3_relu_forward_tc.argtypes = L.dg_nn_conv3x3_forward_tc.argtypes
             L.dg_nn_conv3x3_backward_tc.argtypes = [vp, vp, vp, vp, vp, vp, i32, i32, i32, i32, i32, vp, vp]
             L.dg_nn_conv3x3_tc_scratch.argtypes = [i32, i32, i32, i32, i32]
@@ -510,6 +514,26 @@ def dg_nn_conv3x3_forward_tc(x, w, b, y, scratch=None, stream=None, relu=False):
         raise ValueError("dg_nn_conv3x3_forward_tc: shape mismatch")
     f = lib().dg_nn_conv3x3_relu_forward_tc if relu else lib().dg_nn_conv3x3_forward_tc
     _nn_check(f(_ptr(x), _ptr(w), _ptr(b), _ptr(y), B, Ci, Co, H, W, _ptr(scratch), _stream(stream, x)))
+
+
+def dg_nn_forward_tc(x, params, stream=None):
+    """The output of a network's convolutions on the tensor cores (params: its
+    layers' (w, b), relu between them) in one call, or None where that call does
+    not take the shape (the layers one by one say why)."""
+    import torch
+    B, _, H, W = x.shape
+    n = len(params)
+    ch = (C.c_int32 * (n + 1))(*([x.shape[1]] + [w.shape[0] for w, _ in params]))
+    need = int(lib().dg_nn_forward_tc_scratch(ch, n, B, H, W))
+    if need < 0 or any(tuple(w.shape) != (ch[k + 1], ch[k], 3, 3) or tuple(b.shape) != (ch[k + 1],)
+                       for k, (w, b) in enumerate(params)):
+        return None
+    y = torch.empty((B, ch[n], H, W), dtype=torch.float32, device=x.device)
+    scratch = torch.empty(max(1, need), dtype=torch.float32, device=x.device)
+    _f32(x, y, scratch, *(t for p in params for t in p))
+    ws, bs = ((C.c_void_p * n)(*(p[k].data_ptr() for p in params)) for k in (0, 1))
+    _nn_check(lib().dg_nn_forward_tc(_ptr(x), ws, bs, ch, n, _ptr(y), B, H, W, _ptr(scratch), _stream(stream, x)))
+    return y
 
 
 def dg_nn_conv3x3_backward_tc(x, w, dy, dx, dw, db, scratch=None, stream=None):

@@ -78,16 +78,17 @@ class ProposalNet:
         """Logits (B, 1, H, W) for x (B, C_in, H, W), float32 CUDA. keep=True
         holds the activations for backward()."""
         torch = self.torch
+        if self.tc and not keep:
+            h = dg.dg_nn_forward_tc(x, self.params)
+            if h is not None:
+                self._acts = None
+                return h
         B, _, H, W = x.shape
         acts = [x]
         h = x
         L = len(self.params)
         for k, (w, b) in enumerate(self.params):
             z = torch.empty((B, w.shape[0], H, W), dtype=torch.float32, device=x.device)
-            if self.tc and not keep and k < L - 1:  # nothing needs the values before the relu
-                dg.dg_nn_conv3x3_forward_tc(h, w, b, z, relu=True)
-                h = z
-                continue
             (dg.dg_nn_conv3x3_forward_tc if self.tc else dg.dg_nn_conv3x3_forward)(h, w, b, z)
             if k < L - 1:
                 hk = torch.empty_like(z) if keep else z

@@ -47,3 +47,23 @@ def test_conv_tc_over_the_tile_schedule(shape):
     lim = 9 * Ci * 2.0 ** -22 * conv(x.abs(), w.abs()) + 2.0 ** -23 * ref.abs() + 1e-30
     assert bool(((y.double() - ref).abs() <= lim).all())
     assert torch.equal(z, h)
+
+
+@pytest.mark.parametrize("channels,shape", [([3, 1], (2, 9, 40)), ([20, 32, 1], (1, 33, 130)),
+                                            ([5, 40, 130, 24, 1], (2, 7, 129))])
+def test_network_in_one_call_is_its_layers_one_by_one(channels, shape):
+    from paper_2508_06672_gb300.proposal import ProposalNet
+    P = package()
+    torch = torch_cuda()
+    net = ProposalNet(channels, seed=4, tc=True)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    x = torch.randn(shape[0], channels[0], *shape[1:], generator=g, device="cuda")
+    h = x
+    for k, (w, b) in enumerate(net.params):
+        z = torch.empty((shape[0], channels[k + 1], *shape[1:]), device="cuda")
+        P.dg_nn_conv3x3_forward_tc(h, w, b, z, relu=k + 1 < len(net.params))
+        h = z
+    y = net.forward(x)
+    P.dg_nn_tc_check()
+    assert torch.equal(y, h)
+    assert torch.equal(net.forward(x, keep=True), h)
