@@ -370,7 +370,8 @@ static dg_status map_plan(dg_ctx *c);
 static dg_status run_surface_map(dg_ctx *c, void *out);
 static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *surf, void *out,
                                  bool refine, bool *done);
-static dg_status refine_map(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *out, bool *done);
+static dg_status refine_map(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *out, bool *done,
+                            const GridDev *mains, int nmains);
 
 // Surfaces whose candidates look their correlations up in delay-Doppler maps
 // (dg_map.cu) instead of the per-lag DFT rows of the contraction: the main
@@ -395,7 +396,7 @@ dg_status run_surface(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G
     }
     if (refine && map_options(c)) {
         bool done = false;
-        if ((st = refine_map(c, gd, xyz, G, out, &done)) != DG_OK || done) return st;
+        if ((st = refine_map(c, gd, xyz, G, out, &done, &c->gd, 1)) != DG_OK || done) return st;
     }
     if (c->opt.algo == DG_ALGO_CDFT) return run_surface_cdft(c, gd, xyz, G, surf, out, refine);
     if (c->opt.prec == DG_PREC_FP32 && c->opt.delay == DG_DELAY_INTEGER) {
@@ -1586,11 +1587,10 @@ static dg_status run_surface_map(dg_ctx *c, void *out)
 struct RefineBound {
     double rho = 1e300, sep = 0.0, vel = 0.0, dv = 0.0;
 };
-static RefineBound refine_bound(const dg_ctx *c)
+static RefineBound refine_bound(const dg_ctx *c, const GridDev &g)
 {
     for (int side : {3, 17}) {
         RefineBound b;
-        const GridDev &g = c->gd;
         const int ni = std::min(side, g.nrows), nj = std::min(side, g.nlon);
         std::vector<double> p(3 * (size_t)ni * nj);
         for (int i = 0; i < ni; ++i)
@@ -1624,9 +1624,11 @@ static RefineBound refine_bound(const dg_ctx *c)
 }
 
 // A refinement surface from a table of few lags (k_map_few), planned from the
-// grid's shape and bounds that hold anywhere on the main grid (its centre is
-// known on the device only). *done = false where the shape does not suit it.
-static dg_status refine_map(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *out, bool *done)
+// grid's shape and bounds that hold anywhere on the main grids (its centre, a node
+// of one of them, is known on the device only). *done = false where the shape does
+// not suit it.
+static dg_status refine_map(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *out, bool *done,
+                            const GridDev *mains, int nmains)
 {
     *done = false;
     if (!(gd.nlat & 1) || gd.nlat != gd.nlon || gd.nrows != gd.nlat) return DG_OK;  // the centre is a node
@@ -1637,10 +1639,16 @@ static dg_status refine_map(dg_ctx *c, const GridDev &gd, const double *xyz, int
         nmax = std::max(nmax, (int)c->steps[k].n);
         c64 |= c->steps[k].fmt == DG_IQ_C64;
     }
-    const RefineBound rb = refine_bound(c);
     // the farthest node: half a diagonal of the lattice in metres, with 2 % for
     // the parallels' change of radius over up to 20 km at 80 degrees
-    if (std::fabs(c->gd.lat0_rad) + 0.5 * c->gd.nlat * c->gd.dlat_m / 6.33e6 > 1.39) return DG_OK;
+    RefineBound rb;
+    for (int i = 0; i < nmains; ++i) {
+        if (std::fabs(mains[i].lat0_rad) + 0.5 * mains[i].nlat * mains[i].dlat_m / 6.33e6 > 1.39) return DG_OK;
+        const RefineBound q = refine_bound(c, mains[i]);
+        const double rho = std::min(rb.rho, q.rho);
+        rb = q;
+        rb.rho = rho;
+    }
     const double half = (gd.nlat - 1) / 2, r = 1.02 * half * std::hypot(gd.dlat_m, gd.dlon_m);
     const double rho = rb.rho - r;
     if (!(rho > 0.0) || r > 2e4) return DG_OK;
@@ -2083,6 +2091,7 @@ static dg_status ensure_post(dg_ctx *c, int half, dg_fix **fix_dev, dg_fix **fix
 static dg_status step_device_post(dg_ctx *c, const void *cost, double spacing_m, int half, dg_fix *fix_dev,
                                   dg_fix *fix_host, const ArgmaxResult *known);
 static dg_status read_fix(dg_ctx *c, const dg_fix *fix_host, dg_fix *out);
+static dg_status copy_fix(dg_ctx *c, const dg_fix *fix_host, dg_fix *out);
 
 static dg_status argmax_refine(dg_ctx *c, const void *cost, double spacing_m, double window_m, dg_fix *out,
                                const ArgmaxResult *known)
@@ -2260,8 +2269,13 @@ static dg_status step_device_post(dg_ctx *c, const void *cost, double spacing_m,
 static dg_status read_fix(dg_ctx *c, const dg_fix *fix_host, dg_fix *out)
 {
     CK(c, cudaStreamSynchronize(c->stream));
-    dg_status st = check_latched(c);
-    if (st != DG_OK) return st;
+    const dg_status st = check_latched(c);
+    return st != DG_OK ? st : copy_fix(c, fix_host, out);
+}
+
+// The fix of a step that has been waited for.
+static dg_status copy_fix(dg_ctx *c, const dg_fix *fix_host, dg_fix *out)
+{
     if (fix_host->index < 0) return fail(c, DG_EINVAL, "the surface holds no finite value");
     if (fix_host->refine_n > 0 && fix_host->ri < 0)
         return fail(c, DG_EINVAL, "the refinement surface holds no finite value");
@@ -3326,6 +3340,41 @@ static dg_status regions_map(dg_ctx *c, const dg_grid *regions, int n, float *co
     return DG_OK;
 }
 
+// The refinement around the best of n regions, whose records are on the device, up
+// to its fix in fix_host_sync, with nothing read by the host in between. *done =
+// false (and nothing kept) where refine_map does not serve it.
+static dg_status refine_best(dg_ctx *c, const dg_grid *regions, int n, double spacing_m, int half, bool *done)
+{
+    *done = false;
+    if (half == 0 || !map_options(c)) return DG_OK;
+    std::vector<GridDev> mains((size_t)n);
+    for (int r = 0; r < n; ++r) mains[(size_t)r] = make_griddev(regions[r], 0, regions[r].nlat);
+    dg_status st = ensure_post(c, half, &c->fix_dev_sync, &c->fix_host_sync);
+    if (st != DG_OK) return st;
+    const int side = 2 * half + 1;
+    dg_grid lg = regions[0];  // the centre is replaced on the device
+    lg.dlat_m = lg.dlon_m = spacing_m;
+    lg.nlat = lg.nlon = side;
+    const GridDev lgd = make_griddev(lg, 0, side);
+    const int64_t Gl = (int64_t)side * side;
+    {
+        Timed t(c, DG_K_REFINE);
+        CK(c, launch_best_record(c->reg_res, n, c->amax_res, c->stream));
+        CK(c, launch_grid_ecef(lgd, c->loc.xyz, c->stream, c->amax_res, nullptr, 1, c->gstep + 1));
+        t.done(2);
+    }
+    if ((st = refine_map(c, lgd, c->loc.xyz, Gl, c->loc.cost, done, mains.data(), n)) != DG_OK || !*done) return st;
+    {
+        Timed t(c, DG_K_ARGMAX);
+        int nl = 0;
+        CK(c, launch_argmax(c->loc.cost, Gl, c->opt.prec, lgd, c->gstep + 1, c->amax_tmp, c->amax_fine, &nl, c->stream,
+                            c->amax_res, nullptr, 1, FixOut{c->fix_dev_sync, c->amax_res, mains[0], side}));
+        t.done(nl);
+    }
+    CK(c, cudaMemcpyAsync(c->fix_host_sync, c->fix_dev_sync, sizeof(dg_fix), cudaMemcpyDeviceToHost, c->stream));
+    return DG_OK;
+}
+
 dg_status dg_search_regions(dg_ctx *c, const dg_grid *regions, int32_t n, void *costs, double spacing_m,
                             double window_m, dg_fix *out, int32_t *best)
 {
@@ -3374,6 +3423,11 @@ dg_status dg_search_regions(dg_ctx *c, const dg_grid *regions, int32_t n, void *
         }
     }
     CK(c, cudaMemcpyAsync(c->reg_host, c->reg_res, sizeof(ArgmaxResult) * n, cudaMemcpyDeviceToHost, c->stream));
+    int half = 0;
+    bool refined = false;
+    if (done && refine_half(c, spacing_m, window_m, &half) == DG_OK &&
+        (st = refine_best(c, regions, n, spacing_m, half, &refined)) != DG_OK)
+        return st;
     CK(c, cudaStreamSynchronize(c->stream));
     if ((st = check_latched(c)) != DG_OK) return st;
     c->reg_n = n;
@@ -3384,6 +3438,11 @@ dg_status dg_search_regions(dg_ctx *c, const dg_grid *regions, int32_t n, void *
     // the best region becomes the context's grid; its nodes are there already
     if ((st = set_grid(c, &regions[b], nodes ? c->reg_xyz + 3 * G * b : nullptr, nodes ? c->reg_steps + b : nullptr)) != DG_OK)
         return st;
+    if (refined) {
+        if ((st = copy_fix(c, c->fix_host_sync, out)) != DG_OK) return st;
+        if (best) *best = b;
+        return DG_OK;
+    }
     if ((st = argmax_refine(c, (char *)costs + esz * (size_t)G * b, spacing_m, window_m, out, c->reg_res + b)) != DG_OK)
         return st;
     if (best) *best = b;

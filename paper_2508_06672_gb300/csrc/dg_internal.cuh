@@ -681,6 +681,8 @@ __device__ __forceinline__ void centre_on(GridDev &g, const ArgmaxResult *c)
     g.lon0_rad = (c->lon_rad * (180.0 / kPi)) * (kPi / 180.0);
 }
 
+cudaError_t launch_best_record(const ArgmaxResult *r, int n, ArgmaxResult *out, cudaStream_t s);
+
 // Where the last argmax of a step writes the fix of the step (NULL: no fix):
 // with coarse, the record is the refinement's (side n) and coarse the main
 // surface's over grid g; without, the record is the main surface's.

@@ -212,6 +212,38 @@ __global__ void __launch_bounds__(1024) k_argmax_final(const VI *part, int npart
     }
 }
 
+// The best of n records: the largest value, the first of equal ones (index -1:
+// none has a value).
+__global__ void k_best_record(const ArgmaxResult *__restrict__ r, int n, ArgmaxResult *__restrict__ out)
+{
+    int b = -1;
+    double v = 0.0;
+    for (int i = threadIdx.x; i < n; i += 32)
+        if (r[i].idx >= 0 && (b < 0 || r[i].val > v)) {
+            b = i;
+            v = r[i].val;
+        }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        const int ob = __shfl_xor_sync(0xffffffffu, b, d);
+        const double ov = __shfl_xor_sync(0xffffffffu, v, d);
+        if (ob >= 0 && (b < 0 || ov > v || (ov == v && ob < b))) {
+            b = ob;
+            v = ov;
+        }
+    }
+    if (threadIdx.x == 0) {
+        *out = r[max(b, 0)];
+        if (b < 0) out->idx = -1;
+    }
+}
+
+cudaError_t launch_best_record(const ArgmaxResult *r, int n, ArgmaxResult *out, cudaStream_t s)
+{
+    k_best_record<<<1, 32, 0, s>>>(r, n, out);
+    return cudaGetLastError();
+}
+
 // Nodes that one CTA scans by itself: four loads a thread take less than a second
 // launch (about 5 us).
 constexpr int64_t kArgmaxOne = 4096;
