@@ -10,7 +10,7 @@
 namespace dg {
 
 // A node that its eight neighbours do not rule out (few are left) has its window
-// searched by the whole warp, a row of it at a time: a lane on its own walks (2r +
+// searched by the whole warp, two to four rows at a time: a lane on its own walks (2r +
 // 1)^2 dependent loads while the others wait (512^2 nodes, r = 7: 50 -> 15 us).
 template <typename T>
 __global__ void __launch_bounds__(256) k_detect_mark(const T *__restrict__ v, int nrows, int nlon, double thr, int r,
@@ -40,14 +40,21 @@ __global__ void __launch_bounds__(256) k_detect_mark(const T *__restrict__ v, in
             const int64_t pc = __shfl_sync(0xffffffffu, p, src);
             const T xc = __shfl_sync(0xffffffffu, x, src);
             const int ic = __shfl_sync(0xffffffffu, i, src), jc = __shfl_sync(0xffffffffu, j, src);
-            const int jhi = (int)min((int64_t)nlon - 1, (int64_t)jc + r), ihi = (int)min((int64_t)nrows - 1, (int64_t)ic + r);
+            // windows of at most 16 columns take two rows at a time
+            const int jlo = max(0, jc - r), jhi = (int)min((int64_t)nlon - 1, (int64_t)jc + r);
+            const int ihi = (int)min((int64_t)nrows - 1, (int64_t)ic + r), two = r <= 7 ? 1 : 0;
             bool beaten = false;
-            for (int ii = max(0, ic - r); ii <= ihi && !beaten; ++ii) {
-                const T *row = v + (int64_t)ii * nlon;
+            for (int i0 = max(0, ic - r); i0 <= ihi && !beaten; i0 += 2 << two) {
                 bool b = false;
-                for (int jj = max(0, jc - r) + lane; jj <= jhi; jj += 32) {
-                    const T y = row[jj];
-                    b = b || y > xc || (y == xc && (int64_t)ii * nlon + jj < pc);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int ii = two ? i0 + 2 * u + (lane >> 4) : i0 + u;
+                    if (ii > ihi) continue;
+                    const T *row = v + (int64_t)ii * nlon;
+                    for (int jj = jlo + (two ? lane & 15 : lane); jj <= jhi; jj += 32) {
+                        const T y = row[jj];
+                        b = b || y > xc || (y == xc && (int64_t)ii * nlon + jj < pc);
+                    }
                 }
                 beaten = __any_sync(0xffffffffu, b);
             }

@@ -441,7 +441,7 @@ constexpr int kExpWarps = 8;
 // narrow tables (few bins) take more lags per CTA. U and the phases are staged
 // kExpRows (block, node) rows at a time, so a stage's barrier is paid once for
 // several blocks where a block has few nodes.
-constexpr int kExpRows = 24;
+constexpr int kExpRows = 48;
 template <int NQ, int LW> __global__ void __launch_bounds__(32 * kExpWarps) k_map_expand(MapArgs a)
 {
     constexpr int QW = kExpWarps / LW, NB = NQ * QW, H = NQ / 2, T = 32 * kExpWarps, NLC = 32 * LW;

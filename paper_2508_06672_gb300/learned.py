@@ -168,6 +168,22 @@ class LearnedSearch:
         n = 2 * self.half + 1
         return dict(lat0_deg=lat, lon0_deg=lon, dlat_m=step_lat / dlat, dlon_m=step_lon / dlon, nlat=n, nlon=n)
 
+    def region_grids(self, peaks):
+        """region_grid of each peak, as dg_grid records; the full grid's own
+        numbers are taken once for all of them."""
+        g = self.grid
+        lat0, lon0, nlat, nlon = float(g["lat0_deg"]), float(g["lon0_deg"]), int(g["nlat"]), int(g["nlon"])
+        dlat0, dlon0 = degrees_per_metre(lat0)
+        step_lat, step_lon = dlat0 * float(g["dlat_m"]), dlon0 * float(g["dlon_m"])
+        n, mi, mj, out = 2 * self.half + 1, 0.5 * (nlat - 1), 0.5 * (nlon - 1), []
+        for p in peaks:
+            i = min(max(int(round((p["lat_deg"] - lat0) / step_lat + mi)), 0), nlat - 1)
+            j = min(max(int(round((p["lon_deg"] - lon0) / step_lon + mj)), 0), nlon - 1)
+            lat = lat0 + (i - mi) * step_lat
+            dlat, dlon = degrees_per_metre(lat)
+            out.append(dg.dg_grid(lat, lon0 + (j - mj) * step_lon, step_lat / dlat, step_lon / dlon, n, n))
+        return out
+
     def doubtful(self, fix):
         """True when a region's fix cannot be trusted: its argmax lies within
         ``edge`` nodes of the region's border."""
@@ -215,7 +231,7 @@ class LearnedSearch:
             n = 2 * self.half + 1
             if self.cost is None:
                 self.cost = self.torch.empty((self.regions, n, n), dtype=self.torch.float32, device=self.geo.device)
-            regions = [self.region_grid(p["lat_deg"], p["lon_deg"]) for p in peaks]
+            regions = self.region_grids(peaks)
             fix, best, costs = self.geo.search_regions(regions, *self.refine, costs=self.cost)
             if not fallback or not (self.doubtful(fix) or
                                     self.unsure(peaks, costs[:len(regions)], self.geo.region_maxima(len(regions)))):
