@@ -439,9 +439,9 @@ constexpr int kExpWarps = 8;
 
 // LW of the CTA's warps lie along the lags (32 each), 8 / LW along the bins:
 // narrow tables (few bins) take more lags per CTA. U and the phases are staged
-// kExpRows (block, node) rows at a time, so a stage's barrier is paid once for
+// exp_rows (block, node) rows at a time, so a stage's barrier is paid once for
 // several blocks where a block has few nodes.
-constexpr int kExpRows = 48;
+__host__ __device__ constexpr int exp_rows(int NQ) { return NQ >= 16 ? 96 : 48; }
 template <int NQ, int LW> __global__ void __launch_bounds__(32 * kExpWarps) k_map_expand(MapArgs a)
 {
     constexpr int QW = kExpWarps / LW, NB = NQ * QW, H = NQ / 2, T = 32 * kExpWarps, NLC = 32 * LW;
@@ -449,7 +449,7 @@ template <int NQ, int LW> __global__ void __launch_bounds__(32 * kExpWarps) k_ma
     const int s = blockIdx.z, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const StepDesc sd = a.sd[s % a.ksd];
     const MapSnap ms = a.snap[s];
-    const int qb = blockIdx.y * NB, P = a.P, CS = max(1, kExpRows / P);  // blocks per stage
+    const int qb = blockIdx.y * NB, P = a.P, CS = max(1, exp_rows(NQ) / P);  // blocks per stage
     const int l0 = blockIdx.x * NLC;
     if (l0 >= ms.NL) return;
     float *sT = sm_f;                                              // [P][NB]
@@ -1150,7 +1150,7 @@ cudaError_t launch_chunk_sums(const MapArgs &a, cudaStream_t st, int *launches)
 template <int NQ, int LW> static cudaError_t launch_expand(const MapArgs &a, cudaStream_t st)
 {
     constexpr int NB = NQ * kExpWarps / LW, NLC = 32 * LW;
-    const int CS = a.P < kExpRows ? kExpRows / a.P : 1;
+    const int CS = a.P < exp_rows(NQ) ? exp_rows(NQ) / a.P : 1;
     const size_t smem = sizeof(float) * (size_t)a.P * NB + sizeof(float2) * 3 * (size_t)CS * (NB + a.P * NLC);
     const cudaError_t e = cudaFuncSetAttribute(k_map_expand<NQ, LW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
