@@ -290,9 +290,23 @@ struct NetWeights {
     int64_t off[kNetLayers];  // of the layer's blocks in wimg (elements)
     int CI[kNetLayers], CO[kNetLayers], NT[kNetLayers];
 };
-__global__ void k_net_tc_wimg(NetWeights n, uint16_t *__restrict__ wimg)
+// With planes > 0 the last rows of blocks zero the borders of the BF16 tensors: that
+// many planes of (H + 2) x (W + 2) 16-byte pixels from act on.
+__global__ void k_net_tc_wimg(NetWeights n, uint16_t *__restrict__ wimg, int layers, uint4 *__restrict__ act, int64_t planes,
+                              int H, int W)
 {
     const int l = blockIdx.y;
+    if (l == layers) {
+        const int64_t ring = 2 * (int64_t)(W + 2) + 2 * (int64_t)H;
+        for (int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; it < planes * ring;
+             it += (int64_t)gridDim.x * blockDim.x) {
+            const int64_t p = it / ring, r = it % ring;
+            const int64_t px = r < W + 2 ? r : r < 2 * (W + 2) ? (int64_t)(H + 1) * (W + 2) + r - (W + 2)
+                               : ((r - 2 * (W + 2)) / 2 + 1) * (W + 2) + ((r & 1) ? W + 1 : 0);
+            act[p * (int64_t)(H + 2) * (W + 2) + px] = make_uint4(0, 0, 0, 0);
+        }
+        return;
+    }
     convert_weights<false>(n.w[l], wimg + n.off[l], n.CI[l], n.CO[l], n.NT[l]);
 }
 
@@ -346,10 +360,18 @@ __device__ __forceinline__ void stage_halo(unsigned char *hb, const float *__res
 // nh staging buffers and nw weight slots (nw = all of the layer's blocks when
 // they are resident; then there is one block of output channels). relu: write
 // max(y, 0).
-template <bool WIDE>
+//
+// Between the layers of one call (dg_nn_forward_tc) the activations wait as the
+// BF16 values the products take, already rounded as the staging rounds them (the
+// same results bit for bit), in the staging's own layout: IN16 / OUT16 tensors are
+// [image][channels / 8][H + 2][W + 2][8] with a border of zeros, channels a
+// multiple of 32. A staged row is then one bulk copy of consecutive bytes, and an
+// output pixel's 32 channels are four 16-byte stores: no conversion, half the bytes
+// and no registers on the way in (network at 512 x 512: 238 -> 145 us).
+template <bool WIDE, bool IN16, bool OUT16>
 __global__ void __launch_bounds__(kConvThreads, 1)
-    k_conv3x3_tc(const float *__restrict__ x, const uint16_t *__restrict__ wimg, const float *__restrict__ b,
-                 float *__restrict__ y, int CI, int CO, int H, int W, int NT, int nh, int nw, int64_t tiles, int relu,
+    k_conv3x3_tc(const void *__restrict__ xv, const uint16_t *__restrict__ wimg, const float *__restrict__ b,
+                 void *__restrict__ yv, int CI, int CO, int H, int W, int NT, int nh, int nw, int64_t tiles, int relu,
                  unsigned *err)
 {
     extern __shared__ __align__(1024) unsigned char nsm[];
@@ -368,6 +390,9 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     struct Tile {
         int n, obi, i0, j0;
     };
+    const float *x = reinterpret_cast<const float *>(xv);
+    float *y = reinterpret_cast<float *>(yv);
+    const int64_t plane = (int64_t)(H + 2) * (W + 2) * 16;  // bytes of 8 channels of a BF16 tensor
     auto tile_of = [&](int64_t v) {
         Tile o;
         o.j0 = (int)(v % tx) * kRowsTc;
@@ -384,7 +409,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
             nn_mbar_init(smem_addr(&wempty[k]), 1);
         }
         for (int k = 0; k < nh; ++k) {
-            nn_mbar_init(smem_addr(&hfull[k]), kProdWarps);
+            nn_mbar_init(smem_addr(&hfull[k]), IN16 ? 1 : kProdWarps);
             nn_mbar_init(smem_addr(&hempty[k]), 1);
         }
         for (int k = 0; k < 2; ++k) {
@@ -400,8 +425,37 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     nn_after_sync();
     const uint32_t tmem = tslot;
     bool ok = true;
-    int64_t copied = 0;  // weight blocks whose copy this thread has issued
-    if (warp < kProdWarps) {
+    int64_t copied = 0;  // weight blocks (or BF16 input stages) whose copies this thread has issued
+    if (IN16 && warp < kProdWarps) {
+        if (warp == 0) {
+            int s = 0;
+            uint32_t ph = 1;
+            for (int64_t v = blockIdx.x; v < tiles && ok; v += gridDim.x) {
+                const Tile o = tile_of(v);
+                const int rows = min(kHaloRows + 2, H + 2 - o.i0);  // those of the bordered image
+                const uint32_t len = (uint32_t)min(kHaloQ, W + 2 - o.j0) * 16;
+                const int rr = lane / (kHaloCB / 8), g = lane % (kHaloCB / 8);
+                const char *src = reinterpret_cast<const char *>(xv) + (int64_t)o.n * (CI / 8) * plane + (int64_t)g * plane +
+                                  ((int64_t)(o.i0 + rr) * (W + 2) + o.j0) * 16;
+                for (int cb = 0; cb < ncb; ++cb, src += (kHaloCB / 8) * plane) {
+                    ok = __all_sync(0xffffffffu, nn_wait(smem_addr(&hempty[s]), ph));
+                    if (!ok) break;
+                    if (lane == 0) {
+                        nn_expect_tx(smem_addr(&hfull[s]), (uint32_t)(rows * (kHaloCB / 8)) * len);
+                        ++copied;
+                    }
+                    __syncwarp();
+                    if (rr < rows)
+                        nn_bulk_g2s(smem_addr(nsm + (size_t)s * kHaloBytes + (size_t)lane * kHaloQ * 16), src, len,
+                                    smem_addr(&hfull[s]));
+                    if (++s == nh) {
+                        s = 0;
+                        ph ^= 1;
+                    }
+                }
+            }
+        }
+    } else if (warp < kProdWarps) {
         int s = 0;
         uint32_t ph = 1;  // parity of the buffer's last release; a fresh barrier passes parity 1
         for (int64_t v = blockIdx.x; v < tiles && ok; v += gridDim.x) {
@@ -449,7 +503,20 @@ __global__ void __launch_bounds__(kConvThreads, 1)
                     const float val = __uint_as_float(rv[e]) + __shfl_sync(0xffffffffu, bl, e);
                     rv[e] = __float_as_uint(relu ? fmaxf(val, 0.f) : val);
                 }
-                if (i < H && jp < W) {
+                if (OUT16) {
+                    if (i < H && jp < W) {
+                        char *dst = reinterpret_cast<char *>(yv) + ((int64_t)o.n * (CO / 8) + (o0 + c0) / 8) * plane +
+                                    ((int64_t)(i + 1) * (W + 2) + jp + 1) * 16;
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {
+                            uint32_t pk[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                pk[e] = bf16_pair(__uint_as_float(rv[8 * g + 2 * e]), __uint_as_float(rv[8 * g + 2 * e + 1]));
+                            if (8 * g < nc) *reinterpret_cast<uint4 *>(dst + g * plane) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                        }
+                    }
+                } else if (i < H && jp < W) {
                     char *dst = reinterpret_cast<char *>(yn + (int64_t)(o0 + c0) * HW);
                     const int64_t off = WIDE ? 4 * ((int64_t)i * W + jp) : (int64_t)o32;
                     if (nc == 32) {
@@ -543,6 +610,9 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     __syncwarp();
     // before tensor memory and shared memory are released the MMAs and copies
     // issued have landed, also where a wait gave up
+    if (IN16 && t == 0)
+        for (int64_t g = copied > nh ? copied - nh : 0; g < copied; ++g)
+            ok = nn_wait(smem_addr(&hfull[g % nh]), (uint32_t)(g / nh) & 1u) && ok;
     if (t == 32 * (kProdWarps + kOutWarps))
         for (int64_t g = copied > nw ? copied - nw : 0; g < copied; ++g)
             ok = nn_wait(smem_addr(&wfull[g % nw]), (uint32_t)(g / nw) & 1u) && ok;
@@ -893,8 +963,8 @@ unsigned *err_word()
 }
 
 // The convolution on converted weights.
-cudaError_t launch_conv_blocks(const float *x, const uint16_t *wimg, const float *b, float *y, int B, int CI, int CO, int H,
-                               int W, cudaStream_t s, int relu)
+cudaError_t launch_conv_blocks(const void *x, const uint16_t *wimg, const float *b, void *y, int B, int CI, int CO, int H,
+                               int W, cudaStream_t s, int relu, bool in16 = false, bool out16 = false)
 {
     unsigned *err = err_word();
     if (!err) return cudaErrorInvalidSymbol;
@@ -909,7 +979,10 @@ cudaError_t launch_conv_blocks(const float *x, const uint16_t *wimg, const float
     const int smem = nh * kHaloBytes + nw * wbytes;
     // 32 planes and a row of pixels each, in bytes, against the 32-bit offsets
     const bool wide = 4.0 * (kHaloCB * (double)H * W + 8.0 * W + 4096.0) > 4294967295.0;
-    auto kernel = wide ? k_conv3x3_tc<true> : k_conv3x3_tc<false>;
+    auto kernel = in16 ? (out16 ? (wide ? k_conv3x3_tc<true, true, true> : k_conv3x3_tc<false, true, true>)
+                                : (wide ? k_conv3x3_tc<true, true, false> : k_conv3x3_tc<false, true, false>))
+                       : (out16 ? (wide ? k_conv3x3_tc<true, false, true> : k_conv3x3_tc<false, false, true>)
+                                : (wide ? k_conv3x3_tc<true, false, false> : k_conv3x3_tc<false, false, false>));
     if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
         return e;
     const int64_t tiles = (int64_t)((W + kRowsTc - 1) / kRowsTc) * ((H + kHaloRows - 1) / kHaloRows) * B * ob;
@@ -930,9 +1003,17 @@ cudaError_t launch_conv_tc(bool tr, const float *x, const float *w, const float 
     return e != cudaSuccess ? e : launch_conv_blocks(x, wimg, b, y, B, CI, CO, H, W, s, relu);
 }
 
+// Whether a network's hidden layers wait as BF16 tensors (k_conv3x3_tc).
+bool net16(const int32_t *ch, int L)
+{
+    for (int l = 1; l < L; ++l)
+        if (ch[l] % kHaloCB) return false;
+    return L > 1;
+}
+
 // Scratch of a whole network (floats): every layer's blocks, then two buffers of
-// the widest hidden layer; off: the layers' blocks (elements). -1: a shape out of
-// range.
+// the widest hidden layer (act floats each); off: the layers' blocks (elements). -1:
+// a shape out of range.
 int64_t net_scratch(const int32_t *ch, int L, int B, int H, int W, int64_t *off, int64_t *act)
 {
     if (!ch || L < 1 || L > kNetLayers) return -1;
@@ -944,7 +1025,7 @@ int64_t net_scratch(const int32_t *ch, int L, int B, int H, int W, int64_t *off,
         e += (wimg_elems(ch[l], ch[l + 1], nt_of(ch[l + 1])) + 7) / 8 * 8;
         if (l > 0) wide = std::max(wide, ch[l]);
     }
-    const int64_t a = ((int64_t)B * wide * H * W + 3) / 4 * 4;
+    const int64_t a = net16(ch, L) ? (int64_t)B * (wide / 8) * (H + 2) * (W + 2) * 4 : ((int64_t)B * wide * H * W + 3) / 4 * 4;
     if (act) *act = a;
     return e / 2 + (L > 2 ? 2 : L > 1 ? 1 : 0) * a;
 }
@@ -1018,13 +1099,19 @@ dg_status dg_nn_forward_tc(const float *x, const float *const *w, const float *c
     }
     cudaStream_t s = (cudaStream_t)stream;
     uint16_t *wimg = reinterpret_cast<uint16_t *>(scratch);
-    dg::k_net_tc_wimg<<<dim3((unsigned)std::min<int64_t>((most + 255) / 256, 152 * 8), (unsigned)layers), 256, 0, s>>>(n, wimg);
-    cudaError_t e = cudaGetLastError();
+    const bool b16 = dg::net16(channels, layers);
     float *buf[2] = {scratch + elems / 2, scratch + elems / 2 + act};
+    // both buffers' planes follow one another
+    const int64_t planes = b16 ? act / 4 * (layers > 2 ? 2 : 1) / ((int64_t)(H + 2) * (W + 2)) : 0;
+    if (b16) most = std::max(most, planes * 2 * ((int64_t)W + 2 + H));
+    dg::k_net_tc_wimg<<<dim3((unsigned)std::min<int64_t>((most + 255) / 256, 152 * 2), (unsigned)(layers + (b16 ? 1 : 0))), 256, 0, s>>>(
+        n, wimg, layers, reinterpret_cast<uint4 *>(buf[0]), planes, H, W);
+    cudaError_t e = cudaGetLastError();
     const float *h = x;
     for (int l = 0; l < layers && e == cudaSuccess; ++l) {
         float *z = l + 1 == layers ? y : buf[l & 1];
-        e = dg::launch_conv_blocks(h, wimg + n.off[l], b[l], z, B, channels[l], channels[l + 1], H, W, s, l + 1 < layers);
+        e = dg::launch_conv_blocks(h, wimg + n.off[l], b[l], z, B, channels[l], channels[l + 1], H, W, s, l + 1 < layers,
+                                   b16 && l > 0, b16 && l + 1 < layers);
         h = z;
     }
     return dg::nn_done(e, "dg_nn_forward_tc");

@@ -50,7 +50,9 @@ def test_conv_tc_over_the_tile_schedule(shape):
 
 
 @pytest.mark.parametrize("channels,shape", [([3, 1], (2, 9, 40)), ([20, 32, 1], (1, 33, 130)),
-                                            ([5, 40, 130, 24, 1], (2, 7, 129))])
+                                            ([5, 40, 130, 24, 1], (2, 7, 129)),
+                                            ([7, 32, 64, 160, 32, 1], (3, 21, 257)), ([4, 96, 32, 1], (2, 1, 1)),
+                                            ([33, 128, 64, 1], (1, 130, 128))])
 def test_network_in_one_call_is_its_layers_one_by_one(channels, shape):
     from paper_2508_06672_gb300.proposal import ProposalNet
     P = package()
