@@ -75,7 +75,14 @@ enum { DG_PREC_FP32 = 0, DG_PREC_FP64 = 1 };
  * interpolation being linear in y2, each candidate sums the correlations of
  * lags L - 1 .. L + 2 weighted by its 4-tap weights. Its error against the
  * definition is bounded by the bin interpolation and by the arithmetic of the
- * contraction (DG_CONTRACT_*). */
+ * contraction (DG_CONTRACT_*).
+ * With chunk = 0, DG_TILES_AUTO and an arithmetic that is FP32 or claims its
+ * accuracy (DG_CONTRACT_FP32, _BF16X3, _FP16X3), a main grid of at least 8192
+ * nodes takes the same interpolation from one table per snapshot instead: the
+ * correlation of Eq. 11 at every lag and Doppler bin of the grid's ranges,
+ * computed in FP32 through FFTs, in which every candidate interpolates (error
+ * about 2e-7 of the surface). A refinement grid of few lags takes a small
+ * table summed directly. */
 enum { DG_ALGO_DIRECT = 0, DG_ALGO_CDFT = 1 };
 
 /* Tiles of the CDFT tensor-core contraction.
@@ -142,7 +149,9 @@ typedef struct {
                         the batch keeps 16 lag tiles per SM (dg_cdft_chunks);
                         at most 256 on the refinement grid of
                         dg_argmax_refine (few lags: shorter chunks give the
-                        contraction more tiles). DG_TILES_LAGS needs a chunk
+                        contraction more tiles). 0 also lets large grids
+                        take delay-Doppler tables (DG_ALGO_CDFT above), a
+                        chunk keeps the contraction. DG_TILES_LAGS needs one
                         <= 1024 or a multiple of 1024, DG_TILES_HANKEL one
                         <= 1024                                               */
     int32_t bins;    /* CDFT: Doppler bins per lag; 0 = 64 (the only value)   */
@@ -152,7 +161,8 @@ typedef struct {
                         snapshots (per-candidate arrays and per-lag DFTs),
                         MiB; 0 = 12288. Fewer snapshots per batch below it
                         (at least one); many contexts sharing a GPU lower it */
-    int32_t rows;    /* DIRECT: grid rows per thread, i.e. candidates per
+    int32_t rows;    /* DIRECT (not FP32 with INTEGER delay, whose candidates
+                        are grouped by lag): grid rows per thread, i.e. candidates per
                         thread (a CTA takes 8 warps x rows grid rows x 32
                         grid columns of one snapshot); 0 = 8 (FP32,
                         INTEGER delay) or 4 (FP32 LAGRANGE4, FP64); FP32
@@ -238,10 +248,12 @@ dg_status dg_set_grid(dg_ctx *ctx, const dg_grid *grid);
  * regions (host array, all with the same nlat x nlon), the context moves to
  * it (dg_set_grid) and the cost surface of Algorithm 1 is written to
  * costs + r * nlat * nlon (device, the context's precision, room for
- * n * nlat * nlon values) with its argmax, all stream-ordered; then one host
- * synchronisation, and the region whose argmax holds the largest cost (ties:
- * the first) gets the dense re-evaluation of dg_argmax_refine, whose fix is
- * written to *out (host). *best (host, may be NULL) receives that region's
+ * n * nlat * nlon values) with its argmax, all stream-ordered (regions that take
+ * delay-Doppler tables share their launches: the same values as one by one
+ * within rounding). The region whose argmax holds the largest cost (ties: the
+ * first) gets the dense re-evaluation of dg_argmax_refine, whose fix is
+ * written to *out (host), with one host synchronisation, or two where the
+ * refinement does not take a table of few lags. *best (host, may be NULL) receives that region's
  * index. The context is left on that region's grid. Needs a context over the
  * whole grid and every snapshot loaded. */
 dg_status dg_search_regions(dg_ctx *ctx, const dg_grid *regions, int32_t n, void *costs,
@@ -331,7 +343,8 @@ dg_status dg_graph_fix(dg_ctx *ctx, dg_fix *out);
  * work list over (capture, snapshot, tile)), with each context's plan
  * before it and its combine after it on the context's own branch. Rounds =
  * the most snapshot batches of any context (dg_batch_rounds; 0 when the
- * contractions are per context). Refinement surfaces stay per context. */
+ * contractions are per context, or a context takes delay-Doppler tables).
+ * Refinement surfaces stay per context. */
 typedef struct dg_batch dg_batch;
 dg_status dg_batch_capture(dg_ctx *const *ctxs, int32_t n, void *const *costs, double refine_spacing_m,
                            double refine_window_m, void *stream, dg_batch **out);
@@ -401,12 +414,14 @@ dg_status dg_kernel_time(dg_ctx *ctx, int32_t kernel_class, double *ms, int64_t 
  * summed over snapshots: lag-bucket x chunk pairs contracted (each a
  * chunk-by-bins complex DFT) and candidate x super-chunk pairs combined (the
  * combine merges chunks at the bin frequencies into the longest power-of-two
- * multiple of the chunk whose length x bin spacing stays <= 5e-2 cycles).
+ * multiple of the chunk whose length x bin spacing stays <= 5e-2 cycles). On
+ * delay-Doppler tables: lag x block pairs and candidates looked up.
  * Host pointers, may be NULL; zeros before the first CDFT surface. */
 dg_status dg_cdft_work(const dg_ctx *ctx, int64_t *bucket_chunks, int64_t *candidate_chunks);
 
 /* Shortest and longest chunk (samples) the last CDFT surface used, 0 if none
- * has been computed; with opt.chunk = 0 they follow each batch's FDOA spans.
+ * has been computed; with opt.chunk = 0 they follow each batch's FDOA spans
+ * (on delay-Doppler tables: the chunks the contraction would take).
  * Host only; either pointer may be NULL. */
 dg_status dg_cdft_chunks(const dg_ctx *ctx, int32_t *min_chunk, int32_t *max_chunk);
 
@@ -596,7 +611,9 @@ const char *dg_nn_last_error(void);
  * fixed quota). dg_create allocates; this call does not.
  *
  * It computes the same surface as dg_create + dg_load_capture (every
- * snapshot) + dg_cost_surface, with the same kernels and options. Scratch
+ * snapshot) + dg_cost_surface, with the same options; it keeps the kernel of one
+ * candidate per lane where dg_cost_surface groups candidates by lag (FP32,
+ * INTEGER delay), so there the two agree within rounding. Scratch
  * (candidate ECEF, per-snapshot surfaces, snapshot table, ephemerides, an
  * error word) lives in one static device array of DG_NOALLOC_SCRATCH_BYTES
  * owned by the library; it is reserved on every GPU that loads the library's

@@ -18,6 +18,10 @@
 // 4.9e-3 (2 pi M Delta)^6 of the coherent sum; the snapshot is rejected
 // (DG_EUNSUPPORTED) if M * Delta > kCdftMDelta.
 //
+// Main grids of many nodes with FP32 arithmetic and automatic launch shapes take
+// the tables of dg_map.cu instead; what runs here are explicit chunks and tiles,
+// the single 16-bit forms, and grids too small for a table.
+//
 // All snapshots of a batch are processed by the same launches:
 //   geo      FP64 geometry once per (candidate, snapshot): lag and FDOA kept,
 //            per-snapshot lag and FDOA ranges by atomics (the host sizes the
