@@ -79,9 +79,9 @@ __global__ void k_coarse_init(int *lmm, unsigned long long *nmm, int K)
 }
 
 // Nodes of snapshot k = blockIdx.y, about eight per thread, the next one loaded
-// while the current one is computed (228 -> 82 us for 20 snapshots of 513^2 nodes
-// with that and the minima kept in FP32; bound by instruction issue, about 520 a
-// node): Eq. 3-10 in double-float
+// while the current one is computed (228 -> 76 us for 20 snapshots of 513^2 nodes
+// with that, the minima kept in FP32 and both receivers in packed operations; bound
+// by the FP32 pipe): Eq. 3-10 in double-float
 // arithmetic on the FP32 pipes (ranges to about 1e-7 m), the lag of Eq. 9
 // (round half away from zero; decided by the FP64 expression where D lies
 // within 1e-6 of a rounding boundary) and the FDOA rounded to FP32; block

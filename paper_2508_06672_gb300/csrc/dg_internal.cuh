@@ -120,24 +120,6 @@ __device__ __forceinline__ dfl df_add_fast(dfl a, dfl b)
     return df_fast_two_sum(s.hi, s.lo + (a.lo + b.lo));
 }
 __device__ __forceinline__ dfl df_sub_fast(dfl a, dfl b) { return df_add_fast(a, {-b.hi, -b.lo}); }
-// sqrt of a double-float: one Newton correction of the FP32 root. The
-// residual a.hi - y^2 of y = sqrtf(a.hi) is exact in FP32, so one FMA gives it.
-__device__ __forceinline__ dfl df_sqrt(dfl a)
-{
-    const float y = sqrtf(a.hi);
-    const float r = fmaf(-y, y, a.hi) + a.lo;
-    return df_fast_two_sum(y, __fdividef(r, 2.f * y));
-}
-
-// a / b for a double-float quotient: the FP32 quotient plus one correction
-// from the exact-by-FMA residual (relative error ~1e-14).
-__device__ __forceinline__ dfl df_div_fast(dfl a, dfl b)
-{
-    const float q1 = __fdividef(a.hi, b.hi);
-    const float r = fmaf(-q1, b.hi, a.hi) + (a.lo - q1 * b.lo);
-    return df_fast_two_sum(q1, __fdividef(r, b.hi));
-}
-
 // Eq. 3-10 for the chunked-DFT plan. The lag needs D = (rho2 - rho1) fs / c
 // to ~1e-7 samples (so that Eq. 9 rounds it as the FP64 expression does
 // wherever D is farther than 1e-6 from a rounding boundary), i.e. the ranges
@@ -156,7 +138,8 @@ __device__ __forceinline__ dfl df_div_fast(dfl a, dfl b)
 // are double-float too, and nu is rounded to FP32 once, at the end.
 //
 // Both receivers run through the same operations, so they share Blackwell's packed
-// FP32 instructions, one in each half: about 260 instructions a node for 520.
+// FP32 instructions, one in each half: about 350 instructions a node of the
+// coarse maps for 520, each packed one two slots of the FP32 pipe.
 __device__ __forceinline__ float2 pk_fma(float2 a, float2 b, float2 c)
 {
     unsigned long long r, x, y, z;
@@ -213,13 +196,17 @@ __device__ __forceinline__ dfl2 df2_mul(dfl2 a, dfl2 b)
     e = pk_fma(a.lo, b.hi, e);
     return df2_fast_two_sum(p, e);
 }
-__device__ __forceinline__ dfl2 df2_sqrt(dfl2 a)  // as df_sqrt
+// sqrt of double-floats: one Newton correction of the FP32 root. The residual
+// a.hi - y^2 of y = sqrtf(a.hi) is exact in FP32, so one FMA gives it.
+__device__ __forceinline__ dfl2 df2_sqrt(dfl2 a)
 {
     const float2 y = make_float2(sqrtf(a.hi.x), sqrtf(a.hi.y));
     const float2 r = pk_add(pk_fma(make_float2(-y.x, -y.y), y, a.hi), a.lo);
     return df2_fast_two_sum(y, make_float2(__fdividef(r.x, 2.f * y.x), __fdividef(r.y, 2.f * y.y)));
 }
-__device__ __forceinline__ dfl2 df2_div_fast(dfl2 a, dfl2 b)  // as df_div_fast
+// a / b: the FP32 quotient plus one correction from the exact-by-FMA residual
+// (relative error ~1e-14).
+__device__ __forceinline__ dfl2 df2_div_fast(dfl2 a, dfl2 b)
 {
     const float2 q = make_float2(__fdividef(a.hi.x, b.hi.x), __fdividef(a.hi.y, b.hi.y)), n = make_float2(-q.x, -q.y);
     const float2 r = pk_add(pk_fma(n, b.hi, a.hi), pk_fma(n, b.lo, a.lo));
