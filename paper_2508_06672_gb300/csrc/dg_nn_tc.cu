@@ -424,6 +424,11 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     __syncthreads();
     nn_after_sync();
     const uint32_t tmem = tslot;
+    // Everything above runs while the kernel before still drains (launch_waiting);
+    // its outputs, and what this one overwrites, are safe from here on. Dependents are let in only after
+    // that wait, so a kernel's predecessors but one have always finished.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     bool ok = true;
     int64_t copied = 0;  // weight blocks (or BF16 input stages) whose copies this thread has issued
     if (IN16 && warp < kProdWarps) {
@@ -962,6 +967,25 @@ unsigned *err_word()
     return cudaGetSymbolAddress(&p, g_nn_tc_err) == cudaSuccess ? (unsigned *)p : nullptr;
 }
 
+// Launch of a kernel that itself waits for the one before it in the stream
+// (griddepcontrol.wait), so that its setup and its launch overlap that one's end: the
+// five layers of the proposal network 145 -> 131 us.
+template <typename... P, typename... A>
+cudaError_t launch_waiting(void (*kernel)(P...), dim3 grid, int threads, int smem, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // The convolution on converted weights.
 cudaError_t launch_conv_blocks(const void *x, const uint16_t *wimg, const float *b, void *y, int B, int CI, int CO, int H,
                                int W, cudaStream_t s, int relu, bool in16 = false, bool out16 = false)
@@ -986,9 +1010,8 @@ cudaError_t launch_conv_blocks(const void *x, const uint16_t *wimg, const float 
     if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
         return e;
     const int64_t tiles = (int64_t)((W + kRowsTc - 1) / kRowsTc) * ((H + kHaloRows - 1) / kHaloRows) * B * ob;
-    kernel<<<(unsigned)std::min<int64_t>(tiles, 152), kConvThreads, smem, s>>>(x, wimg, b, y, CI, CO, H, W, NT, nh, nw, tiles,
-                                                                               relu, err);
-    return cudaGetLastError();
+    return launch_waiting(kernel, dim3((unsigned)std::min<int64_t>(tiles, 152)), kConvThreads, smem, s, x, wimg, b, y, CI, CO, H,
+                          W, NT, nh, nw, tiles, relu, err);
 }
 
 cudaError_t launch_conv_tc(bool tr, const float *x, const float *w, const float *b, float *y, int B, int CI, int CO,
