@@ -3284,7 +3284,10 @@ static dg_status regions_map(dg_ctx *c, const dg_grid *regions, int n, float *co
     const double budget = (double)(c->opt.scratch_mib ? c->opt.scratch_mib : 12288) * 1048576.0;
     const int nr = (int)std::min((double)std::min(n, (int)(65535 / K)), std::floor(budget / ((double)K * map_bytes(m))));
     if (nr < 1) return DG_OK;
-    c->mp.gen = 0;  // the tables of the main grid's plan are replaced
+    // the tables of the main grid's plan are replaced, also where the search fails
+    // later on: the plan, and graphs and batches that replay on them, are stale
+    c->mp.gen = 0;
+    ++c->steps_gen;
     if ((st = map_buffers(c, m, K * (size_t)nr, snap)) != DG_OK) return st;
     if ((st = push_steps(c)) != DG_OK) return st;
     if (!all) {
