@@ -327,14 +327,38 @@ dg_status release(dg_ctx *c, void *p)
     return DG_OK;
 }
 
-dg_status ensure(dg_ctx *c, void **p, size_t *cap, size_t bytes)
+// Device and pinned host memory. A failed call leaves *p NULL, and no error for
+// the next launch's cudaGetLastError to find.
+template <typename P> cudaError_t device_alloc(dg_ctx *c, P **p, size_t bytes)
+{
+    const cudaError_t e = cudaMallocAsync((void **)p, bytes, c->stream);
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();
+    }
+    return e;
+}
+template <typename P> cudaError_t pinned_alloc(P **p, size_t bytes)
+{
+    const cudaError_t e = cudaMallocHost((void **)p, bytes);
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();
+    }
+    return e;
+}
+
+// At least `bytes` at *p. key (optional): what the buffer holds; 0 once it is
+// replaced, so that a failure here or later leaves no description of what is gone.
+dg_status ensure(dg_ctx *c, void **p, size_t *cap, size_t bytes, int *key = nullptr)
 {
     if (*cap >= bytes && *p) return DG_OK;
-    const dg_status st = release(c, *p);
-    if (st != DG_OK) return st;
-    *p = nullptr;
+    if (key) *key = 0;
     *cap = 0;
-    CK(c, cudaMallocAsync(p, bytes, c->stream));
+    const dg_status st = release(c, *p);
+    *p = nullptr;
+    if (st != DG_OK) return st;
+    CK(c, device_alloc(c, p, bytes));
     *cap = bytes;
     return DG_OK;
 }
@@ -370,6 +394,11 @@ static dg_status map_plan(dg_ctx *c);
 static dg_status run_surface_map(dg_ctx *c, void *out);
 static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *surf, void *out,
                                  bool refine, bool *done);
+// A dg_set_grid that found no memory leaves the context without nodes.
+static dg_status need_nodes(dg_ctx *c)
+{
+    return c->xyz ? DG_OK : fail(c, DG_ENOMEM, "no memory was left for the grid's nodes: set a grid first");
+}
 static dg_status refine_map(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *out, bool *done,
                             const GridDev *mains, int nmains);
 
@@ -389,7 +418,8 @@ static bool map_eligible(const dg_ctx *c) { return map_options(c) && c->G >= kMa
 dg_status run_surface(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *surf, void *out,
                       bool refine)
 {
-    dg_status st;
+    dg_status st = need_nodes(c);
+    if (st != DG_OK) return st;
     if (!refine && map_eligible(c)) {
         if ((st = map_plan(c)) != DG_OK) return st;
         if (c->mp.ok) return run_surface_map(c, out);
@@ -453,13 +483,15 @@ dg_status run_surface(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G
 }
 
 
+// n elements in place of what *p holds. Capacities that describe *p are 0 while it
+// is replaced (the caller's, set again once all of its buffers are there).
 template <typename P>
 dg_status grow(dg_ctx *c, P **p, size_t n)
 {
     const dg_status st = release(c, *p);
-    if (st != DG_OK) return st;
     *p = nullptr;
-    CK(c, cudaMallocAsync((void **)p, sizeof(P) * (n ? n : 1), c->stream));
+    if (st != DG_OK) return st;
+    CK(c, device_alloc(c, p, sizeof(P) * (n ? n : 1)));
     return DG_OK;
 }
 
@@ -713,7 +745,6 @@ static dg_status cdft_layout(dg_ctx *c, const GridDev &gd, int64_t G, CdftLayout
     if (L.G == G && L.diam >= diam && !L.batches.empty()) return DG_OK;
     int *old_bb = L.bbase, *old_gb = L.gbase;
     L = CdftLayout{};
-    L.G = G;
     L.diam = diam;
     L.bbase = old_bb;
     L.gbase = old_gb;
@@ -726,6 +757,7 @@ static dg_status cdft_layout(dg_ctx *c, const GridDev &gd, int64_t G, CdftLayout
     // pageable sources: staged before the calls return
     CK(c, cudaMemcpyAsync(L.bbase, bb.data(), sizeof(int) * bb.size(), cudaMemcpyHostToDevice, c->stream));
     CK(c, cudaMemcpyAsync(L.gbase, gb.data(), sizeof(int) * gb.size(), cudaMemcpyHostToDevice, c->stream));
+    L.G = G;  // its tables are in place
     return DG_OK;
 }
 
@@ -740,7 +772,6 @@ static dg_status ensure_ephf(dg_ctx *c)
     if (b.ephf_cap >= (size_t)c->K) return DG_OK;
     dg_status st;
     if ((st = grow(c, &b.ephf, 24 * (size_t)c->K)) != DG_OK) return st;
-    b.ephf_cap = (size_t)c->K;
     std::vector<float> ef(24 * (size_t)c->K);
     for (int k = 0; k < c->K; ++k) {
         const double *v = &c->eph_host[k].p1[0];
@@ -751,7 +782,15 @@ static dg_status ensure_ephf(dg_ctx *c)
     }
     // pageable source: staged before the call returns
     CK(c, cudaMemcpyAsync(b.ephf, ef.data(), sizeof(float) * ef.size(), cudaMemcpyHostToDevice, c->stream));
+    b.ephf_cap = (size_t)c->K;
     return DG_OK;
+}
+
+// The nodes' double-float split, G of them.
+static dg_status ensure_xyzf(dg_ctx *c, int64_t G)
+{
+    CdftBufs &b = c->cd;
+    return ensure(c, (void **)&b.xyzf, &b.xyzf_cap, sizeof(float) * 6 * (size_t)G);
 }
 
 // Scratch of the lag sort, grown on demand (never inside a captured graph: a
@@ -762,6 +801,7 @@ static dg_status ensure_sort(dg_ctx *c, size_t S, size_t SG, size_t nbt, size_t 
     CdftBufs &b = c->cd;
     dg_status st;
     if (b.s_cap < S) {
+        b.s_cap = 0;
         if ((st = grow(c, &b.lr, 2 * S)) != DG_OK) return st;
         if ((st = grow(c, &b.delta, S)) != DG_OK) return st;
         if ((st = grow(c, &b.nubase, S)) != DG_OK) return st;
@@ -773,6 +813,7 @@ static dg_status ensure_sort(dg_ctx *c, size_t S, size_t SG, size_t nbt, size_t 
         b.s_cap = S;
     }
     if (b.sg_cap < SG) {
+        b.sg_cap = 0;
         if ((st = grow(c, &b.candL, SG)) != DG_OK) return st;
         if ((st = grow(c, &b.candNu, SG)) != DG_OK) return st;
         if ((st = grow(c, &b.order, SG)) != DG_OK) return st;
@@ -780,6 +821,7 @@ static dg_status ensure_sort(dg_ctx *c, size_t S, size_t SG, size_t nbt, size_t 
         b.sg_cap = SG;
     }
     if (b.nb_cap < nbt) {
+        b.nb_cap = 0;
         if ((st = grow(c, &b.count, nbt)) != DG_OK) return st;
         if ((st = grow(c, &b.need, nbt)) != DG_OK) return st;
         if ((st = grow(c, &b.offs, nbt)) != DG_OK) return st;
@@ -787,6 +829,7 @@ static dg_status ensure_sort(dg_ctx *c, size_t S, size_t SG, size_t nbt, size_t 
         b.nb_cap = nbt;
     }
     if (b.g2b_cap < groups) {
+        b.g2b_cap = 0;
         if ((st = grow(c, &b.g2b, groups)) != DG_OK) return st;
         b.g2b_cap = groups;
     }
@@ -906,10 +949,7 @@ static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz
     if ((st = ensure_sort(c, S, SG, (size_t)L.nbt_max, (size_t)L.groups_max)) != DG_OK) return st;
     if (nseg > 1 && (st = ensure(c, (void **)&b.part, &b.part_cap, sizeof(float2) * SG * nseg)) != DG_OK) return st;
     if ((st = ensure_ephf(c)) != DG_OK) return st;
-    if (b.xyzf_cap < (size_t)G) {
-        if ((st = grow(c, &b.xyzf, 6 * (size_t)G)) != DG_OK) return st;
-        b.xyzf_cap = (size_t)G;
-    }
+    if ((st = ensure_xyzf(c, G)) != DG_OK) return st;
     const bool one = L.batches.size() == 1;
     {
         Timed t(c, refine ? DG_K_REFINE : DG_K_CORR);
@@ -1016,11 +1056,13 @@ static dg_status cdft_setup(dg_ctx *c, CdftRun &r)
         if ((st = grow(c, &b.work, 2)) != DG_OK) return st;
     }
     if (c->opt.delay != DG_DELAY_INTEGER && b.mu_cap < (size_t)s_max * G) {
+        b.mu_cap = 0;
         if ((st = grow(c, &b.candMu, (size_t)s_max * G)) != DG_OK) return st;
         if ((st = grow(c, &b.muS, (size_t)s_max * G)) != DG_OK) return st;
         b.mu_cap = (size_t)s_max * G;
     }
     if (!mma && b.v_cap < (size_t)s_max * M_max * 64) {  // the FP32 contraction's DFT table
+        b.v_cap = 0;
         if ((st = grow(c, &b.V, (size_t)s_max * M_max * 64)) != DG_OK) return st;
         b.v_cap = (size_t)s_max * M_max * 64;
     }
@@ -1029,17 +1071,13 @@ static dg_status cdft_setup(dg_ctx *c, CdftRun &r)
         return fail(c, DG_EUNSUPPORTED, "CDFT: the per-lag DFT buffer would exceed 64 GiB (%lld lag slots x %d chunks); "
                     "use a longer chunk or DIRECT", (long long)L.nbt_max, B_max);
     if (b.w_cap < w_elems) {
+        b.w_cap = 0;
         if ((st = grow(c, &b.W, w_elems)) != DG_OK) return st;
         b.w_cap = w_elems;
     }
     if (mma) {
         const size_t bt = (size_t)s_max * cdft_btab_bytes(c->opt.contract, M_max);
-        if (b.btab_cap < bt) {
-            unsigned char *p = reinterpret_cast<unsigned char *>(b.btab);
-            if ((st = grow(c, &p, bt)) != DG_OK) return st;
-            b.btab = p;
-            b.btab_cap = bt;
-        }
+        if ((st = ensure(c, &b.btab, &b.btab_cap, bt)) != DG_OK) return st;
     }
     const int kplan = refine ? DG_K_REFINE : DG_K_CDFT_PLAN;
     if (!refine) {
@@ -1048,10 +1086,7 @@ static dg_status cdft_setup(dg_ctx *c, CdftRun &r)
         c->cd_chunk_max = 0;
     }
     if ((st = ensure_ephf(c)) != DG_OK) return st;
-    if (b.xyzf_cap < (size_t)G) {
-        if ((st = grow(c, &b.xyzf, 6 * (size_t)G)) != DG_OK) return st;
-        b.xyzf_cap = (size_t)G;
-    }
+    if ((st = ensure_xyzf(c, G)) != DG_OK) return st;
     {
         Timed t(c, kplan);
         CK(c, launch_ecef_split(xyz, G, b.xyzf, c->stream));
@@ -1400,8 +1435,8 @@ static dg_status map_buffers(dg_ctx *c, const MapPlan &m, size_t S, const std::v
     const size_t n = (size_t)1 << m.logn;
     dg_status st;
     if ((st = ensure(c, (void **)&d.snap, &d.snap_cap, sizeof(MapSnap) * snap.size())) != DG_OK) return st;
-    if ((st = ensure(c, (void **)&d.tw, &d.tw_cap, sizeof(float2) * n)) != DG_OK) return st;
-    if ((st = ensure(c, (void **)&d.T, &d.T_cap, sizeof(float) * (size_t)m.P * m.Q)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&d.tw, &d.tw_cap, sizeof(float2) * n, &d.tw_logn)) != DG_OK) return st;
+    if ((st = ensure(c, (void **)&d.T, &d.T_cap, sizeof(float) * (size_t)m.P * m.Q, &d.T_P)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&d.F2, &d.F2_cap, sizeof(float2) * S * m.ntile * m.Cmax * n)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&d.U, &d.U_cap, sizeof(float2) * S * m.Cmax * m.P * m.NLpad)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&d.X, &d.X_cap, sizeof(float2) * S * m.Q * m.NLpad)) != DG_OK) return st;
@@ -1411,6 +1446,7 @@ static dg_status map_buffers(dg_ctx *c, const MapPlan &m, size_t S, const std::v
     // pageable sources: staged before the calls return
     CK(c, cudaMemcpyAsync(d.snap, snap.data(), sizeof(MapSnap) * snap.size(), cudaMemcpyHostToDevice, c->stream));
     if (d.tw_logn != m.logn) {
+        d.tw_logn = 0;
         CK(c, launch_map_twiddles(d.tw, m.logn, c->stream));
         ++c->launches;
         d.tw_logn = m.logn;
@@ -1425,6 +1461,7 @@ static dg_status map_buffers(dg_ctx *c, const MapPlan &m, size_t S, const std::v
                     if (r != p) t *= (x - m.xnode[r]) / (m.xnode[p] - m.xnode[r]);
                 T[(size_t)p * m.Q + q] = (float)t;
             }
+        d.T_P = 0;
         CK(c, cudaMemcpyAsync(d.T, T.data(), sizeof(float) * T.size(), cudaMemcpyHostToDevice, c->stream));
         d.T_P = m.P;
         d.T_Q = m.Q;
@@ -1457,12 +1494,9 @@ static bool map_chunks(dg_ctx *c, int *lo, int *hi)
     return (double)L.nbt_max * (double)B * 512.0 <= (double)((size_t)64 << 30);
 }
 
-static dg_status map_plan(dg_ctx *c)
+static dg_status make_map_plan(dg_ctx *c)
 {
     MapPlan &m = c->mp;
-    if (m.gen == c->steps_gen) return DG_OK;
-    m = MapPlan{};
-    m.gen = c->steps_gen;  // whatever the outcome, it holds until the shapes change
     CdftBufs &b = c->cd;
     if (!map_chunks(c, &m.chunk_min, &m.chunk_max)) return DG_OK;
     std::vector<MapSnap> snap;
@@ -1478,11 +1512,12 @@ static dg_status map_plan(dg_ctx *c)
     if (pr) {
         MapBufs &d = c->mb;
         const size_t fb = sizeof(float) * kPolyTerms * kPolyPts;
-        if ((st = ensure(c, (void **)&d.fit, &d.fit_cap, fb)) != DG_OK) return st;
+        if ((st = ensure(c, (void **)&d.fit, &d.fit_cap, fb, &d.fit_rows)) != DG_OK) return st;
         if ((st = ensure(c, (void **)&d.coef, &d.coef_cap, sizeof(float) * kPolyStride * (size_t)ptiles * m.S)) != DG_OK)
             return st;
         if (d.fit_rows != pr) {
             const std::vector<float> fit = poly_fit(m.poly);
+            d.fit_rows = 0;
             CK(c, cudaMemcpyAsync(d.fit, fit.data(), fb, cudaMemcpyHostToDevice, c->stream));
             d.fit_rows = pr;
         }
@@ -1490,6 +1525,15 @@ static dg_status map_plan(dg_ctx *c)
     if ((st = map_buffers(c, m, (size_t)m.S, snap)) != DG_OK) return st;
     m.ok = true;
     return DG_OK;
+}
+static dg_status map_plan(dg_ctx *c)
+{
+    if (c->mp.gen == c->steps_gen) return DG_OK;
+    c->mp = MapPlan{};
+    const dg_status st = make_map_plan(c);
+    // tables or not, the outcome holds until the shapes change; an error is tried again
+    if (st == DG_OK) c->mp.gen = c->steps_gen;
+    return st;
 }
 
 // The arguments every table shares: captures and ephemerides from snapshot k0
@@ -1906,15 +1950,15 @@ dg_status dg_create(const dg_grid *grid, const dg_ephem *eph, int32_t K, double 
     } while (0)
     CKC(cudaGetDevice(&c->device));
     CKC(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device));
-    CKC(cudaMallocAsync((void **)&c->xyz, sizeof(double) * 3 * (size_t)c->G, c->stream));
+    CKC(device_alloc(c, &c->xyz, sizeof(double) * 3 * (size_t)c->G));
     c->xyz_cap = c->G;
-    CKC(cudaMallocAsync((void **)&c->gstep, 2 * sizeof(GridStep), c->stream));
-    CKC(cudaMallocAsync((void **)&c->eph, sizeof(double) * 12 * (size_t)K, c->stream));
-    CKC(cudaMallocAsync((void **)&c->steps_d, sizeof(StepDesc) * (size_t)K, c->stream));
-    CKC(cudaMallocAsync((void **)&c->amax_res, sizeof(ArgmaxResult), c->stream));
-    CKC(cudaMallocAsync((void **)&c->err_d, sizeof(unsigned), c->stream));
-    CKC(cudaMallocHost((void **)&c->amax_host, sizeof(ArgmaxResult)));
-    CKC(cudaMallocHost((void **)&c->err_h, sizeof(unsigned)));
+    CKC(device_alloc(c, &c->gstep, 2 * sizeof(GridStep)));
+    CKC(device_alloc(c, &c->eph, sizeof(double) * 12 * (size_t)K));
+    CKC(device_alloc(c, &c->steps_d, sizeof(StepDesc) * (size_t)K));
+    CKC(device_alloc(c, &c->amax_res, sizeof(ArgmaxResult)));
+    CKC(device_alloc(c, &c->err_d, sizeof(unsigned)));
+    CKC(pinned_alloc(&c->amax_host, sizeof(ArgmaxResult)));
+    CKC(pinned_alloc(&c->err_h, sizeof(unsigned)));
     *c->err_h = 0;
     CKC(cudaMemsetAsync(c->err_d, 0, sizeof(unsigned), c->stream));
     CKC(cudaMemcpyAsync(c->eph, c->eph_host.data(), sizeof(dg_ephem) * (size_t)K, cudaMemcpyHostToDevice,
@@ -1970,10 +2014,12 @@ static dg_status set_grid(dg_ctx *c, const dg_grid *grid, const double *xyz, con
         return fail(c, DG_EUNSUPPORTED, "dg_set_grid needs a context over the whole grid (no row shard)");
     const int64_t G = (int64_t)grid->nlat * grid->nlon;
     if (G > c->xyz_cap) {
-        CK(c, cudaFreeAsync(c->xyz, c->stream));
+        void *old = c->xyz;  // no nodes (need_nodes) until the new buffer is there
         c->xyz = nullptr;
         c->xyz_cap = 0;
-        CK(c, cudaMallocAsync((void **)&c->xyz, sizeof(double) * 3 * (size_t)G, c->stream));
+        ++c->steps_gen;
+        if (old) CK(c, cudaFreeAsync(old, c->stream));
+        CK(c, device_alloc(c, &c->xyz, sizeof(double) * 3 * (size_t)G));
         c->xyz_cap = G;
     }
     const bool same = same_grid(c->grid, *grid);
@@ -2013,15 +2059,16 @@ dg_status dg_load_capture(dg_ctx *c, int32_t step, int32_t fmt, const void *y1, 
     Step &s = c->steps[step];
     const size_t bytes = bps * (size_t)n;
     if (s.cap < bytes) {
-        if (s.y1) CK(c, cudaFreeAsync(s.y1, c->stream));
-        if (s.y2) CK(c, cudaFreeAsync(s.y2, c->stream));
+        void *const old[2] = {s.y1, s.y2};
         s.y1 = s.y2 = nullptr;
         s.cap = 0;
         s.loaded = false;
-        CK(c, cudaMallocAsync(&s.y1, bytes, c->stream));
-        CK(c, cudaMallocAsync(&s.y2, bytes, c->stream));
+        ++c->steps_gen;  // also where the allocation fails: captured steps read the old buffers
+        for (void *p : old)
+            if (p) CK(c, cudaFreeAsync(p, c->stream));
+        CK(c, device_alloc(c, &s.y1, bytes));
+        CK(c, device_alloc(c, &s.y2, bytes));
         s.cap = bytes;
-        ++c->steps_gen;
     }
     const cudaMemcpyKind kind = is_device_ptr ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     CK(c, cudaMemcpyAsync(s.y1, y1, bytes, kind, c->stream));
@@ -2066,9 +2113,9 @@ static dg_status ensure_local(dg_ctx *c, int64_t G)
             (st = release(c, c->loc.cost)) != DG_OK)
             return st;
         c->loc = LocalGrid{};
-        CK(c, cudaMallocAsync((void **)&c->loc.xyz, sizeof(double) * 3 * G, c->stream));
-        CK(c, cudaMallocAsync(&c->loc.surf, esz * G * c->K + 8, c->stream));
-        CK(c, cudaMallocAsync(&c->loc.cost, esz * G + 8, c->stream));
+        CK(c, device_alloc(c, &c->loc.xyz, sizeof(double) * 3 * G));
+        CK(c, device_alloc(c, &c->loc.surf, esz * G * c->K + 8));
+        CK(c, device_alloc(c, &c->loc.cost, esz * G + 8));
         c->loc.g_cap = (size_t)G;
     }
     return DG_OK;
@@ -2138,11 +2185,9 @@ dg_status dg_detect(dg_ctx *c, const void *cost, double threshold, int32_t relat
         thr = threshold * r.val;
     }
     const size_t out_bytes = sizeof(DetectPeak) * kCap + sizeof(int);  // records, then their count
-    if (!c->det_out) {
-        CK(c, cudaMallocAsync((void **)&c->det_cand, sizeof(int64_t) * kCap, c->stream));
-        CK(c, cudaMallocAsync((void **)&c->det_out, out_bytes, c->stream));
-    }
-    if (!c->det_host) CK(c, cudaMallocHost((void **)&c->det_host, out_bytes));
+    if (!c->det_cand) CK(c, device_alloc(c, &c->det_cand, sizeof(int64_t) * kCap));
+    if (!c->det_out) CK(c, device_alloc(c, &c->det_out, out_bytes));
+    if (!c->det_host) CK(c, pinned_alloc(&c->det_host, out_bytes));
     int *const count_d = reinterpret_cast<int *>(c->det_out + max_peaks);  // behind the records asked for
     const DetectPeak *const pk = c->det_host;
     int count = 0;
@@ -2195,9 +2240,9 @@ static dg_status ensure_post(dg_ctx *c, int half, dg_fix **fix_dev, dg_fix **fix
     if ((st = ensure(c, &c->amax_tmp, &c->amax_tmp_bytes, argmax_tmp_bytes(std::max<int64_t>(c->G, Gl)))) != DG_OK)
         return st;
     if (half > 0 && (st = ensure_local(c, Gl)) != DG_OK) return st;
-    if (!c->amax_fine) CK(c, cudaMallocAsync((void **)&c->amax_fine, sizeof(ArgmaxResult), c->stream));
-    if (!*fix_dev) CK(c, cudaMallocAsync((void **)fix_dev, sizeof(dg_fix), c->stream));
-    if (!*fix_host) CK(c, cudaMallocHost((void **)fix_host, sizeof(dg_fix)));
+    if (!c->amax_fine) CK(c, device_alloc(c, &c->amax_fine, sizeof(ArgmaxResult)));
+    if (!*fix_dev) CK(c, device_alloc(c, fix_dev, sizeof(dg_fix)));
+    if (!*fix_host) CK(c, pinned_alloc(fix_host, sizeof(dg_fix)));
     return DG_OK;
 }
 
@@ -2334,8 +2379,16 @@ static dg_status tc_rounds(dg_ctx *const *ctxs, int n, TcRounds &R, bool &ok)
         }
     }
     dg_ctx *c0 = ctxs[0];
-    CK(c0, cudaMalloc((void **)&R.jobs, sizeof(TcJob) * jobs.size()));
-    CK(c0, cudaMalloc((void **)&R.job_tiles, sizeof(int) * (jobs.size() + rounds)));
+    auto table = [](auto **p, size_t bytes) {  // NULL where it fails (tc_rounds_free)
+        const cudaError_t e = cudaMalloc((void **)p, bytes);
+        if (e != cudaSuccess) {
+            *p = nullptr;
+            cudaGetLastError();
+        }
+        return e;
+    };
+    CK(c0, table(&R.jobs, sizeof(TcJob) * jobs.size()));
+    CK(c0, table(&R.job_tiles, sizeof(int) * (jobs.size() + rounds)));
     CK(c0, cudaMemcpy(R.jobs, jobs.data(), sizeof(TcJob) * jobs.size(), cudaMemcpyHostToDevice));
     R.fmt = fmt;
     R.contract = contract;
@@ -2794,6 +2847,7 @@ dg_status dg_grid_ecef(dg_ctx *c, double *xyz_out)
     if (!c) return fail(nullptr, DG_EINVAL, "ctx is NULL");
     c->err.clear();
     if (!xyz_out) return fail(c, DG_EINVAL, "xyz_out is NULL");
+    if (need_nodes(c) != DG_OK) return DG_ENOMEM;
     CK(c, cudaMemcpyAsync(xyz_out, c->xyz, sizeof(double) * 3 * (size_t)c->G, cudaMemcpyDeviceToDevice,
                           c->stream));
     return DG_OK;
@@ -2804,6 +2858,7 @@ dg_status dg_step_geometry(dg_ctx *c, int32_t step, int32_t *lag, double *D, dou
     if (!c) return fail(nullptr, DG_EINVAL, "ctx is NULL");
     c->err.clear();
     if (step < 0 || step >= c->K) return fail(c, DG_EINVAL, "step %d outside [0, %d)", step, c->K);
+    if (need_nodes(c) != DG_OK) return DG_ENOMEM;
     {
         Timed t(c, DG_K_GRID);
         CK(c, launch_step_geometry(c->gd, c->xyz, c->eph + 12 * (size_t)step, c->fs, c->lambda,
@@ -3042,7 +3097,9 @@ dg_status dg_coarse_maps(dg_ctx *c, int32_t bins, int32_t chunk, float *maps)
     }
     const size_t KG = (size_t)c->K * (size_t)c->G, K = (size_t)c->K;
     CoarseBufs &b = c->co;
-    dg_status st;
+    dg_status st = need_nodes(c);
+    if (st != DG_OK) return st;
+    b.Q = 0;  // the last maps' buffers may go
     if ((st = ensure(c, (void **)&b.lag, &b.lag_cap, sizeof(int) * KG)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&b.nu, &b.nu_cap, sizeof(float) * KG)) != DG_OK) return st;
     if ((st = ensure(c, (void **)&b.lmm, &b.lmm_cap, sizeof(int) * 2 * K)) != DG_OK) return st;
@@ -3050,10 +3107,7 @@ dg_status dg_coarse_maps(dg_ctx *c, int32_t bins, int32_t chunk, float *maps)
     if ((st = ensure(c, (void **)&b.st, &b.st_cap, sizeof(CoarseStep) * K)) != DG_OK) return st;
     if ((st = push_steps(c)) != DG_OK) return st;
     if ((st = ensure_ephf(c)) != DG_OK) return st;
-    if (c->cd.xyzf_cap < (size_t)c->G) {
-        if ((st = grow(c, &c->cd.xyzf, 6 * (size_t)c->G)) != DG_OK) return st;
-        c->cd.xyzf_cap = (size_t)c->G;
-    }
+    if ((st = ensure_xyzf(c, c->G)) != DG_OK) return st;
     CoarseArgs a{};
     a.xyz = c->xyz;
     a.xyzf = c->cd.xyzf;
@@ -3106,7 +3160,7 @@ dg_status dg_coarse_maps(dg_ctx *c, int32_t bins, int32_t chunk, float *maps)
     int nlag_cap = 0;
     for (int k = 0; k < c->K; ++k) nlag_cap = std::max(nlag_cap, lag_slots(c->eph_host[k], c->fs, diam));
     MapArgs f{};
-    const bool fft = coarse_fft(c, nmax, M, nb_max, nlag_cap, f);
+    bool fft = coarse_fft(c, nmax, M, nb_max, nlag_cap, f);
     a.Q = Q;
     a.M = M;
     a.nlag_cap = nlag_cap;
@@ -3125,15 +3179,23 @@ dg_status dg_coarse_maps(dg_ctx *c, int32_t bins, int32_t chunk, float *maps)
     a.pool = b.pool;
     a.turn = b.turn;
     a.part = b.part;
+    bool c64 = false;
+    for (int k = 0; k < c->K; ++k) c64 |= c->steps[k].fmt == DG_IQ_C64;
     if (fft) {
         const size_t n = (size_t)1 << f.logn;
-        bool c64 = false;
-        for (int k = 0; k < c->K; ++k) c64 |= c->steps[k].fmt == DG_IQ_C64;
-        if ((st = ensure(c, (void **)&b.snap, &b.snap_cap, sizeof(MapSnap) * K)) != DG_OK) return st;
-        if ((st = ensure(c, (void **)&b.F2, &b.F2_cap, sizeof(float2) * K * ((size_t)nb_max + f.nwin) * n)) != DG_OK) return st;
-        if (c64 && (st = ensure(c, (void **)&b.bad, &b.bad_cap, sizeof(int) * 4 * K)) != DG_OK) return st;
+        st = ensure(c, (void **)&b.snap, &b.snap_cap, sizeof(MapSnap) * K);
+        if (st == DG_OK) st = ensure(c, (void **)&b.F2, &b.F2_cap, sizeof(float2) * K * ((size_t)nb_max + f.nwin) * n);
+        if (st == DG_OK && c64) st = ensure(c, (void **)&b.bad, &b.bad_cap, sizeof(int) * 4 * K);
+        if (st == DG_OK) st = ensure(c, (void **)&b.tw, &b.tw_cap, sizeof(float2) * n, &b.tw_logn);
+        if (st != DG_OK && st != DG_ENOMEM) return st;
+        if (st == DG_ENOMEM) {  // the direct kernel needs none of these
+            c->err.clear();
+            fft = false;
+        }
+    }
+    if (fft) {
         if (b.tw_logn != f.logn) {
-            if ((st = ensure(c, (void **)&b.tw, &b.tw_cap, sizeof(float2) * n)) != DG_OK) return st;
+            b.tw_logn = 0;
             CK(c, launch_map_twiddles(b.tw, f.logn, c->stream));
             ++c->launches;
             b.tw_logn = f.logn;
@@ -3396,6 +3458,8 @@ dg_status dg_search_regions(dg_ctx *c, const dg_grid *regions, int32_t n, void *
     const int64_t G = (int64_t)regions[0].nlat * regions[0].nlon;
     const size_t esz = c->opt.prec == DG_PREC_FP64 ? 8 : 4;
     if (c->reg_cap < (size_t)n) {
+        c->reg_cap = 0;
+        c->reg_n = 0;
         if (c->reg_res) CK(c, cudaFreeAsync(c->reg_res, c->stream));
         c->reg_res = nullptr;
         if (c->reg_host) {
@@ -3403,15 +3467,20 @@ dg_status dg_search_regions(dg_ctx *c, const dg_grid *regions, int32_t n, void *
             cudaFreeHost(c->reg_host);
             c->reg_host = nullptr;
         }
-        c->reg_cap = 0;
-        CK(c, cudaMallocAsync((void **)&c->reg_res, sizeof(ArgmaxResult) * n, c->stream));
-        CK(c, cudaMallocHost((void **)&c->reg_host, sizeof(ArgmaxResult) * n));
+        CK(c, device_alloc(c, &c->reg_res, sizeof(ArgmaxResult) * n));
+        CK(c, pinned_alloc(&c->reg_host, sizeof(ArgmaxResult) * n));
         c->reg_cap = (size_t)n;
     }
     dg_status st;
     bool done = false, nodes = false;
     c->reg_n = 0;
-    if ((st = regions_map(c, regions, n, (float *)costs, &done, &nodes)) != DG_OK) return st;
+    st = regions_map(c, regions, n, (float *)costs, &done, &nodes);
+    if (st == DG_ENOMEM) {  // no memory for all regions' tables: one region after the other
+        c->err.clear();
+        done = nodes = false;
+    } else if (st != DG_OK) {
+        return st;
+    }
     for (int r = 0; r < n && !done; ++r) {
         if ((st = dg_set_grid(c, &regions[r])) != DG_OK) return st;
         if ((st = ensure_surf(c)) != DG_OK) return st;
