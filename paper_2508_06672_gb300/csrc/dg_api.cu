@@ -91,10 +91,16 @@ struct MapBufs {  // their device tables and scratch, grown on demand
     int tw_logn = 0, T_P = 0, T_Q = 0;  // what tw and T hold
 };
 
+struct LagRule {  // tiles_faster's answer for one grid
+    GridDev g{};
+    bool known = false, tiles = false;
+};
+
 struct CdftBufs {  // chunked-DFT scratch, grown on demand
     int *lr = nullptr;
     CdftLayout main_layout, loc_layout;
     CdftLayout dmain_layout, dloc_layout;  // the direct path's lag groups
+    LagRule dmain_rule, dloc_rule;
     float2 *part = nullptr;                // and its segments' sums
     size_t part_cap = 0;
     std::vector<double> main_span;  // FDOA span estimates per snapshot (main grid)
@@ -882,10 +888,67 @@ static void sort_args(dg_ctx *c, const CdftLayout::Batch &bt, const CdftLayout &
     a.ngroups = (int)bt.groups;
 }
 
+// Whether the tile kernel (k_corr_direct) is the faster one for an FP32 surface
+// with integer delays: where few candidates share a lag. k_corr_lag takes a warp
+// per group however few candidates it has, 5.1e-6 us per group and sample on 152
+// SMs; the tile kernel takes a CTA per rows x 256 candidates, on widely spread lags
+// 0.145 us per tile of an SM and sample plus 0.1, 0.36 at least (tiles of 8 rows;
+// lower envelopes of what it took, so that no grid is slower than on its tiles).
+// Measured, grouped against tiles, by candidates per group: 401^2 nodes and 16
+// snapshots of 16384 samples 7.2 against 19.0 ms (46), 10.7 / 26.2 (25), 24.8 / 26.0
+// (8.6), 29.2 / 26.4 (7.3), 51.6 / 33.1 (4.1), 125 / 37.8 (1.7); 201^2 and 8 of 32768
+// 13.1 / 14.3 (4.1), 18.2 / 21.6 (3.0), 20.5 / 15.5 (2.6), 36.7 / 17.5 (1.5); 101^2 and
+// 8 of 32768, which leave most SMs without a tile, 12.1 / 12.7 (1.2).
+// The groups are estimated from the lags at a lattice of 9 x 9 nodes (0.88 of what an
+// even spread over their range would give, as counted on those grids) of the
+// whole grid, so that every row shard of it takes the same kernel. A refinement
+// grid (gd) is judged as if on the main grid's centre.
+static bool tiles_faster(const dg_ctx *c, const GridDev &gd, LagRule &rule)
+{
+    GridDev g = gd;
+    g.row0 = 0;
+    g.nrows = g.nlat;
+    const GridDev &o = rule.g;
+    if (rule.known && o.lat0_rad == g.lat0_rad && o.lon0_rad == g.lon0_rad && o.dlat_m == g.dlat_m && o.dlon_m == g.dlon_m &&
+        o.nlat == g.nlat && o.nlon == g.nlon)
+        return rule.tiles;
+    const int ni = std::min(9, g.nlat), nj = std::min(9, g.nlon);
+    std::vector<double> p(3 * (size_t)ni * nj);
+    for (int i = 0; i < ni; ++i)
+        for (int j = 0; j < nj; ++j)
+            host_node_ecef(g, ni > 1 ? (double)i * (g.nlat - 1) / (ni - 1) : 0.0, nj > 1 ? (double)j * (g.nlon - 1) / (nj - 1) : 0.0,
+                           &p[3 * ((size_t)i * nj + j)]);
+    const double G = (double)g.nlat * g.nlon;
+    double groups = 0.0;
+    for (int k = 0; k < c->K; ++k) {
+        const dg_ephem &e = c->eph_host[k];
+        double lo = 1e300, hi = -1e300;
+        for (size_t q = 0; q < p.size(); q += 3) {
+            const double *x = &p[q];
+            double r[2];
+            for (int t = 0; t < 2; ++t) {
+                const double *s = t ? e.p2 : e.p1;
+                r[t] = std::sqrt((s[0] - x[0]) * (s[0] - x[0]) + (s[1] - x[1]) * (s[1] - x[1]) + (s[2] - x[2]) * (s[2] - x[2]));
+            }
+            lo = std::min(lo, r[1] - r[0]);
+            hi = std::max(hi, r[1] - r[0]);
+        }
+        const double lags = (hi - lo) * c->fs / kC + 1.0;
+        groups += 0.88 * (lags * -std::expm1(-G / lags) + G / kDirectGroup);  // the lags that hold a candidate
+    }
+    const int rows = c->opt.rows ? c->opt.rows : 8;
+    const double tiles = std::ceil(g.nlat / (8.0 * rows)) * std::ceil(g.nlon / 32.0) * c->K / c->sm_count;
+    rule.g = g;
+    rule.known = true;
+    rule.tiles = groups * 5.1e-6 * 152.0 / c->sm_count > std::max(0.36, 0.1 + 0.145 * tiles) * rows / 8.0;
+    return rule.tiles;
+}
+
 // The direct FP32 surface with the candidates grouped by lag (k_corr_lag):
 // per batch of snapshots (within 4 GiB of sort arrays) the chunked-DFT path's
-// geometry and lag sort, then the correlation. *done = false where the lag
-// slots or the captures are out of its range (the tile kernel serves those).
+// geometry and lag sort, then the correlation. *done = false where the tile kernel
+// is the faster one (tiles_faster), and where the lag slots or the captures are out of
+// its range.
 static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *surf, void *out,
                                  bool refine, bool *done)
 {
@@ -894,6 +957,7 @@ static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz
     CdftLayout &L = refine ? b.dloc_layout : b.dmain_layout;
     for (int k = 0; k < c->K; ++k)
         if (c->steps[k].n > (1 << 24) || !c->steps[k].loaded) return DG_OK;
+    if (tiles_faster(c, gd, refine ? b.dloc_rule : b.dmain_rule)) return DG_OK;
     GridDev shape = gd;  // as in cdft_setup: a captured refinement's centre is known on the device only
     if (refine) {
         shape.lat0_rad = c->gd.lat0_rad;

@@ -56,3 +56,42 @@ def test_lag_groups_of_uneven_captures(fmt):
                                   idx=idx, acc_mode=1)
     ok = ~lag_boundary_mask(s, idx)
     assert rel_err(c[idx][ok], ref[ok], 0.01) < FP32_TOL
+
+
+def _launches(g):
+    P = package()
+    n0 = P.lib().dg_launch_count(g.ctx)
+    g.cost_surface()
+    return P.lib().dg_launch_count(g.ctx) - n0
+
+
+@pytest.mark.parametrize("acc", [0, 1], ids=["power", "mag"])
+def test_sparse_lags_keep_the_tile_kernel(acc):
+    """Where few candidates share a lag the tile kernel (and the sum over the
+    snapshots) runs: its rows per thread change no bit, a row shard is the whole
+    grid's rows, and the surface is the oracle's. The same grid on a short baseline
+    is grouped by lag."""
+    torch = torch_cuda()
+    kw = dict(seed=63, fs_hz=60e6, n_samples=50001, k_steps=8, fmt="ci8", waveform="noise", snr_db=-3.0, grid_n=201,
+              grid_spacing_m=2000.0, bw_hz=40e6)
+    s = sim.make_scene(formation=sim.Formation(sep_m=200e3), **kw)
+    D = oracle.node_geometry(s.grid, s.ephem, s.fs_hz, s.fc_hz)[0]
+    assert np.abs(D).min() < 45000 and s.G / np.ptp(D[0]) < 3.0
+    opts = dict(acc=["power", "mag"][acc])
+    g, c = gpu_surface(s, **opts)
+    assert _launches(g) == 2
+    g.close()
+    _check(s, c, acc, 150)
+    for rows in (4, 16):
+        h, x = gpu_surface(s, rows=rows, **opts)
+        assert _launches(h) == 2
+        h.close()
+        assert np.array_equal(x, c)
+    h, x = gpu_surface(s, row0=50, nrows=70, **opts)
+    assert _launches(h) == 2
+    h.close()
+    assert np.array_equal(x, c[50:120])
+    near = sim.make_scene(formation=sim.Formation(sep_m=10e3), **kw)
+    g, _ = gpu_surface(near, **opts)
+    assert _launches(g) > 2
+    g.close()
