@@ -160,9 +160,12 @@ typedef struct {
     int32_t scratch_mib; /* CDFT: target for the scratch of one batch of
                         snapshots (per-candidate arrays and per-lag DFTs),
                         MiB; 0 = 12288. Fewer snapshots per batch below it
-                        (at least one); many contexts sharing a GPU lower it */
-    int32_t rows;    /* DIRECT (not FP32 with INTEGER delay, whose candidates
-                        are grouped by lag): grid rows per thread, i.e. candidates per
+                        (at least one); many contexts sharing a GPU lower it.
+                        DIRECT, FP32 and INTEGER delay: the lag sort's
+                        scratch; where it does not fit one snapshot the
+                        candidates are not grouped                           */
+    int32_t rows;    /* DIRECT (FP32 with INTEGER delay only where its candidates
+                        are not grouped by lag: few to a lag, small scratch): grid rows per thread, i.e. candidates per
                         thread (a CTA takes 8 warps x rows grid rows x 32
                         grid columns of one snapshot); 0 = 8 (FP32,
                         INTEGER delay) or 4 (FP32 LAGRANGE4, FP64); FP32

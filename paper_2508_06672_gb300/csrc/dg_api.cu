@@ -45,6 +45,7 @@ struct CdftLayout {  // batches and bucket / group bases of one grid size
         int64_t nbt, groups;  // lag slots and combine groups (upper bounds)
     };
     int64_t G = -1;
+    int nseg = 0;           // segments of samples (direct surfaces)
     double diam = 0.0;      // grid diameter bound the lag slots were sized for
     std::vector<Batch> batches;
     int s_max = 0;
@@ -101,6 +102,7 @@ struct CdftBufs {  // chunked-DFT scratch, grown on demand
     CdftLayout main_layout, loc_layout;
     CdftLayout dmain_layout, dloc_layout;  // the direct path's lag groups
     LagRule dmain_rule, dloc_rule;
+    uint64_t no_sort = 0;                  // steps_gen at which the sort found no memory
     float2 *part = nullptr;                // and its segments' sums
     size_t part_cap = 0;
     std::vector<double> main_span;  // FDOA span estimates per snapshot (main grid)
@@ -944,32 +946,27 @@ static bool tiles_faster(const dg_ctx *c, const GridDev &gd, LagRule &rule)
     return rule.tiles;
 }
 
-// The direct FP32 surface with the candidates grouped by lag (k_corr_lag):
-// per batch of snapshots (within 4 GiB of sort arrays) the chunked-DFT path's
-// geometry and lag sort, then the correlation. *done = false where the tile kernel
-// is the faster one (tiles_faster), and where the lag slots or the captures are out of
-// its range.
-static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *surf, void *out,
-                                 bool refine, bool *done)
+// The batches of snapshots of a grouped surface, their lag tables, and the buffers of
+// its sort, within the scratch target: 24 bytes a node, and per snapshot (4 GiB at
+// most) 16 a node, a lag slot and a group, and 8 a node and segment of samples.
+// *fits = false where one snapshot needs more.
+static dg_status lag_batches(dg_ctx *c, CdftLayout &L, int64_t G, double diam, int nseg, bool *fits)
 {
-    *done = false;
     CdftBufs &b = c->cd;
-    CdftLayout &L = refine ? b.dloc_layout : b.dmain_layout;
-    for (int k = 0; k < c->K; ++k)
-        if (c->steps[k].n > (1 << 24) || !c->steps[k].loaded) return DG_OK;
-    if (tiles_faster(c, gd, refine ? b.dloc_rule : b.dmain_rule)) return DG_OK;
-    GridDev shape = gd;  // as in cdft_setup: a captured refinement's centre is known on the device only
-    if (refine) {
-        shape.lat0_rad = c->gd.lat0_rad;
-        shape.lon0_rad = c->gd.lon0_rad;
-    }
-    const double diam = grid_diameter(shape);
     dg_status st;
-    if (!(L.G == G && L.diam >= diam && !L.batches.empty())) {
+    *fits = false;
+    if (!(L.G == G && L.nseg == nseg && L.diam >= diam && !L.batches.empty())) {
+        const double budget = (double)(c->opt.scratch_mib > 0 ? c->opt.scratch_mib : 12288) * 1048576.0;
         CdftLayout n;
         n.G = G;
+        n.nseg = nseg;
         n.diam = diam;
-        const int s_max = (int)std::max(1.0, std::min((double)std::min(c->K, 65535), std::floor(4294967296.0 / (16.0 * (double)G))));
+        int slots_max = 1;
+        for (int k = 0; k < c->K; ++k) slots_max = std::max(slots_max, lag_slots(c->eph_host[k], c->fs, diam));
+        const double seg = nseg > 1 ? 8.0 * (double)G * nseg : 0.0;
+        const double per = 16.0 * ((double)G + 2.0 * slots_max + (double)G / kDirectGroup + 2.0) + seg;
+        const double sorts = std::min(4294967296.0, budget - 24.0 * (double)G);
+        const int s_max = (int)std::max(1.0, std::min((double)std::min(c->K, 65535), std::floor(sorts / per)));
         std::vector<int> bb, gb;
         for (int k0 = 0; k0 < c->K; k0 += s_max) {
             const int S = std::min(s_max, c->K - k0);
@@ -988,6 +985,7 @@ static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz
             n.nbt_max = std::max(n.nbt_max, t.nbt);
             n.groups_max = std::max(n.groups_max, t.groups);
         }
+        if (24.0 * (double)G + per * n.s_max > budget) return DG_OK;
         n.bbase = L.bbase;
         n.gbase = L.gbase;
         L = n;
@@ -999,6 +997,31 @@ static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz
         CK(c, cudaMemcpyAsync(L.gbase, gb.data(), sizeof(int) * gb.size(), cudaMemcpyHostToDevice, c->stream));
         L.G = G;
     }
+    const size_t S = (size_t)L.s_max, SG = S * (size_t)G;
+    if ((st = ensure_sort(c, S, SG, (size_t)L.nbt_max, (size_t)L.groups_max)) != DG_OK) return st;
+    if (nseg > 1 && (st = ensure(c, (void **)&b.part, &b.part_cap, sizeof(float2) * SG * nseg)) != DG_OK) return st;
+    if ((st = ensure_ephf(c)) != DG_OK) return st;
+    if ((st = ensure_xyzf(c, G)) != DG_OK) return st;
+    *fits = true;
+    return DG_OK;
+}
+
+// The direct FP32 surface with the candidates grouped by lag (k_corr_lag):
+// per batch of snapshots (lag_batches) the chunked-DFT path's
+// geometry and lag sort, then the correlation. *done = false where the tile kernel
+// is the faster one (tiles_faster), where the lag slots or the captures are out of
+// its range, and where the sort does not fit the scratch target, or the memory there
+// is: then until the shapes change, so that a captured step takes the same route.
+static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz, int64_t G, void *surf, void *out,
+                                 bool refine, bool *done)
+{
+    *done = false;
+    CdftBufs &b = c->cd;
+    CdftLayout &L = refine ? b.dloc_layout : b.dmain_layout;
+    for (int k = 0; k < c->K; ++k)
+        if (c->steps[k].n > (1 << 24) || !c->steps[k].loaded) return DG_OK;
+    if (tiles_faster(c, gd, refine ? b.dloc_rule : b.dmain_rule)) return DG_OK;
+    if (b.no_sort == c->steps_gen) return DG_OK;
     // segments of samples: enough warps for about 8 rounds of the chip at 48
     // warps per SM, from the whole grid's size (a row shard sums alike), in
     // multiples of 256 samples
@@ -1008,12 +1031,21 @@ static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz
     const int want = (int)std::min(64.0, std::ceil(8.0 * 48.0 * 152.0 / std::max(warps, 1.0)));
     const int seg_len = std::max(1, (nmax + 256 * want - 1) / (256 * want)) * 256;
     const int nseg = (nmax + seg_len - 1) / seg_len;
-    if ((st = push_steps(c)) != DG_OK) return st;
-    const size_t S = (size_t)L.s_max, SG = S * (size_t)G;
-    if ((st = ensure_sort(c, S, SG, (size_t)L.nbt_max, (size_t)L.groups_max)) != DG_OK) return st;
-    if (nseg > 1 && (st = ensure(c, (void **)&b.part, &b.part_cap, sizeof(float2) * SG * nseg)) != DG_OK) return st;
-    if ((st = ensure_ephf(c)) != DG_OK) return st;
-    if ((st = ensure_xyzf(c, G)) != DG_OK) return st;
+    GridDev shape = gd;  // as in cdft_setup: a captured refinement's centre is known on the device only
+    if (refine) {
+        shape.lat0_rad = c->gd.lat0_rad;
+        shape.lon0_rad = c->gd.lon0_rad;
+    }
+    dg_status st = push_steps(c);
+    if (st != DG_OK) return st;
+    bool fits = false;
+    st = lag_batches(c, L, G, grid_diameter(shape), nseg, &fits);
+    if (st == DG_ENOMEM) {
+        c->err.clear();
+        b.no_sort = c->steps_gen;
+        return DG_OK;
+    }
+    if (st != DG_OK || !fits) return st;
     const bool one = L.batches.size() == 1;
     {
         Timed t(c, refine ? DG_K_REFINE : DG_K_CORR);

@@ -11,6 +11,7 @@ namespace fake {
 std::map<char *, size_t> blocks;
 long allocations = 0, fail_at = 0, fail_count = 1;  // fail allocations fail_at .. fail_at + fail_count - 1
 bool failed = false, capturing = false;
+int sorts = 0;  // lag sorts launched
 cudaError_t error = cudaSuccess;  // what cudaGetLastError returns, once
 
 cudaError_t last()
@@ -170,6 +171,7 @@ cudaError_t launch_ecef_split(const double *xyz, int64_t G, float *xyzf, cudaStr
 }
 static void sorted(const CdftBatch &a)
 {
+    ++fake::sorts;
     const double SG = (double)a.S * a.G;
     bases(a);
     NEED(a.candL, SG), NEED(a.candNu, SG), NEED(a.order, SG), NEED(a.nuS, SG), NEED(a.g2b, a.ngroups);
@@ -509,8 +511,61 @@ static bool program(const dg_options &o, const std::vector<dg_grid> &grids, int 
     return good;
 }
 
+// The grouped direct surface keeps its sort within the scratch target, and a surface
+// that finds no memory for it is computed on the tiles.
+static void direct_scratch()
+{
+    dg_options o;
+    dg_options_default(&o);
+    const dg_grid g = grid_of(300, 301, 200.0);
+    const double G = 300.0 * 301.0;
+    const int K = 3, n = 4096;
+    std::vector<dg_ephem> eph((size_t)K);
+    for (dg_ephem &e : eph) {
+        e = dg_ephem{};
+        e.p1[0] = e.p2[0] = 6.9e6;
+        e.p2[1] = 5e4;
+        e.v1[1] = e.v2[1] = 7500.0;
+    }
+    std::vector<float> y((size_t)2 * n, 1.f);
+    float *cost = (float *)std::malloc(4 * (size_t)G);
+    fake::blocks[(char *)cost] = 4 * (size_t)G;
+    auto live = [] {
+        double b = 0.0;
+        for (const auto &x : fake::blocks) b += (double)x.second;
+        return b;
+    };
+    struct {
+        int mib, fail;
+        bool sorted;
+    } cases[] = {{0, 0, true}, {1, 0, false}, {4, 0, false}, {9, 0, true}, {16, 0, true}, {0, 2, false}, {0, 5, false}};
+    for (const auto &t : cases) {
+        fake::op = "direct scratch " + std::to_string(t.mib) + " " + std::to_string(t.fail);
+        o.scratch_mib = t.mib;
+        dg_ctx *c = nullptr;
+        if (dg_create(&g, eph.data(), K, 12.5e6, 1575.42e6, &o, (void *)0x100, &c) != DG_OK) fake::fault("dg_create", "");
+        for (int k = 0; k < K; ++k) dg_load_capture(c, k, DG_IQ_C64, y.data(), y.data(), n, 0);
+        const double before = live() + 4.0 * K * G;
+        fake::allocations = 0;
+        fake::fail_at = t.fail;
+        fake::sorts = 0;
+        for (int r = 0; r < 2; ++r, fake::fail_at = 0)
+            if (dg_cost_surface(c, cost) != DG_OK) fake::fault("dg_cost_surface", dg_last_error(c));
+        const double used = live() - before;
+        if ((fake::sorts > 0) != t.sorted) fake::fault("the wrong kernel", "");
+        if (t.mib && used > 1048576.0 * t.mib + 65536.0) fake::fault("scratch beyond its target", std::to_string(used).c_str());
+        dg_destroy(c);
+    }
+    fake::blocks.erase((char *)cost);
+    std::free(cost);
+}
+
 int main(int argc, char **argv)
 {
+    if (argc > 1 && std::string(argv[1]) == "scratch") {
+        direct_scratch();
+        return fake::faults ? 1 : 0;
+    }
     dg_options o;
     dg_options_default(&o);
     const std::string what = argc > 1 ? argv[1] : "maps";

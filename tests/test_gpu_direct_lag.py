@@ -95,3 +95,20 @@ def test_sparse_lags_keep_the_tile_kernel(acc):
     g, _ = gpu_surface(near, **opts)
     assert _launches(g) > 2
     g.close()
+
+
+def test_lag_groups_in_batches_of_snapshots():
+    """A small scratch target sorts one or two snapshots at a time, and a smaller
+    one takes the tile kernel: the grouped surfaces are equal bit for bit."""
+    s = sim.make_scene(seed=64, fs_hz=12.5e6, n_samples=3000, k_steps=5, fmt="ci16", waveform="noise", snr_db=-3.0,
+                       grid_n=(190, 181), grid_spacing_m=150.0, bw_hz=10e6)
+    surfs, launches = [], []
+    for mib in (0, 6, 4, 1):
+        g, c = gpu_surface(s, scratch_mib=mib)
+        surfs.append(c)
+        launches.append(_launches(g))
+        g.close()
+    assert launches[0] < launches[1] < launches[2] and launches[3] == 2
+    assert np.array_equal(surfs[1], surfs[0]) and np.array_equal(surfs[2], surfs[0])
+    _check(s, surfs[0])
+    _check(s, surfs[3])

@@ -32,3 +32,8 @@ def test_no_launch_on_buffers_that_a_failed_allocation_took(fake_device, what):
         out = r.communicate(timeout=300)[0]
         assert r.returncode == 0, out[-3000:]
         assert int(out.split(":")[1].split()[0]) > 100, out
+
+
+def test_direct_sort_keeps_to_the_scratch_target(fake_device):
+    r = subprocess.run([fake_device, "scratch"], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stdout
