@@ -521,7 +521,7 @@ static int lag_slots(const dg_ephem &e, double fs, double diam)
 {
     const double dx = e.p2[0] - e.p1[0], dy = e.p2[1] - e.p1[1], dz = e.p2[2] - e.p1[2];
     const double span = std::min(2.0 * std::sqrt(dx * dx + dy * dy + dz * dz), 2.0 * diam) * fs / kC;
-    return (int)std::ceil(span) + 6;
+    return (int)std::min(std::ceil(span), 1.0e9) + 6;
 }
 
 // FP64 WGS-84 node position on the host (planning only).
@@ -554,6 +554,20 @@ static double grid_diameter(const GridDev &g)
             d = std::max(d, std::sqrt((p[a][0] - p[b][0]) * (p[a][0] - p[b][0]) + (p[a][1] - p[b][1]) * (p[a][1] - p[b][1]) +
                                       (p[a][2] - p[b][2]) * (p[a][2] - p[b][2])));
     return 1.1 * d + 1.0;
+}
+
+// The diameter behind the lag slots of a direct surface over `shape`, the context's grid
+// or a refinement of it centred on any of its nodes: any two nodes' where the rows
+// come within 10 degrees of a pole, the longitudes go around half of the Earth or the
+// refinement is wide (there three rows and columns, or another centre's, bound
+// nothing; the slots then follow from the receivers' separation).
+static double direct_diameter(const dg_ctx *c, const GridDev &shape, bool refine)
+{
+    const GridDev &g = c->gd;
+    const double half = 0.5 * g.nlat * g.dlat_m / 6.33e6, ref = refine ? 0.5 * shape.nlat * shape.dlat_m / 6.33e6 : 0.0;
+    const double lon = shape.nlon * shape.dlon_m / (6.33e6 * std::cos(refine ? 1.39 : g.lat0_rad));
+    if (std::fabs(g.lat0_rad) + half + ref > 1.39 || ref > 0.02 || lon > 3.0) return 2.0 * kA;
+    return grid_diameter(shape);
 }
 
 // Curvature bounds of D (samples) and the FDOA (cycles per sample) at
@@ -1039,7 +1053,7 @@ static dg_status run_surface_lag(dg_ctx *c, const GridDev &gd, const double *xyz
     dg_status st = push_steps(c);
     if (st != DG_OK) return st;
     bool fits = false;
-    st = lag_batches(c, L, G, grid_diameter(shape), nseg, &fits);
+    st = lag_batches(c, L, G, direct_diameter(c, shape, refine), nseg, &fits);
     if (st == DG_ENOMEM) {
         c->err.clear();
         b.no_sort = c->steps_gen;

@@ -112,3 +112,20 @@ def test_lag_groups_in_batches_of_snapshots():
     assert np.array_equal(surfs[1], surfs[0]) and np.array_equal(surfs[2], surfs[0])
     _check(s, surfs[0])
     _check(s, surfs[3])
+
+
+@pytest.mark.parametrize("lat,grid,turns", [(78.0, (1, 301), 2.0), (84.0, (3, 257), 1.0), (85.5, (61, 67), 0.9)])
+def test_lag_slots_of_grids_around_a_pole(lat, grid, turns):
+    """Grids whose longitudes go around the Earth once or twice, so that their
+    corners and edge midpoints lie close together, and one over the pole."""
+    la = np.radians(lat)
+    radius = sim.WGS84_A / np.sqrt(1.0 - sim.WGS84_E2 * np.sin(la) ** 2) * np.cos(la)
+    spacing = turns * 2.0 * np.pi * radius / (grid[1] - 1)
+    s = sim.make_scene(seed=65, fs_hz=12.5e6, n_samples=4096, k_steps=2, fmt="ci16", waveform="noise", snr_db=-3.0,
+                       grid_n=grid, grid_spacing_m=spacing, bw_hz=10e6, emitter=(lat, 30.0))
+    g, c = gpu_surface(s)
+    assert _launches(g) > 2
+    fix = g.argmax_refine(g.cost_surface(), 100.0, 1000.0)
+    assert fix["refine_n"] == 21
+    g.close()
+    _check(s, c)
