@@ -592,6 +592,9 @@ static Curvature field_curvature(const dg_ctx *c, double rho, double sep, double
     return {d2 * c->fs / kC, n2 / (c->lambda * c->fs)};
 }
 
+// Longitudes of a grid's columns, from the first to the last (radians, a little more).
+static double lon_extent(const GridDev &g) { return g.nlon * g.dlon_m / (6.33e6 * std::cos(g.lat0_rad)); }
+
 // FDOA span of every snapshot over the shard, from a lattice of nodes (its
 // corners, edges and interior; the FDOA field is smooth at these scales): up
 // to 65 x 65 nodes, fewer on small shards (at least 9 x 9, about one lattice
@@ -612,7 +615,8 @@ static void fdoa_spans(const dg_ctx *c, const GridDev &g, std::vector<double> &s
             host_node_ecef(g, std::round(i), std::round(j), &p[3 * ((size_t)a * nj + b)]);
         }
     double h = 0.0;  // half the longest cell diagonal, with 5 % for the curvature within a cell
-    const bool low = std::fabs(g.lat0_rad) + 0.5 * g.nlat * g.dlat_m / 6.33e6 < 1.39;  // within 80 degrees
+    // within 80 degrees, and at most once around: lattice nodes whole turns apart bound nothing
+    const bool low = std::fabs(g.lat0_rad) + 0.5 * g.nlat * g.dlat_m / 6.33e6 < 1.39 && lon_extent(g) < 2.0 * kPi;
     if (range) {
         auto dist2 = [&](size_t q, size_t r) {
             const double *x = &p[3 * q], *y = &p[3 * r];
@@ -1797,7 +1801,8 @@ static dg_status refine_map(dg_ctx *c, const GridDev &gd, const double *xyz, int
     // the parallels' change of radius over up to 20 km at 80 degrees
     RefineBound rb;
     for (int i = 0; i < nmains; ++i) {
-        if (std::fabs(mains[i].lat0_rad) + 0.5 * mains[i].nlat * mains[i].dlat_m / 6.33e6 > 1.39) return DG_OK;
+        if (std::fabs(mains[i].lat0_rad) + 0.5 * mains[i].nlat * mains[i].dlat_m / 6.33e6 > 1.39 || lon_extent(mains[i]) > 3.0)
+            return DG_OK;
         const RefineBound q = refine_bound(c, mains[i]);
         const double rho = std::min(rb.rho, q.rho);
         rb = q;
@@ -3377,7 +3382,8 @@ dg_status dg_coarse_inspect(dg_ctx *c, float *caf, dg_coarse_step *steps, int32_
 // it (field_curvature); false where none hold.
 static bool region_range(const dg_ctx *c, const GridDev &g, GridRange *out)
 {
-    if (std::fabs(g.lat0_rad) + 0.5 * g.nlat * g.dlat_m / 6.33e6 > 1.39) return false;
+    // three columns bound less than half a turn
+    if (std::fabs(g.lat0_rad) + 0.5 * g.nlat * g.dlat_m / 6.33e6 > 1.39 || lon_extent(g) > 3.0) return false;
     double p[9][3], hi = 0.0, hj = 0.0;
     auto norm = [](double x, double y, double z) { return std::sqrt(x * x + y * y + z * z); };
     auto dist = [&](int a, int b) { return norm(p[a][0] - p[b][0], p[a][1] - p[b][1], p[a][2] - p[b][2]); };

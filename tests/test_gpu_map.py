@@ -181,3 +181,25 @@ def test_regions_searched_together_match_fresh_contexts():
     g.set_grid(s.grid)  # the context goes on on its own grid
     assert torch.equal(g.cost_surface(), before)
     g.close()
+
+
+def test_regions_that_go_around_the_earth():
+    """Regions whose first, middle and last columns coincide (two turns): three
+    columns bound nothing there, and the regions are searched as fresh contexts."""
+    torch = torch_cuda()
+    P = package()
+    spacing = 4.0 * np.pi * sim.WGS84_A / 2730
+    s = sim.make_scene(seed=46, fs_hz=12.5e6, n_samples=4096, k_steps=2, fmt="ci16", waveform="noise", snr_db=-3.0,
+                       grid_n=(3, 2731), grid_spacing_m=spacing, bw_hz=10e6, emitter=(0.0, 30.0))
+    regions = [dict(s.grid, lon0_deg=s.grid["lon0_deg"] + d) for d in (0.0, 1.0)]
+    g = P.Geolocator(s.grid, s.ephem, s.fs_hz, s.fc_hz, algo="cdft", contract="fp16x3")
+    g.load_captures(s.fmt, torch.from_numpy(s.y1).cuda(), torch.from_numpy(s.y2).cuda())
+    _, _, costs = g.search_regions(regions, 100.0, 1000.0)
+    for reg, c in zip(regions, costs.double().cpu().numpy()):
+        idx = np.unique(np.random.default_rng(5).integers(0, s.G, 700))
+        ref = oracle.cost_points(reg, s.ephem, s.fs_hz, s.fc_hz, oracle.iq_to_f64(s.y1), oracle.iq_to_f64(s.y2), idx=idx)
+        ok = ~lag_boundary_mask(s, idx) if reg is regions[0] else np.ones(idx.size, bool)
+        D = oracle.node_geometry(reg, s.ephem, s.fs_hz, s.fc_hz)[0].reshape(s.k_steps, -1)[:, idx]
+        ok &= (np.abs(D - np.floor(D) - 0.5) > 1e-6).all(axis=0)
+        assert rel_err(c.ravel()[idx][ok], ref[ok], 0.01) < FP32_TOL
+    g.close()
