@@ -571,10 +571,20 @@ __device__ __forceinline__ void weights6(float s, float (&w)[6])
     w[5] = fmaf(s, c.y, c.x);
 }
 
+// Whether a table of NL lags and Q bins holds lag l (from its first) and the six bins
+// around bin coordinate U0 + u (Lagrange4 reads the lags l - 1 .. l + 2).
+template <bool FRAC> __device__ __forceinline__ bool in_table(int l, int NL, int U0, float u, int Q)
+{
+    int k;
+    round_magic(u - 0.5f, k);
+    return (unsigned)(FRAC ? l - 1 : l) < (unsigned)(FRAC ? NL - 3 : NL) && (unsigned)(U0 + k - 2) <= (unsigned)(Q - 6);
+}
+
 // One candidate and snapshot, at bin coordinate U0 + u: |C|^2 or |C|. BAD:
 // some capture may hold samples that are not finite. The host's bounds keep
-// lag and bins inside the table; an index that still falls outside reads its
-// start.
+// lag and bins inside the table, which the callers check (in_table: a node outside
+// reports itself, as to the lag sort of the contraction); an index that falls
+// outside of its memory reads its start.
 template <bool FRAC, bool BAD>
 __device__ __forceinline__ float map_value(const MapArgs &a, const float2 *__restrict__ X, int s, int L0, int L,
                                            float mu, int U0, float u)
@@ -667,6 +677,7 @@ __device__ __forceinline__ float2 poly_offset(const MapArgs &a, int r, int c)  /
 }
 
 constexpr int kPolyWarps = 8;
+static_assert(4 + 2 * kPolyTerms + 2 <= kPolyStride, "the flag lies behind the terms");
 __global__ void __launch_bounds__(32 * kPolyWarps) k_map_poly(MapArgs a, int tiles_j, int64_t pairs)
 {
     __shared__ float s_fit[kPolyTerms][kPolyPts + 1];
@@ -714,8 +725,8 @@ __global__ void __launch_bounds__(32 * kPolyWarps) k_map_poly(MapArgs a, int til
     s_val[warp][lane] = make_float2(((D.hi - I0) - fmaf(gr, o.x, gc * o.y)) + D.lo, du);
     __syncwarp();
     float *out = a.coef + (size_t)w * kPolyStride;
+    float2 c = make_float2(0.f, 0.f);
     if (lane < kPolyTerms) {
-        float2 c = make_float2(0.f, 0.f);
 #pragma unroll 8
         for (int i = 0; i < kPolyPts; ++i) {
             const float2 v = s_val[warp][i];
@@ -725,6 +736,24 @@ __global__ void __launch_bounds__(32 * kPolyWarps) k_map_poly(MapArgs a, int til
         *reinterpret_cast<float2 *>(out + 4 + 2 * lane) = c;
     } else if (lane == kPolyTerms) {
         *reinterpret_cast<float4 *>(out) = make_float4(I0, U0, gr, gc);
+    }
+    // D and the bin coordinate over the tile: the constant terms and the sums of the
+    // others' magnitudes (the offsets are at most 1). 1 behind the terms where
+    // that does not put every node of the tile inside the table: the lookup then checks
+    // each (checking all of them there cost 7 % of the large lookup).
+    const float2 mid0 = make_float2(__shfl_sync(all, c.x, 0), __shfl_sync(all, c.y, 0));
+    float rd = lane ? fabsf(c.x) : fabsf(gr) * hr + fabsf(gc) * hc, ru = lane ? fabsf(c.y) : 0.f;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        rd += __shfl_xor_sync(all, rd, d);
+        ru += __shfl_xor_sync(all, ru, d);
+    }
+    if (lane == kPolyTerms + 1) {
+        const bool frac = a.delay != DG_DELAY_INTEGER;
+        const float dm = (I0 - (float)ms.L0) + mid0.x, um = U0 + mid0.y;
+        const float m = frac ? 1.01f : 0.51f, p = frac ? 2.01f : 0.51f;
+        const bool in = dm - rd > m && dm + rd < (float)(ms.NL - 1) - p && um - ru > 2.01f && um + ru < (float)a.Q - 3.01f;
+        *reinterpret_cast<float2 *>(out + 4 + 2 * kPolyTerms) = make_float2(in ? 0.f : 1.f, 0.f);
     }
 }
 
@@ -758,6 +787,7 @@ __global__ void __launch_bounds__(256, 4) k_map_lookup_poly(MapArgs a, int tiles
         // polynomials in the row offset: x D, y bin coordinate; terms of
         // r^0 (c^0..5), r^1 (c^0..4), r^2 (c^0..3), ...
         float2 cr[6];
+        bool check;
         {
             float2 m[22];
 #pragma unroll
@@ -775,9 +805,28 @@ __global__ void __launch_bounds__(256, 4) k_map_lookup_poly(MapArgs a, int tiles
                 cr[e] = h;
                 at += 6 - e;
             }
+            check = m[21].x != 0.f;  // k_map_poly: some node of the tile may lie outside the table
         }
         const float lin_c = head.w * o.y;
         const int I0 = (int)head.x, U0 = (int)head.y;
+        if (check) {
+            const int NL = a.snap[s].NL;
+#pragma unroll 1
+            for (int r = 0; r < R; ++r) {
+                const float rr = o.x + 4.f * r, un = rr * (2.f / (float)(TR - 1));
+                const float2 un2 = make_float2(un, un);
+                float2 h = cr[5];
+#pragma unroll
+                for (int e = 4; e >= 0; --e) h = fma2(h, un2, cr[e]);
+                const float lin = fmaf(head.z, rr, lin_c);
+                int n1, n2;
+                const float t = (lin - round_magic(lin, n1)) + h.x;
+                round_magic(FRAC ? t - 0.5f : t, n2);
+                // an integer lag next to its rounding boundary may be the next one
+                if (i0 + 4 * r < a.nrows && j < a.nlon && !in_table<FRAC>(I0 + n1 + n2 - L0, NL, U0, h.y, a.Q))
+                    atomicOr(a.err, ERR_LAG_RANGE);
+            }
+        }
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const float rr = o.x + 4.f * r;
@@ -844,6 +893,7 @@ template <bool FRAC, bool BAD, int WK> __global__ void __launch_bounds__(256) k_
             if (map_node<FRAC>(a, ms, s, xyz_r + p, xyz, L, mu, u)) {
                 int U0;
                 const float uf = round_magic(u, U0);
+                if (!in_table<FRAC>(L - ms.L0, ms.NL, U0, u - uf, a.Q) && ok) atomicOr(a.err, ERR_LAG_RANGE);
                 v = map_value<FRAC, BAD>(a, X + (size_t)s * a.Q * a.NLpad, s, ms.L0, L, mu, U0, u - uf);
             } else if (ok) {
                 atomicOr(a.err, ERR_LAG_RANGE);
