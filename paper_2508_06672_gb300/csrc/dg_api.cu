@@ -12,7 +12,9 @@
 #include <atomic>
 #include <climits>
 #include <cstring>
+#include <list>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -46,6 +48,7 @@ struct CdftLayout {  // batches and bucket / group bases of one grid size
     };
     int64_t G = -1;
     int nseg = 0;           // segments of samples (direct surfaces)
+    bool direct = false;    // lag groups of direct surfaces
     double diam = 0.0;      // grid diameter bound the lag slots were sized for
     std::vector<Batch> batches;
     int s_max = 0;
@@ -92,6 +95,12 @@ struct MapBufs {  // their device tables and scratch, grown on demand
     int tw_logn = 0, T_P = 0, T_Q = 0;  // what tw and T hold
 };
 
+struct BatchHold {  // a batch's replays read a context's buffers
+    cudaEvent_t last = nullptr;  // recorded behind its latest replay
+    uint64_t gen = 0;            // the context's steps_gen that the replays need
+    std::atomic<bool> alive{true};
+};
+
 struct LagRule {  // tiles_faster's answer for one grid
     GridDev g{};
     bool known = false, tiles = false;
@@ -101,6 +110,7 @@ struct CdftBufs {  // chunked-DFT scratch, grown on demand
     int *lr = nullptr;
     CdftLayout main_layout, loc_layout;
     CdftLayout dmain_layout, dloc_layout;  // the direct path's lag groups
+    std::list<CdftLayout> kept;            // layouts of other shapes, while a captured step may read their tables
     LagRule dmain_rule, dloc_rule;
     uint64_t no_sort = 0;                  // steps_gen at which the sort found no memory
     float2 *part = nullptr;                // and its segments' sums
@@ -225,8 +235,8 @@ struct dg_ctx {
     int64_t graph_launches = 0;         // kernels per replay
     uint64_t steps_gen = 1, graph_gen = 0;  // capture buffers / formats / lengths generation
     std::string err;
-    bool captured = false;              // a graph or a batch holds pointers into this context's buffers
-    std::vector<void *> retired;        // buffers replaced since: freed with the context
+    std::vector<std::shared_ptr<BatchHold>> holds;  // of batches that hold pointers into this context's buffers
+    std::vector<void *> retired;        // buffers replaced while a captured step may replay on them (held)
     int64_t launches = 0;
     std::vector<TimedLaunch> pending;
     double ms[DG_K_NCLASS] = {};
@@ -322,17 +332,77 @@ dg_status check_latched(dg_ctx *c)
     return DG_OK;
 }
 
-// Give a buffer back, or keep it until the context goes when a captured step
-// may still replay on it.
+// Whether a captured step may still read this context's buffers: its own graph while
+// it can be launched (its replays lie before what is freed on the stream), a batch
+// while it can be launched or runs on its own stream.
+static bool held(dg_ctx *c)
+{
+    auto runs = [](const BatchHold &h) {
+        const bool busy = cudaEventQuery(h.last) != cudaSuccess;
+        if (busy) cudaGetLastError();  // not an error of the next launch's
+        return busy;
+    };
+    for (size_t i = 0; i < c->holds.size();) {
+        const BatchHold &h = *c->holds[i];
+        if (!h.alive || (h.gen != c->steps_gen && !runs(h))) {
+            c->holds[i] = c->holds.back();
+            c->holds.pop_back();
+        } else {
+            ++i;
+        }
+    }
+    return !c->holds.empty() || (c->graph && c->graph_gen == c->steps_gen);
+}
+
+// The buffers that were kept for captured steps, once no such step is left.
+static dg_status give_back(dg_ctx *c)
+{
+    if ((c->retired.empty() && c->cd.kept.empty()) || held(c)) return DG_OK;
+    for (void *p : c->retired) CK(c, cudaFreeAsync(p, c->stream));
+    c->retired.clear();
+    for (const CdftLayout &L : c->cd.kept)
+        for (int *p : {L.bbase, L.gbase})
+            if (p) CK(c, cudaFreeAsync(p, c->stream));
+    c->cd.kept.clear();
+    return DG_OK;
+}
+
+// Give a buffer back, or keep it while a captured step may still replay on it.
 dg_status release(dg_ctx *c, void *p)
 {
-    if (!p) return DG_OK;
-    if (c->captured) {
+    const dg_status st = give_back(c);
+    if (st != DG_OK || !p) return st;
+    if (held(c)) {
         c->retired.push_back(p);
         return DG_OK;
     }
     CK(c, cudaFreeAsync(p, c->stream));
     return DG_OK;
+}
+
+// Make room for another layout in L: the old one is kept where a captured step may
+// read its tables, one of the shape asked for comes back (then true): a program
+// that alternates between refinement windows holds one layout of each.
+static bool swap_layout(dg_ctx *c, CdftLayout &L, int64_t G, int nseg, double diam, bool direct)
+{
+    auto fits = [&](const CdftLayout &k) {
+        return k.G == G && k.nseg == nseg && k.diam >= diam && k.direct == direct && !k.batches.empty();
+    };
+    if (fits(L)) return true;
+    if (L.G >= 0 && L.bbase && held(c)) {
+        c->cd.kept.push_back(L);
+        L = CdftLayout{};
+    }
+    for (auto k = c->cd.kept.begin(); k != c->cd.kept.end(); ++k) {
+        if (!fits(*k)) continue;
+        int *const old[2] = {L.bbase, L.gbase};
+        L = *k;
+        c->cd.kept.erase(k);
+        for (int *p : old)
+            if (p && release(c, p) != DG_OK) break;
+        return true;
+    }
+    return false;
 }
 
 // Device and pinned host memory. A failed call leaves *p NULL, and no error for
@@ -768,7 +838,7 @@ static dg_status cdft_batches(dg_ctx *c, int64_t G, double diam, CdftLayout &L, 
 static dg_status cdft_layout(dg_ctx *c, const GridDev &gd, int64_t G, CdftLayout &L)
 {
     const double diam = grid_diameter(gd);
-    if (L.G == G && L.diam >= diam && !L.batches.empty()) return DG_OK;
+    if (swap_layout(c, L, G, 0, diam, false)) return DG_OK;
     int *old_bb = L.bbase, *old_gb = L.gbase;
     L = CdftLayout{};
     L.diam = diam;
@@ -973,11 +1043,12 @@ static dg_status lag_batches(dg_ctx *c, CdftLayout &L, int64_t G, double diam, i
     CdftBufs &b = c->cd;
     dg_status st;
     *fits = false;
-    if (!(L.G == G && L.nseg == nseg && L.diam >= diam && !L.batches.empty())) {
+    if (!swap_layout(c, L, G, nseg, diam, true)) {
         const double budget = (double)(c->opt.scratch_mib > 0 ? c->opt.scratch_mib : 12288) * 1048576.0;
         CdftLayout n;
         n.G = G;
         n.nseg = nseg;
+        n.direct = true;
         n.diam = diam;
         int slots_max = 1;
         for (int k = 0; k < c->K; ++k) slots_max = std::max(slots_max, lag_slots(c->eph_host[k], c->fs, diam));
@@ -2133,7 +2204,7 @@ static dg_status set_grid(dg_ctx *c, const dg_grid *grid, const double *xyz, con
         c->xyz = nullptr;
         c->xyz_cap = 0;
         ++c->steps_gen;
-        if (old) CK(c, cudaFreeAsync(old, c->stream));
+        if ((st = release(c, old)) != DG_OK) return st;
         CK(c, device_alloc(c, &c->xyz, sizeof(double) * 3 * (size_t)G));
         c->xyz_cap = G;
     }
@@ -2179,8 +2250,10 @@ dg_status dg_load_capture(dg_ctx *c, int32_t step, int32_t fmt, const void *y1, 
         s.cap = 0;
         s.loaded = false;
         ++c->steps_gen;  // also where the allocation fails: captured steps read the old buffers
-        for (void *p : old)
-            if (p) CK(c, cudaFreeAsync(p, c->stream));
+        for (void *p : old) {
+            const dg_status st = release(c, p);
+            if (st != DG_OK) return st;
+        }
         CK(c, device_alloc(c, &s.y1, bytes));
         CK(c, device_alloc(c, &s.y2, bytes));
         s.cap = bytes;
@@ -2651,6 +2724,7 @@ dg_status dg_graph_capture(dg_ctx *c, void *cost, double spacing_m, double windo
         cudaGraphExecDestroy(c->graph);
         c->graph = nullptr;
     }
+    if ((st = give_back(c)) != DG_OK) return st;
     // one uncaptured step allocates and plans everything; then the capture
     if ((st = prepare_step(c, half)) != DG_OK) return st;
     if ((st = step_device(c, cost, spacing_m, half)) != DG_OK) return st;
@@ -2661,7 +2735,6 @@ dg_status dg_graph_capture(dg_ctx *c, void *cost, double spacing_m, double windo
     if ((st = capture_steps(cs, 1, costs, spacing_m, &half, c->stream, &c->graph, &c->graph_launches)) != DG_OK)
         return st;
     c->graph_gen = c->steps_gen;
-    c->captured = true;
     return DG_OK;
 }
 
@@ -2692,6 +2765,8 @@ struct dg_batch {
     std::vector<dg_ctx *> ctxs;
     std::vector<uint64_t> gens;
     std::vector<cudaEvent_t> ready;  // work queued on each context's stream
+    std::vector<std::shared_ptr<BatchHold>> holds;  // of the contexts
+    cudaEvent_t last = nullptr;      // behind the latest replay
     cudaStream_t stream = nullptr;
     cudaGraphExec_t graph = nullptr;
     int64_t launches = 0;
@@ -2731,13 +2806,12 @@ dg_status dg_batch_capture(dg_ctx *const *ctxs, int32_t n, void *const *costs, d
     b->ctxs.assign(ctxs, ctxs + n);
     for (int i = 0; i < n; ++i) b->gens.push_back(ctxs[i]->steps_gen);
     b->ready.assign((size_t)n, nullptr);
-    for (auto &e : b->ready)
-        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
-            for (auto &x : b->ready)
-                if (x) cudaEventDestroy(x);
-            delete b;
-            return fail(nullptr, DG_ECUDA, "event creation failed");
-        }
+    bool events = cudaEventCreateWithFlags(&b->last, cudaEventDisableTiming) == cudaSuccess;
+    for (auto &e : b->ready) events = events && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+    if (!events) {
+        dg_batch_destroy(b);
+        return fail(nullptr, DG_ECUDA, "event creation failed");
+    }
     b->stream = s;
     dg_status st = tc_rounds(ctxs, n, b->rounds, b->shared);
     if (st == DG_OK)
@@ -2745,12 +2819,16 @@ dg_status dg_batch_capture(dg_ctx *const *ctxs, int32_t n, void *const *costs, d
                            b->shared ? &b->rounds : nullptr);
     if (st != DG_OK) {
         const std::string m = ctxs[0]->err;
-        for (auto &e : b->ready) cudaEventDestroy(e);
-        tc_rounds_free(b->rounds);
-        delete b;
+        dg_batch_destroy(b);
         return fail(nullptr, st, "%s", m.c_str());
     }
-    for (int i = 0; i < n; ++i) ctxs[i]->captured = true;
+    for (int i = 0; i < n; ++i) {
+        auto h = std::make_shared<BatchHold>();
+        h->last = b->last;
+        h->gen = ctxs[i]->steps_gen;
+        b->holds.push_back(h);
+        ctxs[i]->holds.push_back(h);
+    }
     *out = b;
     return DG_OK;
 }
@@ -2770,6 +2848,8 @@ dg_status dg_batch_launch(dg_batch *b)
     }
     const cudaError_t e = cudaGraphLaunch(b->graph, b->stream);
     if (e != cudaSuccess) return fail(nullptr, DG_ECUDA, "cudaGraphLaunch: %s", cudaGetErrorString(e));
+    const cudaError_t r = cudaEventRecord(b->last, b->stream);
+    if (r != cudaSuccess) return fail(nullptr, DG_ECUDA, "cudaEventRecord: %s", cudaGetErrorString(r));
     return DG_OK;
 }
 
@@ -2798,7 +2878,11 @@ int64_t dg_batch_launch_count(const dg_batch *b) { return b ? b->launches : -1; 
 dg_status dg_batch_destroy(dg_batch *b)
 {
     if (!b) return DG_OK;
+    // the contexts may free what its replays read once they are done
+    if (b->last) cudaEventSynchronize(b->last);
+    for (auto &h : b->holds) h->alive = false;
     if (b->graph) cudaGraphExecDestroy(b->graph);
+    if (b->last) cudaEventDestroy(b->last);
     for (auto &e : b->ready)
         if (e) cudaEventDestroy(e);
     tc_rounds_free(b->rounds);
@@ -3064,6 +3148,10 @@ dg_status dg_destroy(dg_ctx *c)
         if (p) cudaFreeAsync(p, s);
     };
     for (void *p : c->retired) fr(p);
+    for (const CdftLayout &L : c->cd.kept) {
+        fr(L.bbase);
+        fr(L.gbase);
+    }
     fr(c->xyz);
     fr(c->gstep);
     fr(c->reg_steps);

@@ -11,7 +11,8 @@ namespace fake {
 std::map<char *, size_t> blocks;
 long allocations = 0, fail_at = 0, fail_count = 1;  // fail allocations fail_at .. fail_at + fail_count - 1
 bool failed = false, capturing = false;
-int sorts = 0;  // lag sorts launched
+int sorts = 0;      // lag sorts launched
+bool busy = false;  // a batch's replay still runs
 cudaError_t error = cudaSuccess;  // what cudaGetLastError returns, once
 
 cudaError_t last()
@@ -117,6 +118,10 @@ RUNTIME(cudaError_t, cudaEventDestroy, (cudaEvent_t)) { return cudaSuccess; }
 RUNTIME(cudaError_t, cudaEventElapsedTime, (float *t, cudaEvent_t, cudaEvent_t)) { return *t = 1.f, cudaSuccess; }
 RUNTIME(cudaError_t, cudaEventRecord, (cudaEvent_t, cudaStream_t)) { return cudaSuccess; }
 RUNTIME(cudaError_t, cudaEventSynchronize, (cudaEvent_t)) { return cudaSuccess; }
+RUNTIME(cudaError_t, cudaEventQuery, (cudaEvent_t))
+{
+    return fake::busy ? fake::error = cudaErrorNotReady : cudaSuccess;
+}
 RUNTIME(cudaError_t, cudaStreamWaitEvent, (cudaStream_t, cudaEvent_t, unsigned)) { return cudaSuccess; }
 RUNTIME(cudaError_t, cudaStreamBeginCapture, (cudaStream_t, cudaStreamCaptureMode)) { return fake::capturing = true, cudaSuccess; }
 RUNTIME(cudaError_t, cudaStreamEndCapture, (cudaStream_t, cudaGraph_t *g))
@@ -560,8 +565,90 @@ static void direct_scratch()
     std::free(cost);
 }
 
+// Buffers replaced while a captured step may read them are kept, and given back once
+// it cannot be launched and does not run any more: a program that alternates between
+// windows and grids beside its graph or batch holds no more and more of them.
+static void kept_buffers(bool cdft)
+{
+    dg_options o;
+    dg_options_default(&o);
+    if (cdft) {
+        o.algo = DG_ALGO_CDFT;
+        o.contract = DG_CONTRACT_FP16X3;
+        o.chunk = 512;
+    }
+    const dg_grid a = grid_of(40, 41, 200.0), b = grid_of(44, 45, 300.0);
+    const int K = 2, n = 4096;
+    std::vector<dg_ephem> eph((size_t)K);
+    for (dg_ephem &e : eph) {
+        e = dg_ephem{};
+        e.p1[0] = e.p2[0] = 6.9e6;
+        e.p2[1] = 5e4;
+        e.v1[1] = e.v2[1] = 7500.0;
+    }
+    std::vector<float> y((size_t)2 * n, 1.f);
+    float *cost = (float *)std::malloc(4 * 45 * 45);
+    fake::blocks[(char *)cost] = 4 * 45 * 45;
+    dg_ctx *c = nullptr;
+    dg_fix fix;
+    fake::fail_at = 0;
+    auto ok = [&](dg_status st, const char *what) {
+        if (st != DG_OK) fake::fault(dg_last_error(c), what);
+    };
+    ok(dg_create(&a, eph.data(), K, 12.5e6, 1575.42e6, &o, (void *)0x100, &c), "dg_create");
+    for (int k = 0; k < K; ++k) ok(dg_load_capture(c, k, DG_IQ_C64, y.data(), y.data(), n, 0), "dg_load_capture");
+    auto windows = [&](int times) {
+        for (int i = 0; i < times; ++i)
+            for (double w : {60.0, 100.0, 140.0}) {
+                ok(dg_cost_surface(c, cost), "dg_cost_surface");
+                ok(dg_argmax_refine(c, cost, 20.0, w, &fix), "dg_argmax_refine");
+            }
+    };
+    auto grids = [&](int times) {
+        for (int i = 0; i < times; ++i)
+            for (const dg_grid *g : {&b, &a}) {
+                ok(dg_set_grid(c, g), "dg_set_grid");
+                windows(1);
+            }
+    };
+    auto growth = [&](const char *what, auto f) {  // blocks that 20 further rounds add
+        fake::op = what;
+        f(2);
+        const size_t before = fake::blocks.size();
+        f(20);
+        if (fake::blocks.size() > before) fake::fault(what, "keeps more and more buffers");
+        return fake::blocks.size();
+    };
+    const size_t none = growth("no captured step", grids);
+    ok(dg_graph_capture(c, cost, 20.0, 60.0), "dg_graph_capture");
+    growth("windows beside a graph", windows);
+    ok(dg_graph_launch(c), "dg_graph_launch");
+    if (growth("grids beside a stale graph", grids) > none + 2) fake::fault("a stale graph", "keeps its buffers");
+    dg_batch *bt = nullptr;
+    void *costs[1] = {cost};
+    ok(dg_batch_capture(&c, 1, costs, 20.0, 60.0, (void *)0x200, &bt), "dg_batch_capture");
+    growth("windows beside a batch", windows);
+    ok(dg_batch_launch(bt), "dg_batch_launch");
+    fake::busy = true;  // its replay still reads the old grid's tables
+    const size_t at = fake::blocks.size();
+    grids(1);
+    if (fake::blocks.size() <= at) fake::fault("a running batch", "lost its buffers");
+    fake::busy = false;
+    if (growth("grids beside a stale batch", grids) > none + 2) fake::fault("a stale batch", "keeps its buffers");
+    dg_batch_destroy(bt);
+    dg_destroy(c);
+    fake::blocks.erase((char *)cost);
+    std::free(cost);
+    fake::op = "the end";
+    if (!fake::blocks.empty()) fake::fault("buffers never given back,", std::to_string(fake::blocks.size()).c_str());
+}
+
 int main(int argc, char **argv)
 {
+    if (argc > 1 && std::string(argv[1]).rfind("kept", 0) == 0) {
+        kept_buffers(std::string(argv[1]) == "kept-cdft");
+        return fake::faults ? 1 : 0;
+    }
     if (argc > 1 && std::string(argv[1]) == "scratch") {
         direct_scratch();
         return fake::faults ? 1 : 0;

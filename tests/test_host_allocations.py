@@ -37,3 +37,9 @@ def test_no_launch_on_buffers_that_a_failed_allocation_took(fake_device, what):
 def test_direct_sort_keeps_to_the_scratch_target(fake_device):
     r = subprocess.run([fake_device, "scratch"], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout
+
+
+@pytest.mark.parametrize("what", ["kept-direct", "kept-cdft"])
+def test_buffers_of_captured_steps_are_given_back(fake_device, what):
+    r = subprocess.run([fake_device, what], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stdout
