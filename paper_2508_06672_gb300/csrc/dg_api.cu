@@ -49,6 +49,7 @@ struct CdftLayout {  // batches and bucket / group bases of one grid size
     int64_t G = -1;
     int nseg = 0;           // segments of samples (direct surfaces)
     bool direct = false;    // lag groups of direct surfaces
+    std::vector<int> fmts;  // the captures' formats (a batch of the contraction has one)
     double diam = 0.0;      // grid diameter bound the lag slots were sized for
     std::vector<Batch> batches;
     int s_max = 0;
@@ -386,7 +387,10 @@ dg_status release(dg_ctx *c, void *p)
 static bool swap_layout(dg_ctx *c, CdftLayout &L, int64_t G, int nseg, double diam, bool direct)
 {
     auto fits = [&](const CdftLayout &k) {
-        return k.G == G && k.nseg == nseg && k.diam >= diam && k.direct == direct && !k.batches.empty();
+        if (k.G != G || k.nseg != nseg || k.diam < diam || k.direct != direct || k.batches.empty()) return false;
+        for (size_t i = 0; i < k.fmts.size(); ++i)
+            if (k.fmts[i] != c->steps[i].fmt) return false;
+        return true;
     };
     if (fits(L)) return true;
     if (L.G >= 0 && L.bbase && held(c)) {
@@ -842,6 +846,7 @@ static dg_status cdft_layout(dg_ctx *c, const GridDev &gd, int64_t G, CdftLayout
     int *old_bb = L.bbase, *old_gb = L.gbase;
     L = CdftLayout{};
     L.diam = diam;
+    for (const Step &t : c->steps) L.fmts.push_back(t.fmt);
     L.bbase = old_bb;
     L.gbase = old_gb;
     std::vector<int> bb, gb;

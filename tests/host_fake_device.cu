@@ -225,17 +225,19 @@ cudaError_t launch_cdft_tiles(const CdftBatch &a, cudaStream_t)
     NEED(a.tbase, a.S + 1), NEED(a.hbase, a.S + 1), NEED(a.layout, a.S), NEED(a.Mcs, a.S);
     return fake::last();
 }
-static cudaError_t contract(const CdftBatch &a)
+static cudaError_t contract(const CdftBatch &a, int fmt)
 {
+    for (int s = 0; NEED(a.sd, a.S) && s < a.S; ++s)
+        if (a.sd[s].fmt != fmt) fake::fault("a capture", "of another format than its batch's");
     captures(a.sd, a.S);
     bases(a);
     NEED(a.tbase, a.S + 1), NEED(a.nubase, a.S), NEED(a.delta, a.S);
     if (NEED(a.bbase, a.S + 1)) NEED(a.W, (double)a.bbase[a.S] * a.Bmax * 128), NEED(a.need, a.bbase[a.S]);
     return fake::last();
 }
-cudaError_t launch_cdft_contract_fp32(const CdftBatch &a, int, int, cudaStream_t) { return contract(a); }
-cudaError_t launch_cdft_contract_mma(const CdftBatch &a, int, int, int, cudaStream_t) { return contract(a); }
-cudaError_t launch_cdft_contract_hankel(const CdftBatch &a, int, int, int, cudaStream_t) { return contract(a); }
+cudaError_t launch_cdft_contract_fp32(const CdftBatch &a, int, int fmt, cudaStream_t) { return contract(a, fmt); }
+cudaError_t launch_cdft_contract_mma(const CdftBatch &a, int, int fmt, int, cudaStream_t) { return contract(a, fmt); }
+cudaError_t launch_cdft_contract_hankel(const CdftBatch &a, int, int fmt, int, cudaStream_t) { return contract(a, fmt); }
 size_t cdft_btab_bytes(int, int M) { return (size_t)M * 256; }
 cudaError_t launch_cdft_btab(const CdftBatch &a, int mode, void *btab, cudaStream_t)
 {
@@ -620,6 +622,13 @@ static void kept_buffers(bool cdft)
         return fake::blocks.size();
     };
     const size_t none = growth("no captured step", grids);
+    fake::op = "another format";  // the batches of snapshots have one each
+    for (int k : {1, 0, 1}) {
+        ok(dg_load_capture(c, k, k ? DG_IQ_CI8 : DG_IQ_C64, y.data(), y.data(), n, 0), "dg_load_capture");
+        windows(1);
+    }
+    ok(dg_load_capture(c, 1, DG_IQ_C64, y.data(), y.data(), n, 0), "dg_load_capture");
+    windows(1);
     ok(dg_graph_capture(c, cost, 20.0, 60.0), "dg_graph_capture");
     growth("windows beside a graph", windows);
     ok(dg_graph_launch(c), "dg_graph_launch");
