@@ -33,7 +33,7 @@ __all__ = [
     "DG_K_CDFT_PLAN", "DG_K_CDFT_CONTRACT", "DG_K_CDFT_COMBINE",
     "dg_nn_conv3x3_forward", "dg_nn_conv3x3_backward", "dg_nn_relu_forward", "dg_nn_relu_backward",
     "dg_nn_bce_logits", "dg_nn_adam", "dg_nn_last_error", "dg_coarse_step", "DG_K_COARSE",
-    "dg_nn_conv3x3_forward_tc", "dg_nn_conv3x3_backward_tc", "dg_nn_tc_check",
+    "dg_nn_conv3x3_forward_tc", "dg_nn_conv3x3_backward_tc", "dg_nn_forward_tc", "dg_nn_tc_check",
 ]
 
 DG_OK, DG_EINVAL, DG_ENOMEM, DG_ECUDA, DG_ESTATE, DG_ETIMEOUT, DG_EUNSUPPORTED = range(7)
@@ -466,6 +466,14 @@ def _stream(stream, t):
     return C.c_void_p(s.cuda_stream)
 
 
+def _floats(shape, t, stream):
+    """Uninitialised floats on t's device that belong to the stream of the call: freed
+    on return, they are not handed out again before its kernels are done with them."""
+    import torch
+    with torch.cuda.stream(stream):  # None: the current stream
+        return torch.empty(shape, dtype=torch.float32, device=t.device)
+
+
 def dg_nn_conv3x3_forward(x, w, b, y, stream=None):
     """y = conv3x3(x, w) + b (NCHW; w: Co x Ci x 3 x 3)."""
     _f32(x, w, b, y)
@@ -480,14 +488,13 @@ def dg_nn_conv3x3_forward(x, w, b, y, stream=None):
 def dg_nn_conv3x3_backward(x, w, dy, dx, dw, db, scratch=None, stream=None):
     """Gradients of sum(dy * conv3x3(x, w, b)): dx (None: skipped), dw, db.
     scratch: dg_nn_conv3x3_scratch floats (allocated here when None)."""
-    import torch
     B, Ci, H, W = x.shape
     Co = w.shape[0]
     need = int(lib().dg_nn_conv3x3_scratch(B, Ci, Co, H, W))
     if need < 0:
         raise ValueError("dg_nn_conv3x3_backward: shape out of range")
     if scratch is None:
-        scratch = torch.empty(max(1, need), dtype=torch.float32, device=x.device)
+        scratch = _floats(max(1, need), x, stream)
     _f32(x, w, dy, dx, dw, db, scratch)
     if (tuple(dy.shape) != (B, Co, H, W) or tuple(dw.shape) != (Co, Ci, 3, 3) or tuple(db.shape) != (Co,)
             or (dx is not None and tuple(dx.shape) != tuple(x.shape)) or scratch.numel() < need):
@@ -500,14 +507,13 @@ def dg_nn_conv3x3_forward_tc(x, w, b, y, scratch=None, stream=None, relu=False):
     """dg_nn_conv3x3_forward on the tensor cores: BF16 operands, FP32 sums;
     scratch: dg_nn_conv3x3_tc_scratch floats (allocated here when None).
     relu: y = max(y, 0) in the same pass."""
-    import torch
     B, Ci, H, W = x.shape
     Co = w.shape[0]
     need = int(lib().dg_nn_conv3x3_tc_scratch(B, Ci, Co, H, W))
     if need < 0:
         raise ValueError("dg_nn_conv3x3_forward_tc: shape out of range")
     if scratch is None:
-        scratch = torch.empty(max(1, need), dtype=torch.float32, device=x.device)
+        scratch = _floats(max(1, need), x, stream)
     _f32(x, w, b, y, scratch)
     if (tuple(w.shape) != (Co, Ci, 3, 3) or tuple(b.shape) != (Co,) or tuple(y.shape) != (B, Co, H, W)
             or scratch.numel() < need):
@@ -520,7 +526,6 @@ def dg_nn_forward_tc(x, params, stream=None):
     """The output of a network's convolutions on the tensor cores (params: its
     layers' (w, b), relu between them) in one call, or None where that call does
     not take the shape (the layers one by one say why)."""
-    import torch
     B, _, H, W = x.shape
     n = len(params)
     ch = (C.c_int32 * (n + 1))(*([x.shape[1]] + [w.shape[0] for w, _ in params]))
@@ -528,8 +533,8 @@ def dg_nn_forward_tc(x, params, stream=None):
     if need < 0 or any(tuple(w.shape) != (ch[k + 1], ch[k], 3, 3) or tuple(b.shape) != (ch[k + 1],)
                        for k, (w, b) in enumerate(params)):
         return None
-    y = torch.empty((B, ch[n], H, W), dtype=torch.float32, device=x.device)
-    scratch = torch.empty(max(1, need), dtype=torch.float32, device=x.device)
+    y = _floats((B, ch[n], H, W), x, stream)
+    scratch = _floats(max(1, need), x, stream)
     _f32(x, y, scratch, *(t for p in params for t in p))
     ws, bs = ((C.c_void_p * n)(*(p[k].data_ptr() for p in params)) for k in (0, 1))
     _nn_check(lib().dg_nn_forward_tc(_ptr(x), ws, bs, ch, n, _ptr(y), B, H, W, _ptr(scratch), _stream(stream, x)))
@@ -539,14 +544,13 @@ def dg_nn_forward_tc(x, params, stream=None):
 def dg_nn_conv3x3_backward_tc(x, w, dy, dx, dw, db, scratch=None, stream=None):
     """dg_nn_conv3x3_backward on the tensor cores: BF16 operands, FP32 sums;
     scratch: dg_nn_conv3x3_tc_scratch floats (allocated here when None)."""
-    import torch
     B, Ci, H, W = x.shape
     Co = w.shape[0]
     need = int(lib().dg_nn_conv3x3_tc_scratch(B, Ci, Co, H, W))
     if need < 0:
         raise ValueError("dg_nn_conv3x3_backward_tc: shape out of range")
     if scratch is None:
-        scratch = torch.empty(max(1, need), dtype=torch.float32, device=x.device)
+        scratch = _floats(max(1, need), x, stream)
     _f32(x, w, dy, dx, dw, db, scratch)
     if (tuple(dy.shape) != (B, Co, H, W) or tuple(dw.shape) != (Co, Ci, 3, 3) or tuple(db.shape) != (Co,)
             or (dx is not None and tuple(dx.shape) != tuple(x.shape)) or scratch.numel() < need):
@@ -577,10 +581,9 @@ def dg_nn_relu_backward(z, dh, dz, stream=None):
 def dg_nn_bce_logits(z, t, pos_weight, grad, loss, scratch=None, stream=None):
     """Mean weighted BCE on logits into loss (1 float) and its gradient into
     grad; scratch: dg_nn_bce_scratch(n) floats (allocated here when None)."""
-    import torch
     n = z.numel()
     if scratch is None:
-        scratch = torch.empty(max(1, int(lib().dg_nn_bce_scratch(n))), dtype=torch.float32, device=z.device)
+        scratch = _floats(max(1, int(lib().dg_nn_bce_scratch(n))), z, stream)
     _f32(z, t, grad, loss, scratch)
     if not (t.numel() == n == grad.numel()) or loss.numel() < 1 or scratch.numel() < lib().dg_nn_bce_scratch(n):
         raise ValueError("dg_nn_bce_logits: size mismatch")

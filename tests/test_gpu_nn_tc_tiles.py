@@ -69,3 +69,29 @@ def test_network_in_one_call_is_its_layers_one_by_one(channels, shape):
     P.dg_nn_tc_check()
     assert torch.equal(y, h)
     assert torch.equal(net.forward(x, keep=True), h)
+
+
+def _network():
+    from paper_2508_06672_gb300.proposal import ProposalNet
+    torch = torch_cuda()
+    net = ProposalNet([20, 32, 64, 32, 1], seed=5, tc=True)
+    x = torch.randn(1, 20, 129, 150, generator=torch.Generator(device="cuda").manual_seed(6), device="cuda")
+    return torch, package(), net, x
+
+
+def test_network_on_a_stream_of_its_own():
+    """The call on another stream than the current one: its scratch and output belong
+    to that stream, so nothing allocated meanwhile takes their place before the
+    kernels, held up behind other work, have run."""
+    torch, P, net, x = _network()
+    ref = P.dg_nn_forward_tc(x, net.params)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(50_000_000)
+    y = P.dg_nn_forward_tc(x, net.params, stream=s)
+    held = [torch.full((n,), float("nan"), device="cuda") for n in (1 << 14, 1 << 17, 1 << 20, 1 << 21, 1 << 22) for _ in range(3)]
+    torch.cuda.current_stream().synchronize()
+    s.synchronize()
+    assert torch.equal(y, ref)
+    del held
