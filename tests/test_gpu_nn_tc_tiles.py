@@ -95,3 +95,26 @@ def test_network_on_a_stream_of_its_own():
     s.synchronize()
     assert torch.equal(y, ref)
     del held
+
+
+def test_network_under_capture():
+    """The network's launches, each let in before the one before it ends, recorded
+    in a graph: replays give the call's output, also on new inputs."""
+    torch, P, net, x = _network()
+    g = torch.cuda.CUDAGraph()
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        for _ in range(2):
+            net.forward(x)
+    torch.cuda.current_stream().wait_stream(s)
+    with torch.cuda.graph(g):
+        y = net.forward(x)
+    for seed in (6, 7, 8):
+        x.copy_(torch.randn(x.shape, generator=torch.Generator(device="cuda").manual_seed(seed), device="cuda"))
+        y.zero_()
+        for _ in range(3):
+            g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y, net.forward(x))
+    P.dg_nn_tc_check()
