@@ -987,7 +987,8 @@ static void sort_args(dg_ctx *c, const CdftLayout::Batch &bt, const CdftLayout &
 // with integer delays: where few candidates share a lag. k_corr_lag takes a warp
 // per group however few candidates it has, 5.1e-6 us per group and sample on 152
 // SMs; the tile kernel takes a CTA per rows x 256 candidates, on widely spread lags
-// 0.145 us per tile of an SM and sample plus 0.1, 0.36 at least (tiles of 8 rows;
+// 0.145 us per tile of an SM and sample plus 0.1, 0.36 at least (tiles of 8 rows,
+// whatever dg_options.rows asks for: a surface is the same bits for every value;
 // lower envelopes of what it took, so that no grid is slower than on its tiles).
 // Measured, grouped against tiles, by candidates per group: 401^2 nodes and 16
 // snapshots of 16384 samples 7.2 against 19.0 ms (46), 10.7 / 26.2 (25), 24.8 / 26.0
@@ -1031,11 +1032,10 @@ static bool tiles_faster(const dg_ctx *c, const GridDev &gd, LagRule &rule)
         const double lags = (hi - lo) * c->fs / kC + 1.0;
         groups += 0.88 * (lags * -std::expm1(-G / lags) + G / kDirectGroup);  // the lags that hold a candidate
     }
-    const int rows = c->opt.rows ? c->opt.rows : 8;
-    const double tiles = std::ceil(g.nlat / (8.0 * rows)) * std::ceil(g.nlon / 32.0) * c->K / c->sm_count;
+    const double tiles = std::ceil(g.nlat / 64.0) * std::ceil(g.nlon / 32.0) * c->K / c->sm_count;
     rule.g = g;
     rule.known = true;
-    rule.tiles = groups * 5.1e-6 * 152.0 / c->sm_count > std::max(0.36, 0.1 + 0.145 * tiles) * rows / 8.0;
+    rule.tiles = groups * 5.1e-6 * 152.0 / c->sm_count > std::max(0.36, 0.1 + 0.145 * tiles);
     return rule.tiles;
 }
 

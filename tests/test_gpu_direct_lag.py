@@ -129,3 +129,18 @@ def test_lag_slots_of_grids_around_a_pole(lat, grid, turns):
     assert fix["refine_n"] == 21
     g.close()
     _check(s, c)
+
+
+@pytest.mark.parametrize("spacing", [2500.0, 4000.0, 7000.0, 12000.0, 20000.0])
+def test_rows_do_not_choose_the_kernel(spacing):
+    """Grids on both sides of the rule: one surface for every dg_options.rows."""
+    s = sim.make_scene(formation=sim.Formation(sep_m=200e3), seed=66, fs_hz=60e6, n_samples=3000, k_steps=8, fmt="ci8",
+                       waveform="noise", snr_db=-3.0, grid_n=101, grid_spacing_m=spacing, bw_hz=40e6)
+    surfs, launches = [], []
+    for rows in (0, 4, 8, 16):
+        g, c = gpu_surface(s, rows=rows)
+        surfs.append(c)
+        launches.append(_launches(g))
+        g.close()
+    assert len(set(launches)) == 1
+    assert all(np.array_equal(c, surfs[0]) for c in surfs[1:])
