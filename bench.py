@@ -567,10 +567,11 @@ def run_dg(a, rank, world, local_rank):
             "data": "synthetic",
             "config": {"workload": desc, "G": G_rank * world, "K": scene.k_steps, "N": scene.n_samples,
                        "fmt": scene.fmt, "delay": "integer", "algo": a.algo, "acc": "power",
+                       # delay-Doppler tables have no chunk, contraction or tiles
                        "chunk": ((a.chunk if a.chunk else f"auto: {chunk_lo}..{chunk_hi}" if chunk_lo != chunk_hi
-                                  else f"auto: {chunk_hi}") if a.algo == "cdft" else None),
-                       "contract": a.contract if a.algo == "cdft" else None,
-                       "tiles": a.tiles if a.algo == "cdft" else None,
+                                  else f"auto: {chunk_hi}") if a.algo == "cdft" and not maps else None),
+                       "contract": ("none: FP32 delay-Doppler tables" if maps else a.contract) if a.algo == "cdft" else None,
+                       "tiles": a.tiles if a.algo == "cdft" and not maps else None,
                        "refine": f"{REFINE_SPACING_M:g} m spacing, +-{REFINE_WINDOW_M:g} m",
                        "l2": "flushed between timed steps (256 MB write outside the events)",
                        "parallelism": f"grid rows sharded over {world} GPU(s)", "seed": scene.meta["seed"]},

@@ -80,9 +80,12 @@ enum { DG_PREC_FP32 = 0, DG_PREC_FP64 = 1 };
  * accuracy (DG_CONTRACT_FP32, _BF16X3, _FP16X3), a main grid of at least 8192
  * nodes takes the same interpolation from one table per snapshot instead: the
  * correlation of Eq. 11 at every lag and Doppler bin of the grid's ranges,
- * computed in FP32 through FFTs, in which every candidate interpolates (error
- * about 2e-7 of the surface). A refinement grid of few lags takes a small
- * table summed directly. */
+ * computed in FP32 through FFTs, in which every candidate interpolates. Its
+ * error is about 2e-7 to 4e-7 of the surface (2-norm, up to 7e-7 with 4000
+ * bins); an FFT rounds relative to the energy of its block, so captures with
+ * isolated pulses of 600 times the noise leave a node off by 2e-6 of its own
+ * value (median; 1.5e-5 at 6000 times) where sums of its own products stay at
+ * 1e-6. A refinement grid of few lags takes a small table summed directly. */
 enum { DG_ALGO_DIRECT = 0, DG_ALGO_CDFT = 1 };
 
 /* Tiles of the CDFT tensor-core contraction.
@@ -367,7 +370,12 @@ dg_status dg_batch_destroy(dg_batch *batch);
  * interpolation bound, so the choice changes speed, not the error class.
  * DG_ALGO_DIRECT: the grid rows per thread (dg_options.rows: 4, 8, 16 in
  * FP32, 16 not with LAGRANGE4; 2, 4 in FP64), i.e. the candidates per CTA;
- * the surface is the same, bit for bit, for every value.
+ * the surface is the same, bit for bit, for every value, and where its
+ * candidates are grouped by lag (FP32, INTEGER delay) so is the time.
+ * The CDFT shapes are the contraction's: a context that takes delay-Doppler
+ * tables (chunk 0, DG_TILES_AUTO) leaves them for the shape chosen, which is
+ * slower on every grid measured (6.8 against 81 ms on 4001^2 nodes and 50
+ * snapshots), so it is for programs that want the contraction.
  * It times dg_cost_surface into cost (device, the context's precision; its
  * contents are overwritten) with CUDA events on the context's stream: one
  * untimed run, then reps >= 1 timed runs, keeping the median. The fastest

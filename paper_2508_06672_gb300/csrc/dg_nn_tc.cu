@@ -969,7 +969,7 @@ unsigned *err_word()
 
 // Launch of a kernel that itself waits for the one before it in the stream
 // (griddepcontrol.wait), so that its setup and its launch overlap that one's end: the
-// five layers of the proposal network 145 -> 131 us.
+// five layers of the proposal network 145 -> 132 us.
 template <typename... P, typename... A>
 cudaError_t launch_waiting(void (*kernel)(P...), dim3 grid, int threads, int smem, cudaStream_t s, A... args)
 {

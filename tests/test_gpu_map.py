@@ -224,3 +224,26 @@ def test_tables_of_thousands_of_bins(delay):
     ok &= ref < 10 * np.median(ref)
     assert ok.sum() > 900
     assert np.linalg.norm(c.ravel()[idx][ok] - ref[ok]) < 4e-6 * np.linalg.norm(ref[ok])
+
+
+@pytest.mark.parametrize("fmt,amp", [("ci16", 30000.0), ("c64", 3e5)])
+def test_captures_with_pulses(fmt, amp):
+    """Isolated pulses hundreds and thousands of times the noise, in both captures:
+    an FFT's rounding is relative to the energy of its block, and the surface stays
+    within the FP32 bound."""
+    torch = torch_cuda()
+    P = package()
+    s = _scene(48, 200.0, 20000, k=1, fs=12.5e6, grid=(91, 93))
+    rng = np.random.default_rng(7)
+    y = [rng.normal(0.0, 50.0, (1, 20000, 2)) for _ in range(2)]
+    for q in y:
+        q[0, rng.integers(0, 20000, 20)] = amp
+    y = [np.rint(q).astype(np.int16 if fmt == "ci16" else np.float32) for q in y]
+    g = P.Geolocator(s.grid, s.ephem, s.fs_hz, s.fc_hz, algo="cdft")
+    g.load_captures(fmt, torch.from_numpy(y[0]).cuda(), torch.from_numpy(y[1]).cuda())
+    c = g.cost_surface().double().cpu().numpy().ravel()
+    g.close()
+    idx = np.unique(rng.integers(0, s.G, 1200))
+    ref = oracle.cost_points(s.grid, s.ephem, s.fs_hz, s.fc_hz, oracle.iq_to_f64(y[0]), oracle.iq_to_f64(y[1]), idx=idx)
+    ok = ~lag_boundary_mask(s, idx)
+    assert rel_err(c[idx][ok], ref[ok], 0.01) < FP32_TOL
