@@ -342,6 +342,10 @@ dg_status dg_graph_fix(dg_ctx *ctx, dg_fix *out);
  * for it and writes n fixes (host); a context whose step failed gets
  * index = -1 and the first failure is returned. A context must not be used
  * by other calls while a launch of its batch is in flight.
+ * A DIRECT context (FP32, INTEGER delay) whose candidates share few lags may
+ * group them by lag alone and not in a batch, whose other contexts fill the GPU:
+ * the same values within rounding. While the batch can be launched the
+ * context's own calls go the batch's way, so its fixes equal theirs.
  * When every context runs CDFT on the tensor cores (lag or row tiles) with
  * one capture format and one contraction arithmetic, the contractions of
  * the main surfaces are shared: round r is one persistent launch over the

@@ -100,10 +100,12 @@ struct BatchHold {  // a batch's replays read a context's buffers
     cudaEvent_t last = nullptr;  // recorded behind its latest replay
     uint64_t gen = 0;            // the context's steps_gen that the replays need
     std::atomic<bool> alive{true};
+    double fill = 0.0;           // tiles_faster: tiles per SM of the whole batch
 };
 
 struct LagRule {  // tiles_faster's answer for one grid
     GridDev g{};
+    double fill = 0.0;
     bool known = false, tiles = false;
 };
 
@@ -113,6 +115,7 @@ struct CdftBufs {  // chunked-DFT scratch, grown on demand
     CdftLayout dmain_layout, dloc_layout;  // the direct path's lag groups
     std::list<CdftLayout> kept;            // layouts of other shapes, while a captured step may read their tables
     LagRule dmain_rule, dloc_rule;
+    double fill = 0.0;                     // while a batch is being captured: BatchHold::fill
     uint64_t no_sort = 0;                  // steps_gen at which the sort found no memory
     float2 *part = nullptr;                // and its segments' sums
     size_t part_cap = 0;
@@ -983,6 +986,12 @@ static void sort_args(dg_ctx *c, const CdftLayout::Batch &bt, const CdftLayout &
     a.ngroups = (int)bt.groups;
 }
 
+// Tiles per SM of a whole grid and all snapshots (k_corr_direct at 8 rows a thread).
+static double grid_tiles(const dg_ctx *c, const GridDev &g)
+{
+    return std::ceil(g.nlat / 64.0) * std::ceil(g.nlon / 32.0) * c->K / c->sm_count;
+}
+
 // Whether the tile kernel (k_corr_direct) is the faster one for an FP32 surface
 // with integer delays: where few candidates share a lag. k_corr_lag takes a warp
 // per group however few candidates it has, 5.1e-6 us per group and sample on 152
@@ -998,14 +1007,23 @@ static void sort_args(dg_ctx *c, const CdftLayout::Batch &bt, const CdftLayout &
 // The groups are estimated from the lags at a lattice of 9 x 9 nodes (0.88 of what an
 // even spread over their range would give, as counted on those grids) of the
 // whole grid, so that every row shard of it takes the same kernel. A refinement
-// grid (gd) is judged as if on the main grid's centre.
+// grid (gd) is judged as if on the main grid's centre. In a batch the other
+// contexts' work fills the SMs that a small grid's tiles leave: a context's tiles
+// then cost their share of the whole batch's (32 contexts of 101^2 nodes, 4
+// snapshots of 16384 samples: 10.2 / 15.7 ms at 15 candidates a group, 33.7 / 22.9 at
+// 3.6, 48.0 / 21.3 at 2.5), and its synchronising calls go the same way while the
+// batch can be launched.
 static bool tiles_faster(const dg_ctx *c, const GridDev &gd, LagRule &rule)
 {
     GridDev g = gd;
     g.row0 = 0;
     g.nrows = g.nlat;
+    const double tiles = grid_tiles(c, g);
+    double fill = std::max(tiles, c->cd.fill);
+    for (const auto &h : c->holds)
+        if (h->alive && h->gen == c->steps_gen) fill = std::max(fill, h->fill);
     const GridDev &o = rule.g;
-    if (rule.known && o.lat0_rad == g.lat0_rad && o.lon0_rad == g.lon0_rad && o.dlat_m == g.dlat_m && o.dlon_m == g.dlon_m &&
+    if (rule.known && rule.fill == fill && o.lat0_rad == g.lat0_rad && o.lon0_rad == g.lon0_rad && o.dlat_m == g.dlat_m && o.dlon_m == g.dlon_m &&
         o.nlat == g.nlat && o.nlon == g.nlon)
         return rule.tiles;
     const int ni = std::min(9, g.nlat), nj = std::min(9, g.nlon);
@@ -1032,10 +1050,10 @@ static bool tiles_faster(const dg_ctx *c, const GridDev &gd, LagRule &rule)
         const double lags = (hi - lo) * c->fs / kC + 1.0;
         groups += 0.88 * (lags * -std::expm1(-G / lags) + G / kDirectGroup);  // the lags that hold a candidate
     }
-    const double tiles = std::ceil(g.nlat / 64.0) * std::ceil(g.nlon / 32.0) * c->K / c->sm_count;
     rule.g = g;
+    rule.fill = fill;
     rule.known = true;
-    rule.tiles = groups * 5.1e-6 * 152.0 / c->sm_count > std::max(0.36, 0.1 + 0.145 * tiles);
+    rule.tiles = groups * 5.1e-6 * 152.0 / c->sm_count > std::max(0.36, 0.1 + 0.145 * fill) * tiles / fill;
     return rule.tiles;
 }
 
@@ -2792,6 +2810,20 @@ dg_status dg_batch_capture(dg_ctx *const *ctxs, int32_t n, void *const *costs, d
     if (!s || s == cudaStreamLegacy || s == cudaStreamPerThread)
         return fail(nullptr, DG_EUNSUPPORTED, "graph capture needs a non-default stream");
     std::vector<int> half((size_t)n);
+    double fill = 0.0;
+    for (int i = 0; i < n; ++i)
+        if (ctxs[i]) fill += grid_tiles(ctxs[i], ctxs[i]->gd);
+    struct Filled {  // the steps below are planned for the whole batch's work
+        dg_ctx *const *ctxs;
+        int n;
+        void set(double f)
+        {
+            for (int i = 0; i < n; ++i)
+                if (ctxs[i]) ctxs[i]->cd.fill = f;
+        }
+        ~Filled() { set(0.0); }
+    } filled{ctxs, n};
+    filled.set(fill);
     for (int i = 0; i < n; ++i) {
         dg_ctx *c = ctxs[i];
         if (!c || !costs[i]) return fail(nullptr, DG_EINVAL, "context or cost %d is NULL", i);
@@ -2830,6 +2862,7 @@ dg_status dg_batch_capture(dg_ctx *const *ctxs, int32_t n, void *const *costs, d
     for (int i = 0; i < n; ++i) {
         auto h = std::make_shared<BatchHold>();
         h->last = b->last;
+        h->fill = fill;
         h->gen = ctxs[i]->steps_gen;
         b->holds.push_back(h);
         ctxs[i]->holds.push_back(h);

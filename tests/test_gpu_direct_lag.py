@@ -144,3 +144,45 @@ def test_rows_do_not_choose_the_kernel(spacing):
         g.close()
     assert len(set(launches)) == 1
     assert all(np.array_equal(c, surfs[0]) for c in surfs[1:])
+
+
+def test_sparse_lags_in_a_batch():
+    """Small sparse grids group their lags alone, where their tiles leave most SMs
+    idle, and keep the tiles in a batch that fills the GPU; the contexts' own calls
+    follow the batch while it lives."""
+    torch = torch_cuda()
+    P = package()
+    gs, costs, alone = [], [], []
+    for i in range(40):
+        s = sim.make_scene(seed=70 + i % 4, fs_hz=20e6, n_samples=2048, k_steps=4, fmt="ci8", waveform="noise", snr_db=-3.0,
+                           grid_n=(101, 103), grid_spacing_m=8000.0, bw_hz=16e6)
+        g = P.Geolocator(s.grid, s.ephem, s.fs_hz, s.fc_hz, stream=torch.cuda.Stream())
+        y1, y2 = torch.from_numpy(s.y1).cuda(), torch.from_numpy(s.y2).cuda()
+        torch.cuda.synchronize()
+        g.load_captures(s.fmt, y1, y2)
+        gs.append(g)
+        costs.append(torch.empty((g.nrows, g.nlon), dtype=g.dtype, device=g.device))
+
+    def own(g):
+        with torch.cuda.stream(g.stream):
+            n = _launches(g)
+            c = g.cost_surface()
+            fix = g.argmax_refine(c, 100.0, 1000.0)
+        return n, fix, c.double().cpu().numpy()
+
+    torch.cuda.synchronize()
+    alone = [own(g) for g in gs[:4]]
+    assert all(n > 2 for n, _, _ in alone)
+    b = P.Batch(gs, costs, 100.0, 1000.0)
+    b.launch()
+    fixes = b.fixes()
+    for i in range(4):
+        n, fix, c = own(gs[i])
+        assert n == 2 and fix == fixes[i]
+        assert np.array_equal(costs[i].double().cpu().numpy(), c)
+        assert rel_err(c, alone[i][2], 0.01) < 2 * FP32_TOL
+    b.close()
+    n, fix, c = own(gs[0])
+    assert n == alone[0][0] and fix == alone[0][1] and np.array_equal(c, alone[0][2])
+    for g in gs:
+        g.close()
